@@ -20,6 +20,7 @@
 #include "dbt_fused.cuh"
 #include "dbt_gemm_tc.cuh"
 #include "dbt_gemm_persist.cuh"
+#include "dbt_gemm_prompt.cuh"
 #include "dbt_kernels.cuh"
 
 using namespace dbt;
@@ -100,6 +101,7 @@ struct dbt_model {
     int cur_rows;          // primary rows (sequences x positions) of the launch plan being built
     bool moe_fuse_swiglu;  // the persistent per-expert gate|up launch applies the SwiGLU itself (DBT_MOE_FUSE_SWIGLU=0: a kernel of its own)
     bool prompt_fuse_swiglu;  // prompt chunks: SwiGLU in the gate|up GEMM's epilogue (DBT_PROMPT_FUSE_SWIGLU=0: a kernel of its own)
+    bool prompt_pairs;        // prompt chunks on the paired-SM GEMMs (dense bf16 chain)
     bool prompt_attn_off;  // DBT_PROMPT_ATTN=tile: prompt chunks through the 16-row kernel's packed tiles (the earlier form)
     bool fuse_qkv;     // decode steps: the attention kernel does the Q|K|V epilogue itself (DBT_FUSE_QKV=0 keeps the kernel)
     int num_sms;
@@ -258,7 +260,8 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
         w.P_floats = want < cap ? want : cap;
         if (w.P_floats < (size_t)Rmax * widest) w.P_floats = (size_t)Rmax * widest;
         w.P = k.take<float>(w.P_floats);
-        w.ss = k.take<float>((size_t)((d + 127) / 128) * Rmax);
+        // shares of sum(S^2): 256 columns each in decode steps, half a 256-feature tile in prompt chunks
+        w.ss = k.take<float>((size_t)((d + 255) / 256 * 2) * Rmax);
         if (moe) {
             size_t Rk = (size_t)Rmax * kmax_of(c);
             w.Xs = k.take<__nv_bfloat16>(2 * Rk * d);
@@ -1318,6 +1321,130 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
     return DBT_OK;
 }
 
+// ---- prompt chunks of dense bf16 models: paired-SM GEMMs with their epilogues -----------------------
+
+// The 3-D one-box view of a two-plane GEMM input, built on first use.
+const CUtensorMap *act_view(dbt_model *m, const CUtensorMap *X, int box_rows, int K) {
+    auto reg = m->act_base.find(X);
+    if (reg == m->act_base.end()) return nullptr;
+    auto key = std::make_tuple(X, box_rows, m->Rmax);
+    auto hit = m->act3d.find(key);
+    if (hit == m->act3d.end()) {
+        CUtensorMap t;
+        if (!make_act_map(&t, reg->second.base, (uint64_t)m->Rmax, (uint64_t)K, box_rows)) return nullptr;
+        hit = m->act3d.emplace(key, t).first;
+    }
+    return &hit->second;
+}
+
+template <int N, int MODE>
+dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *const (&W)[3], const CUtensorMap *X, const PgParams &p,
+                              double bytes) {
+    const int pairs = m->num_sms / 2, grid = 2 * (p.tiles < pairs ? p.tiles : pairs);
+    LAUNCH(m, tag, bytes, (gemm_prompt_kernel<N, MODE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *W[0], *W[1], *W[2], *X, p);
+    return DBT_OK;
+}
+
+// One GEMM of a prompt chunk.  p carries the epilogue's operands; n_out the features of up to three matrices
+// (PG_GATEUP: of the gate matrix, the up matrix has as many).
+template <int MODE>
+dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
+                           const int (&n_out)[3], int nseg, const CUtensorMap *X, int K, int R, PgParams p) {
+    constexpr int N = 256, kTileF = MODE == PG_GATEUP ? N / 2 : N;
+    const CUtensorMap *x = act_view(m, X, 128, K);
+    if (!x) return fail(m, DBT_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", tag);
+    p.K = K;
+    p.R = R;
+    p.m_tiles = (R + kPgM - 1) / kPgM;
+    p.nseg = nseg;
+    int nt = 0, col = 0;
+    double bytes = 0;
+    for (int s = 0; s < nseg; s++) {
+        p.seg[s] = PgSeg{nt, n_out[s], col};
+        col += n_out[s];
+        nt += (n_out[s] + kTileF - 1) / kTileF;
+        bytes += (double)n_out[s] * K * 2 * (MODE == PG_GATEUP ? 2 : 1);
+    }
+    p.tiles = nt * p.m_tiles;
+    p.status = m->ws.status;
+    const CUtensorMap *const W[3] = {W0, W1 ? W1 : W0, W2 ? W2 : W0};
+    return launch_gemm_prompt<N, MODE>(m, tag, W, x, p, bytes);
+}
+
+// One chunk of a prompt through all layers: five kernels per layer.
+dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
+    typedef __nv_bfloat16 WT;
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const int R = rm.B * rm.cn, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ff;
+    const size_t pool_layer_elems = (size_t)2 * c.num_pages * c.n_kv_heads * c.page_size * c.head_dim;
+    const size_t lo_x = (size_t)m->Rmax * d, lo_h = (size_t)m->Rmax * F;
+    double kv_bytes = 0;
+    for (int b = 0; b < rm.B; b++)
+        for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * sizeof(WT);
+    dbt_status st;
+    int ss_tiles = wide_ss_tiles(m);  // the embedding kernel's; the residual epilogues leave two shares per feature tile
+    const int ss_next = 2 * ((d + 255) / 256);
+    auto base = [&] {
+        PgParams p{};
+        p.ss_in = w.ss;
+        p.ss_tiles = ss_tiles;
+        p.ss_ld = m->Rmax;
+        p.d_norm = d;
+        p.eps = c.rms_eps;
+        return p;
+    };
+    auto resid = [&](const float *g_next) {
+        PgParams p{};
+        p.S = w.S;
+        p.g_next = g_next;
+        p.X = w.Xb;
+        p.x_lo = lo_x;
+        p.ss_out = w.ss;
+        p.ss_ld = m->Rmax;
+        p.d = d;
+        return p;
+    };
+    for (int l = 0; l < c.n_layers; l++) {
+        const dbt_layer_weights &lw = m->layers[l];
+        const LayerMaps &mp = m->maps[l];
+        PgParams q = base();
+        q.Q = w.Q;
+        q.B = rm.B; q.cn = rm.cn; q.dh = c.head_dim; q.n_q = c.n_q_heads; q.n_kv = c.n_kv_heads;
+        q.num_pages = c.num_pages; q.pt_stride = m->pages_per_seq_max;
+        q.rope = w.rope; q.seq_len = w.seq_len; q.page_table = w.page_table;
+        q.kpool = reinterpret_cast<WT *>(m->kv_pool) + (size_t)l * pool_layer_elems;
+        q.vpool = q.kpool + pool_layer_elems / 2;
+        if ((st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, R, q)) != DBT_OK) return st;
+        st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, 0, l, kv_bytes, nullptr, true, false)
+                               : run_attention_mma<64>(m, rm, 0, l, kv_bytes, nullptr, true, false);
+        if (st != DBT_OK) return st;
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, resid(lw.mlp_norm_g))) != DBT_OK)
+            return st;
+        ss_tiles = ss_next;
+        if (m->prompt_fuse_swiglu) {
+            PgParams g = base();
+            g.H = w.Hb;
+            g.h_lo = lo_h;
+            g.F = F;
+            st = run_gemm_prompt<PG_GATEUP>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, 0, 0}, 1, &m->map_Xb, d, R, g);
+        } else {
+            PgParams g{};
+            g.P = w.P;
+            g.ldp = 2 * F;
+            st = run_gemm_prompt<PG_STORE>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, F, 0}, 2, &m->map_Xb, d, R, g);
+            if (st == DBT_OK)
+                LAUNCH(m, "swiglu_couple", 0, swiglu_rows_kernel, dim3(R, (F + 1023) / 1024), 256, 0, w.P, 1, (size_t)0, F, w.Hb, lo_h,
+                       (const float *)w.ss, ss_tiles, m->Rmax, d, c.rms_eps);
+        }
+        if (st != DBT_OK) return st;
+        const float *g_next = l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr);
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R, resid(g_next))) != DBT_OK)
+            return st;
+    }
+    return DBT_OK;
+}
+
 dbt_status run_head_wide(dbt_model *m, const RowMap &rm, int grouped, int n_tile) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
@@ -1387,7 +1514,8 @@ dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, f
         RowMap rm{B, cn};
         int R = B * cn, n_tile = pad_rows(R < 256 ? R : 256);
         if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, n_tile)) != DBT_OK) return st;
-        if ((st = run_layers_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
+        const bool pairs = m->prompt_pairs && cn > 1 && R > 256;
+        if ((st = pairs ? run_layers_prompt(m, rm) : run_layers_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
         if (last_logits && p0 + cn >= n) {
             if ((st = run_head_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
             CUDA_TRY(m, cudaMemcpyAsync(last_logits, w.Z, sizeof(float) * (size_t)B * c.vocab, cudaMemcpyDeviceToDevice,
@@ -1413,6 +1541,14 @@ bool allow_smem_all() {
                cudaSuccess &&
            cudaFuncSetAttribute(gemm_tc_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<64, 2>::kSmemBytes) ==
                cudaSuccess;
+}
+
+template <int N, int MODE>
+bool allow_smem_pg() {
+    return cudaFuncSetAttribute(gemm_prompt_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PgCfg<N>::kSmemBytes) == cudaSuccess;
+}
+bool allow_smem_prompt() {
+    return allow_smem_pg<256, PG_STORE>() && allow_smem_pg<256, PG_QKV>() && allow_smem_pg<256, PG_RESID>() && allow_smem_pg<256, PG_GATEUP>();
 }
 
 // Build the TMA descriptors of a bf16 model.  Returns false when the path cannot be used.
@@ -1494,6 +1630,7 @@ bool setup_tc(dbt_model *m) {
     // Default chain of a dense bf16 model: the RMSNorm factor is applied after the GEMM, so no kernel
     // reduces over a whole row.
     m->wide = ok && m->att_fast && !moe;
+    m->prompt_pairs = m->wide && allow_smem_prompt();
     m->act_parts = 2;
     return ok;
 }

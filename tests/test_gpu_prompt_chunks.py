@@ -1,0 +1,58 @@
+"""GPU: prompt chunks at the edges of the paired-SM GEMMs' 256 x 256 tiles and of the prompt attention's 128-row query
+and 128-key tiles, against the oracle's position-by-position primary pass."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import assert_logits_close, make_gpu_model
+from paper_2608_12385_b200.inputs import ModelConfig, make_tokens, make_weights
+
+pytestmark = pytest.mark.gpu
+
+
+def cfg_of(**kw):
+    base = dict(d_model=256, n_layers=2, n_q_heads=8, n_kv_heads=2, head_dim=64, d_ff=712, vocab=500, weight_dtype="bf16")
+    base.update(kw)
+    return ModelConfig(**base)
+
+
+@pytest.mark.parametrize("cfg,B,n,past", [
+    (cfg_of(), 1, 257, 0),                                       # one row past a row tile
+    (cfg_of(), 1, 512, 0),                                       # whole row tiles, whole key tiles
+    (cfg_of(), 2, 300, 0),                                       # a row tile that spans two sequences
+    (cfg_of(), 1, 300, 133),                                     # behind a cached prefix that ends inside a page
+    (cfg_of(d_model=328, d_ff=1032), 1, 385, 0),                 # ragged feature tiles in every matrix
+    (cfg_of(n_q_heads=2, n_kv_heads=2), 1, 400, 0),              # one head per KV head: 128 positions per query tile
+    (cfg_of(n_q_heads=16, n_kv_heads=2, n_layers=1), 3, 130, 1),  # eight heads per KV head: 16 positions per query tile
+    (cfg_of(n_q_heads=4, n_kv_heads=2, head_dim=128, n_layers=1), 1, 650, 0),
+])
+def test_prompt_chunk_edges_match_the_oracle(cfg, B, n, past):
+    w = make_weights(cfg, seed=91, matrix_std=0.05)
+    total = past + n
+    tok = make_tokens(cfg, B, total, seed=92)
+    om = oracle.OracleModel(cfg, w, B, total)
+    gm = make_gpu_model(cfg, w, B, total)
+    want = om.prefill(tok.numpy())
+    if past:
+        gm.prefill(tok[:, :past].cuda().contiguous())
+    # logits are the last position's own pass; n - 1 positions go through as one chunk
+    got = gm.prefill(tok[:, past:].cuda().contiguous(), want_logits=True)
+    assert_logits_close(got, want, "bf16", "prompt logits")
+    k_dev, v_dev = gm.export_kv(B, total)
+    # bf16 storage (2^-9 relative) on top of the logit-level error of fp32 sums
+    np.testing.assert_allclose(k_dev.float().numpy(), om.k_cache[:, :B, :total], rtol=2.0 ** -8, atol=5e-3)
+    np.testing.assert_allclose(v_dev.float().numpy(), om.v_cache[:, :B, :total], rtol=2.0 ** -8, atol=5e-3)
+    assert gm.sync_status() == (0, 0)
+
+
+def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
+    """Pages past the last key hold whatever the pool held before; NaN there must change nothing."""
+    cfg = cfg_of()
+    w = make_weights(cfg, seed=93, matrix_std=0.05)
+    tok = make_tokens(cfg, 1, 333, seed=94).cuda().contiguous()
+    a, b = make_gpu_model(cfg, w, 1, 512), make_gpu_model(cfg, w, 1, 512)
+    b.kv_pool.fill_(float("nan"))
+    za, zb = a.prefill(tok, want_logits=True), b.prefill(tok, want_logits=True)
+    assert torch.equal(za, zb) and torch.isfinite(za).all()
+    assert torch.equal(a.export_kv(1, 333)[0], b.export_kv(1, 333)[0])
