@@ -88,6 +88,10 @@ struct dbt_model {
     bool tc;
     std::vector<LayerMaps> maps;
     CUtensorMap map_lm, map_Xb, map_Ob, map_Hb, map_kv, map_Xs, map_Hs;
+    CUtensorMap map_pq, map_pkv;  // prompt attention: queries, pages
+    // prompt chunks take attn_prompt_kernel (bf16 queries, see prompt_q); off for head ratios that do not divide 16 and by
+    // DBT_PROMPT_ATTN=tile: the 16-row kernel's packed tiles
+    bool prompt_attn_tc;
     bool moe_tc;  // MoE experts on the tensor cores
     bool att_fast;  // TMA + mma.sync attention over the bf16 pool
     bool wide;      // dense bf16: RMSNorm factor applied after the GEMM, no row-wide reduction kernel
@@ -101,8 +105,6 @@ struct dbt_model {
     int cur_rows;          // primary rows (sequences x positions) of the launch plan being built
     bool moe_fuse_swiglu;  // the persistent per-expert gate|up launch applies the SwiGLU itself (DBT_MOE_FUSE_SWIGLU=0: a kernel of its own)
     bool prompt_fuse_swiglu;  // prompt chunks: SwiGLU in the gate|up GEMM's epilogue (DBT_PROMPT_FUSE_SWIGLU=0: a kernel of its own)
-    bool prompt_pairs;        // prompt chunks on the paired-SM GEMMs (dense bf16 chain)
-    bool prompt_attn_off;  // DBT_PROMPT_ATTN=tile: prompt chunks through the 16-row kernel's packed tiles (the earlier form)
     bool fuse_qkv;     // decode steps: the attention kernel does the Q|K|V epilogue itself (DBT_FUSE_QKV=0 keeps the kernel)
     int num_sms;
     int act_parts;  // 2: GEMM inputs carried as hi + lo bf16 terms (the operator-level GEMM entry uses 1: plain bf16)
@@ -596,10 +598,6 @@ struct TcCall {
     // *fused tells the caller whether it did
     const SwigluEpi *swiglu;
     bool *fused;
-    // dense gate|up launch over a prompt chunk: gate and up tiles of the same features in one CTA, SwiGLU in the
-    // epilogue (see GuEpi); *gu_fused tells the caller whether it was taken
-    const GuEpi *gu;
-    bool *gu_fused;
 };
 
 int norm_threads(int d) { return d >= 1024 ? 1024 : d >= 512 ? 512 : 256; }
@@ -697,9 +695,6 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
         if (16 * w2 < 10 * w1) mt = 2;
     }
     if (c.grp_cnt && c.grp_mt2 && n_tile == 64) mt = 2;
-    const bool gu_pair = !c.grp_cnt && c.R > 256 && c.gu && c.gu_fused && c.nseg == 2 && c.n_out[0] == c.n_out[1] && c.n_out[0] % 8 == 0 &&
-                         m->prompt_fuse_swiglu;
-    if (gu_pair) mt = 2;
     for (int s = 0; s < c.nseg; s++) {
         p.seg[s] = TcSeg{tiles, c.n_out[s], c.rows[s], col};
         tiles += (c.n_out[s] + kTcM * mt - 1) / (kTcM * mt);
@@ -707,14 +702,6 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
         if (!c.grp_cnt) bytes += (double)c.n_out[s] * c.K * 2;  // per-expert launches: the loaded set is known on the device only
     }
     p.nseg = c.nseg;
-    if (gu_pair) {  // tiles of 128 features, each with its gate and its up rows
-        p.seg[0] = TcSeg{0, c.n_out[0], c.rows[0], 0};
-        p.nseg = 1;
-        tiles = (c.n_out[0] + kTcM - 1) / kTcM;
-        p.gu = *c.gu;
-        p.gu.on = 1;
-        *c.gu_fused = true;
-    }
     p.K = c.K;
     p.ldp = col;
     p.R = c.R;
@@ -781,6 +768,11 @@ bool attn_deep(const dbt_model *m, int items) {
     return paths_of(c) * G <= 8 && 2 * pairs > m->num_sms && pairs <= m->num_sms;
 }
 
+// Queries of a prompt chunk as the prompt attention kernel reads them: bf16 [rows][q_dim] in the memory of Q, times
+// log2(e) / sqrt(d_h) (nullptr: that kernel is not used and Q is fp32).
+__nv_bfloat16 *prompt_q(const dbt_model *m) { return m->prompt_attn_tc ? reinterpret_cast<__nv_bfloat16 *>(m->ws.Q) : nullptr; }
+float prompt_q_scale(const dbt_model *m) { return kLog2e / sqrtf((float)m->cfg.head_dim); }
+
 // The attention work split of a decode step, once for all its layers.
 dbt_status run_attention_plan(dbt_model *m, const RowMap &rm) {
     const dbt_config &c = m->cfg;
@@ -833,10 +825,8 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
     }
     // prompt chunks: 16 / G consecutive positions of a sequence share a query tile (the 16-row kernel)
     const bool packed = pack_prompt && !grouped && !qf && rm.cn > 1;
-    if (packed && 16 % G == 0 && !m->prompt_attn_off) {
-        // the prompt kernel: eight query tiles per CTA share every page the CTA brings in
+    if (packed && m->prompt_attn_tc) {
         PromptAttnParams q{};
-        q.Q = w.Q;
         q.B = rm.B;
         q.cn = rm.cn;
         q.G = G;
@@ -844,14 +834,15 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
         q.num_pages = c.num_pages;
         q.pt_stride = m->pages_per_seq_max;
         q.k_row0 = p.k_row0;
+        q.v_row0 = p.k_row0 + plane;
         q.page_table = w.page_table;
         q.seq_len = w.seq_len;
         q.Ob = w.Ob;
         q.lo_off = p.lo_off;
         q.status = w.status;
-        q.nqb = (rm.cn + kPaWarps * (16 / G) - 1) / (kPaWarps * (16 / G));
+        q.nqb = (rm.cn + 256 / G - 1) / (256 / G);
         dim3 gp(rm.B * c.n_kv_heads * q.nqb);
-        LAUNCH(m, "attention", kv_bytes, attn_prompt_kernel<DH>, gp, (kPaWarps + 1) * 32, PromptAttCfg<DH>::kSmemBytes, m->map_kv, q);
+        LAUNCH(m, "attention", kv_bytes, attn_prompt_kernel<DH>, gp, kPaThreads, PromptAttCfg<DH>::kSmemBytes, m->map_pq, m->map_pkv, q);
         return DBT_OK;
     }
     if (packed) {
@@ -879,6 +870,90 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
     return DBT_OK;
 }
 
+// ---- GEMMs of prompt chunks on pairs of SMs (dbt_gemm_prompt.cuh) -----------------------------------------
+
+// The 3-D one-box view of a two-plane GEMM input, built on first use.
+const CUtensorMap *act_view(dbt_model *m, const CUtensorMap *X, int box_rows, int K) {
+    auto reg = m->act_base.find(X);
+    if (reg == m->act_base.end()) return nullptr;
+    auto key = std::make_tuple(X, box_rows, m->Rmax);
+    auto hit = m->act3d.find(key);
+    if (hit == m->act3d.end()) {
+        CUtensorMap t;
+        if (!make_act_map(&t, reg->second.base, (uint64_t)m->Rmax, (uint64_t)K, box_rows)) return nullptr;
+        hit = m->act3d.emplace(key, t).first;
+    }
+    return &hit->second;
+}
+
+template <int N, int MODE>
+dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *const (&W)[3], const CUtensorMap *X, const PgParams &p,
+                              double bytes) {
+    const int pairs = m->num_sms / 2, grid = 2 * (p.tiles < pairs ? p.tiles : pairs);
+    LAUNCH(m, tag, bytes, (gemm_prompt_kernel<N, MODE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *W[0], *W[1], *W[2], *X, p);
+    return DBT_OK;
+}
+
+// One GEMM of a prompt chunk.  p carries the epilogue's operands; n_out the features of up to three matrices
+// (PG_GATEUP: of the gate matrix, the up matrix has as many).
+template <int MODE>
+dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
+                           const int (&n_out)[3], int nseg, const CUtensorMap *X, int K, int R, PgParams p) {
+    constexpr int N = 256, kTileF = MODE == PG_GATEUP ? N / 2 : N;
+    const CUtensorMap *x = act_view(m, X, 128, K);
+    if (!x) return fail(m, DBT_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", tag);
+    p.K = K;
+    p.R = R;
+    p.m_tiles = (R + kPgM - 1) / kPgM;
+    p.nseg = nseg;
+    int nt = 0, col = 0;
+    double bytes = 0;
+    for (int s = 0; s < nseg; s++) {
+        p.seg[s] = PgSeg{nt, n_out[s], col};
+        col += n_out[s];
+        nt += (n_out[s] + kTileF - 1) / kTileF;
+        bytes += (double)n_out[s] * K * 2 * (MODE == PG_GATEUP ? 2 : 1);
+    }
+    p.tiles = nt * p.m_tiles;
+    p.status = m->ws.status;
+    const CUtensorMap *const W[3] = {W0, W1 ? W1 : W0, W2 ? W2 : W0};
+    return launch_gemm_prompt<N, MODE>(m, tag, W, x, p, bytes);
+}
+
+// The operands of a Q|K|V epilogue for layer l (1/rms, RoPE, queries, cache append).
+PgParams prompt_qkv_params(dbt_model *m, const RowMap &rm, int l, int ss_tiles) {
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const size_t pool_layer_elems = (size_t)2 * c.num_pages * c.n_kv_heads * c.page_size * c.head_dim;
+    PgParams q{};
+    q.ss_in = w.ss; q.ss_tiles = ss_tiles; q.ss_ld = m->Rmax; q.d_norm = c.d_model; q.eps = c.rms_eps;
+    q.Q = w.Q;
+    q.Qb = prompt_q(m);
+    q.q_scale = prompt_q_scale(m);
+    q.B = rm.B; q.cn = rm.cn; q.dh = c.head_dim; q.n_q = c.n_q_heads; q.n_kv = c.n_kv_heads;
+    q.num_pages = c.num_pages; q.pt_stride = m->pages_per_seq_max;
+    q.rope = w.rope; q.seq_len = w.seq_len; q.page_table = w.page_table;
+    q.kpool = reinterpret_cast<__nv_bfloat16 *>(m->kv_pool) + (size_t)l * pool_layer_elems;
+    q.vpool = q.kpool + pool_layer_elems / 2;
+    return q;
+}
+
+// The operands of a residual epilogue that prepares a GEMM input with the gain g_next.
+PgParams prompt_resid_params(dbt_model *m, const float *g_next) {
+    const Workspace &w = m->ws;
+    PgParams p{};
+    p.S = w.S;
+    p.g_next = g_next;
+    p.X = w.Xb;
+    p.x_lo = (size_t)m->Rmax * m->cfg.d_model;
+    p.ss_out = w.ss;
+    p.ss_ld = m->Rmax;
+    p.d = m->cfg.d_model;
+    return p;
+}
+// Shares of sum(S^2) that a residual epilogue leaves per row.
+int prompt_ss_tiles(const dbt_model *m) { return 2 * ((m->cfg.d_model + 255) / 256); }
+
 // MoE sub-layer on the tensor cores (Eq. moe_layer, Eq. moe_budget, Section 4.3).  Rows of both
 // paths are sorted by expert; one grouped GEMM launch covers all experts (blockIdx.z), CTAs of
 // experts nobody selected exit before touching their weights, so each selected expert's
@@ -887,7 +962,7 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
 // consumer of a GEMM on them applies the row's factor itself, and the combine leaves the next layer's
 // input in the same form when it is given that layer's gain g_next.
 dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool record_experts, bool wide,
-                      const float *g_next) {
+                      const float *g_next, int ss_tiles) {
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
@@ -903,7 +978,7 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
     size_t lo_x = m->act_parts == 2 ? (size_t)m->Rmax * d : 0;
     size_t lo_xs = m->act_parts == 2 ? (size_t)Rk * d : 0, lo_hs = m->act_parts == 2 ? (size_t)Rk * Fe : 0;
     const float *ssp = wide ? w.ss : nullptr;
-    const int ss_tiles = (d + 255) / 256, ss_ld = m->Rmax;
+    const int ss_ld = m->Rmax;
     dbt_status st;
     // shared expert(s) on every row of both paths; b couples its hidden state
     const float *Psh = nullptr;
@@ -1072,19 +1147,19 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
         qkv.W[1] = &mp.wk; qkv.n_out[1] = kvd; qkv.rows[1] = Bc;
         qkv.W[2] = &mp.wv; qkv.n_out[2] = kvd; qkv.rows[2] = Bc;
         qkv.nseg = 3; qkv.X = &m->map_Xb; qkv.K = d; qkv.R = Ra; qkv.P = w.P; qkv.P_floats = w.P_floats; qkv.parts = m->act_parts; qkv.lo_row0 = m->Rmax; qkv.tag = "gemm_qkv";
-        if ((st = run_gemm_tc(m, qkv, n_tile, &nsp, &sstride)) != DBT_OK) return st;
+        if (rows_form)
+            st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, Bc,
+                                         prompt_qkv_params(m, rm, l, mss_tiles));
+        else
+            st = run_gemm_tc(m, qkv, n_tile, &nsp, &sstride);
+        if (st != DBT_OK) return st;
         const bool fuse = m->fuse_qkv && m->att_fast && rm.cn == 1;
         QkvFuse qf{w.P, nsp, sstride, mwide ? w.ss : nullptr, mwide ? mss_tiles : 0, mwide ? m->Rmax : 0, lw.coup_a};
-        if (rows_form)
-            LAUNCH(m, "qkv_epilogue", 0, qkv_rows_kernel, dim3(Bc, ((c.n_q_heads + c.n_kv_heads) * (c.head_dim / 8) + 255) / 256), 256, 0,
-                   w.P, nsp, sstride, w.Q, rm, c.n_q_heads, c.n_kv_heads, c.head_dim, w.rope, w.seq_len, w.page_table,
-                   m->pages_per_seq_max, c.num_pages, c.page_size, kpool, vpool, w.status, (const float *)w.ss, mss_tiles, m->Rmax, d,
-                   c.rms_eps);
-        else if (!fuse)
+        if (!rows_form && !fuse)
             LAUNCH(m, "qkv_epilogue", 0, qkv_epilogue_kernel<WT>, dim3(Bc, c.n_q_heads + c.n_kv_heads, branch_blocks(ga)), 64, 0, w.P, nsp, sstride, w.Q, rm, ga, c.n_q_heads,
                    c.n_kv_heads, c.head_dim, lw.coup_a, w.rope, w.seq_len, w.page_table, m->pages_per_seq_max, c.num_pages,
                    c.page_size, kpool, vpool, w.status, mwide ? (const float *)w.ss : (const float *)nullptr, mwide ? mss_tiles : 0,
-                   mwide ? m->Rmax : 0, d, c.rms_eps);
+                   mwide ? m->Rmax : 0, d, c.rms_eps, (__nv_bfloat16 *)nullptr, 0.f);
         if (m->att_fast)
             st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, ga, l, kv_bytes, fuse ? &qf : nullptr, rows_form, m->att_planned)
                                    : run_attention_mma<64>(m, rm, ga, l, kv_bytes, fuse ? &qf : nullptr, rows_form, m->att_planned);
@@ -1096,12 +1171,15 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
         TcCall op{};
         op.W[0] = &mp.wo; op.n_out[0] = d; op.rows[0] = Ra; op.nseg = 1; op.X = &m->map_Ob; op.K = qd; op.R = Ra;
         op.P = w.P; op.P_floats = w.P_floats; op.parts = m->act_parts; op.lo_row0 = m->Rmax; op.tag = "gemm_o";
-        if ((st = run_gemm_tc(m, op, n_tile, &nsp, &sstride)) != DBT_OK) return st;
-        // S-bar_i = S_i + Attn_i W_O (matched: S-bar_2 = S_2 + g_A * Attn_1 W_O) ; RMSNorm for the MLP
         if (rows_form)
-            LAUNCH(m, "resid_wide", 0, resid_rows_kernel, dim3((Bc + 3) / 4, mss_tiles), 256, 0, w.S, w.P, nsp, sstride, lw.mlp_norm_g, Bc, d,
-                   w.Xb, lo_x, w.ss, m->Rmax);
-        else if (mwide)
+            st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, Bc,
+                                           prompt_resid_params(m, lw.mlp_norm_g));
+        else
+            st = run_gemm_tc(m, op, n_tile, &nsp, &sstride);
+        if (st != DBT_OK) return st;
+        // S-bar_i = S_i + Attn_i W_O (matched: S-bar_2 = S_2 + g_A * Attn_1 W_O) ; RMSNorm for the MLP
+        if (rows_form) {
+        } else if (mwide)
             LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, mss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, nsp, sstride, matched ? 3 : 1,
                    matched ? lw.gate_a : (const float *)nullptr, Bc, grouped, lw.mlp_norm_g, d, w.Xb, lo_x, w.ss, m->Rmax);
         else
@@ -1125,7 +1203,8 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
             mode = 2;
         } else {
             st = m->moe_tc ? run_moe_tc(m, l, rm, grouped, record_experts, mwide,
-                                        l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : nullptr)
+                                        l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : nullptr,
+                                        rows_form ? prompt_ss_tiles(m) : mss_tiles)
                            : run_moe<WT>(m, l, rm, grouped, record_experts);
             if (st != DBT_OK) return st;
             mode = 0;
@@ -1230,9 +1309,6 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
     size_t pool_layer_elems = (size_t)2 * c.num_pages * c.n_kv_heads * c.page_size * c.head_dim;
     size_t lo_x = m->act_parts == 2 ? (size_t)m->Rmax * d : 0, lo_h = m->act_parts == 2 ? (size_t)m->Rmax * F : 0;
     int ss_tiles = wide_ss_tiles(m), ss_ld = m->Rmax;
-    // prompt chunks of more than one row tile: the kernels between the GEMMs stream tens of MB and take
-    // their vector form (four elements per thread)
-    const bool rows_form = !grouped && rm.cn > 1 && Bc > 256 && d % 4 == 0 && F % 4 == 0 && c.head_dim % 8 == 0 && ((size_t)m->Rmax * d) % 4 == 0;
     double kv_bytes = 0;
     for (int b = 0; b < rm.B; b++)
         for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * sizeof(WT);
@@ -1258,16 +1334,11 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
         if ((st = run_gemm_tc(m, qkv, n_tile, &nsp, &sstride)) != DBT_OK) return st;
         const bool fuse = m->fuse_qkv && rm.cn == 1;
         QkvFuse qf{w.P, nsp, sstride, w.ss, ss_tiles, ss_ld, lw.coup_a};
-        if (rows_form)
-            LAUNCH(m, "qkv_epilogue", 0, qkv_rows_kernel, dim3(Bc, ((c.n_q_heads + c.n_kv_heads) * (c.head_dim / 8) + 255) / 256), 256, 0,
-                   w.P, nsp, sstride, w.Q, rm, c.n_q_heads, c.n_kv_heads, c.head_dim, w.rope, w.seq_len, w.page_table,
-                   m->pages_per_seq_max, c.num_pages, c.page_size, kpool, vpool, w.status, (const float *)w.ss, ss_tiles, ss_ld, d,
-                   c.rms_eps);
-        else if (!fuse)
+        if (!fuse)
             LAUNCH(m, "qkv_epilogue", 0, qkv_epilogue_kernel<WT>, dim3(Bc, c.n_q_heads + c.n_kv_heads, branch_blocks(grouped)), 64, 0, w.P, nsp, sstride,
                    w.Q, rm, grouped, c.n_q_heads, c.n_kv_heads, c.head_dim, lw.coup_a, w.rope, w.seq_len, w.page_table,
                    m->pages_per_seq_max, c.num_pages, c.page_size, kpool, vpool, w.status, (const float *)w.ss, ss_tiles, ss_ld, d,
-                   c.rms_eps);
+                   c.rms_eps, rm.cn > 1 ? prompt_q(m) : (__nv_bfloat16 *)nullptr, prompt_q_scale(m));
         st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, grouped, l, kv_bytes, fuse ? &qf : nullptr, true, m->att_planned)
                                : run_attention_mma<64>(m, rm, grouped, l, kv_bytes, fuse ? &qf : nullptr, true, m->att_planned);
         if (st != DBT_OK) return st;
@@ -1275,10 +1346,6 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
         op.W[0] = &mp.wo; op.n_out[0] = d; op.rows[0] = R; op.nseg = 1;
         {
             if ((st = run_gemm_tc(m, op, n_tile, &nsp, &sstride)) != DBT_OK) return st;
-            if (rows_form)
-                LAUNCH(m, "resid_wide", 0, resid_rows_kernel, dim3((Bc + 3) / 4, ss_tiles), 256, 0, w.S, w.P, nsp, sstride, lw.mlp_norm_g, Bc, d,
-                       w.Xb, lo_x, w.ss, ss_ld);
-            else
             LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, ss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, nsp, sstride, 1,
                    (const float *)nullptr, Bc, grouped, lw.mlp_norm_g, d, w.Xb, lo_x, w.ss, ss_ld);
         }
@@ -1287,20 +1354,7 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
         gu.W[1] = &mp.wu; gu.n_out[1] = F; gu.rows[1] = R;
         gu.nseg = 2;
         {
-            bool gu_done = false;
-            GuEpi ge{};
-            if (rows_form) {
-                ge.Hb = w.Hb; ge.lo_off = lo_h; ge.ss = w.ss; ge.ss_tiles = ss_tiles; ge.ss_ld = ss_ld; ge.d_norm = d; ge.F = F;
-                ge.eps = c.rms_eps;
-                gu.gu = &ge;
-                gu.gu_fused = &gu_done;
-            }
             if ((st = run_gemm_tc(m, gu, n_tile, &nsp, &sstride)) != DBT_OK) return st;
-            if (gu_done) {
-            } else if (rows_form)
-                LAUNCH(m, "swiglu_couple", 0, swiglu_rows_kernel, dim3(Bc, (F + 1023) / 1024), 256, 0, w.P, nsp, sstride, F, w.Hb, lo_h,
-                       (const float *)w.ss, ss_tiles, ss_ld, d, c.rms_eps);
-            else
             LAUNCH(m, "swiglu_couple", 0, swiglu_couple_kernel, dim3(Bc, (F + 255) / 256, branch_blocks(grouped)), 256, 0, w.P, nsp, sstride, F, Bc,
                    grouped, lw.coup_b, w.Hb, lo_h, (const float *)w.ss, ss_tiles, ss_ld, d, c.rms_eps);
         }
@@ -1310,10 +1364,6 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
                                                  : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr);
         {
             if ((st = run_gemm_tc(m, dn, n_tile, &nsp, &sstride)) != DBT_OK) return st;
-            if (rows_form)
-                LAUNCH(m, "resid_wide", 0, resid_rows_kernel, dim3((Bc + 3) / 4, ss_tiles), 256, 0, w.S, w.P, nsp, sstride, g_next, Bc, d, w.Xb,
-                       lo_x, w.ss, ss_ld);
-            else
             LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, ss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, nsp, sstride, 2, lw.coup_c, Bc,
                    grouped, g_next, d, w.Xb, lo_x, w.ss, ss_ld);
         }
@@ -1321,55 +1371,7 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
     return DBT_OK;
 }
 
-// ---- prompt chunks of dense bf16 models: paired-SM GEMMs with their epilogues -----------------------
-
-// The 3-D one-box view of a two-plane GEMM input, built on first use.
-const CUtensorMap *act_view(dbt_model *m, const CUtensorMap *X, int box_rows, int K) {
-    auto reg = m->act_base.find(X);
-    if (reg == m->act_base.end()) return nullptr;
-    auto key = std::make_tuple(X, box_rows, m->Rmax);
-    auto hit = m->act3d.find(key);
-    if (hit == m->act3d.end()) {
-        CUtensorMap t;
-        if (!make_act_map(&t, reg->second.base, (uint64_t)m->Rmax, (uint64_t)K, box_rows)) return nullptr;
-        hit = m->act3d.emplace(key, t).first;
-    }
-    return &hit->second;
-}
-
-template <int N, int MODE>
-dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *const (&W)[3], const CUtensorMap *X, const PgParams &p,
-                              double bytes) {
-    const int pairs = m->num_sms / 2, grid = 2 * (p.tiles < pairs ? p.tiles : pairs);
-    LAUNCH(m, tag, bytes, (gemm_prompt_kernel<N, MODE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *W[0], *W[1], *W[2], *X, p);
-    return DBT_OK;
-}
-
-// One GEMM of a prompt chunk.  p carries the epilogue's operands; n_out the features of up to three matrices
-// (PG_GATEUP: of the gate matrix, the up matrix has as many).
-template <int MODE>
-dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
-                           const int (&n_out)[3], int nseg, const CUtensorMap *X, int K, int R, PgParams p) {
-    constexpr int N = 256, kTileF = MODE == PG_GATEUP ? N / 2 : N;
-    const CUtensorMap *x = act_view(m, X, 128, K);
-    if (!x) return fail(m, DBT_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", tag);
-    p.K = K;
-    p.R = R;
-    p.m_tiles = (R + kPgM - 1) / kPgM;
-    p.nseg = nseg;
-    int nt = 0, col = 0;
-    double bytes = 0;
-    for (int s = 0; s < nseg; s++) {
-        p.seg[s] = PgSeg{nt, n_out[s], col};
-        col += n_out[s];
-        nt += (n_out[s] + kTileF - 1) / kTileF;
-        bytes += (double)n_out[s] * K * 2 * (MODE == PG_GATEUP ? 2 : 1);
-    }
-    p.tiles = nt * p.m_tiles;
-    p.status = m->ws.status;
-    const CUtensorMap *const W[3] = {W0, W1 ? W1 : W0, W2 ? W2 : W0};
-    return launch_gemm_prompt<N, MODE>(m, tag, W, x, p, bytes);
-}
+// ---- prompt chunks of dense bf16 models -------------------------------------------------------------
 
 // One chunk of a prompt through all layers: five kernels per layer.
 dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
@@ -1377,14 +1379,12 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
     const int R = rm.B * rm.cn, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ff;
-    const size_t pool_layer_elems = (size_t)2 * c.num_pages * c.n_kv_heads * c.page_size * c.head_dim;
-    const size_t lo_x = (size_t)m->Rmax * d, lo_h = (size_t)m->Rmax * F;
+    const size_t lo_h = (size_t)m->Rmax * F;
     double kv_bytes = 0;
     for (int b = 0; b < rm.B; b++)
         for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * sizeof(WT);
     dbt_status st;
     int ss_tiles = wide_ss_tiles(m);  // the embedding kernel's; the residual epilogues leave two shares per feature tile
-    const int ss_next = 2 * ((d + 255) / 256);
     auto base = [&] {
         PgParams p{};
         p.ss_in = w.ss;
@@ -1394,34 +1394,17 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
         p.eps = c.rms_eps;
         return p;
     };
-    auto resid = [&](const float *g_next) {
-        PgParams p{};
-        p.S = w.S;
-        p.g_next = g_next;
-        p.X = w.Xb;
-        p.x_lo = lo_x;
-        p.ss_out = w.ss;
-        p.ss_ld = m->Rmax;
-        p.d = d;
-        return p;
-    };
     for (int l = 0; l < c.n_layers; l++) {
         const dbt_layer_weights &lw = m->layers[l];
         const LayerMaps &mp = m->maps[l];
-        PgParams q = base();
-        q.Q = w.Q;
-        q.B = rm.B; q.cn = rm.cn; q.dh = c.head_dim; q.n_q = c.n_q_heads; q.n_kv = c.n_kv_heads;
-        q.num_pages = c.num_pages; q.pt_stride = m->pages_per_seq_max;
-        q.rope = w.rope; q.seq_len = w.seq_len; q.page_table = w.page_table;
-        q.kpool = reinterpret_cast<WT *>(m->kv_pool) + (size_t)l * pool_layer_elems;
-        q.vpool = q.kpool + pool_layer_elems / 2;
+        const PgParams q = prompt_qkv_params(m, rm, l, ss_tiles);
         if ((st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, R, q)) != DBT_OK) return st;
         st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, 0, l, kv_bytes, nullptr, true, false)
                                : run_attention_mma<64>(m, rm, 0, l, kv_bytes, nullptr, true, false);
         if (st != DBT_OK) return st;
-        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, resid(lw.mlp_norm_g))) != DBT_OK)
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, prompt_resid_params(m, lw.mlp_norm_g))) != DBT_OK)
             return st;
-        ss_tiles = ss_next;
+        ss_tiles = prompt_ss_tiles(m);
         if (m->prompt_fuse_swiglu) {
             PgParams g = base();
             g.H = w.Hb;
@@ -1439,7 +1422,7 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
         }
         if (st != DBT_OK) return st;
         const float *g_next = l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr);
-        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R, resid(g_next))) != DBT_OK)
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R, prompt_resid_params(m, g_next))) != DBT_OK)
             return st;
     }
     return DBT_OK;
@@ -1514,7 +1497,7 @@ dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, f
         RowMap rm{B, cn};
         int R = B * cn, n_tile = pad_rows(R < 256 ? R : 256);
         if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, n_tile)) != DBT_OK) return st;
-        const bool pairs = m->prompt_pairs && cn > 1 && R > 256;
+        const bool pairs = cn > 1 && R > 256;
         if ((st = pairs ? run_layers_prompt(m, rm) : run_layers_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
         if (last_logits && p0 + cn >= n) {
             if ((st = run_head_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
@@ -1608,7 +1591,7 @@ bool setup_tc(dbt_model *m) {
         m->act_base[&m->map_Hs] = {w.Hs};
     }
     const char *fa = getenv("DBT_ATTN");
-    m->att_fast = ok && !(fa && strcmp(fa, "simt") == 0) &&
+    m->att_fast = ok && allow_smem_prompt() && !(fa && strcmp(fa, "simt") == 0) &&
                   make_kv_page_map(&m->map_kv, m->kv_pool, (uint64_t)c.n_layers * 2 * c.num_pages * c.n_kv_heads * c.page_size,
                                    (uint64_t)c.num_pages * c.n_kv_heads * c.page_size, c.head_dim) &&
                   cudaFuncSetAttribute(attn_prompt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1630,8 +1613,12 @@ bool setup_tc(dbt_model *m) {
     // Default chain of a dense bf16 model: the RMSNorm factor is applied after the GEMM, so no kernel
     // reduces over a whole row.
     m->wide = ok && m->att_fast && !moe;
-    m->prompt_pairs = m->wide && allow_smem_prompt();
     m->act_parts = 2;
+    const char *pa = getenv("DBT_PROMPT_ATTN");
+    const int G = c.n_q_heads / c.n_kv_heads;
+    m->prompt_attn_tc = m->att_fast && 16 % G == 0 && !(pa && strcmp(pa, "tile") == 0) &&
+                        make_prompt_q_map(&m->map_pq, w.Q, m->Rmax, c.n_q_heads, c.head_dim, G) &&
+                        make_prompt_kv_map(&m->map_pkv, m->kv_pool, (uint64_t)c.n_layers * 2 * c.num_pages * c.n_kv_heads * c.page_size, c.head_dim);
     return ok;
 }
 
@@ -1778,8 +1765,6 @@ dbt_status dbt_create(const dbt_config *cfg, const dbt_weights *w, void *kv_pool
         m->moe_fuse_swiglu = !(fs && strcmp(fs, "0") == 0);
         const char *pf = getenv("DBT_PROMPT_FUSE_SWIGLU");
         m->prompt_fuse_swiglu = !(pf && strcmp(pf, "0") == 0);
-        const char *pa = getenv("DBT_PROMPT_ATTN");
-        m->prompt_attn_off = pa && strcmp(pa, "tile") == 0;
     }
     const char *ro = getenv("DBT_READOUT");
     m->readout_row = ro && strcmp(ro, "row") == 0;

@@ -67,6 +67,8 @@ struct PgParams {
     int F;
     // PG_QKV (segments 0, 1, 2 = Q, K, V)
     float *Q;
+    __nv_bfloat16 *Qb;  // the prompt attention kernel's queries: bf16, times q_scale (nullptr: Q, fp32)
+    float q_scale;
     int B, cn, dh, n_q, n_kv, num_pages, pt_stride;
     const float2 *rope;
     const int32_t *seq_len, *page_table;
@@ -463,7 +465,13 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         }
                         if (head >= nh) continue;
                         if (sg == 0) {
-                            if (on) {
+                            if (on && p.Qb) {
+                                __nv_bfloat16 *q0 = p.Qb + (size_t)row * p.n_q * hd + (size_t)head * hd + i0;
+#pragma unroll
+                                for (int i = 0; i < 16; i++) x0[i] *= p.q_scale, x1[i] *= p.q_scale;
+                                store16(q0, x0);
+                                store16(q0 + hh2, x1);
+                            } else if (on) {
                                 float *q0 = p.Q + (size_t)row * p.n_q * hd + (size_t)head * hd + i0;
 #pragma unroll
                                 for (int i = 0; i < 4; i++) {
