@@ -21,6 +21,7 @@
 #include "dbt_gemm_tc.cuh"
 #include "dbt_gemm_persist.cuh"
 #include "dbt_gemm_prompt.cuh"
+#include "dbt_gemm_group.cuh"
 #include "dbt_kernels.cuh"
 
 using namespace dbt;
@@ -61,6 +62,7 @@ struct LayerMaps {
     CUtensorMap wq, wk, wv, wo, wg, wu, wd;  // dense MLP; for MoE wg/wu/wd hold the shared expert
     CUtensorMap eg, eu, ed;                  // all routed experts as [E*Fe, d], [E*Fe, d], [E*d, Fe]
     CUtensorMap rt;                          // router [E, d]
+    CUtensorMap eg64, eu64, rt32;            // the same matrices in boxes of 64 / 32 rows (prompt chunks)
 };
 
 }  // namespace
@@ -104,7 +106,6 @@ struct dbt_model {
     int moe_persist;       // per-expert GEMMs as persistent CTAs over the units that have work: -1 by the batch, DBT_MOE_PERSIST=0/1 off/on
     int cur_rows;          // primary rows (sequences x positions) of the launch plan being built
     bool moe_fuse_swiglu;  // the persistent per-expert gate|up launch applies the SwiGLU itself (DBT_MOE_FUSE_SWIGLU=0: a kernel of its own)
-    bool prompt_fuse_swiglu;  // prompt chunks: SwiGLU in the gate|up GEMM's epilogue (DBT_PROMPT_FUSE_SWIGLU=0: a kernel of its own)
     bool fuse_qkv;     // decode steps: the attention kernel does the Q|K|V epilogue itself (DBT_FUSE_QKV=0 keeps the kernel)
     int num_sms;
     int act_parts;  // 2: GEMM inputs carried as hi + lo bf16 terms (the operator-level GEMM entry uses 1: plain bf16)
@@ -157,13 +158,24 @@ int npaths(int grouped) { return grouped > 1 ? grouped : 1; }
 // Kernels that pair a primary row with one branch row run a block per branch in grid.z.
 unsigned branch_blocks(int grouped) { return grouped > 1 ? (unsigned)(grouped - 1) : 1u; }
 int kmax_of(const dbt_config &c) { return c.k_primary > c.k_branch ? c.k_primary : c.k_branch; }
-// Rows of the activation buffers: all paths of a full batch in a decode step, or one prompt chunk of the
-// prefill (2048 rows for dense bf16 models, whose GEMMs sweep several row tiles per weight tile and whose
-// causal attention packs consecutive positions into a query tile; 256 otherwise).
+// Rows that the decode kernels and the short prompt chunks in their form work on.
+int decode_rows(const dbt_config &c) { return paths_of(c) * c.max_batch > 256 ? paths_of(c) * c.max_batch : 256; }
+// Rows of the activation buffers of bf16 models: a decode step's, or one prompt chunk.  A chunk is at most 37 row tiles
+// of 256: with the 74 pairs of SMs the tiles of a GEMM of any even number of feature tiles are then whole waves (a 1B
+// layer's four GEMMs take 1.22 tile times per row tile; 1.34 at 8 row tiles, 1.31 at 32), an expert's matrices serve
+// four times the rows of a 2048-row chunk, and the buffers stay below a gigabyte at the 1B width.
+constexpr int kPromptRows = 37 * 256;
 int prefill_rows(const dbt_config &c) {
-    // rows of a prompt chunk: bf16 models 2048, everything else 256
-    int chunk = c.weight_dtype != DBT_DTYPE_BF16 ? 256 : 2048;
-    return paths_of(c) * c.max_batch > chunk ? paths_of(c) * c.max_batch : chunk;
+    if (c.weight_dtype != DBT_DTYPE_BF16) return decode_rows(c);
+    const long long all = ((long long)c.max_batch * c.max_seq + 255) / 256 * 256;
+    const int chunk = all < kPromptRows ? (int)all : kPromptRows;
+    return decode_rows(c) > chunk ? decode_rows(c) : chunk;
+}
+// Expert-sorted rows of the two-plane buffers: every selection of a decode step's rows, or of a prompt chunk's (the
+// primary path alone, fan-out k_1).
+size_t sorted_rows(const dbt_config &c) {
+    const size_t dec = (size_t)decode_rows(c) * kmax_of(c), pro = (size_t)prefill_rows(c) * c.k_primary;
+    return dec > pro ? dec : pro;
 }
 
 const char *check_config(const dbt_config *c, dbt_status *st) {
@@ -204,6 +216,7 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
     Carver k{base, 0};
     Workspace w{};
     int Rmax = prefill_rows(c);
+    const int Rd = decode_rows(c);  // the generic kernels' buffers and the split-K partials: prompt chunks do not use them
     int d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
     bool moe = c.n_experts > 0;
     int Fs = moe ? c.n_shared_experts * c.d_expert : 0;
@@ -212,13 +225,13 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
     int att_rows = att_rows_of(c);
     int part_items = att_rows * c.n_kv_heads + 8 * 148;  // attention partial slots: up to three rounds of 2 x 148 segments plus one per pair
     w.S = k.take<float>((size_t)Rmax * d);
-    w.X = k.take<float>((size_t)Rmax * d);
+    w.X = k.take<float>((size_t)Rd * d);
     w.Q = k.take<float>((size_t)Rmax * qd);
-    w.Kn = k.take<float>((size_t)Rmax * kvd);
-    w.Vn = k.take<float>((size_t)Rmax * kvd);
-    w.O = k.take<float>((size_t)Rmax * qd);
-    w.G1 = k.take<float>((size_t)Rmax * F);
-    w.M = k.take<float>((size_t)Rmax * d);
+    w.Kn = k.take<float>((size_t)Rd * kvd);
+    w.Vn = k.take<float>((size_t)Rd * kvd);
+    w.O = k.take<float>((size_t)Rd * qd);
+    w.G1 = k.take<float>((size_t)Rd * F);
+    w.M = k.take<float>((size_t)Rd * d);
     w.Z = k.take<float>((size_t)paths_of(c) * c.max_batch * c.vocab);
     w.Zrows = k.take<float>((size_t)paths_of(c) * c.max_batch * d);
     w.part = k.take<float>((size_t)part_items * 16 * (c.head_dim + 2));
@@ -241,10 +254,10 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
         w.rlogits = k.take<float>((size_t)Rmax * c.n_experts);
         w.rwts = k.take<float>((size_t)Rmax * km);
         w.ridx = k.take<int32_t>((size_t)Rmax * km);
-        w.Hexp = k.take<float>((size_t)Rmax * km * c.d_expert);
-        w.Yexp = k.take<float>((size_t)Rmax * km * d);
-        w.Msh = k.take<float>((size_t)Rmax * d);
-        w.Hsh = k.take<float>((size_t)Rmax * (Fs > 0 ? Fs : 8));
+        w.Hexp = k.take<float>((size_t)Rd * km * c.d_expert);
+        w.Yexp = k.take<float>(sorted_rows(c) * d);
+        w.Msh = k.take<float>((size_t)Rd * d);
+        w.Hsh = k.take<float>((size_t)Rd * (Fs > 0 ? Fs : 8));
         w.ecnt = k.take<int32_t>(c.n_experts);
         w.elist = k.take<int32_t>((size_t)c.n_experts * Rmax);
         w.last_experts = k.take<int32_t>((size_t)c.n_layers * paths_of(c) * c.max_batch * km);
@@ -257,24 +270,24 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
         w.Hb = k.take<__nv_bfloat16>((size_t)2 * Rmax * F);
         // room for the widest GEMM output at a few splits, capped
         size_t widest = (size_t)(moe ? (qd + 2 * kvd > 2 * F ? qd + 2 * kvd : 2 * F) : (2 * F > qd + 2 * kvd ? 2 * F : qd + 2 * kvd));
-        size_t want = (size_t)Rmax * widest * 6;
+        size_t want = (size_t)Rd * widest * 8;
         size_t cap = (size_t)24 << 20;  // floats (96 MB)
         w.P_floats = want < cap ? want : cap;
-        if (w.P_floats < (size_t)Rmax * widest) w.P_floats = (size_t)Rmax * widest;
+        if (w.P_floats < (size_t)Rd * widest) w.P_floats = (size_t)Rd * widest;
         w.P = k.take<float>(w.P_floats);
         // shares of sum(S^2): 256 columns each in decode steps, half a 256-feature tile in prompt chunks
         w.ss = k.take<float>((size_t)((d + 255) / 256 * 2) * Rmax);
         if (moe) {
-            size_t Rk = (size_t)Rmax * kmax_of(c);
+            const size_t Rk = sorted_rows(c);
             w.Xs = k.take<__nv_bfloat16>(2 * Rk * d);
             w.Hs = k.take<__nv_bfloat16>(2 * Rk * c.d_expert);
-            w.Pe = k.take<float>(Rk * 2 * c.d_expert);
+            w.Pe = k.take<float>((size_t)Rd * kmax_of(c) * 2 * c.d_expert);
             size_t wide2 = (size_t)(2 * Fs > d ? 2 * Fs : d);
-            w.P2_floats = Fs > 0 ? (size_t)Rmax * wide2 * 6 : 0;
+            w.P2_floats = Fs > 0 ? (size_t)Rd * wide2 * 6 : 0;
             if (w.P2_floats > ((size_t)8 << 20)) w.P2_floats = (size_t)8 << 20;
-            if (Fs > 0 && w.P2_floats < (size_t)Rmax * wide2) w.P2_floats = (size_t)Rmax * wide2;
+            if (Fs > 0 && w.P2_floats < (size_t)Rd * wide2) w.P2_floats = (size_t)Rd * wide2;
             w.P2 = k.take<float>(w.P2_floats);
-            w.epos = k.take<int32_t>(Rk);
+            w.epos = k.take<int32_t>((size_t)Rmax * kmax_of(c));
             w.eoff = k.take<int32_t>(c.n_experts + 1);
             w.rs_sorted = k.take<float>(Rk);
         }
@@ -593,7 +606,6 @@ struct TcCall {
     int grp_w_rows, n_groups;
     int grp_row_tiles;  // per-expert mode: row tiles of n_tile rows per expert (0: one tile holds any list)
     int grp_prewait;    // per-expert mode: the lists are final before this launch can be resident (see TcParams)
-    int grp_mt2;        // per-expert mode, 64-row tiles: two weight tiles per CTA share each activation box (prompt chunks)
     // per-expert gate|up launch: where it runs as persistent CTAs it may apply the SwiGLU itself (see SwigluEpi);
     // *fused tells the caller whether it did
     const SwigluEpi *swiglu;
@@ -694,7 +706,6 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
         const int w1 = (t1 * rt + sms - 1) / sms, w2 = (t2 * rt + sms - 1) / sms;
         if (16 * w2 < 10 * w1) mt = 2;
     }
-    if (c.grp_cnt && c.grp_mt2 && n_tile == 64) mt = 2;
     for (int s = 0; s < c.nseg; s++) {
         p.seg[s] = TcSeg{tiles, c.n_out[s], c.rows[s], col};
         tiles += (c.n_out[s] + kTcM * mt - 1) / (kTcM * mt);
@@ -742,7 +753,7 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     switch (n_tile) {
         case 16: return launch_gemm_tc<16>(m, c, p, e, grid, bytes);
         case 32: return launch_gemm_tc<32>(m, c, p, e, grid, bytes);
-        case 64: return mt == 2 ? launch_gemm_tc<64, 2>(m, c, p, e, grid, bytes) : launch_gemm_tc<64>(m, c, p, e, grid, bytes);
+        case 64: return launch_gemm_tc<64>(m, c, p, e, grid, bytes);
         case 128: return launch_gemm_tc<128>(m, c, p, e, grid, bytes);
         case 256: return mt == 2 ? launch_gemm_tc<256, 2>(m, c, p, e, grid, bytes) : launch_gemm_tc<256>(m, c, p, e, grid, bytes);
     }
@@ -896,10 +907,10 @@ dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *
 
 // One GEMM of a prompt chunk.  p carries the epilogue's operands; n_out the features of up to three matrices
 // (PG_GATEUP: of the gate matrix, the up matrix has as many).
-template <int MODE>
+template <int MODE, int N = 256>
 dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
                            const int (&n_out)[3], int nseg, const CUtensorMap *X, int K, int R, PgParams p) {
-    constexpr int N = 256, kTileF = MODE == PG_GATEUP ? N / 2 : N;
+    constexpr int kTileF = MODE == PG_GATEUP ? N / 2 : N;
     const CUtensorMap *x = act_view(m, X, 128, K);
     if (!x) return fail(m, DBT_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", tag);
     p.K = K;
@@ -915,6 +926,8 @@ dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0,
         bytes += (double)n_out[s] * K * 2 * (MODE == PG_GATEUP ? 2 : 1);
     }
     p.tiles = nt * p.m_tiles;
+    const int groups = (p.m_tiles + 8) / 9;
+    p.m_group = (p.m_tiles + groups - 1) / groups;
     p.status = m->ws.status;
     const CUtensorMap *const W[3] = {W0, W1 ? W1 : W0, W2 ? W2 : W0};
     return launch_gemm_prompt<N, MODE>(m, tag, W, x, p, bytes);
@@ -962,14 +975,15 @@ int prompt_ss_tiles(const dbt_model *m) { return 2 * ((m->cfg.d_model + 255) / 2
 // consumer of a GEMM on them applies the row's factor itself, and the combine leaves the next layer's
 // input in the same form when it is given that layer's gain g_next.
 dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool record_experts, bool wide,
-                      const float *g_next, int ss_tiles) {
+                      const float *g_next) {
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
     const dbt_layer_weights &lw = m->layers[l];
     const LayerMaps &mp = m->maps[l];
     int Bc = rm.B * rm.cn, R = npaths(grouped) * Bc, d = c.d_model;
-    int E = c.n_experts, Fe = c.d_expert, km = kmax_of(c), Fs = c.n_shared_experts * Fe, Rk = m->Rmax * km;
+    int E = c.n_experts, Fe = c.d_expert, km = kmax_of(c), Fs = c.n_shared_experts * Fe, Rk = (int)sorted_rows(c);
+    const int Rkd = decode_rows(c) * km;  // rows of the fp32 buffers behind the per-expert GEMMs
     // Row tile (and with it the resident-CTA count that sizes the split-K factors of the router and the shared
     // expert) from the batch, never from the mode: a primary-only step uses the tile of the grouped step, so both
     // add the same partials in the same order and write the same K/V bits.
@@ -978,7 +992,7 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
     size_t lo_x = m->act_parts == 2 ? (size_t)m->Rmax * d : 0;
     size_t lo_xs = m->act_parts == 2 ? (size_t)Rk * d : 0, lo_hs = m->act_parts == 2 ? (size_t)Rk * Fe : 0;
     const float *ssp = wide ? w.ss : nullptr;
-    const int ss_ld = m->Rmax;
+    const int ss_tiles = (d + 255) / 256, ss_ld = m->Rmax;
     dbt_status st;
     // shared expert(s) on every row of both paths; b couples its hidden state
     const float *Psh = nullptr;
@@ -1038,9 +1052,9 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
            c.rms_eps, w.rs_sorted);
     // routed experts: gate|up, SwiGLU, down
     TcCall gu{};
-    gu.W[0] = &mp.eg; gu.n_out[0] = Fe; gu.rows[0] = Rk;
-    gu.W[1] = &mp.eu; gu.n_out[1] = Fe; gu.rows[1] = Rk;
-    gu.nseg = 2; gu.X = &m->map_Xs; gu.K = d; gu.R = Rk; gu.P = w.Pe; gu.P_floats = (size_t)Rk * 2 * Fe;
+    gu.W[0] = &mp.eg; gu.n_out[0] = Fe; gu.rows[0] = Rkd;
+    gu.W[1] = &mp.eu; gu.n_out[1] = Fe; gu.rows[1] = Rkd;
+    gu.nseg = 2; gu.X = &m->map_Xs; gu.K = d; gu.R = Rkd; gu.P = w.Pe; gu.P_floats = (size_t)Rkd * 2 * Fe;
     gu.tag = "expert_gateup"; gu.parts = m->act_parts; gu.lo_row0 = Rk;
     gu.grp_cnt = w.ecnt; gu.grp_off = w.eoff; gu.grp_w_rows = Fe; gu.n_groups = E;
     // An expert's list is short on average (rows x k / experts) but may hold every row: row tiles of
@@ -1049,14 +1063,12 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
     // could need, keep two CTAs per SM and their deeper rings at large batches (measured: 4.86 -> 4.53 ms
     // at batch 32, 6.43 -> 4.81 at batch 64).  DBT_MOE_ROWTILE=0: one tile of all rows; 16/32/64: that tile.
     int gt = n_tile, grt = 0;
-    // (prompt chunks of more than 256 rows: tiles of 64 rows, an expert's share of such a chunk)
-    const int want_tile = m->moe_row_tile >= 0 ? m->moe_row_tile : (paths_of(c) * Bc <= 64 ? 16 : Bc <= 256 ? 32 : 64);
+    const int want_tile = m->moe_row_tile >= 0 ? m->moe_row_tile : (paths_of(c) * Bc <= 64 ? 16 : 32);
     if (want_tile > 0 && n_tile > want_tile) {
         gt = want_tile;
         grt = (R + gt - 1) / gt;
     }
     gu.grp_row_tiles = grt;
-    gu.grp_mt2 = (gt == 64 && Bc > 256) ? 1 : 0;
     gu.grp_prewait = m->use_pdl ? 1 : 0;  // the gather kernel before it lets its dependents in only after its own wait
     const SwigluEpi se{w.Hs, lo_hs, wide ? (const float *)w.rs_sorted : (const float *)nullptr, Fe};
     bool swiglu_done = false;
@@ -1067,11 +1079,10 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
         LAUNCH(m, "moe_swiglu", 0, moe_swiglu_kernel, dim3(R * km, (Fe + 255) / 256), 256, 0, w.Pe, w.eoff + E, Fe, w.Hs, lo_hs,
                wide ? (const float *)w.rs_sorted : (const float *)nullptr);
     TcCall dn{};
-    dn.W[0] = &mp.ed; dn.n_out[0] = d; dn.rows[0] = Rk; dn.nseg = 1; dn.X = &m->map_Hs; dn.K = Fe; dn.R = Rk;
-    dn.P = w.Yexp; dn.P_floats = (size_t)Rk * d; dn.tag = "expert_down"; dn.parts = m->act_parts; dn.lo_row0 = Rk;
+    dn.W[0] = &mp.ed; dn.n_out[0] = d; dn.rows[0] = Rkd; dn.nseg = 1; dn.X = &m->map_Hs; dn.K = Fe; dn.R = Rkd;
+    dn.P = w.Yexp; dn.P_floats = (size_t)Rkd * d; dn.tag = "expert_down"; dn.parts = m->act_parts; dn.lo_row0 = Rk;
     dn.grp_cnt = w.ecnt; dn.grp_off = w.eoff; dn.grp_w_rows = d; dn.n_groups = E;
     dn.grp_row_tiles = grt;
-    dn.grp_mt2 = gu.grp_mt2;
     // The lists come from the sort kernel, several launches back.  A CTA of this launch can only be resident once
     // every CTA of the launch before it has started (the SwiGLU kernel, or the gate|up GEMM where that applies the
     // SwiGLU itself), hence once every CTA of the gate|up GEMM is resident, hence once every CTA of the gather kernel
@@ -1081,12 +1092,6 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
     if (Fs > 0 && !overlap && (st = shared_expert(w.P, w.P_floats)) != DBT_OK) return st;
     if (overlap) CUDA_TRY(m, cudaStreamWaitEvent(main_stream, m->ev_join, 0));
     const bool next_in = wide && g_next != nullptr;
-    if (!grouped && wide && rm.cn > 1 && Bc > 256 && d % 4 == 0 && ((size_t)m->Rmax * d) % 4 == 0) {  // prompt chunks: the vector form
-        LAUNCH(m, "moe_combine", 0, moe_combine_rows_kernel, dim3((Bc + 3) / 4, (d + 255) / 256), 256, 0, w.Yexp, Psh, nsp, sstride, w.ridx,
-               w.epos, w.rwts, km, Bc, d, w.S, next_in ? g_next : (const float *)nullptr, next_in ? w.Xb : (__nv_bfloat16 *)nullptr, lo_x,
-               next_in ? w.ss : (float *)nullptr, ss_ld);
-        return DBT_OK;
-    }
     LAUNCH_BR(m, grouped, "moe_combine", 0, moe_combine_sorted_kernel, dim3(Bc, (d + 255) / 256, branch_blocks(grouped)), 256, 0, w.Yexp, Psh, nsp, sstride, w.ridx, w.epos, w.rwts, km,
            Bc, grouped, lw.coup_c, matched ? lw.gate_g : (const float *)nullptr, d, w.S, next_in ? g_next : (const float *)nullptr,
            next_in ? w.Xb : (__nv_bfloat16 *)nullptr, lo_x, next_in ? w.ss : (float *)nullptr, ss_ld);
@@ -1118,10 +1123,6 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
     const bool mwide = moe && m->moe_tc && m->moe_wide;
     const int mss_tiles = (d + 255) / 256;
     size_t lo_x = m->act_parts == 2 ? (size_t)m->Rmax * d : 0;
-    // prompt chunks of more than one row tile (MoE models): the prompt attention kernel and the vector forms of the
-    // kernels around it, as in the dense prompt pass
-    const bool rows_form = mwide && m->att_fast && !grouped && rm.cn > 1 && Bc > 256 && d % 4 == 0 && c.head_dim % 8 == 0 &&
-                           ((size_t)m->Rmax * d) % 4 == 0;
     dbt_status st;
     int mode = 0, nsp = 1;
     size_t sstride = 0;
@@ -1147,22 +1148,17 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
         qkv.W[1] = &mp.wk; qkv.n_out[1] = kvd; qkv.rows[1] = Bc;
         qkv.W[2] = &mp.wv; qkv.n_out[2] = kvd; qkv.rows[2] = Bc;
         qkv.nseg = 3; qkv.X = &m->map_Xb; qkv.K = d; qkv.R = Ra; qkv.P = w.P; qkv.P_floats = w.P_floats; qkv.parts = m->act_parts; qkv.lo_row0 = m->Rmax; qkv.tag = "gemm_qkv";
-        if (rows_form)
-            st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, Bc,
-                                         prompt_qkv_params(m, rm, l, mss_tiles));
-        else
-            st = run_gemm_tc(m, qkv, n_tile, &nsp, &sstride);
-        if (st != DBT_OK) return st;
+        if ((st = run_gemm_tc(m, qkv, n_tile, &nsp, &sstride)) != DBT_OK) return st;
         const bool fuse = m->fuse_qkv && m->att_fast && rm.cn == 1;
         QkvFuse qf{w.P, nsp, sstride, mwide ? w.ss : nullptr, mwide ? mss_tiles : 0, mwide ? m->Rmax : 0, lw.coup_a};
-        if (!rows_form && !fuse)
+        if (!fuse)
             LAUNCH(m, "qkv_epilogue", 0, qkv_epilogue_kernel<WT>, dim3(Bc, c.n_q_heads + c.n_kv_heads, branch_blocks(ga)), 64, 0, w.P, nsp, sstride, w.Q, rm, ga, c.n_q_heads,
                    c.n_kv_heads, c.head_dim, lw.coup_a, w.rope, w.seq_len, w.page_table, m->pages_per_seq_max, c.num_pages,
                    c.page_size, kpool, vpool, w.status, mwide ? (const float *)w.ss : (const float *)nullptr, mwide ? mss_tiles : 0,
                    mwide ? m->Rmax : 0, d, c.rms_eps, (__nv_bfloat16 *)nullptr, 0.f);
         if (m->att_fast)
-            st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, ga, l, kv_bytes, fuse ? &qf : nullptr, rows_form, m->att_planned)
-                                   : run_attention_mma<64>(m, rm, ga, l, kv_bytes, fuse ? &qf : nullptr, rows_form, m->att_planned);
+            st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, ga, l, kv_bytes, fuse ? &qf : nullptr, false, m->att_planned)
+                                   : run_attention_mma<64>(m, rm, ga, l, kv_bytes, fuse ? &qf : nullptr, false, m->att_planned);
         else if (c.head_dim == 128)
             st = run_attention<WT, 128>(m, rm, ga, kpool, vpool, att_split, kv_bytes, true);
         else
@@ -1171,15 +1167,9 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
         TcCall op{};
         op.W[0] = &mp.wo; op.n_out[0] = d; op.rows[0] = Ra; op.nseg = 1; op.X = &m->map_Ob; op.K = qd; op.R = Ra;
         op.P = w.P; op.P_floats = w.P_floats; op.parts = m->act_parts; op.lo_row0 = m->Rmax; op.tag = "gemm_o";
-        if (rows_form)
-            st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, Bc,
-                                           prompt_resid_params(m, lw.mlp_norm_g));
-        else
-            st = run_gemm_tc(m, op, n_tile, &nsp, &sstride);
-        if (st != DBT_OK) return st;
+        if ((st = run_gemm_tc(m, op, n_tile, &nsp, &sstride)) != DBT_OK) return st;
         // S-bar_i = S_i + Attn_i W_O (matched: S-bar_2 = S_2 + g_A * Attn_1 W_O) ; RMSNorm for the MLP
-        if (rows_form) {
-        } else if (mwide)
+        if (mwide)
             LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, mss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, nsp, sstride, matched ? 3 : 1,
                    matched ? lw.gate_a : (const float *)nullptr, Bc, grouped, lw.mlp_norm_g, d, w.Xb, lo_x, w.ss, m->Rmax);
         else
@@ -1203,8 +1193,7 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
             mode = 2;
         } else {
             st = m->moe_tc ? run_moe_tc(m, l, rm, grouped, record_experts, mwide,
-                                        l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : nullptr,
-                                        rows_form ? prompt_ss_tiles(m) : mss_tiles)
+                                        l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : nullptr)
                            : run_moe<WT>(m, l, rm, grouped, record_experts);
             if (st != DBT_OK) return st;
             mode = 0;
@@ -1259,37 +1248,6 @@ dbt_status step_tc(dbt_model *m, const int32_t *tokens_dev, int B, int grouped, 
         CUDA_TRY(m, cudaMemcpyAsync(z2_dev, w.Z + (size_t)B * c.vocab, zb * (npaths(grouped) - 1), cudaMemcpyDeviceToDevice, m->stream));
     for (int b = 0; b < B; b++) m->len_host[b] += 1;
     m->pending_union = c.n_experts > 0;
-    return DBT_OK;
-}
-
-dbt_status prefill_tc(dbt_model *m, const int32_t *tokens_dev, int B, int n, float *last_logits) {
-    typedef __nv_bfloat16 WT;
-    const dbt_config &c = m->cfg;
-    const Workspace &w = m->ws;
-    // chunks of up to Rmax rows where every kernel of the chain takes more than one row tile (the tensor-core MoE
-    // chain with the norm factor behind the GEMMs); 256 rows otherwise
-    const bool big = c.n_experts > 0 && m->moe_tc && m->moe_wide && m->att_fast;
-    int cn_max = (big ? m->Rmax : (m->Rmax < 256 ? m->Rmax : 256)) / B;
-    if (cn_max < 1) cn_max = 1;
-    dbt_status st;
-    for (int p0 = 0; p0 < n; p0 += cn_max) {
-        int cn = n - p0 < cn_max ? n - p0 : cn_max;
-        RowMap rm{B, cn};
-        int R = B * cn, n_tile = pad_rows(R);
-        LAUNCH(m, "embed", 0, embed_norm_kernel<WT>, R, 256, 0, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, (const WT *)m->w.embed_primary,
-               (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S, w.status);
-        int mode, nsp;
-        size_t sstride;
-        if ((st = run_layers_tc(m, rm, 0, n_tile, false, &mode, &nsp, &sstride)) != DBT_OK) return st;
-        bool last = p0 + cn >= n;
-        if (last && last_logits) {
-            if ((st = run_head_tc(m, R, 0, B, cn, cn - 1, pad_rows(B), mode, nsp, sstride)) != DBT_OK) return st;
-            CUDA_TRY(m, cudaMemcpyAsync(last_logits, w.Z, sizeof(float) * (size_t)B * c.vocab, cudaMemcpyDeviceToDevice,
-                                        m->stream));
-        }
-        LAUNCH(m, "advance_len", 0, advance_len_kernel, (B + 127) / 128, 128, 0, w.seq_len, B, cn);
-    }
-    for (int b = 0; b < B; b++) m->len_host[b] += n;
     return DBT_OK;
 }
 
@@ -1385,15 +1343,6 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
         for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * sizeof(WT);
     dbt_status st;
     int ss_tiles = wide_ss_tiles(m);  // the embedding kernel's; the residual epilogues leave two shares per feature tile
-    auto base = [&] {
-        PgParams p{};
-        p.ss_in = w.ss;
-        p.ss_tiles = ss_tiles;
-        p.ss_ld = m->Rmax;
-        p.d_norm = d;
-        p.eps = c.rms_eps;
-        return p;
-    };
     for (int l = 0; l < c.n_layers; l++) {
         const dbt_layer_weights &lw = m->layers[l];
         const LayerMaps &mp = m->maps[l];
@@ -1405,25 +1354,83 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
         if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, prompt_resid_params(m, lw.mlp_norm_g))) != DBT_OK)
             return st;
         ss_tiles = prompt_ss_tiles(m);
-        if (m->prompt_fuse_swiglu) {
-            PgParams g = base();
-            g.H = w.Hb;
-            g.h_lo = lo_h;
-            g.F = F;
-            st = run_gemm_prompt<PG_GATEUP>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, 0, 0}, 1, &m->map_Xb, d, R, g);
-        } else {
-            PgParams g{};
-            g.P = w.P;
-            g.ldp = 2 * F;
-            st = run_gemm_prompt<PG_STORE>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, F, 0}, 2, &m->map_Xb, d, R, g);
-            if (st == DBT_OK)
-                LAUNCH(m, "swiglu_couple", 0, swiglu_rows_kernel, dim3(R, (F + 1023) / 1024), 256, 0, w.P, 1, (size_t)0, F, w.Hb, lo_h,
-                       (const float *)w.ss, ss_tiles, m->Rmax, d, c.rms_eps);
-        }
+        PgParams g{};
+        g.ss_in = w.ss; g.ss_tiles = ss_tiles; g.ss_ld = m->Rmax; g.d_norm = d; g.eps = c.rms_eps;
+        g.H = w.Hb; g.h_lo = lo_h; g.F = F;
+        st = run_gemm_prompt<PG_GATEUP>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, 0, 0}, 1, &m->map_Xb, d, R, g);
         if (st != DBT_OK) return st;
         const float *g_next = l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr);
         if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R, prompt_resid_params(m, g_next))) != DBT_OK)
             return st;
+    }
+    return DBT_OK;
+}
+
+// ---- prompt chunks of MoE models ----------------------------------------------------------------------
+// Whether they take the paired-SM chain (otherwise 256-row chunks through the decode step's kernels).
+bool moe_prompt_ok(const dbt_model *m) {
+    const dbt_config &c = m->cfg;
+    return c.n_experts > 0 && m->moe_tc && m->moe_wide && m->att_fast && c.d_model <= 8192 && c.n_experts % 4 == 0;
+}
+
+// One chunk of a prompt through all layers (Eq. moe_layer, primary path alone: fan-out k_1): Q|K|V, attention, O, router,
+// top-k, sort, gather, the routed experts' gate|up and down, the shared expert's gate|up, and its down projection, whose
+// epilogue also takes the routed experts' rows into the residual.
+dbt_status run_layers_moe_prompt(dbt_model *m, const RowMap &rm) {
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const int R = rm.B * rm.cn, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
+    const int E = c.n_experts, Fe = c.d_expert, Fs = c.n_shared_experts * Fe, km = kmax_of(c), Rk = (int)sorted_rows(c);
+    const size_t lo_x = (size_t)m->Rmax * d, lo_xs = (size_t)Rk * d, lo_hs = (size_t)Rk * Fe;
+    double kv_bytes = 0;
+    for (int b = 0; b < rm.B; b++)
+        for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * 2;
+    dbt_status st;
+    int ss_tiles = wide_ss_tiles(m);
+    for (int l = 0; l < c.n_layers; l++) {
+        const dbt_layer_weights &lw = m->layers[l];
+        const LayerMaps &mp = m->maps[l];
+        if ((st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, R,
+                                          prompt_qkv_params(m, rm, l, ss_tiles))) != DBT_OK)
+            return st;
+        st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, 0, l, kv_bytes, nullptr, true, false)
+                               : run_attention_mma<64>(m, rm, 0, l, kv_bytes, nullptr, true, false);
+        if (st != DBT_OK) return st;
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R,
+                                            prompt_resid_params(m, lw.mlp_norm_g))) != DBT_OK)
+            return st;
+        ss_tiles = prompt_ss_tiles(m);
+        PgParams rt{};
+        rt.ss_in = w.ss; rt.ss_tiles = ss_tiles; rt.ss_ld = m->Rmax; rt.d_norm = d; rt.eps = c.rms_eps;
+        rt.P = w.rlogits; rt.ldp = E;
+        if ((st = run_gemm_prompt<PG_STORE, 64>(m, "router", &mp.rt32, nullptr, nullptr, {E, 0, 0}, 1, &m->map_Xb, d, R, rt)) != DBT_OK) return st;
+        LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.rlogits, 1, (size_t)0, E, R, c.k_primary, c.k_branch, km, 0, w.ridx,
+               w.rwts, (int32_t *)nullptr, 0, (const float *)nullptr, 0, 0, d, c.rms_eps);
+        LAUNCH(m, "moe_sort", 0, moe_sort_kernel, 1, 1024, 0, w.ridx, R, km, E, w.ecnt, w.eoff, w.epos, (int32_t *)nullptr);
+        LAUNCH(m, "moe_gather", 0, moe_gather_rows_kernel, R, 256, 0, w.Xb, lo_x, w.ridx, w.epos, km, c.k_primary, d, w.Xs, lo_xs, w.ss, ss_tiles,
+               m->Rmax, c.rms_eps, w.rs_sorted);
+        GgParams g{};
+        g.E = E; g.cnt = w.ecnt; g.off = w.eoff; g.lo_row0 = Rk; g.status = w.status;
+        g.K = d; g.n_feat = Fe; g.rs = w.rs_sorted; g.H = w.Hs; g.h_lo = lo_hs;
+        const int grid = m->num_sms / 2 * 2;
+        LAUNCH(m, "expert_gateup", 0, gemm_group_kernel<GG_GATEUP>, grid, kPgThreads, kGgSmemBytes, mp.eg64, mp.eu64, m->map_Xs, g);
+        g.K = Fe; g.n_feat = d; g.Y = w.Yexp;
+        LAUNCH(m, "expert_down", 0, gemm_group_kernel<GG_DOWN>, grid, kPgThreads, kGgSmemBytes, mp.ed, mp.ed, m->map_Hs, g);
+        const float *g_next = l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : nullptr;
+        if (Fs > 0) {
+            PgParams sg{};
+            sg.ss_in = w.ss; sg.ss_tiles = ss_tiles; sg.ss_ld = m->Rmax; sg.d_norm = d; sg.eps = c.rms_eps;
+            sg.H = w.Hb; sg.h_lo = (size_t)m->Rmax * Fs; sg.F = Fs;
+            if ((st = run_gemm_prompt<PG_GATEUP>(m, "shared_gateup", &mp.wg, &mp.wu, nullptr, {Fs, 0, 0}, 1, &m->map_Xb, d, R, sg)) != DBT_OK) return st;
+            PgParams sd = prompt_resid_params(m, g_next);
+            sd.Y = w.Yexp; sd.sel_idx = w.ridx; sd.sel_pos = w.epos; sd.sel_wts = w.rwts; sd.kmax = km; sd.k = c.k_primary;
+            if ((st = run_gemm_prompt<PG_COMBINE>(m, "shared_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, Fs, R, sd)) != DBT_OK) return st;
+        } else {
+            LAUNCH(m, "moe_combine", 0, moe_combine_rows_kernel, dim3((R + 3) / 4, (d + 255) / 256), 256, 0, w.Yexp, (const float *)nullptr, 1,
+                   (size_t)0, w.ridx, w.epos, w.rwts, km, R, d, w.S, g_next, g_next ? w.Xb : (__nv_bfloat16 *)nullptr, lo_x,
+                   g_next ? w.ss : (float *)nullptr, m->Rmax);
+            ss_tiles = wide_ss_tiles(m);
+        }
     }
     return DBT_OK;
 }
@@ -1482,6 +1489,41 @@ dbt_status step_wide(dbt_model *m, const int32_t *tokens_dev, int B, int grouped
     return DBT_OK;
 }
 
+dbt_status prefill_tc(dbt_model *m, const int32_t *tokens_dev, int B, int n, float *last_logits) {
+    typedef __nv_bfloat16 WT;
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const bool big = moe_prompt_ok(m);
+    int cn_max = (big ? m->Rmax : (m->Rmax < 256 ? m->Rmax : 256)) / B;
+    if (cn_max < 1) cn_max = 1;
+    dbt_status st;
+    for (int p0 = 0; p0 < n; p0 += cn_max) {
+        int cn = n - p0 < cn_max ? n - p0 : cn_max;
+        RowMap rm{B, cn};
+        int R = B * cn, n_tile = pad_rows(R);
+        const int tok_n = m->tok_stride > 1 ? m->tok_stride : n;
+        int mode = 0, nsp = 1;
+        size_t sstride = 0;
+        if (big && cn > 1 && R > 256) {
+            if ((st = run_embed_wide<WT>(m, tokens_dev, tok_n, p0, rm, R, n_tile)) != DBT_OK) return st;
+            if ((st = run_layers_moe_prompt(m, rm)) != DBT_OK) return st;
+        } else {
+            LAUNCH(m, "embed", 0, embed_norm_kernel<WT>, R, 256, 0, tokens_dev, tok_n, p0, rm, (const WT *)m->w.embed_primary,
+                   (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S, w.status);
+            if ((st = run_layers_tc(m, rm, 0, n_tile, false, &mode, &nsp, &sstride)) != DBT_OK) return st;
+        }
+        bool last = p0 + cn >= n;
+        if (last && last_logits) {
+            if ((st = run_head_tc(m, R, 0, B, cn, cn - 1, pad_rows(B), mode, nsp, sstride)) != DBT_OK) return st;
+            CUDA_TRY(m, cudaMemcpyAsync(last_logits, w.Z, sizeof(float) * (size_t)B * c.vocab, cudaMemcpyDeviceToDevice,
+                                        m->stream));
+        }
+        LAUNCH(m, "advance_len", 0, advance_len_kernel, (B + 127) / 128, 128, 0, w.seq_len, B, cn);
+    }
+    for (int b = 0; b < B; b++) m->len_host[b] += n;
+    return DBT_OK;
+}
+
 dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, float *last_logits) {
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
@@ -1521,8 +1563,6 @@ bool allow_smem() {
 bool allow_smem_all() {
     return allow_smem<16>() && allow_smem<32>() && allow_smem<64>() && allow_smem<128>() && allow_smem<256>() &&
            cudaFuncSetAttribute(gemm_tc_kernel<256, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<256, 2>::kSmemBytes) ==
-               cudaSuccess &&
-           cudaFuncSetAttribute(gemm_tc_kernel<64, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcCfg<64, 2>::kSmemBytes) ==
                cudaSuccess;
 }
 
@@ -1531,7 +1571,10 @@ bool allow_smem_pg() {
     return cudaFuncSetAttribute(gemm_prompt_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PgCfg<N>::kSmemBytes) == cudaSuccess;
 }
 bool allow_smem_prompt() {
-    return allow_smem_pg<256, PG_STORE>() && allow_smem_pg<256, PG_QKV>() && allow_smem_pg<256, PG_RESID>() && allow_smem_pg<256, PG_GATEUP>();
+    return allow_smem_pg<256, PG_QKV>() && allow_smem_pg<256, PG_RESID>() && allow_smem_pg<256, PG_GATEUP>() &&
+           allow_smem_pg<256, PG_COMBINE>() && allow_smem_pg<64, PG_STORE>() &&
+           cudaFuncSetAttribute(gemm_group_kernel<GG_GATEUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess &&
+           cudaFuncSetAttribute(gemm_group_kernel<GG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess;
 }
 
 // Build the TMA descriptors of a bf16 model.  Returns false when the path cannot be used.
@@ -1558,7 +1601,8 @@ bool setup_tc(dbt_model *m) {
     }
     m->moe_tc = false;
     if (moe && ok) {
-        int E = c.n_experts, Fe = c.d_expert, Fs = c.n_shared_experts * Fe, Rk = m->Rmax * kmax_of(c);
+        int E = c.n_experts, Fe = c.d_expert, Fs = c.n_shared_experts * Fe;
+        const size_t Rk = sorted_rows(c);
         const char *mo = getenv("DBT_MOE");
         bool want = !(mo && strcmp(mo, "simt") == 0);
         bool mok = want;
@@ -1568,7 +1612,8 @@ bool setup_tc(dbt_model *m) {
             mok = make_bf16_map(&mp.eg, lw.exp_gate, (uint64_t)E * Fe, d, kTcM) &&
                   make_bf16_map(&mp.eu, lw.exp_up, (uint64_t)E * Fe, d, kTcM) &&
                   make_bf16_map(&mp.ed, lw.exp_down, (uint64_t)E * d, Fe, kTcM) &&
-                  make_bf16_map(&mp.rt, lw.router, E, d, kTcM);
+                  make_bf16_map(&mp.rt, lw.router, E, d, kTcM) && make_bf16_map(&mp.eg64, lw.exp_gate, (uint64_t)E * Fe, d, 64) &&
+                  make_bf16_map(&mp.eu64, lw.exp_up, (uint64_t)E * Fe, d, 64) && make_bf16_map(&mp.rt32, lw.router, E, d, 32);
             if (mok && Fs > 0)
                 mok = make_bf16_map(&mp.wg, lw.sh_gate, Fs, d, kTcM) && make_bf16_map(&mp.wu, lw.sh_up, Fs, d, kTcM) &&
                       make_bf16_map(&mp.wd, lw.sh_down, d, Fs, kTcM);
@@ -1649,7 +1694,7 @@ template <typename WT>
 dbt_status prefill_impl(dbt_model *m, const int32_t *tokens_dev, int B, int n, float *last_logits) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
-    int cn_max = m->Rmax / B;
+    int cn_max = decode_rows(c) / B;
     if (cn_max < 1) cn_max = 1;
     dbt_status st;
     for (int p0 = 0; p0 < n; p0 += cn_max) {
@@ -1763,8 +1808,6 @@ dbt_status dbt_create(const dbt_config *cfg, const dbt_weights *w, void *kv_pool
         m->moe_persist = !mp ? -1 : strcmp(mp, "1") == 0 ? 1 : 0;
         const char *fs = getenv("DBT_MOE_FUSE_SWIGLU");
         m->moe_fuse_swiglu = !(fs && strcmp(fs, "0") == 0);
-        const char *pf = getenv("DBT_PROMPT_FUSE_SWIGLU");
-        m->prompt_fuse_swiglu = !(pf && strcmp(pf, "0") == 0);
     }
     const char *ro = getenv("DBT_READOUT");
     m->readout_row = ro && strcmp(ro, "row") == 0;

@@ -400,37 +400,6 @@ __device__ __forceinline__ float4 sum_splits4(const float *P, size_t split_strid
     return m;
 }
 
-// swiglu_couple_kernel for R primary rows: H = SiLU(rs * gate) * (rs * up) as two planes.
-// grid (R, ceil(F / 1024)).  F % 4 == 0.
-__global__ void __launch_bounds__(256) swiglu_rows_kernel(const float *P, int nsplit, size_t split_stride, int F,
-                                                          __nv_bfloat16 *Hb, size_t lo_off, const float *ss, int ss_tiles,
-                                                          int ss_ld, int d_norm, float eps) {
-    pdl_launch_dependents();
-    __shared__ float rs_s;
-    const int row = blockIdx.x, f = (blockIdx.y * 256 + threadIdx.x) * 4;
-    pdl_wait();
-    float a = 0.f;
-    if (ss && threadIdx.x < 32)
-        for (int t = threadIdx.x; t < ss_tiles; t += 32) a += __ldcg(ss + (size_t)t * ss_ld + row);
-    float4 gt = make_float4(0.f, 0.f, 0.f, 0.f), up = gt;
-    if (f < F) {
-        size_t o = (size_t)row * 2 * F + f;
-        gt = sum_splits4(P, split_stride, nsplit, o);
-        up = sum_splits4(P, split_stride, nsplit, o + F);
-    }
-    if (threadIdx.x < 32) {
-        a = warp_sum(a);
-        if (threadIdx.x == 0) rs_s = ss ? 1.f / sqrtf(a / (float)d_norm + eps) : 1.f;
-    }
-    __syncthreads();
-    if (f < F) {
-        const float rs = rs_s;
-        float4 h = make_float4(silu(rs * gt.x) * (rs * up.x), silu(rs * gt.y) * (rs * up.y), silu(rs * gt.z) * (rs * up.z),
-                               silu(rs * gt.w) * (rs * up.w));
-        store_split4(Hb, (size_t)row * F + f, lo_off, h);
-    }
-}
-
 // Eq. embeddings for the fused path: S^0 = RMSNorm(E[x]) and, for the first layer's Q|K|V GEMM,
 // the input g_next * S^0 as two bf16 planes plus sum(S^0 ^2) per row (tile 0 carries the whole
 // sum, the other tile slots are zeroed).  One block per row.
@@ -576,6 +545,46 @@ __global__ void __launch_bounds__(256) moe_gather_kernel(const __nv_bfloat16 *Xb
         if (lo_out) dst[i + lo_out / 8] = src[i + lo_in / 8];
     }
     DBT_TL_END("moe_gath");
+}
+
+// moe_gather_kernel for a prompt chunk: a block takes a row, requests it before its positions are known, and writes a
+// copy per selection.  d % 8 == 0, d <= 8192.
+__global__ void __launch_bounds__(256) moe_gather_rows_kernel(const __nv_bfloat16 *Xb, size_t lo_in, const int32_t *idx, const int32_t *pos,
+                                                              int kmax, int k, int d, __nv_bfloat16 *Xs, size_t lo_out, const float *ss,
+                                                              int ss_tiles, int ss_ld, float eps, float *rs_sorted) {
+    pdl_enter();
+    const int row = blockIdx.x, nv = d / 8;
+    const uint4 *src = reinterpret_cast<const uint4 *>(Xb + (size_t)row * d);
+    constexpr int NV = 4;
+    uint4 hi[NV], lo[NV];
+#pragma unroll
+    for (int u = 0; u < NV; u++) {
+        const int i = threadIdx.x + u * 256;
+        if (i < nv) {
+            hi[u] = __ldcg(src + i);
+            lo[u] = __ldcg(src + lo_in / 8 + i);
+        }
+    }
+    float a = 0.f;
+    if (threadIdx.x < 32)
+        for (int t = threadIdx.x; t < ss_tiles; t += 32) a += __ldcg(ss + (size_t)t * ss_ld + row);
+    for (int j = 0; j < k; j++) {
+        if (__ldcg(idx + (size_t)row * kmax + j) < 0) continue;
+        const int ps = __ldcg(pos + (size_t)row * kmax + j);
+        uint4 *dst = reinterpret_cast<uint4 *>(Xs + (size_t)ps * d);
+#pragma unroll
+        for (int u = 0; u < NV; u++) {
+            const int i = threadIdx.x + u * 256;
+            if (i < nv) {
+                dst[i] = hi[u];
+                dst[i + lo_out / 8] = lo[u];
+            }
+        }
+        if (threadIdx.x < 32) {
+            const float q = warp_sum(a);
+            if (threadIdx.x == 0) rs_sorted[ps] = 1.f / sqrtf(q / (float)d + eps);
+        }
+    }
 }
 
 // H = SiLU(gate) * up on the sorted rows; Pe rows are [Fe gate | Fe up] (one split).  rs (nullable):

@@ -29,6 +29,8 @@ enum PgMode {
     PG_QKV = 1,     // 1/rms, RoPE on Q and K, Q out, K and V appended to the paged cache
     PG_RESID = 2,   // S += acc; the next GEMM's input g * S (two planes) and each row's share of sum(S^2)
     PG_GATEUP = 3,  // H = SiLU(rs * gate) * (rs * up), two planes
+    PG_COMBINE = 4,  // PG_RESID behind an MoE layer's shared expert: the routed experts' rows join the residual too,
+                     // S += acc + sum_j wts[r][j] Y[pos[r][j]] over the row's k selections (idx < 0: none)
 };
 
 constexpr int kPgM = 256;         // activation rows of a pair's tile
@@ -44,6 +46,10 @@ struct PgSeg {
 
 struct PgParams {
     int K, R, m_tiles, tiles;  // tiles: m_tiles x feature tiles
+    // Order of the tiles: groups of m_group row tiles, in a group feature tile by feature tile.  The pairs that run at
+    // once then share about as many row tiles as weight tiles (9 x 8 of 74), whatever the chunk: with all 32 row tiles of
+    // an 8192-row chunk side by side the 8B shape's gate|up re-read its 134 MB of activations from HBM (97 us per row tile).
+    int m_group;
     PgSeg seg[3];
     int nseg;
     int *status;
@@ -61,6 +67,11 @@ struct PgParams {
     size_t x_lo;
     float *ss_out;  // [feature tile * 2 + half][ss_ld]
     int d;
+    // PG_COMBINE
+    const float *Y;
+    const int32_t *sel_idx, *sel_pos;
+    const float *sel_wts;
+    int kmax, k;
     // PG_GATEUP
     __nv_bfloat16 *H;
     size_t h_lo;
@@ -233,6 +244,12 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
     const uint32_t tmem_base = *tmem_holder;
     pdl_launch_dependents();
 
+    const int n_tiles = p.tiles / p.m_tiles;
+    auto tile_of = [&](int t, int &mt, int &nt) {
+        const int per = p.m_group * n_tiles, gr = t / per, m0 = gr * p.m_group, in = t - gr * per, gm = min(p.m_group, p.m_tiles - m0);
+        nt = in / gm;
+        mt = m0 + in - nt * gm;
+    };
     // feature tile -> matrix, first feature
     auto seg_of = [&](int nt) { return p.nseg > 2 && nt >= p.seg[2].tile0 ? 2 : p.nseg > 1 && nt >= p.seg[1].tile0 ? 1 : 0; };
     constexpr int kTileF = MODE == PG_GATEUP ? N / 2 : N;  // features of one tile (gate|up: N / 2 of each matrix)
@@ -263,15 +280,17 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                 tma2_load_3d(ring + s * Cfg::kStageBytes, &tmX, mapa_u32(full_bar(s), 0), kt * kTcK, mt * kPgM + (int)rank * 128, 0);
             };
             const int npre = pair < p.tiles ? min(STAGES, nkt) : 0;
+            int mt, nt;
+            tile_of(pair, mt, nt);
             for (int i = 0; i < npre; i++) {
                 if (rank == 0) mbar_expect_tx(full_bar(i), 2 * Cfg::kStageBytes);
-                load_w(i, pair / p.m_tiles, i);
+                load_w(i, nt, i);
             }
             pdl_wait();
-            for (int i = 0; i < npre; i++) load_x(i, pair % p.m_tiles, i);
+            for (int i = 0; i < npre; i++) load_x(i, mt, i);
             int it = 0;  // stages requested so far, over all tiles
             for (int t = pair; t < p.tiles && ok; t += npairs) {
-                const int mt = t % p.m_tiles, nt = t / p.m_tiles;
+                tile_of(t, mt, nt);
                 for (int kt = 0; kt < nkt; kt++, it++) {
                     if (it < npre) continue;
                     const int s = it % STAGES;
@@ -322,7 +341,9 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
         pdl_wait();
         int n_acc = 0;
         for (int t = pair; t < p.tiles; t += npairs, n_acc++) {
-            const int a = n_acc & 1, mt = t % p.m_tiles, nt = t / p.m_tiles;
+            const int a = n_acc & 1;
+            int mt, nt;
+            tile_of(t, mt, nt);
             const int sg = seg_of(nt), f0 = (nt - p.seg[sg].tile0) * kTileF;
             const int row0 = mt * kPgM + (int)rank * 128 + quad * 32, row = row0 + lane;
             const bool on = row < p.R;
@@ -330,35 +351,62 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
             if (MODE == PG_QKV || MODE == PG_GATEUP || MODE == PG_STORE)
                 rs = row_scale(p.ss_in, p.ss_tiles, p.ss_ld, on ? row : 0, p.d_norm, p.eps);
             const uint32_t tacc = lane_base + a * N;
-            ok = mbar_wait_cluster(acc_full(a), (n_acc >> 1) & 1);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if constexpr (MODE == PG_STORE || MODE == PG_RESID) {
+            auto acc_ready = [&] {
+                bool r = mbar_wait_cluster(acc_full(a), (n_acc >> 1) & 1);
+                ok = r = __all_sync(0xffffffffu, r);
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                return r;
+            };
+            if constexpr (MODE == PG_STORE || MODE == PG_RESID || MODE == PG_COMBINE) {
                 // Chunks of 32 columns go through a 4 KB staging tile of the warp (16-byte pieces, XOR-swizzled by row),
                 // so that global memory sees 128-byte row pieces: lane l then holds columns 4 (l % 8) .. of row 4 i + l / 8.
+                // What a chunk adds to the accumulator is requested a chunk ahead (the first before the accumulator is
+                // there): the epilogue would otherwise wait for memory once per chunk, longer than the next tile's MMAs take.
+                constexpr bool kResid = MODE != PG_STORE;
+                constexpr int kPre = MODE == PG_COMBINE ? 2 : 0;  // selections whose rows are requested ahead
                 const int c4 = (lane & 7) * 4, rsub = lane >> 3;
                 float sq[8];
 #pragma unroll
                 for (int i = 0; i < 8; i++) sq[i] = 0.f;
                 const int cbase = half * (N / 2);
+                int ps[kPre + 1];
+                float wt[kPre + 1];
+                if (MODE == PG_COMBINE) {  // this lane's own row's first selections
+#pragma unroll
+                    for (int j = 0; j < kPre; j++) {
+                        const size_t o = (size_t)row * p.kmax + j;
+                        const bool sel = on && j < p.k && __ldcg(p.sel_idx + o) >= 0;
+                        ps[j] = sel ? __ldcg(p.sel_pos + o) : -1;
+                        wt[j] = sel ? __ldcg(p.sel_wts + o) : 0.f;
+                    }
+                }
+                float4 s4[8], y4[kPre > 0 ? kPre : 1][8];
+                auto request = [&](int c) {
+                    const int col = f0 + cbase + c + c4;
+                    const bool con = col < p.seg[sg].n_out;
+#pragma unroll
+                    for (int i = 0; i < 8; i++) {
+                        const int rl = i * 4 + rsub, r = row0 + rl;
+                        s4[i] = con && r < p.R ? ldcg4(p.S + (size_t)r * p.d + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int j = 0; j < kPre; j++) {
+                            const int q = __shfl_sync(0xffffffffu, ps[j], rl);
+                            y4[j][i] = con && q >= 0 ? ldcg4(p.Y + (size_t)q * p.d + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                    }
+                };
+                if (kResid) request(0);
+                if (!acc_ready()) break;
 #pragma unroll 1
                 for (int c = 0; c < N / 2; c += 32) {
                     const int col = f0 + cbase + c + c4;  // this lane's first column
                     const bool con = col < p.seg[sg].n_out;
-                    float4 s4[8], gn = make_float4(1.f, 1.f, 1.f, 1.f);
-                    if (MODE == PG_RESID) {
-                        if (p.g_next && con) gn = *reinterpret_cast<const float4 *>(p.g_next + col);
-#pragma unroll
-                        for (int i = 0; i < 8; i++) {
-                            const int r = row0 + i * 4 + rsub;
-                            s4[i] = con && r < p.R ? ldcg4(p.S + (size_t)r * p.d + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-                    }
                     uint32_t v[2][16];
                     __syncwarp();  // the staging tile has been read
                     tmem_ld16_issue(tacc + cbase + c, v[0]);
                     tmem_ld16_issue(tacc + cbase + c + 16, v[1]);
+                    float4 gn = make_float4(1.f, 1.f, 1.f, 1.f);
+                    if (kResid && p.g_next && con) gn = *reinterpret_cast<const float4 *>(p.g_next + col);
                     tmem_ld_wait();
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
@@ -367,6 +415,36 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         *reinterpret_cast<float4 *>(stg + lane * 32 + ((j ^ (lane & 7)) << 2)) = x;
                     }
                     __syncwarp();
+                    float4 add[8];
+                    if (kResid) {
+#pragma unroll
+                        for (int i = 0; i < 8; i++) {
+                            float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                            for (int j = 0; j < kPre; j++) {
+                                const float g = __shfl_sync(0xffffffffu, wt[j], i * 4 + rsub);
+                                m.x = fmaf(g, y4[j][i].x, m.x), m.y = fmaf(g, y4[j][i].y, m.y);
+                                m.z = fmaf(g, y4[j][i].z, m.z), m.w = fmaf(g, y4[j][i].w, m.w);
+                            }
+                            add[i] = make_float4(s4[i].x + m.x, s4[i].y + m.y, s4[i].z + m.z, s4[i].w + m.w);
+                        }
+                        if (MODE == PG_COMBINE && p.k > kPre && con) {  // wider fan-outs: the further selections' rows
+#pragma unroll
+                            for (int i = 0; i < 8; i++) {
+                                const int r = row0 + i * 4 + rsub;
+                                if (r >= p.R) continue;
+                                for (int j = kPre; j < p.k; j++) {
+                                    const size_t o = (size_t)r * p.kmax + j;
+                                    if (__ldcg(p.sel_idx + o) < 0) continue;
+                                    const float g = __ldcg(p.sel_wts + o);
+                                    const float4 y = ldcg4(p.Y + (size_t)__ldcg(p.sel_pos + o) * p.d + col);
+                                    add[i].x = fmaf(g, y.x, add[i].x), add[i].y = fmaf(g, y.y, add[i].y);
+                                    add[i].z = fmaf(g, y.z, add[i].z), add[i].w = fmaf(g, y.w, add[i].w);
+                                }
+                            }
+                        }
+                        if (c + 32 < N / 2) request(c + 32);
+                    }
 #pragma unroll
                     for (int i = 0; i < 8; i++) {
                         const int rl = i * 4 + rsub, r = row0 + rl;
@@ -376,14 +454,14 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                             *reinterpret_cast<float4 *>(p.P + (size_t)r * p.ldp + p.seg[sg].col0 + col) = x;
                         } else {
                             const size_t o = (size_t)r * p.d + col;
-                            x.x += s4[i].x, x.y += s4[i].y, x.z += s4[i].z, x.w += s4[i].w;
+                            x.x += add[i].x, x.y += add[i].y, x.z += add[i].z, x.w += add[i].w;
                             *reinterpret_cast<float4 *>(p.S + o) = x;
                             store_split4(p.X, o, p.x_lo, make_float4(gn.x * x.x, gn.y * x.y, gn.z * x.z, gn.w * x.w));
                             sq[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
                         }
                     }
                 }
-                if (MODE == PG_RESID) {
+                if (kResid) {
 #pragma unroll
                     for (int i = 0; i < 8; i++) {
                         float q = sq[i];
@@ -395,6 +473,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     }
                 }
             } else if constexpr (MODE == PG_GATEUP) {
+                if (!acc_ready()) break;
                 const int fbase = half * (N / 4);
 #pragma unroll 1
                 for (int c = 0; c < N / 4; c += 16) {
@@ -419,6 +498,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     }
                 }
             } else {
+                if (!acc_ready()) break;
                 // PG_QKV: the tile holds N / dh whole heads of one of Q, K, V; the two warps of a lane quadrant take the
                 // first and the second half of every head's rotation pairs (i, i + dh / 2)
                 const int hd = p.dh, hh2 = hd >> 1, span = hd >> 2;

@@ -56,3 +56,14 @@ def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
     za, zb = a.prefill(tok, want_logits=True), b.prefill(tok, want_logits=True)
     assert torch.equal(za, zb) and torch.isfinite(za).all()
     assert torch.equal(a.export_kv(1, 333)[0], b.export_kv(1, 333)[0])
+
+
+@pytest.mark.parametrize("kw,B,n", [
+    (dict(n_experts=4, d_expert=200), 1, 700),                                  # lists of several row tiles of an expert
+    (dict(n_experts=64, d_expert=136, k_branch=2), 2, 150),                     # short lists, some experts without a row
+    (dict(n_experts=8, d_expert=328, n_shared_experts=0, k_branch=8), 1, 513),  # no shared expert: the combine kernel
+    (dict(n_experts=8, d_expert=128, n_shared_experts=2, k_primary=3, d_model=328), 1, 300),
+])
+def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n):
+    from test_gpu_parity import small_moe, test_moe_prompt_chunks_of_more_than_one_row_tile_match_the_oracle as check
+    check(small_moe(**kw), B, n, 0.05)
