@@ -23,6 +23,7 @@
 #include "dbt_gemm_prompt.cuh"
 #include "dbt_gemm_group.cuh"
 #include "dbt_kernels.cuh"
+#include "dbt_small.cuh"
 
 using namespace dbt;
 
@@ -576,6 +577,87 @@ dbt_status run_layers(dbt_model *m, const RowMap &rm, int grouped, bool record_e
     return DBT_OK;
 }
 
+// Whether a decode step of B sequences takes the few-row chain (dbt_small.cuh): fp32 dense models.  Decided from the
+// batch and the model, never from the mode, so that grouped and primary-only steps do the same arithmetic per row.
+bool small_step(const dbt_model *m, int B) {
+    const dbt_config &c = m->cfg;
+    return c.weight_dtype == DBT_DTYPE_F32 && c.n_experts == 0 && paths_of(c) * B <= kSmallRows &&
+           paths_of(c) * (c.n_q_heads / c.n_kv_heads) <= 8;
+}
+
+dbt_status run_small_linear(dbt_model *m, const char *tag, int B, const SmallLin &a) {
+    int total = 0;
+    double bytes = 0;
+    for (int s = 0; s < a.nseg; s++) total += a.n_out[s];
+    const bool swiglu = a.epi == EPI_SWIGLU;
+    bytes = (double)total * a.K * 4 * (swiglu ? 2 : 1);
+    const int grid = (total + kSmallWarps - 1) / kSmallWarps, block = kSmallWarps * 32;
+    const bool few = paths_of(m->cfg) * B <= 4;  // rows in flight at once
+    if (swiglu) {
+        if (few) LAUNCH(m, tag, bytes, (linear_small_kernel<float, 4, true>), grid, block, 0, a);
+        else LAUNCH(m, tag, bytes, (linear_small_kernel<float, 8, true>), grid, block, 0, a);
+    } else {
+        if (few) LAUNCH(m, tag, bytes, (linear_small_kernel<float, 4, false>), grid, block, 0, a);
+        else LAUNCH(m, tag, bytes, (linear_small_kernel<float, 8, false>), grid, block, 0, a);
+    }
+    return DBT_OK;
+}
+
+template <int DH>
+dbt_status run_small_attention(dbt_model *m, const SmallAttn &a, int nsplit, double kv_bytes) {
+    const int nq = paths_of(m->cfg) * a.G;
+    dim3 grid(a.B, a.n_kv, nsplit);
+    if (nq <= 2) LAUNCH(m, "attention", kv_bytes, (attn_small_kernel<2, DH>), grid, kSaThreads, 0, a);
+    else if (nq <= 4) LAUNCH(m, "attention", kv_bytes, (attn_small_kernel<4, DH>), grid, kSaThreads, 0, a);
+    else LAUNCH(m, "attention", kv_bytes, (attn_small_kernel<8, DH>), grid, kSaThreads, 0, a);
+    return DBT_OK;
+}
+
+// The layer stack and the shared output matrix of a decode step at few rows: five kernels per layer.
+dbt_status run_layers_small(dbt_model *m, int B, int grouped) {
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const int R = npaths(grouped) * B, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
+    const size_t pool_layer = (size_t)2 * c.num_pages * c.n_kv_heads * c.page_size * c.head_dim;
+    int nsplit = (2 * 148 + B * c.n_kv_heads - 1) / (B * c.n_kv_heads);
+    nsplit = nsplit < 1 ? 1 : nsplit > 16 ? 16 : nsplit;
+    double kv_bytes = 0;
+    for (int b = 0; b < B; b++) kv_bytes += (double)(m->len_host[b] + 1) * 2 * kvd * 4;
+    dbt_status st;
+    auto lin = [&](const void *W, float *Y, int n_out, const float *X, const float *g, int K, int epi) {
+        SmallLin a{};
+        a.W[0] = W; a.Y[0] = Y; a.n_out[0] = n_out; a.rows[0] = R; a.nseg = 1;
+        a.X = X; a.g = g; a.eps = c.rms_eps; a.K = K; a.epi = epi; a.Bc = B; a.S = w.S;
+        return a;
+    };
+    for (int l = 0; l < c.n_layers; l++) {
+        const dbt_layer_weights &lw = m->layers[l];
+        SmallLin q = lin(lw.wq, w.Q, qd, w.S, lw.attn_norm_g, d, EPI_STORE);
+        q.W[1] = lw.wk; q.Y[1] = w.Kn; q.n_out[1] = kvd; q.rows[1] = B;
+        q.W[2] = lw.wv; q.Y[2] = w.Vn; q.n_out[2] = kvd; q.rows[2] = B;
+        q.nseg = 3;
+        if ((st = run_small_linear(m, "linear_qkv", B, q)) != DBT_OK) return st;
+        SmallAttn t{};
+        t.Q = w.Q; t.Kn = w.Kn; t.Vn = w.Vn;
+        t.B = B; t.P = npaths(grouped); t.G = c.n_q_heads / c.n_kv_heads; t.n_kv = c.n_kv_heads;
+        t.coup_a = lw.coup_a; t.rope = w.rope; t.seq_len = w.seq_len; t.page_table = w.page_table;
+        t.pt_stride = m->pages_per_seq_max; t.num_pages = c.num_pages;
+        t.kpool = reinterpret_cast<float *>(m->kv_pool) + (size_t)l * pool_layer;
+        t.vpool = t.kpool + pool_layer / 2;
+        t.part = w.part; t.tickets = w.att_tickets; t.O = w.O; t.status = w.status;
+        st = c.head_dim == 128 ? run_small_attention<128>(m, t, nsplit, kv_bytes) : run_small_attention<64>(m, t, nsplit, kv_bytes);
+        if (st != DBT_OK) return st;
+        if ((st = run_small_linear(m, "linear_o", B, lin(lw.wo, nullptr, d, w.O, nullptr, qd, EPI_RESID))) != DBT_OK) return st;
+        SmallLin gu = lin(lw.w_gate, w.G1, c.d_ff, w.S, lw.mlp_norm_g, d, EPI_SWIGLU);
+        gu.W[1] = lw.w_up; gu.coup = lw.coup_b;
+        if ((st = run_small_linear(m, "linear_gateup", B, gu)) != DBT_OK) return st;
+        SmallLin dn = lin(lw.w_down, nullptr, d, w.G1, nullptr, c.d_ff, EPI_DOWN);
+        dn.coup = lw.coup_c;
+        if ((st = run_small_linear(m, "linear_down", B, dn)) != DBT_OK) return st;
+    }
+    return run_small_linear(m, "lm_head", B, lin(m->w.lm_head, w.Z, c.vocab, w.S, c.final_norm ? m->w.final_norm_g : nullptr, d, EPI_STORE));
+}
+
 // Final norm + shared output matrix on `rows` rows taken from S (row r*src_mul+src_add).
 template <typename WT>
 dbt_status run_head(dbt_model *m, int rows, int src_mul, int src_add) {
@@ -1046,7 +1128,7 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
                                     m->stream));
     LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.P, rnsp, rstride, E, Bc, c.k_primary, c.k_branch, km,
            c.router_mode == DBT_ROUTER_REPLAY, w.ridx, w.rwts, last, c.max_batch * km, ssp, ss_tiles, ss_ld, d, c.rms_eps);
-    LAUNCH(m, "moe_sort", 0, moe_sort_kernel, 1, R * km > 512 ? 1024 : (E + 31) / 32 * 32 < 64 ? 64 : (E + 31) / 32 * 32, 0, w.ridx, R, km, E, w.ecnt, w.eoff, w.epos,
+    LAUNCH(m, "moe_sort", 0, moe_sort_kernel, 1, R * km > 512 || E > 256 ? 1024 : 256, 0, w.ridx, R, km, E, w.ecnt, w.eoff, w.epos,
            record_experts ? w.union_cnt + l : (int32_t *)nullptr);
     LAUNCH(m, "moe_gather", 0, moe_gather_kernel, R * km, 256, 0, w.Xb, lo_x, w.ridx, w.epos, km, d, w.Xs, lo_xs, ssp, ss_tiles, ss_ld,
            c.rms_eps, w.rs_sorted);
@@ -1677,8 +1759,12 @@ dbt_status step_impl(dbt_model *m, const int32_t *tokens_dev, int B, int grouped
     dbt_status st;
     LAUNCH(m, "embed", 0, embed_norm_kernel<WT>, R, 256, 0, tokens_dev, m->tok_stride, m->tok_p0, rm, (const WT *)m->w.embed_primary,
            (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S, w.status);
-    if ((st = run_layers<WT>(m, rm, grouped, true)) != DBT_OK) return st;
-    if ((st = run_head<WT>(m, R, 1, 0)) != DBT_OK) return st;
+    if (small_step(m, B)) {
+        if ((st = run_layers_small(m, B, grouped)) != DBT_OK) return st;
+    } else {
+        if ((st = run_layers<WT>(m, rm, grouped, true)) != DBT_OK) return st;
+        if ((st = run_head<WT>(m, R, 1, 0)) != DBT_OK) return st;
+    }
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
     if ((st = run_readout(m, B, grouped, next_dev, alpha_dev)) != DBT_OK) return st;
     size_t zb = sizeof(float) * (size_t)B * c.vocab;
