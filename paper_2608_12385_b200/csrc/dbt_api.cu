@@ -63,7 +63,7 @@ struct LayerMaps {
     CUtensorMap wq, wk, wv, wo, wg, wu, wd;  // dense MLP; for MoE wg/wu/wd hold the shared expert
     CUtensorMap eg, eu, ed;                  // all routed experts as [E*Fe, d], [E*Fe, d], [E*d, Fe]
     CUtensorMap rt;                          // router [E, d]
-    CUtensorMap eg64, eu64, rt32;            // the same matrices in boxes of 64 / 32 rows (prompt chunks)
+    CUtensorMap eg64, eu64;                  // the experts' in boxes of 64 rows (prompt chunks)
 };
 
 }  // namespace
@@ -103,6 +103,10 @@ struct dbt_model {
     struct ActBase { const void *base; };
     std::map<const CUtensorMap *, ActBase> act_base;
     std::map<std::tuple<const CUtensorMap *, int, int>, CUtensorMap> act3d;
+    // a weight matrix behind its 128-row map, and its views in boxes of other heights, built on first use
+    struct WeightBase { const void *base; uint64_t rows, K; };
+    std::map<const CUtensorMap *, WeightBase> w_base;
+    std::map<std::pair<const CUtensorMap *, int>, CUtensorMap> w_view;
     bool evict_first;  // weight tiles and K/V pages carry the evict-first L2 hint (DBT_EVICT_FIRST=0 turns it off)
     int moe_persist;       // per-expert GEMMs as persistent CTAs over the units that have work: -1 by the batch, DBT_MOE_PERSIST=0/1 off/on
     int cur_rows;          // primary rows (sequences x positions) of the launch plan being built
@@ -276,8 +280,8 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
         w.P_floats = want < cap ? want : cap;
         if (w.P_floats < (size_t)Rd * widest) w.P_floats = (size_t)Rd * widest;
         w.P = k.take<float>(w.P_floats);
-        // shares of sum(S^2): 256 columns each in decode steps, half a 256-feature tile in prompt chunks
-        w.ss = k.take<float>((size_t)((d + 255) / 256 * 2) * Rmax);
+        // shares of sum(S^2): 256 columns each in decode steps, up to eight per 256-feature tile in prompt chunks
+        w.ss = k.take<float>((size_t)((d + 255) / 256 * 8) * Rmax);
         if (moe) {
             const size_t Rk = sorted_rows(c);
             w.Xs = k.take<__nv_bfloat16>(2 * Rk * d);
@@ -322,15 +326,21 @@ dbt_status fail(dbt_model *m, dbt_status st, const char *fmt, ...) {
 // stream-serialization attribute, so the kernel may start while its predecessor drains.  Each
 // kernel calls griddepcontrol.wait before it touches anything its predecessor produced.
 template <typename... Params, typename... Args>
-cudaError_t launch_kernel(cudaStream_t stream, bool pdl, dim3 grid, dim3 block, size_t smem,
+cudaError_t launch_kernel(cudaStream_t stream, bool pdl, unsigned cluster, dim3 grid, dim3 block, size_t smem,
                           void (*kernel)(Params...), Args &&...args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     int n = 0;
+    if (cluster > 0) {  // (0: the kernel's own compile-time cluster, or none)
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = cluster;
+        attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+        n++;
+    }
     if (pdl) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n].val.programmaticStreamSerializationAllowed = 1;
@@ -366,7 +376,8 @@ cudaEvent_t prof_event(dbt_model *m) {
 }
 
 // tag: kernel family name for the profile; bytes: the algorithmic bytes this launch must move.
-#define LAUNCH(m, tag, bytes, kernel, grid, block, smem, ...)                                            \
+#define LAUNCH(m, tag, bytes, kernel, grid, block, smem, ...) LAUNCH_CLUSTER(m, tag, bytes, 0, kernel, grid, block, smem, __VA_ARGS__)
+#define LAUNCH_CLUSTER(m, tag, bytes, cluster, kernel, grid, block, smem, ...)                           \
     do {                                                                                                 \
         cudaEvent_t p0_ = nullptr, p1_ = nullptr;                                                        \
         if ((m)->prof_on) {                                                                              \
@@ -374,7 +385,7 @@ cudaEvent_t prof_event(dbt_model *m) {
             p1_ = prof_event(m);                                                                         \
             cudaEventRecord(p0_, (m)->stream);                                                           \
         }                                                                                                \
-        cudaError_t e_ = launch_kernel((m)->stream, (m)->use_pdl && !pdl_disabled_for(m, tag), dim3(grid),       \
+        cudaError_t e_ = launch_kernel((m)->stream, (m)->use_pdl && !pdl_disabled_for(m, tag), cluster, dim3(grid), \
                                        dim3(block), smem, kernel, __VA_ARGS__);                          \
         (m)->launches++;                                                                                 \
         if ((m)->prof_on) {                                                                              \
@@ -722,6 +733,131 @@ int split_slots(const dbt_model *m, int n_tile) {
     return (n_tile <= 64 ? 2 : 1) * sms;
 }
 
+// ---- GEMMs of prompt chunks on pairs of SMs (dbt_gemm_prompt.cuh) -----------------------------------------
+
+// The 3-D one-box view of a two-plane GEMM input, built on first use.
+const CUtensorMap *act_view(dbt_model *m, const CUtensorMap *X, int box_rows, int K) {
+    auto reg = m->act_base.find(X);
+    if (reg == m->act_base.end()) return nullptr;
+    auto key = std::make_tuple(X, box_rows, m->Rmax);
+    auto hit = m->act3d.find(key);
+    if (hit == m->act3d.end()) {
+        CUtensorMap t;
+        if (!make_act_map(&t, reg->second.base, (uint64_t)m->Rmax, (uint64_t)K, box_rows)) return nullptr;
+        hit = m->act3d.emplace(key, t).first;
+    }
+    return &hit->second;
+}
+
+const CUtensorMap *weight_view(dbt_model *m, const CUtensorMap *W, int box_rows) {
+    if (box_rows == kTcM) return W;
+    auto reg = m->w_base.find(W);
+    if (reg == m->w_base.end()) return nullptr;
+    auto key = std::make_pair(W, box_rows);
+    auto hit = m->w_view.find(key);
+    if (hit == m->w_view.end()) {
+        CUtensorMap t;
+        if (!make_bf16_map(&t, reg->second.base, reg->second.rows, reg->second.K, box_rows)) return nullptr;
+        hit = m->w_view.emplace(key, t).first;
+    }
+    return &hit->second;
+}
+
+// Tile width and split of one such GEMM, by the time it takes (us, measured on its parts): a k-tile costs the MMAs of N
+// columns (4 N cycles) or what an SM takes in for it (32 KB of rows and 64 N bytes of weights at ~50 bytes per cycle); a
+// tile's first loads and its end 4.5 us, its epilogue up to 4; an exchange 4.4 at N = 256.  Unsplit tiles follow each other
+// on persistent pairs, split ones start anew: 15 clusters of 8 CTAs and about 34 of 4 are resident at a time.
+struct PgPlan {
+    int N, splits;
+};
+PgPlan plan_gemm_prompt(const dbt_model *m, PgMode mode, const int (&n_out)[3], int nseg, int K, int R) {
+    const int widths[] = {256, 192, 128};
+    const int total_kt = (K + kTcK - 1) / kTcK, mt = (R + kPgM - 1) / kPgM;
+    PgPlan best{256, 1};
+    double best_cost = 1e30;
+    for (int N : widths) {
+        if (N == 128 && mode != PG_STORE) continue;
+        if (N == 192 && mode != PG_STORE && mode != PG_GATEUP) continue;
+        for (int S = 1; S <= 4; S *= 2) {
+            if (S > 1 && (mode == PG_GATEUP || mode == PG_COMBINE || N == 192)) continue;  // (slices are multiples of 32 columns)
+            if (mode == PG_QKV && N / S % m->cfg.head_dim) continue;
+            const int kps = (total_kt + S - 1) / S;
+            if ((S - 1) * kps >= total_kt) continue;
+            int tiles = 0;
+            for (int s = 0; s < nseg; s++) tiles += (n_out[s] + (mode == PG_GATEUP ? N / 2 : N) - 1) / (mode == PG_GATEUP ? N / 2 : N);
+            tiles *= mt;
+            const int at_once = S == 1 ? m->num_sms / 2 : S == 2 ? 34 : 15, waves = (tiles + at_once - 1) / at_once;
+            const double feed = (32768.0 + 64.0 * N) / 50, per_kt = (feed > 4.0 * N ? feed : 4.0 * N) / 1900;
+            const double fixed = 4.5 + (S == 1 ? 4.0 : 4.4 + 2.7) * N / 256;
+            const double cost = S == 1 ? waves * kps * per_kt + fixed : waves * (kps * per_kt + fixed);
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = PgPlan{N, S};
+            }
+        }
+    }
+    return best;
+}
+
+template <int N, int MODE>
+dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
+                              const int (&n_out)[3], int nseg, const CUtensorMap *X, int S, PgParams p) {
+    constexpr int kTileF = MODE == PG_GATEUP ? N / 2 : N;
+    const CUtensorMap *x = act_view(m, X, 128, p.K);
+    const CUtensorMap *w[3] = {weight_view(m, W0, N / 2), weight_view(m, W1 ? W1 : W0, N / 2), weight_view(m, W2 ? W2 : W0, N / 2)};
+    if (!x || !w[0] || !w[1] || !w[2]) return fail(m, DBT_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", tag);
+    p.m_tiles = (p.R + kPgM - 1) / kPgM;
+    p.nseg = nseg;
+    p.splits = S;
+    p.kt_per_split = ((p.K + kTcK - 1) / kTcK + S - 1) / S;
+    int nt = 0, col = 0;
+    double bytes = 0;
+    for (int s = 0; s < nseg; s++) {
+        p.seg[s] = PgSeg{nt, n_out[s], col};
+        col += n_out[s];
+        nt += (n_out[s] + kTileF - 1) / kTileF;
+        bytes += (double)n_out[s] * p.K * 2 * (MODE == PG_GATEUP ? 2 : 1);
+    }
+    p.tiles = nt * p.m_tiles;
+    const int groups = (p.m_tiles + 8) / 9, pairs = m->num_sms / 2;
+    p.m_group = (p.m_tiles + groups - 1) / groups;
+    p.status = m->ws.status;
+    const int grid = S > 1 ? 2 * S * p.tiles : 2 * (p.tiles < pairs ? p.tiles : pairs);
+    LAUNCH_CLUSTER(m, tag, bytes, 2 * S, (gemm_prompt_kernel<N, MODE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *w[0], *w[1], *w[2], *x, p);
+    return DBT_OK;
+}
+
+// One GEMM of a prompt chunk (or of a decode step of many rows: PG_STORE).  p carries the epilogue's operands; n_out the
+// features of up to three matrices (PG_GATEUP: of the gate matrix, the up matrix has as many).  *shares: how many shares of
+// sum(S^2) a residual epilogue leaves per row.
+template <PgMode MODE>
+dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
+                           const int (&n_out)[3], int nseg, const CUtensorMap *X, int K, int R, PgParams p, int *shares = nullptr) {
+    p.K = K;
+    p.R = R;
+    int widest = 0;
+    for (int s = 0; s < nseg; s++) widest = n_out[s] > widest ? n_out[s] : widest;
+    PgPlan pl = plan_gemm_prompt(m, MODE, n_out, nseg, K, R);
+    if (shares) *shares = 2 * pl.splits * ((n_out[0] + 255) / 256);
+    if constexpr (MODE == PG_STORE) {
+        if (widest <= 64) return launch_gemm_prompt<64, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, 1, p);
+        if (pl.N == 128) return launch_gemm_prompt<128, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
+    }
+    if constexpr (MODE == PG_STORE || MODE == PG_GATEUP)
+        if (pl.N == 192) return launch_gemm_prompt<192, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
+    return launch_gemm_prompt<256, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
+}
+
+// Outputs of whole 16-byte pieces, and enough of them to fill the pairs.
+bool many_rows_ok(const TcCall &c) {
+    int total = 0;
+    for (int s = 0; s < c.nseg; s++) {
+        if (c.n_out[s] % 4) return false;
+        total += c.n_out[s];
+    }
+    return total >= 1024;
+}
+
 template <int N_TILE, int MT = 1>
 dbt_status launch_gemm_tc(dbt_model *m, const TcCall &c, const TcParams &p, const LmEpi &e, dim3 grid, double bytes) {
     const CUtensorMap *w1 = c.nseg > 1 ? c.W[1] : c.W[0], *w2 = c.nseg > 2 ? c.W[2] : c.W[0];
@@ -772,6 +908,22 @@ dbt_status launch_gemm_tc(dbt_model *m, const TcCall &c, const TcParams &p, cons
 // Y partials P[split][R][ldp]; returns the split count and stride the consumer must use.
 dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_out, size_t *split_stride_out,
                        int force_split = 0, LmEpi e = LmEpi{}, int test_skip_load = 0) {
+    // Many stacked rows (row tiles of 128 and 256): pairs of SMs with the rows on the M side, one finished sum per output.
+    // At 234 rows of the 1B model against row tiles of 256 on one SM with split-K partials, per launch by events: gate|up
+    // 43 -> 27 us, Q|K|V 23 -> 21, O 19 -> 19, output matrix 80 -> 56, down 25 -> 29 (its sums then need no second pass).
+    // (Up to 64 rows the weight stream is the bound and both sides take the same time, but M is 256 whatever the rows.)
+    if (!c.grp_cnt && c.parts == 2 && n_tile >= 128 && many_rows_ok(c)) {
+        PgParams q{};
+        q.P = e.Z ? e.Z : c.P;
+        for (int s = 0; s < c.nseg; s++) q.ldp += c.n_out[s];
+        if (e.Z && e.use_scale) {
+            q.ss_in = e.ss_in; q.ss_tiles = e.ss_tiles; q.ss_ld = e.ss_ld; q.d_norm = e.d_norm; q.eps = e.eps;
+        }
+        if (!e.Z && (size_t)c.R * q.ldp > c.P_floats) return fail(m, DBT_ERR_CAPACITY, "partial buffer too small for %s", c.tag);
+        if (nsplit_out) *nsplit_out = 1;
+        if (split_stride_out) *split_stride_out = (size_t)c.R * q.ldp;
+        return run_gemm_prompt<PG_STORE>(m, c.tag, c.W[0], c.W[1], c.W[2], c.n_out, c.nseg, c.X, c.K, c.R, q);
+    }
     TcParams p{};
     int tiles = 0, col = 0;
     double bytes = 0;
@@ -963,58 +1115,6 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
     return DBT_OK;
 }
 
-// ---- GEMMs of prompt chunks on pairs of SMs (dbt_gemm_prompt.cuh) -----------------------------------------
-
-// The 3-D one-box view of a two-plane GEMM input, built on first use.
-const CUtensorMap *act_view(dbt_model *m, const CUtensorMap *X, int box_rows, int K) {
-    auto reg = m->act_base.find(X);
-    if (reg == m->act_base.end()) return nullptr;
-    auto key = std::make_tuple(X, box_rows, m->Rmax);
-    auto hit = m->act3d.find(key);
-    if (hit == m->act3d.end()) {
-        CUtensorMap t;
-        if (!make_act_map(&t, reg->second.base, (uint64_t)m->Rmax, (uint64_t)K, box_rows)) return nullptr;
-        hit = m->act3d.emplace(key, t).first;
-    }
-    return &hit->second;
-}
-
-template <int N, int MODE>
-dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *const (&W)[3], const CUtensorMap *X, const PgParams &p,
-                              double bytes) {
-    const int pairs = m->num_sms / 2, grid = 2 * (p.tiles < pairs ? p.tiles : pairs);
-    LAUNCH(m, tag, bytes, (gemm_prompt_kernel<N, MODE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *W[0], *W[1], *W[2], *X, p);
-    return DBT_OK;
-}
-
-// One GEMM of a prompt chunk.  p carries the epilogue's operands; n_out the features of up to three matrices
-// (PG_GATEUP: of the gate matrix, the up matrix has as many).
-template <int MODE, int N = 256>
-dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
-                           const int (&n_out)[3], int nseg, const CUtensorMap *X, int K, int R, PgParams p) {
-    constexpr int kTileF = MODE == PG_GATEUP ? N / 2 : N;
-    const CUtensorMap *x = act_view(m, X, 128, K);
-    if (!x) return fail(m, DBT_ERR_CUDA, "cuTensorMapEncodeTiled failed for %s", tag);
-    p.K = K;
-    p.R = R;
-    p.m_tiles = (R + kPgM - 1) / kPgM;
-    p.nseg = nseg;
-    int nt = 0, col = 0;
-    double bytes = 0;
-    for (int s = 0; s < nseg; s++) {
-        p.seg[s] = PgSeg{nt, n_out[s], col};
-        col += n_out[s];
-        nt += (n_out[s] + kTileF - 1) / kTileF;
-        bytes += (double)n_out[s] * K * 2 * (MODE == PG_GATEUP ? 2 : 1);
-    }
-    p.tiles = nt * p.m_tiles;
-    const int groups = (p.m_tiles + 8) / 9;
-    p.m_group = (p.m_tiles + groups - 1) / groups;
-    p.status = m->ws.status;
-    const CUtensorMap *const W[3] = {W0, W1 ? W1 : W0, W2 ? W2 : W0};
-    return launch_gemm_prompt<N, MODE>(m, tag, W, x, p, bytes);
-}
-
 // The operands of a Q|K|V epilogue for layer l (1/rms, RoPE, queries, cache append).
 PgParams prompt_qkv_params(dbt_model *m, const RowMap &rm, int l, int ss_tiles) {
     const dbt_config &c = m->cfg;
@@ -1046,9 +1146,6 @@ PgParams prompt_resid_params(dbt_model *m, const float *g_next) {
     p.d = m->cfg.d_model;
     return p;
 }
-// Shares of sum(S^2) that a residual epilogue leaves per row.
-int prompt_ss_tiles(const dbt_model *m) { return 2 * ((m->cfg.d_model + 255) / 256); }
-
 // MoE sub-layer on the tensor cores (Eq. moe_layer, Eq. moe_budget, Section 4.3).  Rows of both
 // paths are sorted by expert; one grouped GEMM launch covers all experts (blockIdx.z), CTAs of
 // experts nobody selected exit before touching their weights, so each selected expert's
@@ -1352,6 +1449,7 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
     double kv_bytes = 0;
     for (int b = 0; b < rm.B; b++)
         for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * sizeof(WT);
+    const bool many = n_tile >= 128 && d % 4 == 0 && F % 4 == 0;  // (the GEMMs then leave finished sums, see run_gemm_tc)
     dbt_status st;
     int nsp = 1;
     size_t sstride = 0;
@@ -1386,6 +1484,10 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
         op.W[0] = &mp.wo; op.n_out[0] = d; op.rows[0] = R; op.nseg = 1;
         {
             if ((st = run_gemm_tc(m, op, n_tile, &nsp, &sstride)) != DBT_OK) return st;
+            if (many && nsp == 1)
+                LAUNCH(m, "resid_wide", 0, resid_many_kernel, dim3(Bc, (d + 1023) / 1024, branch_blocks(grouped)), 256, 0, w.S, w.P, 1,
+                       (const float *)nullptr, Bc, grouped, lw.mlp_norm_g, d, w.Xb, lo_x, w.ss, ss_ld);
+            else
             LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, ss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, nsp, sstride, 1,
                    (const float *)nullptr, Bc, grouped, lw.mlp_norm_g, d, w.Xb, lo_x, w.ss, ss_ld);
         }
@@ -1395,6 +1497,10 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
         gu.nseg = 2;
         {
             if ((st = run_gemm_tc(m, gu, n_tile, &nsp, &sstride)) != DBT_OK) return st;
+            if (many && nsp == 1)
+                LAUNCH(m, "swiglu_couple", 0, swiglu_many_kernel, dim3(Bc, (F + 1023) / 1024, branch_blocks(grouped)), 256, 0, w.P, F, Bc, grouped,
+                       lw.coup_b, w.Hb, lo_h, (const float *)w.ss, ss_tiles, ss_ld, d, c.rms_eps);
+            else
             LAUNCH(m, "swiglu_couple", 0, swiglu_couple_kernel, dim3(Bc, (F + 255) / 256, branch_blocks(grouped)), 256, 0, w.P, nsp, sstride, F, Bc,
                    grouped, lw.coup_b, w.Hb, lo_h, (const float *)w.ss, ss_tiles, ss_ld, d, c.rms_eps);
         }
@@ -1404,6 +1510,10 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
                                                  : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr);
         {
             if ((st = run_gemm_tc(m, dn, n_tile, &nsp, &sstride)) != DBT_OK) return st;
+            if (many && nsp == 1)
+                LAUNCH(m, "resid_wide", 0, resid_many_kernel, dim3(Bc, (d + 1023) / 1024, branch_blocks(grouped)), 256, 0, w.S, w.P, 2, lw.coup_c, Bc,
+                       grouped, g_next, d, w.Xb, lo_x, w.ss, ss_ld);
+            else
             LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, ss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, nsp, sstride, 2, lw.coup_c, Bc,
                    grouped, g_next, d, w.Xb, lo_x, w.ss, ss_ld);
         }
@@ -1433,16 +1543,15 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
         st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, 0, l, kv_bytes, nullptr, true, false)
                                : run_attention_mma<64>(m, rm, 0, l, kv_bytes, nullptr, true, false);
         if (st != DBT_OK) return st;
-        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, prompt_resid_params(m, lw.mlp_norm_g))) != DBT_OK)
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, prompt_resid_params(m, lw.mlp_norm_g), &ss_tiles)) != DBT_OK)
             return st;
-        ss_tiles = prompt_ss_tiles(m);
         PgParams g{};
         g.ss_in = w.ss; g.ss_tiles = ss_tiles; g.ss_ld = m->Rmax; g.d_norm = d; g.eps = c.rms_eps;
         g.H = w.Hb; g.h_lo = lo_h; g.F = F;
         st = run_gemm_prompt<PG_GATEUP>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, 0, 0}, 1, &m->map_Xb, d, R, g);
         if (st != DBT_OK) return st;
         const float *g_next = l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr);
-        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R, prompt_resid_params(m, g_next))) != DBT_OK)
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R, prompt_resid_params(m, g_next), &ss_tiles)) != DBT_OK)
             return st;
     }
     return DBT_OK;
@@ -1479,13 +1588,12 @@ dbt_status run_layers_moe_prompt(dbt_model *m, const RowMap &rm) {
                                : run_attention_mma<64>(m, rm, 0, l, kv_bytes, nullptr, true, false);
         if (st != DBT_OK) return st;
         if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R,
-                                            prompt_resid_params(m, lw.mlp_norm_g))) != DBT_OK)
+                                            prompt_resid_params(m, lw.mlp_norm_g), &ss_tiles)) != DBT_OK)
             return st;
-        ss_tiles = prompt_ss_tiles(m);
         PgParams rt{};
         rt.ss_in = w.ss; rt.ss_tiles = ss_tiles; rt.ss_ld = m->Rmax; rt.d_norm = d; rt.eps = c.rms_eps;
         rt.P = w.rlogits; rt.ldp = E;
-        if ((st = run_gemm_prompt<PG_STORE, 64>(m, "router", &mp.rt32, nullptr, nullptr, {E, 0, 0}, 1, &m->map_Xb, d, R, rt)) != DBT_OK) return st;
+        if ((st = run_gemm_prompt<PG_STORE>(m, "router", &mp.rt, nullptr, nullptr, {E, 0, 0}, 1, &m->map_Xb, d, R, rt)) != DBT_OK) return st;
         LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.rlogits, 1, (size_t)0, E, R, c.k_primary, c.k_branch, km, 0, w.ridx,
                w.rwts, (int32_t *)nullptr, 0, (const float *)nullptr, 0, 0, d, c.rms_eps);
         LAUNCH(m, "moe_sort", 0, moe_sort_kernel, 1, 1024, 0, w.ridx, R, km, E, w.ecnt, w.eoff, w.epos, (int32_t *)nullptr);
@@ -1506,7 +1614,7 @@ dbt_status run_layers_moe_prompt(dbt_model *m, const RowMap &rm) {
             if ((st = run_gemm_prompt<PG_GATEUP>(m, "shared_gateup", &mp.wg, &mp.wu, nullptr, {Fs, 0, 0}, 1, &m->map_Xb, d, R, sg)) != DBT_OK) return st;
             PgParams sd = prompt_resid_params(m, g_next);
             sd.Y = w.Yexp; sd.sel_idx = w.ridx; sd.sel_pos = w.epos; sd.sel_wts = w.rwts; sd.kmax = km; sd.k = c.k_primary;
-            if ((st = run_gemm_prompt<PG_COMBINE>(m, "shared_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, Fs, R, sd)) != DBT_OK) return st;
+            if ((st = run_gemm_prompt<PG_COMBINE>(m, "shared_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, Fs, R, sd, &ss_tiles)) != DBT_OK) return st;
         } else {
             LAUNCH(m, "moe_combine", 0, moe_combine_rows_kernel, dim3((R + 3) / 4, (d + 255) / 256), 256, 0, w.Yexp, (const float *)nullptr, 1,
                    (size_t)0, w.ridx, w.epos, w.rwts, km, R, d, w.S, g_next, g_next ? w.Xb : (__nv_bfloat16 *)nullptr, lo_x,
@@ -1621,7 +1729,7 @@ dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, f
         RowMap rm{B, cn};
         int R = B * cn, n_tile = pad_rows(R < 256 ? R : 256);
         if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, n_tile)) != DBT_OK) return st;
-        const bool pairs = cn > 1 && R > 256;
+        const bool pairs = cn > 1 && R > 64;
         if ((st = pairs ? run_layers_prompt(m, rm) : run_layers_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
         if (last_logits && p0 + cn >= n) {
             if ((st = run_head_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
@@ -1654,7 +1762,8 @@ bool allow_smem_pg() {
 }
 bool allow_smem_prompt() {
     return allow_smem_pg<256, PG_QKV>() && allow_smem_pg<256, PG_RESID>() && allow_smem_pg<256, PG_GATEUP>() &&
-           allow_smem_pg<256, PG_COMBINE>() && allow_smem_pg<64, PG_STORE>() &&
+           allow_smem_pg<192, PG_GATEUP>() && allow_smem_pg<256, PG_COMBINE>() && allow_smem_pg<64, PG_STORE>() &&
+           allow_smem_pg<128, PG_STORE>() && allow_smem_pg<192, PG_STORE>() && allow_smem_pg<256, PG_STORE>() &&
            cudaFuncSetAttribute(gemm_group_kernel<GG_GATEUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess &&
            cudaFuncSetAttribute(gemm_group_kernel<GG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess;
 }
@@ -1695,7 +1804,7 @@ bool setup_tc(dbt_model *m) {
                   make_bf16_map(&mp.eu, lw.exp_up, (uint64_t)E * Fe, d, kTcM) &&
                   make_bf16_map(&mp.ed, lw.exp_down, (uint64_t)E * d, Fe, kTcM) &&
                   make_bf16_map(&mp.rt, lw.router, E, d, kTcM) && make_bf16_map(&mp.eg64, lw.exp_gate, (uint64_t)E * Fe, d, 64) &&
-                  make_bf16_map(&mp.eu64, lw.exp_up, (uint64_t)E * Fe, d, 64) && make_bf16_map(&mp.rt32, lw.router, E, d, 32);
+                  make_bf16_map(&mp.eu64, lw.exp_up, (uint64_t)E * Fe, d, 64);
             if (mok && Fs > 0)
                 mok = make_bf16_map(&mp.wg, lw.sh_gate, Fs, d, kTcM) && make_bf16_map(&mp.wu, lw.sh_up, Fs, d, kTcM) &&
                       make_bf16_map(&mp.wd, lw.sh_down, d, Fs, kTcM);
@@ -1707,6 +1816,20 @@ bool setup_tc(dbt_model *m) {
         // epilogue never stores)
         m->moe_tc = mok;
     }
+    for (int l = 0; l < c.n_layers; l++) {
+        const dbt_layer_weights &lw = m->layers[l];
+        LayerMaps &mp = m->maps[l];
+        const uint64_t Fd = moe ? (uint64_t)c.n_shared_experts * c.d_expert : (uint64_t)F;
+        m->w_base[&mp.wq] = {lw.wq, (uint64_t)qd, (uint64_t)d};
+        m->w_base[&mp.wk] = {lw.wk, (uint64_t)kvd, (uint64_t)d};
+        m->w_base[&mp.wv] = {lw.wv, (uint64_t)kvd, (uint64_t)d};
+        m->w_base[&mp.wo] = {lw.wo, (uint64_t)d, (uint64_t)qd};
+        m->w_base[&mp.wg] = {moe ? lw.sh_gate : lw.w_gate, Fd, (uint64_t)d};
+        m->w_base[&mp.wu] = {moe ? lw.sh_up : lw.w_up, Fd, (uint64_t)d};
+        m->w_base[&mp.wd] = {moe ? lw.sh_down : lw.w_down, (uint64_t)d, Fd};
+        if (moe) m->w_base[&mp.rt] = {lw.router, (uint64_t)c.n_experts, (uint64_t)d};
+    }
+    m->w_base[&m->map_lm] = {m->w.lm_head, (uint64_t)c.vocab, (uint64_t)d};
     ok = ok && make_bf16_map(&m->map_lm, m->w.lm_head, c.vocab, d, kTcM);
     ok = ok && make_bf16_map(&m->map_Xb, w.Xb, 2 * m->Rmax, d, 16) && make_bf16_map(&m->map_Ob, w.Ob, 2 * m->Rmax, qd, 16);
     if (!moe) ok = ok && make_bf16_map(&m->map_Hb, w.Hb, 2 * m->Rmax, F, 16);

@@ -42,6 +42,10 @@ __device__ __forceinline__ unsigned long long tl_tag(const char *s) {
 #define DBT_TL_DECL unsigned long long tl0_ = gtime(), tl1_ = 0, tlx_[4] = {0, 0, 0, 0}
 #define DBT_TL_WAITED tl1_ = gtime()
 #define DBT_TL_MARK(k) tlx_[k] = gtime()
+// marks of a thread other than thread 0, which stores the record: through shared memory
+#define DBT_TL_SHARED __shared__ unsigned long long tls_[4]; if (threadIdx.x < 4) tls_[threadIdx.x] = 0
+#define DBT_TL_SHARED_MARK(cond, k) if (cond) tls_[k] = gtime()
+#define DBT_TL_SHARED_TAKE for (int k_ = 1; k_ < 4; k_++) tlx_[k_] = tls_[k_]
 #define DBT_TL_END(name) DBT_TL_END_IF(blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0, name)
 #define DBT_TL_END_IF(cond, name)                                                          \
     if (threadIdx.x == 0 && (cond)) {                                                      \
@@ -58,6 +62,9 @@ __device__ __forceinline__ unsigned long long tl_tag(const char *s) {
 #define DBT_TL_DECL
 #define DBT_TL_WAITED
 #define DBT_TL_MARK(k)
+#define DBT_TL_SHARED
+#define DBT_TL_SHARED_MARK(cond, k)
+#define DBT_TL_SHARED_TAKE
 #define DBT_TL_END(name)
 #define DBT_TL_END_IF(cond, name)
 #endif

@@ -70,12 +70,12 @@ __device__ __forceinline__ void sum_splits_k(const float *P, size_t split_stride
 __device__ __forceinline__ float row_scale(const float *ss, int ss_tiles, int ss_ld, int row, int d_norm, float eps) {
     if (!ss) return 1.f;
     float a = 0.f;
-    for (int t0 = 0; t0 < ss_tiles; t0 += 8) {  // eight shares in flight at a time, added in tile order
-        float v[8];
+    for (int t0 = 0; t0 < ss_tiles; t0 += 16) {  // sixteen shares in flight at a time, added in tile order
+        float v[16];
 #pragma unroll
-        for (int j = 0; j < 8; j++) v[j] = t0 + j < ss_tiles ? __ldcg(ss + (size_t)(t0 + j) * ss_ld + row) : 0.f;
+        for (int j = 0; j < 16; j++) v[j] = t0 + j < ss_tiles ? __ldcg(ss + (size_t)(t0 + j) * ss_ld + row) : 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; j++) a += v[j];
+        for (int j = 0; j < 16; j++) a += v[j];
     }
     return 1.f / sqrtf(a / (float)d_norm + eps);
 }
@@ -398,6 +398,101 @@ __device__ __forceinline__ float4 sum_splits4(const float *P, size_t split_strid
         m.x += v.x, m.y += v.y, m.z += v.z, m.w += v.w;
     }
     return m;
+}
+
+// resid_wide_kernel and swiglu_couple_kernel for steps of more than 64 stacked rows, whose GEMMs leave one finished sum per
+// output (no splits): a few MB per launch, so a thread takes four consecutive columns of a row and of its branch twin.
+// At 117 sequences of the 1B model the one-column forms ran in three waves: 6.8 and 11.7 us of the step each.
+// grid (primary rows, ceil(columns / 1024), branches), 256 threads.  Columns % 4 == 0.
+__global__ void __launch_bounds__(256) resid_many_kernel(float *S, const float *P, int mode, const float *__restrict__ coup_c, int Bc,
+                                                         int grouped, const float *__restrict__ g_next, int d, __nv_bfloat16 *Xb,
+                                                         size_t lo_off, float *ss_out, int ss_ld) {
+    pdl_launch_dependents();
+    __shared__ float scratch[16];
+    const int b = blockIdx.x, i = blockIdx.y * 1024 + threadIdx.x * 4, warp = threadIdx.x >> 5;
+    const bool act = i < d, first = blockIdx.z == 0;
+    const int r2 = ((int)blockIdx.z + 1) * Bc + b;
+    float4 gn = make_float4(1.f, 1.f, 1.f, 1.f), cc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (act && g_next) gn = *reinterpret_cast<const float4 *>(g_next + i);
+    if (act && mode >= 2) cc = *reinterpret_cast<const float4 *>(coup_c + i);
+    pdl_wait();
+    float q1 = 0.f, q2 = 0.f;
+    if (act) {
+        const size_t o1 = (size_t)b * d + i, o2 = (size_t)r2 * d + i;
+        float4 s1 = ldcg4(S + o1), m1 = ldcg4(P + o1), s2 = s1, m2 = m1;
+        if (grouped) {
+            s2 = ldcg4(S + o2);
+            if (mode != 3) m2 = ldcg4(P + o2);
+        }
+        s1.x += m1.x, s1.y += m1.y, s1.z += m1.z, s1.w += m1.w;
+        if (first) {
+            *reinterpret_cast<float4 *>(S + o1) = s1;
+            store_split4(Xb, o1, lo_off, make_float4(gn.x * s1.x, gn.y * s1.y, gn.z * s1.z, gn.w * s1.w));
+        }
+        q1 = s1.x * s1.x + s1.y * s1.y + s1.z * s1.z + s1.w * s1.w;
+        if (grouped) {
+            if (mode == 2) m2.x += cc.x * m1.x, m2.y += cc.y * m1.y, m2.z += cc.z * m1.z, m2.w += cc.w * m1.w;
+            if (mode == 3) m2 = make_float4(cc.x * m1.x, cc.y * m1.y, cc.z * m1.z, cc.w * m1.w);  // Eq. matched_attention
+            s2.x += m2.x, s2.y += m2.y, s2.z += m2.z, s2.w += m2.w;
+            *reinterpret_cast<float4 *>(S + o2) = s2;
+            store_split4(Xb, o2, lo_off, make_float4(gn.x * s2.x, gn.y * s2.y, gn.z * s2.z, gn.w * s2.w));
+            q2 = s2.x * s2.x + s2.y * s2.y + s2.z * s2.z + s2.w * s2.w;
+        }
+    }
+    q1 = warp_sum(q1);
+    q2 = warp_sum(q2);
+    if ((threadIdx.x & 31) == 0) {
+        scratch[warp] = q1;
+        scratch[8 + warp] = q2;
+    }
+    __syncthreads();
+    const int t = blockIdx.y * 4 + threadIdx.x;  // share of 256 columns: two warps
+    if (threadIdx.x < 4 && t * 256 < d) {
+        if (first) ss_out[(size_t)t * ss_ld + b] = scratch[2 * threadIdx.x] + scratch[2 * threadIdx.x + 1];
+        if (grouped) ss_out[(size_t)t * ss_ld + r2] = scratch[8 + 2 * threadIdx.x] + scratch[8 + 2 * threadIdx.x + 1];
+    }
+}
+
+__global__ void __launch_bounds__(256) swiglu_many_kernel(const float *P, int F, int Bc, int grouped, const float *__restrict__ coup_b,
+                                                          __nv_bfloat16 *Hb, size_t lo_off, const float *ss, int ss_tiles, int ss_ld,
+                                                          int d_norm, float eps) {
+    pdl_launch_dependents();
+    __shared__ float sh[2];
+    const int b = blockIdx.x, f = blockIdx.y * 1024 + threadIdx.x * 4, lane = threadIdx.x & 31;
+    const bool act = f < F, first = blockIdx.z == 0;
+    const int rb = grouped ? ((int)blockIdx.z + 1) * Bc + b : b;
+    float4 cb = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (act && grouped && coup_b) cb = *reinterpret_cast<const float4 *>(coup_b + f);
+    pdl_wait();
+    float a = 0.f;  // the norm shares of the block's two rows, a half warp each
+    if (ss && threadIdx.x < 32)
+        for (int t = lane & 15; t < ss_tiles; t += 16) a += __ldcg(ss + (size_t)t * ss_ld + (lane < 16 ? b : rb));
+    float4 g1 = make_float4(0.f, 0.f, 0.f, 0.f), u1 = g1, g2 = g1, u2 = g1;
+    if (act) {
+        const float *p1 = P + (size_t)b * 2 * F + f, *p2 = P + (size_t)rb * 2 * F + f;
+        g1 = ldcg4(p1);
+        u1 = ldcg4(p1 + F);
+        if (grouped) {
+            g2 = ldcg4(p2);
+            u2 = ldcg4(p2 + F);
+        }
+    }
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if ((lane & 15) == 0) sh[lane >> 4] = ss ? 1.f / sqrtf(a / (float)d_norm + eps) : 1.f;
+    }
+    __syncthreads();
+    if (!act) return;
+    const float r1 = sh[0], r2 = sh[1];
+    const float4 h1 = make_float4(silu(r1 * g1.x) * (r1 * u1.x), silu(r1 * g1.y) * (r1 * u1.y), silu(r1 * g1.z) * (r1 * u1.z),
+                                  silu(r1 * g1.w) * (r1 * u1.w));
+    if (first) store_split4(Hb, (size_t)b * F + f, lo_off, h1);
+    if (grouped) {
+        const float4 h2 = make_float4(silu(r2 * g2.x) * (r2 * u2.x) + cb.x * h1.x, silu(r2 * g2.y) * (r2 * u2.y) + cb.y * h1.y,
+                                      silu(r2 * g2.z) * (r2 * u2.z) + cb.z * h1.z, silu(r2 * g2.w) * (r2 * u2.w) + cb.w * h1.w);
+        store_split4(Hb, (size_t)rb * F + f, lo_off, h2);
+    }
 }
 
 // Eq. embeddings for the fused path: S^0 = RMSNorm(E[x]) and, for the first layer's Q|K|V GEMM,

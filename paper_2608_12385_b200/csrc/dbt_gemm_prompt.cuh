@@ -15,6 +15,11 @@
 // between: gate|up with SwiGLU 204 -> 122 us (1.55 PFLOP/s of tensor work), down + residual 86 + 15 -> 74, Q|K|V + rotation
 // and append 61 + 25 -> 62, O + residual 41 + 15 -> 39.
 //
+// Few row tiles (decode steps of more than 64 stacked rows, short prompts) leave too few tiles for the chip: the contracted
+// width of a tile is then split over 2 or 4 pairs of one cluster.  Each CTA owns a slice of the tile's columns, the others
+// write their partial sums of it into its (by then idle) ring through distributed shared memory, and it adds them in split
+// order and runs the epilogue of that slice: no partials in memory, no kernel to sum them.
+//
 // Roles: warp 0 TMA producer, warp 1 MMA issuer (of the pair's first CTA) and TMEM owner, warps 2..9 epilogue (two per
 // TMEM lane quadrant, each taking half of the tile's columns).  Every wait is bounded: on expiry the CTA records
 // kStatusWaitExpired, stops storing, and still reaches the cluster barrier that the pair leaves by.
@@ -50,6 +55,7 @@ struct PgParams {
     // once then share about as many row tiles as weight tiles (9 x 8 of 74), whatever the chunk: with all 32 row tiles of
     // an 8192-row chunk side by side the 8B shape's gate|up re-read its 134 MB of activations from HBM (97 us per row tile).
     int m_group;
+    int splits, kt_per_split;  // pairs per tile (1, 2, 4; a cluster is 2 * splits CTAs); k-tiles of each
     PgSeg seg[3];
     int nseg;
     int *status;
@@ -65,7 +71,7 @@ struct PgParams {
     const float *g_next;  // nullptr: 1
     __nv_bfloat16 *X;
     size_t x_lo;
-    float *ss_out;  // [feature tile * 2 + half][ss_ld]
+    float *ss_out;  // [(feature tile * splits + split) * 2 + half][ss_ld]
     int d;
     // PG_COMBINE
     const float *Y;
@@ -90,9 +96,10 @@ template <int N>
 struct PgCfg {
     static constexpr int kBBytes = N / 2 * kTcK * 2;  // this CTA's half of the weight tile
     static constexpr int kStageBytes = kPgABytes + kBBytes;
-    static constexpr int kStages = N == 256 ? 4 : 5;
+    static constexpr int kStages = N >= 128 ? 4 : 5;
     static constexpr int kStagingBytes = kPgEpiWarps * 4096;
-    static constexpr int kTmemCols = 2 * N < 32 ? 32 : 2 * N;
+    static constexpr int kAccStride = N > 128 ? 256 : N;  // TMEM columns between the two accumulators
+    static constexpr int kTmemCols = 2 * kAccStride;
     static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 + 256;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory of one SM");
 };
@@ -162,11 +169,12 @@ __device__ __forceinline__ void umma2_f16(uint32_t tmem_d, uint64_t adesc, uint6
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
         : "memory");
 }
-// Arrive on the barrier at this offset in both CTAs of the pair once the MMAs issued so far are done.
-__device__ __forceinline__ void umma2_commit(uint32_t bar) {
+// Arrive on the barrier at this offset in both CTAs of the pair (mask: their ranks in the cluster) once the MMAs issued so
+// far are done.
+__device__ __forceinline__ void umma2_commit(uint32_t bar, uint32_t mask = 3) {
     asm volatile(
         "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-        "h"((uint16_t)3)
+        "h"((uint16_t)mask)
         : "memory");
 }
 
@@ -197,10 +205,12 @@ __device__ __forceinline__ void store16(__nv_bfloat16 *dst, const float *x) {
 }
 
 template <int N, int MODE>
-__global__ void __launch_bounds__(kPgThreads, 1) __cluster_dims__(2, 1, 1)
+__global__ void __launch_bounds__(kPgThreads, 1)
 gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
                    const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmX, const PgParams p) {
     using Cfg = PgCfg<N>;
+    DBT_TL_DECL;
+    DBT_TL_SHARED;
     constexpr int STAGES = Cfg::kStages;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
@@ -216,9 +226,12 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
     static_assert(8 * (2 * STAGES + 4) + 4 <= 256, "barrier area");
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t rank = cluster_rank();
-    const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-    const int nkt = (p.K + kTcK - 1) / kTcK;
+    // rank in the pair; the pair's first CTA; which part of the contracted width
+    const int S = p.splits;
+    const uint32_t crank = cluster_rank(), rank = crank & 1, lead = crank & ~1u, pair_mask = 3u << lead;
+    const int split = (int)(crank >> 1);
+    const int pair = blockIdx.x / (2 * S), npairs = gridDim.x / (2 * S);  // (splits > 1: one tile per cluster)
+    const int kt0 = split * p.kt_per_split, nkt = min(p.kt_per_split, (p.K + kTcK - 1) / kTcK - kt0);
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; s++) {
@@ -274,20 +287,21 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     tw = sg == 0 ? &tmW0 : sg == 1 ? &tmW1 : &tmW2;
                     row = f0 + (int)rank * (N / 2);
                 }
-                tma2_load_2d_hint(ring + s * Cfg::kStageBytes + kPgABytes, tw, mapa_u32(full_bar(s), 0), kt * kTcK, row, pol);
+                tma2_load_2d_hint(ring + s * Cfg::kStageBytes + kPgABytes, tw, mapa_u32(full_bar(s), lead), kt * kTcK, row, pol);
             };
             auto load_x = [&](int s, int mt, int kt) {
-                tma2_load_3d(ring + s * Cfg::kStageBytes, &tmX, mapa_u32(full_bar(s), 0), kt * kTcK, mt * kPgM + (int)rank * 128, 0);
+                tma2_load_3d(ring + s * Cfg::kStageBytes, &tmX, mapa_u32(full_bar(s), lead), kt * kTcK, mt * kPgM + (int)rank * 128, 0);
             };
             const int npre = pair < p.tiles ? min(STAGES, nkt) : 0;
             int mt, nt;
             tile_of(pair, mt, nt);
             for (int i = 0; i < npre; i++) {
                 if (rank == 0) mbar_expect_tx(full_bar(i), 2 * Cfg::kStageBytes);
-                load_w(i, nt, i);
+                load_w(i, nt, kt0 + i);
             }
             pdl_wait();
-            for (int i = 0; i < npre; i++) load_x(i, mt, i);
+            DBT_TL_WAITED;
+            for (int i = 0; i < npre; i++) load_x(i, mt, kt0 + i);
             int it = 0;  // stages requested so far, over all tiles
             for (int t = pair; t < p.tiles && ok; t += npairs) {
                 tile_of(t, mt, nt);
@@ -297,10 +311,11 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     if (it >= STAGES) ok = mbar_wait_cluster(empty_bar(s), ((it / STAGES) - 1) & 1);
                     if (!ok) break;
                     if (rank == 0) mbar_expect_tx(full_bar(s), 2 * Cfg::kStageBytes);
-                    load_w(s, nt, kt);
-                    load_x(s, mt, kt);
+                    load_w(s, nt, kt0 + kt);
+                    load_x(s, mt, kt0 + kt);
                 }
             }
+            DBT_TL_MARK(0);
             if (!ok) report(p.status, kStatusWaitExpired, 600);
         }
     } else if (warp == 1) {
@@ -313,7 +328,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                 if (n_acc >= 2) ok = mbar_wait_cluster(acc_empty(a), ((n_acc >> 1) - 1) & 1);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t acc = tmem_base + a * N;
+                const uint32_t acc = tmem_base + a * Cfg::kAccStride;
                 for (int kt = 0; kt < nkt; kt++, it++) {
                     const int s = it % STAGES;
                     ok = mbar_wait_cluster(full_bar(s), (it / STAGES) & 1);
@@ -327,11 +342,18 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
 #pragma unroll
                         for (int k = 0; k < kTcK / 16; k++) umma2_f16(acc, adesc + 2 * k, bdesc + 2 * k, idesc, (kt | part | k) != 0);
                     }
-                    umma2_commit(empty_bar(s));
+                    umma2_commit(empty_bar(s), pair_mask);
                 }
-                if (ok) umma2_commit(acc_full(a));
+                if (ok) umma2_commit(acc_full(a), pair_mask);
             }
             if (!ok) report(p.status, kStatusWaitExpired, 601);
+        }
+    }
+    if (warp < 2) {
+        if (S > 1) {  // the exchange's two barriers (acc_ready)
+            __syncwarp();
+            cluster_sync_all();
+            cluster_sync_all();
         }
     } else {
         // ---- epilogue: TMEM lane = row, TMEM column = feature
@@ -350,12 +372,56 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
             float rs = 1.f;
             if (MODE == PG_QKV || MODE == PG_GATEUP || MODE == PG_STORE)
                 rs = row_scale(p.ss_in, p.ss_tiles, p.ss_ld, on ? row : 0, p.d_norm, p.eps);
-            const uint32_t tacc = lane_base + a * N;
+            const uint32_t tacc = lane_base + a * Cfg::kAccStride;
             auto acc_ready = [&] {
                 bool r = mbar_wait_cluster(acc_full(a), (n_acc >> 1) & 1);
                 ok = r = __all_sync(0xffffffffu, r);
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                DBT_TL_SHARED_MARK(warp == 2 && lane == 0, 1);
+                if (S > 1) {
+                    // the slices that other CTAs own go to their rings, [source][4-column group][row][4]
+                    cluster_sync_all();  // every pair's MMAs are done: the rings are idle
+                    if (r) {
+                        const int w = N / S;
+#pragma unroll 1
+                        for (int c = half * (N / 2); c < (half + 1) * (N / 2); c += 16) {
+                            const int o = c / w;
+                            if (o == split) continue;
+                            uint32_t v[16];
+                            __syncwarp();
+                            tmem_ld16_issue(tacc + c, v);
+                            tmem_ld_wait();
+                            const int slot = split < o ? split : split - 1;
+                            const uint32_t dst = mapa_u32(ring + (uint32_t)(((slot * w + c - o * w) * 128 + (quad * 32 + lane) * 4) * 4), (uint32_t)(2 * o) + rank);
+#pragma unroll
+                            for (int q = 0; q < 4; q++)
+                                asm volatile("st.shared::cluster.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst + q * 128 * 16), "r"(v[4 * q]), "r"(v[4 * q + 1]),
+                                             "r"(v[4 * q + 2]), "r"(v[4 * q + 3])
+                                             : "memory");
+                        }
+                    }
+                    __syncwarp();
+                    cluster_sync_all();
+                }
+                DBT_TL_SHARED_MARK(warp == 2 && lane == 0, 2);
                 return r;
+            };
+            // Adds the other splits' sums to 16 columns of this CTA's slice, in split order.
+            auto add_peers = [&](uint32_t (&v)[16], int c) {
+                const int w = N / S, lc = c - split * w;
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int k = 0; k < S; k++) {
+                        float4 y = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]), __uint_as_float(v[4 * q + 2]),
+                                               __uint_as_float(v[4 * q + 3]));
+                        if (k != split)
+                            y = *reinterpret_cast<const float4 *>(gen + (size_t)((((k < split ? k : k - 1) * w + lc + 4 * q) * 128 + (quad * 32 + lane) * 4) * 4));
+                        x.x += y.x, x.y += y.y, x.z += y.z, x.w += y.w;
+                    }
+                    v[4 * q] = __float_as_uint(x.x), v[4 * q + 1] = __float_as_uint(x.y);
+                    v[4 * q + 2] = __float_as_uint(x.z), v[4 * q + 3] = __float_as_uint(x.w);
+                }
             };
             if constexpr (MODE == PG_STORE || MODE == PG_RESID || MODE == PG_COMBINE) {
                 // Chunks of 32 columns go through a 4 KB staging tile of the warp (16-byte pieces, XOR-swizzled by row),
@@ -368,7 +434,8 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                 float sq[8];
 #pragma unroll
                 for (int i = 0; i < 8; i++) sq[i] = 0.f;
-                const int cbase = half * (N / 2);
+                // this warp's columns: half of the CTA's slice, at least 32 (a slice of 32 leaves four warps without)
+                const int wide = max(32, N / (2 * S)), cbase = split * (N / S) + half * wide, cend = half * wide < N / S ? wide : 0;
                 int ps[kPre + 1];
                 float wt[kPre + 1];
                 if (MODE == PG_COMBINE) {  // this lane's own row's first selections
@@ -395,10 +462,10 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         }
                     }
                 };
-                if (kResid) request(0);
+                if (kResid && cend > 0) request(0);
                 if (!acc_ready()) break;
 #pragma unroll 1
-                for (int c = 0; c < N / 2; c += 32) {
+                for (int c = 0; c < cend; c += 32) {
                     const int col = f0 + cbase + c + c4;  // this lane's first column
                     const bool con = col < p.seg[sg].n_out;
                     uint32_t v[2][16];
@@ -408,6 +475,10 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     float4 gn = make_float4(1.f, 1.f, 1.f, 1.f);
                     if (kResid && p.g_next && con) gn = *reinterpret_cast<const float4 *>(p.g_next + col);
                     tmem_ld_wait();
+                    if (S > 1) {
+                        add_peers(v[0], cbase + c);
+                        add_peers(v[1], cbase + c + 16);
+                    }
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
                         float4 x = make_float4(rs * __uint_as_float(v[j >> 2][(j & 3) * 4]), rs * __uint_as_float(v[j >> 2][(j & 3) * 4 + 1]),
@@ -443,7 +514,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                                 }
                             }
                         }
-                        if (c + 32 < N / 2) request(c + 32);
+                        if (c + 32 < cend) request(c + 32);
                     }
 #pragma unroll
                     for (int i = 0; i < 8; i++) {
@@ -469,7 +540,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         q += __shfl_xor_sync(0xffffffffu, q, 2);
                         q += __shfl_xor_sync(0xffffffffu, q, 4);
                         const int r = row0 + i * 4 + rsub;
-                        if ((lane & 7) == 0 && r < p.R) p.ss_out[(size_t)(nt * 2 + half) * p.ss_ld + r] = q;
+                        if ((lane & 7) == 0 && r < p.R) p.ss_out[(size_t)((nt * S + split) * 2 + half) * p.ss_ld + r] = q;
                     }
                 }
             } else if constexpr (MODE == PG_GATEUP) {
@@ -514,7 +585,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     }
                 }
 #pragma unroll 1
-                for (int hc = 0; hc < N / hd; hc++) {
+                for (int hc = split * (N / S) / hd; hc < (split + 1) * (N / S) / hd; hc++) {  // (N / splits holds whole heads)
                     const int head = f0 / hd + hc;
 #pragma unroll 1
                     for (int j = 0; j < span; j += 16) {
@@ -530,6 +601,10 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                             for (int i = 0; i < 8; i++) cs[i] = tab[i];
                         }
                         tmem_ld_wait();
+                        if (S > 1) {
+                            add_peers(v0, hc * hd + i0);
+                            add_peers(v1, hc * hd + hh2 + i0);
+                        }
                         float x0[16], x1[16];
 #pragma unroll
                         for (int i = 0; i < 16; i++) {
@@ -568,10 +643,11 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     }
                 }
             }
+            DBT_TL_SHARED_MARK(warp == 2 && lane == 0, 3);
             // the accumulator may be overwritten: tell the pair's MMA issuer
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(mapa_u32(acc_empty(a), 0));
+            if (lane == 0) mbar_arrive_cluster(mapa_u32(acc_empty(a), lead));
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 610 + warp);
     }
@@ -581,6 +657,8 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
     cluster_sync_all();  // neither CTA leaves while the other may still signal its barriers
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)Cfg::kTmemCols) : "memory");
+    DBT_TL_SHARED_TAKE;
+    DBT_TL_END("gemm_pg");
 }
 
 }  // namespace dbt

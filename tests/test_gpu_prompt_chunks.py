@@ -67,3 +67,17 @@ def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
 def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n):
     from test_gpu_parity import small_moe, test_moe_prompt_chunks_of_more_than_one_row_tile_match_the_oracle as check
     check(small_moe(**kw), B, n, 0.05)
+
+
+@pytest.mark.parametrize("n_out,K,R", [(2048, 2048, 70), (2048, 2048, 256), (1028, 520, 129), (4096, 5632, 234), (1024, 64, 200),
+                                       (11264, 2048, 130)])
+def test_many_row_decode_widths_match_the_oracle(n_out, K, R):
+    """Decode steps of 65 to 256 stacked rows take the paired-SM GEMMs: the split over clusters (2 and 4 pairs per tile),
+    ragged last k-tiles and feature tiles.  One layer whose MLP has the given widths, primary rows and branch rows."""
+    cfg = cfg_of(d_model=K if K <= 2048 else 256, d_ff=max(n_out, K) // 2 // 8 * 8, n_layers=1, vocab=1028)
+    B = (R + 1) // 2
+    w = make_weights(cfg, seed=95, matrix_std=0.02)
+    tok = make_tokens(cfg, B, 3, seed=96)
+    from gpu_util import teacher_forced_compare
+    # tokens: logits may be off by the stated 2e-2 each, so two probabilities closer than e^(2 x 2e-2) - 1 may swap
+    teacher_forced_compare(cfg, w, tok, n_prefill=1, grouped=True, token_margin=4.1e-2)
