@@ -38,7 +38,7 @@ struct Workspace {
     int32_t *seq_len, *page_table, *status, *tokens_stage, *next_stage, *att_tickets, *att_tickets2, *gemm_tickets;
     float *alpha_stage;
     char *kv_stage;  // staging for dbt_kv_export / dbt_kv_import (kKvStageBytes)
-    int32_t *att_plan;  // a decode step's attention work split (attn_plan_kernel), kAttPlanInts
+    int32_t *att_plan;  // a decode step's attention work split (embed_fused_kernel), kAttPlanInts
     // MoE
     float *rlogits, *rwts, *Hexp, *Yexp, *Msh, *Hsh;
     int32_t *ridx, *ecnt, *elist, *last_experts, *union_cnt;
@@ -136,7 +136,7 @@ struct dbt_model {
     std::vector<GraphEntry> graphs;
     // where a decode step finds sequence b's token: tokens[b * tok_stride + tok_p0] (1, 0 except inside dbt_prefill_boundary)
     int tok_stride = 1, tok_p0 = 0;
-    bool att_planned = false;  // inside a decode step whose attention work split has been computed (run_attention_plan)
+    bool att_planned = false;  // inside a decode step whose attention work split has been computed (run_embed_wide)
 };
 
 namespace {
@@ -409,18 +409,23 @@ cudaEvent_t prof_event(dbt_model *m) {
 // Mixture readout (Eq. alpha, Eq. mixloss) and greedy token; also advances the sequence lengths.
 // Rows cut into chunks of at most 2048 logits, one CTA per (sequence, chunk): two short launches
 // instead of one CTA walking a row three times (DBT_READOUT=row keeps that kernel).
-dbt_status run_readout(dbt_model *m, int B, int grouped, int32_t *next_dev, float *alpha_dev) {
+// z1_dev, z2_dev (nullable): where the caller wants the logits.
+dbt_status run_readout(dbt_model *m, int B, int grouped, int32_t *next_dev, float *alpha_dev, float *z1_dev, float *z2_dev) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
     int nc = (c.vocab + kRoChunk - 1) / kRoChunk;
     if (m->readout_row || nc > kRoMaxChunks) {
         LAUNCH(m, "readout", 0, readout_kernel, B, 1024, 0, w.Z, B, c.vocab, grouped, next_dev, alpha_dev, w.seq_len, 1);
+        const size_t zb = sizeof(float) * (size_t)B * c.vocab;
+        if (z1_dev) CUDA_TRY(m, cudaMemcpyAsync(z1_dev, w.Z, zb, cudaMemcpyDeviceToDevice, m->stream));
+        if (z2_dev && grouped)  // the branches' logits, branch-major [K-1][B][V]
+            CUDA_TRY(m, cudaMemcpyAsync(z2_dev, w.Z + (size_t)B * c.vocab, zb * (npaths(grouped) - 1), cudaMemcpyDeviceToDevice, m->stream));
         return DBT_OK;
     }
     int chunk = (c.vocab + nc - 1) / nc;
     if (grouped) LAUNCH(m, "readout_stats", 0, readout_stats_kernel, dim3(B, nc), kRoThreads, 0, w.Z, B, c.vocab, grouped, chunk, w.ro_stats);
     LAUNCH(m, "readout", 0, readout_pick_kernel, dim3(B, nc), kRoThreads, 0, w.Z, B, c.vocab, chunk, grouped, w.ro_stats, w.ro_tickets,
-           next_dev, alpha_dev, w.seq_len, 1);
+           next_dev, alpha_dev, w.seq_len, 1, z1_dev, z2_dev);
     return DBT_OK;
 }
 
@@ -1018,17 +1023,6 @@ bool attn_deep(const dbt_model *m, int items) {
 __nv_bfloat16 *prompt_q(const dbt_model *m) { return m->prompt_attn_tc ? reinterpret_cast<__nv_bfloat16 *>(m->ws.Q) : nullptr; }
 float prompt_q_scale(const dbt_model *m) { return kLog2e / sqrtf((float)m->cfg.head_dim); }
 
-// The attention work split of a decode step, once for all its layers.
-dbt_status run_attention_plan(dbt_model *m, const RowMap &rm) {
-    const dbt_config &c = m->cfg;
-    const int items = rm.B * rm.cn;
-    if (items > kAttMaxItems) return DBT_OK;  // (the attention launch reports the capacity error)
-    LAUNCH(m, "attn_plan", 0, attn_plan_kernel, 1, 32, 0, rm, m->ws.seq_len, c.n_kv_heads,
-           attn_deep(m, items) ? m->num_sms : 2 * m->num_sms, m->ws.att_plan);
-    m->att_planned = true;  // cleared by the step function when its layers have been enqueued
-    return DBT_OK;
-}
-
 template <int DH>
 dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int layer, double kv_bytes,
                              const QkvFuse *qf = nullptr, bool pack_prompt = false, bool planned = false) {
@@ -1277,6 +1271,22 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
     return DBT_OK;
 }
 
+// Embeddings and the first layer's GEMM input; plan: also the attention work split of a decode step, once for all its layers.
+template <typename WT>
+dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0, const RowMap &rm, int R, bool plan) {
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const int items = rm.B * rm.cn;
+    plan = plan && items <= kAttMaxItems;  // (the attention launch reports the capacity error)
+    LAUNCH(m, "embed", 0, embed_fused_kernel<WT>, R + (plan ? 1 : 0), 256, 0, tokens_dev, n, p0, rm, (const WT *)m->w.embed_primary,
+           (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S,
+           m->layers[0].attn_norm_g, w.Xb, m->act_parts == 2 ? (size_t)m->Rmax * c.d_model : (size_t)0, w.ss, m->Rmax,
+           (c.d_model + 255) / 256, w.status, w.seq_len, c.n_kv_heads, attn_deep(m, items) ? m->num_sms : 2 * m->num_sms,
+           plan ? w.att_plan : (int32_t *)nullptr);
+    m->att_planned = plan;  // cleared by the step function when its layers have been enqueued
+    return DBT_OK;
+}
+
 // bf16 layer stack: TMA + tcgen05 GEMMs with the elementwise work between them fused into
 // three small kernels.  On return the last layer's MLP output is still pending in P (dense
 // models): `pending` tells the caller how to fold it into S (mode of resid_norm_kernel).
@@ -1312,12 +1322,8 @@ dbt_status run_layers_tc(dbt_model *m, const RowMap &rm, int grouped, int n_tile
         WT *vpool = kpool + pool_kv_elems;
         // fold the previous layer's MLP output into S (Eq. mlp), N_i = RMSNorm(S_i).  MoE, wide form: the
         // GEMM input is g * S with the 1/rms factor applied behind the GEMM; the previous layer's combine
-        // has left it already, the first layer gets it from the residual kernel with nothing to add.
-        if (mwide) {
-            if (l == 0)
-                LAUNCH_BR(m, grouped, "resid_wide", 0, resid_wide_kernel, dim3(Bc, mss_tiles, branch_blocks(grouped)), 256, 0, w.S, w.P, 0, (size_t)0, 1,
-                       (const float *)nullptr, Bc, grouped, lw.attn_norm_g, d, w.Xb, lo_x, w.ss, m->Rmax);
-        } else {
+        // has left it already, the first layer's comes from the embedding kernel.
+        if (!mwide) {
             LAUNCH(m, "resid_norm", 0, resid_norm_kernel, dim3(Bc, 1, branch_blocks(grouped)), norm_threads(d), 0, w.S, w.P, nsp, sstride, mode,
                    l > 0 ? m->layers[l - 1].coup_c : nullptr, Bc, grouped, lw.attn_norm_g, c.rms_eps, d, 1, 1, 0, w.Xb,
                    lo_x, (float *)nullptr);
@@ -1410,9 +1416,13 @@ dbt_status step_tc(dbt_model *m, const int32_t *tokens_dev, int B, int grouped, 
     int R = npaths(grouped) * B;
     int n_tile = pad_rows(paths_of(c) * B);  // the same instruction shape in both modes
     dbt_status st;
-    if (m->att_fast && (st = run_attention_plan(m, rm)) != DBT_OK) return st;
-    LAUNCH(m, "embed", 0, embed_norm_kernel<WT>, R, 256, 0, tokens_dev, m->tok_stride, m->tok_p0, rm, (const WT *)m->w.embed_primary,
-           (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S, w.status);
+    const bool mwide = c.n_experts > 0 && m->moe_tc && m->moe_wide;  // (see run_layers_tc)
+    if (mwide) {
+        if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, m->att_fast)) != DBT_OK) return st;
+    } else {
+        LAUNCH(m, "embed", 0, embed_norm_kernel<WT>, R, 256, 0, tokens_dev, m->tok_stride, m->tok_p0, rm, (const WT *)m->w.embed_primary,
+               (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S, w.status);
+    }
     int mode, nsp;
     size_t sstride;
     st = run_layers_tc(m, rm, grouped, n_tile, true, &mode, &nsp, &sstride);
@@ -1420,11 +1430,7 @@ dbt_status step_tc(dbt_model *m, const int32_t *tokens_dev, int B, int grouped, 
     if (st != DBT_OK) return st;
     if ((st = run_head_tc(m, B, grouped, B, 1, 0, n_tile, mode, nsp, sstride)) != DBT_OK) return st;
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
-    if ((st = run_readout(m, B, grouped, next_dev, alpha_dev)) != DBT_OK) return st;
-    size_t zb = sizeof(float) * (size_t)B * c.vocab;
-    if (z1_dev) CUDA_TRY(m, cudaMemcpyAsync(z1_dev, w.Z, zb, cudaMemcpyDeviceToDevice, m->stream));
-    if (z2_dev && grouped)  // the branches' logits, branch-major [K-1][B][V]
-        CUDA_TRY(m, cudaMemcpyAsync(z2_dev, w.Z + (size_t)B * c.vocab, zb * (npaths(grouped) - 1), cudaMemcpyDeviceToDevice, m->stream));
+    if ((st = run_readout(m, B, grouped, next_dev, alpha_dev, z1_dev, z2_dev)) != DBT_OK) return st;
     for (int b = 0; b < B; b++) m->len_host[b] += 1;
     m->pending_union = c.n_experts > 0;
     return DBT_OK;
@@ -1644,37 +1650,20 @@ dbt_status run_head_wide(dbt_model *m, const RowMap &rm, int grouped, int n_tile
     return run_gemm_tc(m, lm, n_tile, nullptr, nullptr, 0, e);
 }
 
-template <typename WT>
-dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0, const RowMap &rm, int R, int n_tile) {
-    const dbt_config &c = m->cfg;
-    const Workspace &w = m->ws;
-    LAUNCH(m, "embed", 0, embed_fused_kernel<WT>, R, 256, 0, tokens_dev, n, p0, rm, (const WT *)m->w.embed_primary,
-           (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S,
-           m->layers[0].attn_norm_g, w.Xb, m->act_parts == 2 ? (size_t)m->Rmax * c.d_model : (size_t)0, w.ss, m->Rmax,
-           wide_ss_tiles(m), w.status);
-    return DBT_OK;
-}
-
 dbt_status step_wide(dbt_model *m, const int32_t *tokens_dev, int B, int grouped, int32_t *next_dev, float *z1_dev,
                      float *z2_dev, float *alpha_dev) {
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
-    const Workspace &w = m->ws;
     RowMap rm{B, 1};
     int R = npaths(grouped) * B, n_tile = pad_rows(paths_of(c) * B);
     dbt_status st;
-    if ((st = run_attention_plan(m, rm)) != DBT_OK) return st;
-    if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, n_tile)) != DBT_OK) return st;
+    if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, true)) != DBT_OK) return st;
     st = run_layers_wide(m, rm, grouped, n_tile);
     m->att_planned = false;
     if (st != DBT_OK) return st;
     if ((st = run_head_wide(m, rm, grouped, n_tile)) != DBT_OK) return st;
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
-    if ((st = run_readout(m, B, grouped, next_dev, alpha_dev)) != DBT_OK) return st;
-    size_t zb = sizeof(float) * (size_t)B * c.vocab;
-    if (z1_dev) CUDA_TRY(m, cudaMemcpyAsync(z1_dev, w.Z, zb, cudaMemcpyDeviceToDevice, m->stream));
-    if (z2_dev && grouped)  // the branches' logits, branch-major [K-1][B][V]
-        CUDA_TRY(m, cudaMemcpyAsync(z2_dev, w.Z + (size_t)B * c.vocab, zb * (npaths(grouped) - 1), cudaMemcpyDeviceToDevice, m->stream));
+    if ((st = run_readout(m, B, grouped, next_dev, alpha_dev, z1_dev, z2_dev)) != DBT_OK) return st;
     for (int b = 0; b < B; b++) m->len_host[b] += 1;
     return DBT_OK;
 }
@@ -1695,8 +1684,11 @@ dbt_status prefill_tc(dbt_model *m, const int32_t *tokens_dev, int B, int n, flo
         int mode = 0, nsp = 1;
         size_t sstride = 0;
         if (big && cn > 1 && R > 256) {
-            if ((st = run_embed_wide<WT>(m, tokens_dev, tok_n, p0, rm, R, n_tile)) != DBT_OK) return st;
+            if ((st = run_embed_wide<WT>(m, tokens_dev, tok_n, p0, rm, R, false)) != DBT_OK) return st;
             if ((st = run_layers_moe_prompt(m, rm)) != DBT_OK) return st;
+        } else if (c.n_experts > 0 && m->moe_tc && m->moe_wide) {
+            if ((st = run_embed_wide<WT>(m, tokens_dev, tok_n, p0, rm, R, false)) != DBT_OK) return st;
+            if ((st = run_layers_tc(m, rm, 0, n_tile, false, &mode, &nsp, &sstride)) != DBT_OK) return st;
         } else {
             LAUNCH(m, "embed", 0, embed_norm_kernel<WT>, R, 256, 0, tokens_dev, tok_n, p0, rm, (const WT *)m->w.embed_primary,
                    (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S, w.status);
@@ -1728,7 +1720,7 @@ dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, f
         int cn = p0 < n_bulk ? (n_bulk - p0 < cn_max ? n_bulk - p0 : cn_max) : 1;
         RowMap rm{B, cn};
         int R = B * cn, n_tile = pad_rows(R < 256 ? R : 256);
-        if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, n_tile)) != DBT_OK) return st;
+        if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, false)) != DBT_OK) return st;
         const bool pairs = cn > 1 && R > 64;
         if ((st = pairs ? run_layers_prompt(m, rm) : run_layers_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
         if (last_logits && p0 + cn >= n) {
@@ -1889,11 +1881,7 @@ dbt_status step_impl(dbt_model *m, const int32_t *tokens_dev, int B, int grouped
         if ((st = run_head<WT>(m, R, 1, 0)) != DBT_OK) return st;
     }
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
-    if ((st = run_readout(m, B, grouped, next_dev, alpha_dev)) != DBT_OK) return st;
-    size_t zb = sizeof(float) * (size_t)B * c.vocab;
-    if (z1_dev) CUDA_TRY(m, cudaMemcpyAsync(z1_dev, w.Z, zb, cudaMemcpyDeviceToDevice, m->stream));
-    if (z2_dev && grouped)  // the branches' logits, branch-major [K-1][B][V]
-        CUDA_TRY(m, cudaMemcpyAsync(z2_dev, w.Z + (size_t)B * c.vocab, zb * (npaths(grouped) - 1), cudaMemcpyDeviceToDevice, m->stream));
+    if ((st = run_readout(m, B, grouped, next_dev, alpha_dev, z1_dev, z2_dev)) != DBT_OK) return st;
     for (int b = 0; b < B; b++) m->len_host[b] += 1;
     m->pending_union = c.n_experts > 0;
     return DBT_OK;

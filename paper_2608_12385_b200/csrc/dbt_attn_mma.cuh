@@ -63,7 +63,7 @@ struct AttnParams {
     // limit; a chunk holds cn positions per sequence, nbk = ceil(cn / pack) tiles per sequence, one CTA pass per
     // (tile, KV head) over all its keys, no split.  Q rows and output rows are seq * cn + position.
     int pack, cn, nbk;
-    const int *plan;   // the step's precomputed work split (attn_plan_kernel), or nullptr
+    const int *plan;   // the step's precomputed work split (embed_fused_kernel), or nullptr
     int plan_prewait;  // the plan may be read before the dependency wait
 };
 
@@ -142,7 +142,7 @@ __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 128;
 
 // The work split of one attention launch, computed by one warp from the sequence lengths: cum[i] = stages of the
 // rows before row i, nk[i] = keys visible to row i, segcum[i] = segments (per KV head) of the rows before row i.
-// The same for every layer of a decode step, so a step computes it once (attn_plan_kernel) and the attention
+// The same for every layer of a decode step, so a step computes it once (embed_fused_kernel) and the attention
 // launches copy it; launches without a plan (prompt chunks) compute it themselves.
 __device__ __forceinline__ void att_plan_warp(int lane, int items, RowMap rm, const int32_t *seq_len, int n_kv, int C0_arg,
                                               int *cum, int *nk_s, int *segcum) {
@@ -226,9 +226,47 @@ __device__ __forceinline__ void att_plan_warp(int lane, int items, RowMap rm, co
 
 constexpr int kAttPlanInts = 3 * kAttMaxItems + 2;  // cum [items + 1] | nk [items] | segcum [items + 1], at fixed offsets
 
-__global__ void __launch_bounds__(32) attn_plan_kernel(RowMap rm, const int32_t *seq_len, int n_kv, int C0, int *plan) {
+// Eq. embeddings for the fused path: S^0 = RMSNorm(E[x]) and, for the first layer's Q|K|V GEMM,
+// the input g_next * S^0 as two bf16 planes plus sum(S^0 ^2) per row (tile 0 carries the whole
+// sum, the other tile slots are zeroed).  One block per row; with plan != nullptr (decode steps) one more block computes the
+// step's attention work split, which needs the sequence lengths only (as a launch of its own it was one more link of the chain).
+template <typename WT>
+__global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens, int n, int p0, RowMap rm,
+                                                          const WT *__restrict__ E1, const WT *__restrict__ E2,
+                                                          const float *__restrict__ g, float eps, int d, int V,
+                                                          float *S, const float *__restrict__ g_next,
+                                                          __nv_bfloat16 *Xb, size_t lo_off, float *ss_out, int ss_ld,
+                                                          int ss_tiles, int *status, const int32_t *seq_len, int n_kv, int C0, int *plan) {
     pdl_enter();
-    att_plan_warp(threadIdx.x, rm.Bc(), rm, seq_len, n_kv, C0, plan, plan + kAttMaxItems + 1, plan + 2 * kAttMaxItems + 1);
+    __shared__ float scratch[32];
+    int r = blockIdx.x;
+    if (plan && r == (int)gridDim.x - 1) {
+        if (threadIdx.x < 32)
+            att_plan_warp(threadIdx.x, rm.Bc(), rm, seq_len, n_kv, C0, plan, plan + kAttMaxItems + 1, plan + 2 * kAttMaxItems + 1);
+        return;
+    }
+    int path = r / rm.Bc();  // 0 primary; j >= 1: decode branch j with its own table E2[j-1] (Appendix C.1)
+    int tok = ld_mut(tokens + (size_t)rm.seq(r) * n + p0 + rm.off(r));
+    if (tok < 0 || tok >= V) {
+        if (threadIdx.x == 0) report(status, kStatusBadToken, tok);
+        tok = min(max(tok, 0), V - 1);
+    }
+    const WT *e = (path ? E2 + (size_t)(path - 1) * V * d : E1) + (size_t)tok * d;
+    float ss = 0.f;
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        float x = load1(e + i);
+        ss += x * x;
+    }
+    ss = block_sum(ss, scratch);
+    float inv = 1.f / sqrtf(ss / (float)d + eps), sq = 0.f;
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        float s0 = g[i] * load1(e + i) * inv;
+        S[(size_t)r * d + i] = s0;
+        store_split(Xb, (size_t)r * d + i, lo_off, g_next[i] * s0);
+        sq += s0 * s0;
+    }
+    sq = block_sum(sq, scratch);
+    for (int t = threadIdx.x; t < ss_tiles; t += blockDim.x) ss_out[(size_t)t * ss_ld + r] = t == 0 ? sq : 0.f;
 }
 
 template <int DH, bool NARROW, bool DEEP = false>

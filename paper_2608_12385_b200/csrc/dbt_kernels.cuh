@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(1024) readout_kernel(const float *Z, int B, in
 //     normalisers and alpha (Eq. alpha), evaluates alpha p + (1 - alpha) mean_j q_j (Eq. mixloss;
 //     Appendix C.1 for several branches) over its chunk, and leaves its best (value, index); the last
 //     CTA of the row to arrive picks among the NC candidates (lowest index on ties), writes the token and
-//     alpha and advances the sequence length.
+//     alpha and advances the sequence length.  z1_out, z2_out (nullable): the caller's logits, [B][V] and [K-1][B][V].
 // Primary-only steps skip the first kernel: the pick is the argmax of z1.
 // Record layout (kRoRec floats): [0] m1, [1] s1, [2] sum of squares, [3] best value, [4] best index,
 // [5 + 2j] m of branch j, [6 + 2j] s of branch j.
@@ -551,7 +551,8 @@ __global__ void __launch_bounds__(kRoThreads) readout_stats_kernel(const float *
 
 __global__ void __launch_bounds__(kRoThreads) readout_pick_kernel(const float *Z, int B, int V, int chunk, int P,
                                                                   float *stats, int32_t *tickets, int32_t *next,
-                                                                  float *alpha_out, int32_t *seq_len, int advance) {
+                                                                  float *alpha_out, int32_t *seq_len, int advance, float *z1_out,
+                                                                  float *z2_out) {
     pdl_enter();
     __shared__ float bv[32];
     __shared__ int bi[32];
@@ -568,6 +569,21 @@ __global__ void __launch_bounds__(kRoThreads) readout_pick_kernel(const float *Z
         const int v = v0 + j * kRoThreads + tid;
         a[j] = v < v1 ? __ldcg(z1 + v) : -INFINITY;
         c[j] = (grouped && v < v1) ? __ldcg(z2 + v) : -INFINITY;
+    }
+    // the caller's logits leave from here (two copies behind this kernel were two more links of the step's chain)
+    if (z1_out) {
+#pragma unroll
+        for (int j = 0; j < kRoPer; j++) {
+            const int v = v0 + j * kRoThreads + tid;
+            if (v < v1) z1_out[(size_t)b * V + v] = a[j];
+        }
+    }
+    if (z2_out && grouped) {
+#pragma unroll
+        for (int j = 0; j < kRoPer; j++) {
+            const int v = v0 + j * kRoThreads + tid;
+            if (v < v1) z2_out[(size_t)b * V + v] = c[j];
+        }
     }
     if (grouped && warp == 0) {
         // fold the row's records: maxima first, then the sums rescaled to them (a lane per chunk, fixed tree; one lane
@@ -625,7 +641,10 @@ __global__ void __launch_bounds__(kRoThreads) readout_pick_kernel(const float *Z
 #pragma unroll
             for (int j = 0; j < kRoPer; j++) {
                 const int v = v0 + j * kRoThreads + tid;
-                if (v < v1) qs[j] += expf(__ldcg(zj + v) - mj) / dj;
+                if (v >= v1) continue;
+                const float z = __ldcg(zj + v);
+                qs[j] += expf(z - mj) / dj;
+                if (z2_out) z2_out[(size_t)(jb * B + b) * V + v] = z;
             }
         }
     }
