@@ -38,7 +38,7 @@ struct AttnParams {
     int G, n_kv, num_pages, pt_stride;
     long long k_row0;  // first row of this layer's K plane in the pool's row numbering (the V plane is one plane further)
     const int32_t *page_table, *seq_len;
-    float *part;        // [CTAs + pairs][16][DH + 2] segment partials
+    float *part;        // [CTAs + pairs] segment partials: [16][DH] outputs, then [16][2] (m, l)
     int *tickets;       // [rows][n_kv] arrival counters (zero between launches)
     int *tickets2;      // [rows][n_kv][kAttMaxGroups] arrival counters of the segment groups
     __nv_bfloat16 *Ob;  // [rows][q_dim] attention output, hi plane (+ lo plane at lo_off)
@@ -772,11 +772,11 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                             } else {
     #pragma unroll
                                 for (int nb = 0; nb < NB; nb++)
-                                    *reinterpret_cast<float2 *>(out + (size_t)q * (DH + 2) + nb * 8 + c) =
+                                    *reinterpret_cast<float2 *>(out + (size_t)q * DH + nb * 8 + c) =
                                         make_float2(o[nb][2 * h], o[nb][2 * h + 1]);
                                 if ((lane & 3) == 0) {
-                                    out[(size_t)q * (DH + 2) + DH] = m_run[h];  // base-2 units
-                                    out[(size_t)q * (DH + 2) + DH + 1] = l_run[h];
+                                    out[16 * DH + 2 * q] = m_run[h];  // base-2 units
+                                    out[16 * DH + 2 * q + 1] = l_run[h];
                                 }
                             }
                         }
@@ -969,12 +969,12 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                             } else {
 #pragma unroll
                                 for (int mb = 0; mb < MB; mb++) {
-                                    out[(size_t)q * (DH + 2) + mb * 16 + g8] = o[mb][j];
-                                    out[(size_t)q * (DH + 2) + mb * 16 + g8 + 8] = o[mb][2 + j];
+                                    out[(size_t)q * DH + mb * 16 + g8] = o[mb][j];
+                                    out[(size_t)q * DH + mb * 16 + g8 + 8] = o[mb][2 + j];
                                 }
                                 if (g8 == 0) {
-                                    out[(size_t)q * (DH + 2) + DH] = m_run[j];  // base-2 units
-                                    out[(size_t)q * (DH + 2) + DH + 1] = l_run[j];
+                                    out[16 * DH + 2 * q] = m_run[j];  // base-2 units
+                                    out[16 * DH + 2 * q + 1] = l_run[j];
                                 }
                             }
                         }
@@ -991,47 +991,50 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         // long one on a single CTA (a pair of a 32k-token sequence has ~35 segments).
         // merge n partials at slots pbase + j * slot_stride; final: normalise and write the output,
         // else leave the merged (unnormalised) state in the first slot
+        // A thread takes four consecutive outputs of up to two query rows, eight partials of each in flight: up to eight
+        // query rows need one round of loads per eight partials.  (Two single outputs per thread took a round per 256
+        // outputs: 5 us behind the last segment at 4 query rows, 9 at 8; now about 2.)
         auto merge = [&](float *pbase, int slot_stride, int n, bool final) {
             const size_t sstr = (size_t)slot_stride * 16 * (DH + 2);
-            for (int idx0 = tid; idx0 < nq_act * DH; idx0 += 2 * 128) {
-                // two outputs per thread, eight partials of each in flight
-                const float *pq[2];
-                float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f}, X[2] = {0.f, 0.f};
+            constexpr int VQ = DH / 4;  // 16-byte pieces of a query row
+            for (int idx0 = tid; idx0 < nq_act * VQ; idx0 += 2 * 128) {
+                float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f};
+                float4 X[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
                 bool act[2];
                 int ee[2], qq[2];
 #pragma unroll
                 for (int a = 0; a < 2; a++) {
-                    int idx = idx0 + a * 128;
-                    act[a] = idx < nq_act * DH;
-                    qq[a] = act[a] ? idx / DH : 0;
-                    ee[a] = act[a] ? idx % DH : 0;
-                    pq[a] = pbase + (size_t)qq[a] * (DH + 2);
+                    const int idx = idx0 + a * 128;
+                    act[a] = idx < nq_act * VQ;
+                    qq[a] = act[a] ? idx / VQ : 0;
+                    ee[a] = act[a] ? idx % VQ * 4 : 0;
                 }
                 for (int sb = 0; sb < n; sb += 8) {
-                    float mv[2][8], lv[2][8], ov[2][8];
+                    float2 ml[2][8];
+                    float4 ov[2][8];
 #pragma unroll
                     for (int a = 0; a < 2; a++)
 #pragma unroll
                         for (int j = 0; j < 8; j++) {
-                            bool on = act[a] && sb + j < n;
-                            const float *pp = pq[a] + (size_t)(sb + j) * sstr;
-                            mv[a][j] = on ? __ldcg(pp + DH) : -INFINITY;
-                            lv[a][j] = on ? __ldcg(pp + DH + 1) : 0.f;
-                            ov[a][j] = on ? __ldcg(pp + ee[a]) : 0.f;
+                            const bool on = act[a] && sb + j < n;
+                            const float *pp = pbase + (size_t)(sb + j) * sstr;
+                            ml[a][j] = on ? __ldcg(reinterpret_cast<const float2 *>(pp + 16 * DH) + qq[a]) : make_float2(-INFINITY, 0.f);
+                            ov[a][j] = on ? ldcg4(pp + (size_t)qq[a] * DH + ee[a]) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
 #pragma unroll
                     for (int a = 0; a < 2; a++) {
                         float Mn = M[a];
 #pragma unroll
-                        for (int j = 0; j < 8; j++) Mn = fmaxf(Mn, mv[a][j]);
-                        float sc = M[a] == -INFINITY ? 0.f : exp2f(M[a] - Mn);
+                        for (int j = 0; j < 8; j++) Mn = fmaxf(Mn, ml[a][j].x);
+                        const float sc = M[a] == -INFINITY ? 0.f : exp2f(M[a] - Mn);
                         L[a] *= sc;
-                        X[a] *= sc;
+                        X[a].x *= sc, X[a].y *= sc, X[a].z *= sc, X[a].w *= sc;
 #pragma unroll
                         for (int j = 0; j < 8; j++) {
-                            float f = mv[a][j] == -INFINITY ? 0.f : exp2f(mv[a][j] - Mn);
-                            L[a] = fmaf(lv[a][j], f, L[a]);
-                            X[a] = fmaf(ov[a][j], f, X[a]);
+                            const float f = ml[a][j].x == -INFINITY ? 0.f : exp2f(ml[a][j].x - Mn);
+                            L[a] = fmaf(ml[a][j].y, f, L[a]);
+                            X[a].x = fmaf(ov[a][j].x, f, X[a].x), X[a].y = fmaf(ov[a][j].y, f, X[a].y);
+                            X[a].z = fmaf(ov[a][j].z, f, X[a].z), X[a].w = fmaf(ov[a][j].w, f, X[a].w);
                         }
                         M[a] = Mn;
                     }
@@ -1040,16 +1043,13 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 for (int a = 0; a < 2; a++) {
                     if (!act[a]) continue;
                     if (final) {
-                        int row = packed ? item_row0(item) + qq[a] / p.G : (qq[a] / p.G) * Bc + item;
-                        int h = g * p.G + qq[a] % p.G;
-                        size_t o_idx = (size_t)row * q_dim + (size_t)h * DH + ee[a];
-                        float x = X[a] / L[a];
-                        __nv_bfloat16 hi = __float2bfloat16_rn(x);
-                        p.Ob[o_idx] = hi;
-                        if (p.lo_off) p.Ob[o_idx + p.lo_off] = __float2bfloat16_rn(x - __bfloat162float(hi));
+                        const int row = packed ? item_row0(item) + qq[a] / p.G : (qq[a] / p.G) * Bc + item;
+                        const int h = g * p.G + qq[a] % p.G;
+                        store_split4(p.Ob, (size_t)row * q_dim + (size_t)h * DH + ee[a], p.lo_off,
+                                     make_float4(X[a].x / L[a], X[a].y / L[a], X[a].z / L[a], X[a].w / L[a]));
                     } else {
-                        // this thread is the only reader of the first slot's element (q, e)
-                        pbase[(size_t)qq[a] * (DH + 2) + ee[a]] = X[a];
+                        // this thread is the only reader of the first slot's elements (q, e..)
+                        *reinterpret_cast<float4 *>(pbase + (size_t)qq[a] * DH + ee[a]) = X[a];
                         if (ee[a] == 0) {
                             sc_m[qq[a]] = M[a];
                             sc_l[qq[a]] = L[a];
@@ -1060,8 +1060,8 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
             if (!final) {
                 consumer_sync();  // every thread has read the first slot's (m, l): now they may change
                 if (tid < nq_act) {
-                    pbase[(size_t)tid * (DH + 2) + DH] = sc_m[tid];
-                    pbase[(size_t)tid * (DH + 2) + DH + 1] = sc_l[tid];
+                    pbase[16 * DH + 2 * tid] = sc_m[tid];
+                    pbase[16 * DH + 2 * tid + 1] = sc_l[tid];
                 }
                 __threadfence();
             }
