@@ -8,8 +8,11 @@
 //
 // Work decomposition.  A (row, KV head) pair of u 64-token stages is cut into n ~ u / q equal
 // segments (q: a target length chosen so that the segments fill one to three rounds of the
-// grid); the segments of all pairs, in (row, KV head, segment) order, are dealt to a fixed grid
-// of CTAs (two per SM) round robin.
+// grid); the segments of all pairs, in (row, KV head, segment) order with the rows by falling length,
+// are dealt to a fixed grid of CTAs (two per SM), every second round backwards: the CTAs' shares then
+// differ little however the lengths do, and the pairs of an incomplete last round are cut to fill it.
+// (An equal share of all stages per CTA, cutting pairs at its borders, was measured: 16 % slower on 117
+// ragged sequences, as every CTA pays for one more query build, fold and merge.)
 // A CTA never straddles two pairs (the per-segment costs -- building the queries, folding the
 // warps, the merge -- are then paid once per CTA for equal-length batches), and the split depends
 // on the lengths only.  A segment's un-normalised partial (m, l, O) goes to the slot of its
@@ -76,6 +79,7 @@ constexpr int kAttMaxSeg = 256;    // most segments a (sequence, KV head) pair i
 constexpr int kAttGroup = 8;       // segments merged at once (one round of loads)
 constexpr int kAttSingle = 16;     // up to this many segments, one CTA merges them all (two rounds of loads)
 constexpr int kAttMaxGroups = kAttMaxSeg / kAttGroup;
+constexpr unsigned kAttKeyMask = (1u << 24) - 1;  // keys of a row in the plan; its row index above
 constexpr float kLog2e = 1.4426950408889634f;
 
 // DEEP: one CTA per SM with a ring twice as deep instead of two CTAs per SM: the same bytes in flight per SM,
@@ -140,21 +144,17 @@ __device__ __forceinline__ void tma_load_4d_hint(uint32_t dst, const CUtensorMap
 }
 __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
 
-// The work split of one attention launch, computed by one warp from the sequence lengths: cum[i] = stages of the
-// rows before row i, nk[i] = keys visible to row i, segcum[i] = segments (per KV head) of the rows before row i.
+// The work split of one attention launch, computed by one warp from the keys nk[i] = keys | row << 24 of its rows in the
+// order in which they are dealt (by falling length where the step's plan sorts them): cum[i] = stages of the rows before
+// place i, segcum[i] = segments (per KV head) of the rows before place i.
 // The same for every layer of a decode step, so a step computes it once (embed_fused_kernel) and the attention
 // launches copy it; launches without a plan (prompt chunks) compute it themselves.
-__device__ __forceinline__ void att_plan_warp(int lane, int items, RowMap rm, const int32_t *seq_len, int n_kv, int C0_arg,
-                                              int *cum, int *nk_s, int *segcum) {
+__device__ __forceinline__ void att_plan_warp(int lane, int items, int n_kv, int C0_arg, int *cum, const unsigned *nk_s, int *segcum) {
     int running = 0, longest = 0;
     if (lane == 0) cum[0] = 0;
     for (int base = 0; base < items; base += 32) {
-        int i = base + lane, nk = 0, u = 0;
-        if (i < items) {
-            nk = ld_mut(seq_len + rm.seq(i)) + rm.off(i) + 1;
-            u = (nk + kAttTile - 1) / kAttTile;
-            nk_s[i] = nk;
-        }
+        int i = base + lane, u = 0;
+        if (i < items) u = ((int)(nk_s[i] & kAttKeyMask) + kAttTile - 1) / kAttTile;
         int incl = u, mx = u;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -208,11 +208,22 @@ __device__ __forceinline__ void att_plan_warp(int lane, int items, RowMap rm, co
         // the plain split fits one round, or every pair is already whole: take it (the common cases)
         if (cand == 0 && (rounds == 1 || sg == items * n_kv)) break;
     }
+    // Whole pairs in several rounds: the rows of an incomplete last round are cut to fill it (936 equal pairs on 296 CTAs
+    // would take four rounds for 3.16).
+    const int pairs = items * n_kv, rem = pairs % C0;
+    int tail0 = items, tail_n = 1;
+    if (best_sg == pairs && pairs > C0 && rem > 0) {
+        const int t0 = (pairs - rem + n_kv - 1) / n_kv;
+        if (t0 < items && C0 / ((items - t0) * n_kv) > 1) {
+            tail0 = t0;
+            tail_n = min(C0 / ((items - t0) * n_kv), kAttGroup);
+        }
+    }
     int run2 = 0;
     if (lane == 0) segcum[0] = 0;
     for (int base = 0; base < items; base += 32) {
         int i = base + lane, n = 0;
-        if (i < items) n = seg_count(cum[i + 1] - cum[i], best_q, best_mode);
+        if (i < items) n = i >= tail0 ? max(1, min(tail_n, (cum[i + 1] - cum[i]) / kAttMinUnits)) : seg_count(cum[i + 1] - cum[i], best_q, best_mode);
         int incl = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -225,6 +236,32 @@ __device__ __forceinline__ void att_plan_warp(int lane, int items, RowMap rm, co
 }
 
 constexpr int kAttPlanInts = 3 * kAttMaxItems + 2;  // cum [items + 1] | nk [items] | segcum [items + 1], at fixed offsets
+
+// A decode step's plan (one position per sequence), by one block of at least 256 threads: rows by falling length.
+__device__ __forceinline__ void att_plan_block(int B, const int32_t *seq_len, int n_kv, int C0, int *plan) {
+    __shared__ int len[kAttMaxItems], cum[kAttMaxItems + 1], segcum[kAttMaxItems + 1];
+    __shared__ unsigned nk[kAttMaxItems];
+    const int i = threadIdx.x;
+    if (i < B) len[i] = ld_mut(seq_len + i) + 1;
+    __syncthreads();
+    if (i < B) {
+        int rank = 0;
+        for (int j = 0; j < B; j++) rank += len[j] > len[i] || (len[j] == len[i] && j < i);
+        nk[rank] = (unsigned)len[i] | (unsigned)i << 24;
+    }
+    __syncthreads();
+    if (i < 32) att_plan_warp(i, B, n_kv, C0, cum, nk, segcum);
+    __syncthreads();
+    if (i <= B && i <= kAttMaxItems) {
+        plan[i] = cum[i];
+        plan[2 * kAttMaxItems + 1 + i] = segcum[i];
+        if (i < B) plan[kAttMaxItems + 1 + i] = (int)nk[i];
+    }
+    if (i == 0 && B == kAttMaxItems) {  // (256 threads: the last place of 257)
+        plan[B] = cum[B];
+        plan[2 * kAttMaxItems + 1 + B] = segcum[B];
+    }
+}
 
 // Eq. embeddings for the fused path: S^0 = RMSNorm(E[x]) and, for the first layer's Q|K|V GEMM,
 // the input g_next * S^0 as two bf16 planes plus sum(S^0 ^2) per row (tile 0 carries the whole
@@ -241,8 +278,7 @@ __global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens,
     __shared__ float scratch[32];
     int r = blockIdx.x;
     if (plan && r == (int)gridDim.x - 1) {
-        if (threadIdx.x < 32)
-            att_plan_warp(threadIdx.x, rm.Bc(), rm, seq_len, n_kv, C0, plan, plan + kAttMaxItems + 1, plan + 2 * kAttMaxItems + 1);
+        att_plan_block(rm.B, seq_len, n_kv, C0, plan);
         return;
     }
     int path = r / rm.Bc();  // 0 primary; j >= 1: decode branch j with its own table E2[j-1] (Appendix C.1)
@@ -286,8 +322,8 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
     float *sc_l = sc_m + 16;                                                        // [16]
     int *flag = reinterpret_cast<int *>(sc_l + 16);                                 // [0] last?, [1] longest pair, [8..15] 1/rms per path
     int *cum = flag + 16;                // [items + 1] prefix of tiles per row
-    int *nk_s = cum + kAttMaxItems + 1;  // [items] visible keys per row
-    int *segcum = nk_s + kAttMaxItems;   // [items + 1] prefix of segments per row (per KV head)
+    unsigned *nk_s = reinterpret_cast<unsigned *>(cum + kAttMaxItems + 1);  // [items] visible keys per row | row << 24
+    int *segcum = cum + 2 * kAttMaxItems + 1;   // [items + 1] prefix of segments per row (per KV head)
     __nv_bfloat16 *kv_new =  // [2][DH] this step's K, V row (16-byte aligned)
         reinterpret_cast<__nv_bfloat16 *>((reinterpret_cast<uintptr_t>(segcum + kAttMaxItems + 1) + 15) & ~(uintptr_t)15);
 
@@ -321,10 +357,13 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         for (int i = tid; i <= items; i += blockDim.x) {
             cum[i] = ld_mut(p.plan + i);
             segcum[i] = ld_mut(p.plan + 2 * kAttMaxItems + 1 + i);
-            if (i < items) nk_s[i] = ld_mut(p.plan + kAttMaxItems + 1 + i);
+            if (i < items) nk_s[i] = (unsigned)ld_mut(p.plan + kAttMaxItems + 1 + i);
         }
     } else if (warp == 0 && !packed) {
-        att_plan_warp(lane, items, p.rm, p.seq_len, p.n_kv, (int)gridDim.x, cum, nk_s, segcum);
+        for (int i = lane; i < items; i += 32)
+            nk_s[i] = (unsigned)(ld_mut(p.seq_len + p.rm.seq(i)) + p.rm.off(i) + 1) | (unsigned)i << 24;
+        __syncwarp();
+        att_plan_warp(lane, items, p.n_kv, (int)gridDim.x, cum, nk_s, segcum);
     }
     __syncthreads();
     if (use_plan && p.plan_prewait) pdl_wait();
@@ -332,36 +371,36 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
     const int C = gridDim.x, Sg = packed ? items * p.n_kv : segcum[items] * p.n_kv;  // all segments, ordered (row, KV head, segment)
     DBT_TL_MARK(3);
     if ((int)blockIdx.x >= Sg) return;
-    // segment sidx -> its row, KV head, stage range and the pair's segment count
-    auto item_nkeys = [&](int i) {
-        if (!packed) return nk_s[i];
-        return ld_mut(p.seq_len + i / p.nbk) + (i % p.nbk) * p.pack + item_npos(i);
-    };
-    auto locate = [&](int sidx, int &item, int &g, int &seg, int &n, int &ui, int &t0, int &t1) {
+    // segment sidx -> its row and the keys it sees, KV head, stage range and the pair's segment count
+    auto locate = [&](int sidx, int &item, int &nkeys, int &g, int &seg, int &n, int &ui, int &t0, int &t1) {
         if (packed) {  // one pass per (tile, KV head) over all its keys
             item = sidx / p.n_kv;
+            nkeys = ld_mut(p.seq_len + item / p.nbk) + (item % p.nbk) * p.pack + item_npos(item);
             g = sidx % p.n_kv;
             seg = 0;
             n = 1;
-            ui = (item_nkeys(item) + kAttTile - 1) / kAttTile;
+            ui = (nkeys + kAttTile - 1) / kAttTile;
             t0 = 0;
             t1 = ui;
             return;
         }
         int lo = 0, hi = items - 1;
-        while (lo < hi) {  // largest row whose first segment is <= sidx
+        while (lo < hi) {  // largest place whose first segment is <= sidx
             int mid = (lo + hi + 1) >> 1;
             if (segcum[mid] * p.n_kv <= sidx) lo = mid; else hi = mid - 1;
         }
-        item = lo;
-        n = segcum[item + 1] - segcum[item];
-        int rel = sidx - segcum[item] * p.n_kv;
+        item = (int)(nk_s[lo] >> 24);
+        nkeys = (int)(nk_s[lo] & kAttKeyMask);
+        n = segcum[lo + 1] - segcum[lo];
+        int rel = sidx - segcum[lo] * p.n_kv;
         g = rel / n;
         seg = rel % n;
-        ui = cum[item + 1] - cum[item];
+        ui = cum[lo + 1] - cum[lo];
         t0 = (int)(((long long)seg * ui) / n);
         t1 = (int)(((long long)(seg + 1) * ui) / n);
     };
+    // this CTA's segment of a round: every second round is dealt backwards
+    auto dealt = [&](int round) { return round * C + ((round & 1) ? C - 1 - (int)blockIdx.x : (int)blockIdx.x); };
 
     if (warp == kAttWarps) {
         // ---- producer: walks the same segments as the consumers.  Lane 0 waits for the stage and
@@ -371,10 +410,10 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         const uint64_t pol = l2_evict_first_policy();
         bool ok = true;
         int it = 0;
-        for (int sidx = blockIdx.x; sidx < Sg && ok; sidx += C) {
-            int item, g, seg, n, ui, t0, t1;
-            locate(sidx, item, g, seg, n, ui, t0, t1);
-            int seq = item_seq(item), total_pages = (item_nkeys(item) + 15) >> 4;
+        for (int round = 0, sidx; ok && (sidx = dealt(round)) < Sg; round++) {
+            int item, nkeys, g, seg, n, ui, t0, t1;
+            locate(sidx, item, nkeys, g, seg, n, ui, t0, t1);
+            int seq = item_seq(item), total_pages = (nkeys + 15) >> 4;
             // page ids 32 at a time (eight stages' worth, one coalesced load): a lookup per stage would put an
             // L2 round trip on every stage of this loop and cap a CTA at one stage per ~0.7 us
             int pt_base = -(1 << 30), my_page = 0;
@@ -411,7 +450,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 // at once instead, with the small loads issued first, was measured slower: the queries are ready
                 // 0.8 us sooner but the stream then runs 10 % slower; pausing after one, two, four or six stages
                 // gave 1.0446, 1.0384, 1.0420 and 1.0462 ms per step of the 1B model at batch 16.)
-                if (it == kAttPauseAt || (it < kAttPauseAt && sidx + C >= Sg && t == t1 - 1)) asm volatile("bar.sync 2, 160;" ::: "memory");
+                if (it == kAttPauseAt || (it < kAttPauseAt && dealt(round + 1) >= Sg && t == t1 - 1)) asm volatile("bar.sync 2, 160;" ::: "memory");
             }
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 300);
@@ -435,10 +474,9 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         }
         __syncwarp();
     };
-    for (int sidx = blockIdx.x; sidx < Sg; sidx += C) {
-        int item, g, seg, nseg, ui, t0, t1;
-        locate(sidx, item, g, seg, nseg, ui, t0, t1);
-        int nkeys = item_nkeys(item);
+    for (int round = 0, sidx; (sidx = dealt(round)) < Sg; round++) {
+        int item, nkeys, g, seg, nseg, ui, t0, t1;
+        locate(sidx, item, nkeys, g, seg, nseg, ui, t0, t1);
         if (packed) nq_act = item_npos(item) * p.G;  // rows: position-major, the G heads of each position
 
         // Query tile (16 rows x DH, fp32) into shared memory, then mma A fragments (bf16),
@@ -567,7 +605,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
             }
         }
         consumer_sync();
-        if (sidx == (int)blockIdx.x) {
+        if (round == 0) {
             asm volatile("bar.arrive 2, 160;" ::: "memory");  // the producer may stream on
             DBT_TL_MARK(0);
         }
@@ -983,7 +1021,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 }
             }
         }
-        if (sidx == (int)blockIdx.x) DBT_TL_MARK(1);
+        if (round == 0) DBT_TL_MARK(1);
         // ---- merging a pair's segments.  Up to kAttSingle segments: the last one to arrive merges them
         // all, in segment order, and writes the output.  More: the segments form groups of kAttGroup;
         // the last arrival of a group merges it in place into the group's first slot, and the last
@@ -1093,7 +1131,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 }
             }
         }
-        if (sidx == (int)blockIdx.x) DBT_TL_MARK(2);
+        if (round == 0) DBT_TL_MARK(2);
     }
 #ifdef DBT_TL_ATT_ALL
     {  // every CTA leaves a record: mark 3 carries (SM id << 16 | block index)
