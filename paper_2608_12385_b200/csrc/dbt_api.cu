@@ -913,11 +913,12 @@ dbt_status launch_gemm_tc(dbt_model *m, const TcCall &c, const TcParams &p, cons
 // Y partials P[split][R][ldp]; returns the split count and stride the consumer must use.
 dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_out, size_t *split_stride_out,
                        int force_split = 0, LmEpi e = LmEpi{}, int test_skip_load = 0) {
-    // Many stacked rows (row tiles of 128 and 256): pairs of SMs with the rows on the M side, one finished sum per output.
-    // At 234 rows of the 1B model against row tiles of 256 on one SM with split-K partials, per launch by events: gate|up
-    // 43 -> 27 us, Q|K|V 23 -> 21, O 19 -> 19, output matrix 80 -> 56, down 25 -> 29 (its sums then need no second pass).
-    // (Up to 64 rows the weight stream is the bound and both sides take the same time, but M is 256 whatever the rows.)
-    if (!c.grp_cnt && c.parts == 2 && n_tile >= 128 && many_rows_ok(c)) {
+    // Many stacked rows (more than 128): pairs of SMs with the rows on the M side, one finished sum per output.  At 234
+    // rows of the 1B model against row tiles of 256 on one SM with split-K partials, per launch by events: gate|up 43 -> 27
+    // us, Q|K|V 23 -> 21, O 19 -> 19, output matrix 80 -> 56, down 25 -> 29 (its sums then need no second pass); a step is
+    // 5 % faster at 132 rows, 20 % at 234.  Up to 128 rows half of M would be idle and the row tile of 128 keeps four stages
+    // of both planes as one operand: a step of 128 rows is 13 % faster that way, of 80 rows 17 %.
+    if (!c.grp_cnt && c.parts == 2 && n_tile >= 256 && many_rows_ok(c)) {
         PgParams q{};
         q.P = e.Z ? e.Z : c.P;
         for (int s = 0; s < c.nseg; s++) q.ldp += c.n_out[s];
@@ -1455,7 +1456,7 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
     double kv_bytes = 0;
     for (int b = 0; b < rm.B; b++)
         for (int j = 0; j < rm.cn; j++) kv_bytes += (double)(m->len_host[b] + j + 1) * 2 * kvd * sizeof(WT);
-    const bool many = n_tile >= 128 && d % 4 == 0 && F % 4 == 0;  // (the GEMMs then leave finished sums, see run_gemm_tc)
+    const bool many = n_tile >= 256 && d % 4 == 0 && F % 4 == 0;  // (the GEMMs then leave finished sums, see run_gemm_tc)
     dbt_status st;
     int nsp = 1;
     size_t sstride = 0;
@@ -1721,7 +1722,8 @@ dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, f
         RowMap rm{B, cn};
         int R = B * cn, n_tile = pad_rows(R < 256 ? R : 256);
         if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, false)) != DBT_OK) return st;
-        const bool pairs = cn > 1 && R > 64;
+        // (measured on the 1B model: 128 rows 7 % slower than the decode step's kernels, 199 rows 23 % faster)
+        const bool pairs = cn > 1 && R > 128;
         if ((st = pairs ? run_layers_prompt(m, rm) : run_layers_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
         if (last_logits && p0 + cn >= n) {
             if ((st = run_head_wide(m, rm, 0, n_tile)) != DBT_OK) return st;
@@ -1833,7 +1835,7 @@ bool setup_tc(dbt_model *m) {
         m->act_base[&m->map_Hs] = {w.Hs};
     }
     const char *fa = getenv("DBT_ATTN");
-    m->att_fast = ok && allow_smem_prompt() && !(fa && strcmp(fa, "simt") == 0) &&
+    m->att_fast = ok && allow_smem_prompt() && c.max_seq < (1 << 24) && !(fa && strcmp(fa, "simt") == 0) &&
                   make_kv_page_map(&m->map_kv, m->kv_pool, (uint64_t)c.n_layers * 2 * c.num_pages * c.n_kv_heads * c.page_size,
                                    (uint64_t)c.num_pages * c.n_kv_heads * c.page_size, c.head_dim) &&
                   cudaFuncSetAttribute(attn_prompt_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -72,7 +72,7 @@ def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n):
 @pytest.mark.parametrize("n_out,K,R", [(2048, 2048, 70), (2048, 2048, 256), (1028, 520, 129), (4096, 5632, 234), (1024, 64, 200),
                                        (11264, 2048, 130)])
 def test_many_row_decode_widths_match_the_oracle(n_out, K, R):
-    """Decode steps of 65 to 256 stacked rows take the paired-SM GEMMs: the split over clusters (2 and 4 pairs per tile),
+    """Decode steps of 129 to 256 stacked rows take the paired-SM GEMMs (fewer: row tiles of 128 on one SM): the split over clusters (2 and 4 pairs per tile),
     ragged last k-tiles and feature tiles.  One layer whose MLP has the given widths, primary rows and branch rows."""
     cfg = cfg_of(d_model=K if K <= 2048 else 256, d_ff=max(n_out, K) // 2 // 8 * 8, n_layers=1, vocab=1028)
     B = (R + 1) // 2
