@@ -136,6 +136,7 @@ struct dbt_model {
     std::vector<GraphEntry> graphs;
     // where a decode step finds sequence b's token: tokens[b * tok_stride + tok_p0] (1, 0 except inside dbt_prefill_boundary)
     int tok_stride = 1, tok_p0 = 0;
+    bool cluster16 = false;    // clusters of 16 CTAs can run here (see small_cluster)
     bool att_planned = false;  // inside a decode step whose attention work split has been computed (run_embed_wide)
 };
 
@@ -629,7 +630,42 @@ dbt_status run_small_attention(dbt_model *m, const SmallAttn &a, int nsplit, dou
     return DBT_OK;
 }
 
-// The layer stack and the shared output matrix of a decode step at few rows: five kernels per layer.
+// Shared memory of the cluster kernel behind each attention launch for steps of B sequences, 0 where the model or the rows do
+// not fit it.  Sized for all paths, whatever the mode, so that both modes do the same arithmetic per row.
+size_t small_cluster(const dbt_model *m, int B) {
+    const dbt_config &c = m->cfg;
+    const int qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim;
+    return m->cluster16 ? small_cluster_smem(paths_of(c) * B, c.d_model, qd, c.d_ff, qd + 2 * kvd) : 0;
+}
+
+// Whether the cluster kernel may run here: 16 CTAs per cluster are beyond the portable size.
+bool allow_small_cluster() {
+    for (const void *f : {(const void *)small_mlp_kernel<4>, (const void *)small_mlp_kernel<8>})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kScMaxSmem) != cudaSuccess ||
+            cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kScCtas);
+    cfg.blockDim = dim3(kScThreads);
+    cfg.dynamicSmemBytes = kScMaxSmem;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = kScCtas;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, small_mlp_kernel<8>, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return n > 0;
+}
+
+// The layer stack and the shared output matrix of a decode step at few rows: five kernels per layer, two where the cluster
+// kernel takes all that lies between two attention launches.
 dbt_status run_layers_small(dbt_model *m, int B, int grouped) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
@@ -646,13 +682,14 @@ dbt_status run_layers_small(dbt_model *m, int B, int grouped) {
         a.X = X; a.g = g; a.eps = c.rms_eps; a.K = K; a.epi = epi; a.Bc = B; a.S = w.S;
         return a;
     };
+    const size_t csm = small_cluster(m, B);
     for (int l = 0; l < c.n_layers; l++) {
         const dbt_layer_weights &lw = m->layers[l];
         SmallLin q = lin(lw.wq, w.Q, qd, w.S, lw.attn_norm_g, d, EPI_STORE);
         q.W[1] = lw.wk; q.Y[1] = w.Kn; q.n_out[1] = kvd; q.rows[1] = B;
         q.W[2] = lw.wv; q.Y[2] = w.Vn; q.n_out[2] = kvd; q.rows[2] = B;
         q.nseg = 3;
-        if ((st = run_small_linear(m, "linear_qkv", B, q)) != DBT_OK) return st;
+        if ((csm == 0 || l == 0) && (st = run_small_linear(m, "linear_qkv", B, q)) != DBT_OK) return st;
         SmallAttn t{};
         t.Q = w.Q; t.Kn = w.Kn; t.Vn = w.Vn;
         t.B = B; t.P = npaths(grouped); t.G = c.n_q_heads / c.n_kv_heads; t.n_kv = c.n_kv_heads;
@@ -663,6 +700,25 @@ dbt_status run_layers_small(dbt_model *m, int B, int grouped) {
         t.part = w.part; t.tickets = w.att_tickets; t.O = w.O; t.status = w.status;
         st = c.head_dim == 128 ? run_small_attention<128>(m, t, nsplit, kv_bytes) : run_small_attention<64>(m, t, nsplit, kv_bytes);
         if (st != DBT_OK) return st;
+        if (csm) {
+            SmallMlp a{};
+            a.O = w.O; a.wo = (const float *)lw.wo; a.g_mlp = lw.mlp_norm_g;
+            a.wg = (const float *)lw.w_gate; a.wu = (const float *)lw.w_up; a.coup_b = lw.coup_b;
+            a.wd = (const float *)lw.w_down; a.coup_c = lw.coup_c;
+            a.S = w.S; a.R = R; a.Bc = B; a.d = d; a.qd = qd; a.F = c.d_ff; a.eps = c.rms_eps; a.status = w.status;
+            float *const y[3] = {w.Q, w.Kn, w.Vn};
+            const int n[3] = {qd, kvd, kvd}, rows[3] = {R, B, B};
+            for (int s = 0; s < 3; s++) a.y_next[s] = y[s], a.n_next[s] = n[s], a.rows_next[s] = rows[s];
+            if (l + 1 < c.n_layers) {
+                const dbt_layer_weights &nw = m->layers[l + 1];
+                a.g_next = nw.attn_norm_g;
+                a.w_next[0] = (const float *)nw.wq; a.w_next[1] = (const float *)nw.wk; a.w_next[2] = (const float *)nw.wv;
+            }
+            const double bytes = ((double)2 * d * qd + 2.0 * d * kvd + 3.0 * d * c.d_ff) * 4;
+            if (paths_of(c) * B <= 4) LAUNCH_CLUSTER(m, "small_mlp", bytes, kScCtas, small_mlp_kernel<4>, kScCtas, kScThreads, csm, a);
+            else LAUNCH_CLUSTER(m, "small_mlp", bytes, kScCtas, small_mlp_kernel<8>, kScCtas, kScThreads, csm, a);
+            continue;
+        }
         if ((st = run_small_linear(m, "linear_o", B, lin(lw.wo, nullptr, d, w.O, nullptr, qd, EPI_RESID))) != DBT_OK) return st;
         SmallLin gu = lin(lw.w_gate, w.G1, c.d_ff, w.S, lw.mlp_norm_g, d, EPI_SWIGLU);
         gu.W[1] = lw.w_up; gu.coup = lw.coup_b;
@@ -671,7 +727,14 @@ dbt_status run_layers_small(dbt_model *m, int B, int grouped) {
         dn.coup = lw.coup_c;
         if ((st = run_small_linear(m, "linear_down", B, dn)) != DBT_OK) return st;
     }
-    return run_small_linear(m, "lm_head", B, lin(m->w.lm_head, w.Z, c.vocab, w.S, c.final_norm ? m->w.final_norm_g : nullptr, d, EPI_STORE));
+    const SmallLin lm = lin(m->w.lm_head, w.Z, c.vocab, w.S, c.final_norm ? m->w.final_norm_g : nullptr, d, EPI_STORE);
+    if (paths_of(c) * B <= 8 && d <= 256) {
+        const double bytes = (double)c.vocab * d * 4;
+        if (paths_of(c) * B <= 4) LAUNCH(m, "lm_head", bytes, logits_small_kernel<4>, (c.vocab + 31) / 32, 256, 0, lm);
+        else LAUNCH(m, "lm_head", bytes, logits_small_kernel<8>, (c.vocab + 31) / 32, 256, 0, lm);
+        return DBT_OK;
+    }
+    return run_small_linear(m, "lm_head", B, lm);
 }
 
 // Final norm + shared output matrix on `rows` rows taken from S (row r*src_mul+src_add).
@@ -1998,6 +2061,7 @@ dbt_status dbt_create(const dbt_config *cfg, const dbt_weights *w, void *kv_pool
         m->num_sms = sms > 0 && sms <= 148 ? sms : 148;  // the partial buffer is sized for 2 x 148 CTAs
     }
     m->tc = setup_tc(m);
+    m->cluster16 = cfg->weight_dtype == DBT_DTYPE_F32 && !moe && allow_small_cluster();
     {
         const char *ef = getenv("DBT_EVICT_FIRST");
         m->evict_first = !(ef && strcmp(ef, "0") == 0);

@@ -9,10 +9,12 @@
 //                         KV head) pair is split over blocks by its own length and merged by the last one to arrive;
 //   linear_small          O + residual; gate|up with the norm, SwiGLU and b; down with c and residual -- a warp keeps a
 //                         feature of all rows, so a branch row finds its primary twin in the same warp.
-// Measured on the tiny fp32 model (4 layers, batch 2, context 64..80): 192 -> 128 us per step, copies of the outputs included.
+// Measured on the tiny fp32 model (4 layers, batch 2, context 64..80), copies of the outputs included: 192 -> 126 us per step;
+// with the cluster kernel behind each attention launch (its phases take 1.5, 3.1, 2.2 and 2.0 us) 90.
 #pragma once
 
 #include "dbt_fused.cuh"
+#include "dbt_gemm_prompt.cuh"
 #include "dbt_kernels.cuh"
 
 namespace dbt {
@@ -151,11 +153,14 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
     __shared__ __align__(16) float red[kSaThreads / 32][NQ][DH];
     __shared__ float m_s[NQ], l_s[NQ], corr_s[NQ];
     __shared__ int last_s;
+    __shared__ int page_s[kSaChunk / 16 + 1];  // the pass's pages: one load instead of one in front of every key
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x, g = blockIdx.y, sp = blockIdx.z, nsplit = gridDim.z;
     const int nq = a.P * a.G, q_dim = a.n_kv * a.G * DH, kv_dim = a.n_kv * DH, half = DH / 2;
     pdl_launch_dependents();
+    DBT_TL_DECL;
     pdl_wait();
+    DBT_TL_WAITED;
     const int pos = ld_mut(a.seq_len + b), nkeys = pos + 1;
     const int n_act = min(nsplit, (nkeys + kSaSplitKeys - 1) / kSaSplitKeys);  // by the sequence's own length
     if (sp >= n_act) return;
@@ -163,14 +168,19 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
     const int jbeg = min(nkeys, sp * pps * 16), jend = min(nkeys, jbeg + pps * 16);
     const bool owns_new = pos >= jbeg && pos < jend;
     const int32_t *pt = a.page_table + (size_t)b * a.pt_stride;
-    auto row_of = [&](int j) {  // pool row of key j of this head
-        int page = pt[j >> 4];
-        if (page < 0 || page >= a.num_pages) {
-            report(a.status, kStatusBadPage, page);
-            page = 0;
+    auto fetch_pages = [&](int j0) {  // jbeg, and with it every pass, starts on a page border
+        if (tid < kSaChunk / 16 && j0 + tid * 16 < jend) {
+            int page = pt[(j0 >> 4) + tid];
+            if (page < 0 || page >= a.num_pages) {
+                report(a.status, kStatusBadPage, page);
+                page = -1;
+            }
+            page_s[tid] = page;
         }
-        return (((size_t)page * a.n_kv + g) * 16 + (j & 15)) * DH;
     };
+    fetch_pages(jbeg);
+    // pool row of key j0 + j of this head (a bad page id was reported: the step runs on with page 0)
+    auto row_of = [&](int j) { return (((size_t)max(page_s[j >> 4], 0) * a.n_kv + g) * 16 + (j & 15)) * DH; };
     // the new key and value: rotated, appended by the split that holds the position
     if (owns_new && tid < half) {
         const float2 t = a.rope[(size_t)pos * half + tid];
@@ -178,7 +188,7 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
         const float x0 = __ldcg(kn + tid), x1 = __ldcg(kn + tid + half), v0 = __ldcg(vn + tid), v1 = __ldcg(vn + tid + half);
         const int page = pt[pos >> 4];
         if (page >= 0 && page < a.num_pages) {
-            const size_t r = row_of(pos);
+            const size_t r = (((size_t)page * a.n_kv + g) * 16 + (pos & 15)) * DH;
             a.kpool[r + tid] = x0 * t.x - x1 * t.y;
             a.kpool[r + tid + half] = x1 * t.x + x0 * t.y;
             a.vpool[r + tid] = v0;
@@ -209,6 +219,7 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
         m_s[tid] = -INFINITY;
         l_s[tid] = 0.f;
     }
+    DBT_TL_MARK(0);
     __syncthreads();  // (the appended row too: written by this block)
     const int dl = (lane % LPK) * 4, ksub = warp * KPW + lane / LPK;  // this thread's four dims; its key within KPB
     float o[NQ][4];
@@ -216,19 +227,23 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
     for (int q = 0; q < NQ; q++) o[q][0] = o[q][1] = o[q][2] = o[q][3] = 0.f;
     for (int j0 = jbeg; j0 < jend; j0 += kSaChunk) {
         const int cnt = min(kSaChunk, jend - j0);
+        if (j0 > jbeg) {
+            fetch_pages(j0);
+            __syncthreads();
+        }
         constexpr int U = 4;  // keys in flight per lane group
         float4 vv[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {  // the first values travel with the first keys
             const int j = ksub + u * KPB;
-            vv[u] = j < cnt ? ldcg4(a.vpool + row_of(j0 + j) + dl) : make_float4(0.f, 0.f, 0.f, 0.f);
+            vv[u] = j < cnt ? ldcg4(a.vpool + row_of(j) + dl) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         for (int k0 = 0; k0 < cnt; k0 += U * KPB) {
             float4 kk[U];
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 const int j = k0 + ksub + u * KPB;
-                kk[u] = j < cnt ? ldcg4(a.kpool + row_of(j0 + j) + dl) : make_float4(0.f, 0.f, 0.f, 0.f);
+                kk[u] = j < cnt ? ldcg4(a.kpool + row_of(j) + dl) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
             for (int u = 0; u < U; u++) {
@@ -274,7 +289,7 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
 #pragma unroll
                 for (int u = 0; u < U; u++) {
                     const int j = k0 + ksub + u * KPB;
-                    vv[u] = j < cnt ? ldcg4(a.vpool + row_of(j0 + j) + dl) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    vv[u] = j < cnt ? ldcg4(a.vpool + row_of(j) + dl) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
             }
 #pragma unroll
@@ -292,6 +307,7 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
         }
         __syncthreads();  // the scores are free again
     }
+    DBT_TL_MARK(1);
     // fold the key subsets: within a warp, then the warps in order
 #pragma unroll
     for (int q = 0; q < NQ; q++) {
@@ -315,6 +331,7 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
         else
             part[(size_t)q * (DH + 2) + e] = t;
     }
+    DBT_TL_END("attsmall");
     if (n_act == 1) return;
     if (tid < nq) {
         part[(size_t)tid * (DH + 2) + DH] = m_s[tid];
@@ -344,6 +361,316 @@ __global__ void __launch_bounds__(kSaThreads) attn_small_kernel(const SmallAttn 
         }
         a.O[(size_t)((q / a.G) * a.B + b) * q_dim + (size_t)(g * a.G + q % a.G) * DH + e] = t / L;
     }
+}
+
+// Everything between two attention launches in one: O projection + residual, gate|up with norm, SwiGLU and b, down with c
+// and residual, and the next layer's Q|K|V -- four dependent linear layers, which as launches of their own are four links of
+// about 4.5 us each.  One cluster of 16 CTAs: each holds a sixteenth of every matrix in shared memory (bulk copies issued
+// before the dependency wait, so they pass while the attention kernel runs) and sends what it computes to all 16 through
+// distributed shared memory; between the layers each waits for the other slices' bytes instead of a kernel boundary.
+// Taken where a layer's matrices fit the cluster's shared memory beside the rows (small_cluster_smem).
+struct SmallMlp {
+    const float *O, *wo, *g_mlp, *wg, *wu, *coup_b, *wd, *coup_c;
+    const float *g_next, *w_next[3];  // the next layer's norm gain and Q, K, V matrices (g_next == nullptr: last layer)
+    float *S, *y_next[3];
+    int n_next[3], rows_next[3];
+    int R, Bc, d, qd, F;
+    float eps;
+    int *status;
+};
+constexpr int kScCtas = 16, kScThreads = 512, kScMaxRows = 8, kScMaxSmem = 227 * 1024 - 256;  // (static shared memory beside it)
+
+// Floats of one CTA's slices and row buffers.
+struct SmallClusterLayout {
+    int dO, Fs, qs;                           // features per CTA: O and down, gate (and up), next Q|K|V
+    int wo, wg, wu, wd, wn, x, s, h, g1, g2, cb, cc, total;  // offsets
+};
+__host__ __device__ inline SmallClusterLayout small_cluster_layout(int R, int d, int qd, int F, int n_next) {
+    SmallClusterLayout l;
+    l.dO = d / kScCtas;
+    l.Fs = F / kScCtas;
+    l.qs = n_next / kScCtas;
+    l.wo = 0;
+    l.wg = l.wo + l.dO * qd;
+    l.wu = l.wg + l.Fs * d;
+    l.wd = l.wu + l.Fs * d;
+    l.wn = l.wd + l.dO * F;
+    l.x = l.wn + l.qs * d;
+    l.s = l.x + R * (qd > d ? qd : d);
+    l.h = l.s + R * d;
+    l.g1 = l.h + R * F;
+    l.g2 = l.g1 + d;
+    l.cb = l.g2 + d;
+    l.cc = l.cb + l.Fs;
+    l.total = l.cc + l.dO;
+    return l;
+}
+// Dynamic shared memory of a CTA; 0: the shape does not go this way.
+inline size_t small_cluster_smem(int R, int d, int qd, int F, int n_next) {
+    if (R > kScMaxRows || d > 256 || d % (4 * kScCtas) || F % (4 * kScCtas) || n_next % kScCtas || qd % 8) return 0;
+    const size_t bytes = (size_t)small_cluster_layout(R, d, qd, F, n_next).total * 4;
+    return bytes <= (size_t)kScMaxSmem ? bytes : 0;
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const float *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes),
+                 "r"(bar)
+                 : "memory");
+}
+// Sixteen bytes into another CTA's shared memory, counted by its barrier.
+__device__ __forceinline__ void st_async4(uint32_t addr, float4 v, uint32_t bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1,%2,%3,%4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w), "r"(bar)
+                 : "memory");
+}
+
+// The sums over the warp of RM (4 or 8) values per lane: lane l returns that of value l / (32 / RM).  A value halves with
+// every exchange, 6 or 9 shuffles instead of 5 RM.
+template <int RM>
+__device__ __forceinline__ float warp_sum_rows(const float (&v)[RM]) {
+    const int lane = threadIdx.x & 31;
+    float t[RM];
+#pragma unroll
+    for (int r = 0; r < RM; r++) t[r] = v[r];
+    int n = RM, o = 16;
+#pragma unroll
+    for (int step = 0; step < (RM == 8 ? 3 : 2); step++) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int r = 0; r < RM / 2; r++)
+            if (r < n / 2) {
+                const float keep = up ? t[r + n / 2] : t[r], give = up ? t[r] : t[r + n / 2];
+                t[r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+        n /= 2;
+        o /= 2;
+    }
+    float s = t[0];
+#pragma unroll
+    for (; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// w . x[row] over K (a multiple of 4) for the row of this lane (warp_sum_rows), by one warp, both in shared memory.
+template <int RM>
+__device__ __forceinline__ float sc_dot(const float *w, const float *x, int K, int R) {
+    const int lane = threadIdx.x & 31;
+    float acc[RM];
+#pragma unroll
+    for (int r = 0; r < RM; r++) acc[r] = 0.f;
+    for (int k = lane * 4; k < K; k += 128) {
+        const float4 a = *reinterpret_cast<const float4 *>(w + k);
+#pragma unroll
+        for (int r = 0; r < RM; r++) {
+            const float4 b = *reinterpret_cast<const float4 *>(x + (size_t)min(r, R - 1) * K + k);
+            acc[r] = fmaf(a.x, b.x, fmaf(a.y, b.y, fmaf(a.z, b.z, fmaf(a.w, b.w, acc[r]))));
+        }
+    }
+    return warp_sum_rows<RM>(acc);
+}
+
+// Normalised rows in registers, for several features of one warp: g * S of all rows (at most 256 columns), and 1/rms of this
+// lane's row, which the products are multiplied by.
+// kGlobal: the rows lie in memory that the kernel before has written.
+template <int RM, bool kGlobal = false>
+struct ScRows {
+    float4 x[RM][2];
+    float inv;
+    // norm = false: the rows as they are (g is not read)
+    __device__ __forceinline__ void load(const float *S, const float *g, int K, int R, float eps, bool norm = true) {
+        float ss[RM];
+#pragma unroll
+        for (int r = 0; r < RM; r++) ss[r] = 0.f;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = (threadIdx.x & 31) * 4 + u * 128;
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), gv = !norm ? make_float4(1.f, 1.f, 1.f, 1.f) : k < K ? *reinterpret_cast<const float4 *>(g + k) : z;
+#pragma unroll
+            for (int r = 0; r < RM; r++) {
+                const float *p = S + (size_t)min(r, R - 1) * K + k;
+                const float4 v = k < K ? (kGlobal ? ldcg4(p) : *reinterpret_cast<const float4 *>(p)) : z;
+                ss[r] = fmaf(v.x, v.x, fmaf(v.y, v.y, fmaf(v.z, v.z, fmaf(v.w, v.w, ss[r]))));
+                x[r][u] = make_float4(v.x * gv.x, v.y * gv.y, v.z * gv.z, v.w * gv.w);
+            }
+        }
+        inv = norm ? 1.f / sqrtf(warp_sum_rows<RM>(ss) / (float)K + eps) : 1.f;
+    }
+    static __device__ __forceinline__ void weights(const float *w, int K, float4 (&a)[2]) {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int k = (threadIdx.x & 31) * 4 + u * 128;
+            a[u] = k < K ? *reinterpret_cast<const float4 *>(w + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    __device__ __forceinline__ float dot(const float *w, int K) const {
+        float4 a[2];
+        weights(w, K, a);
+        return dot(a);
+    }
+    __device__ __forceinline__ float dot(const float4 (&wa)[2]) const {
+        float acc[RM];
+#pragma unroll
+        for (int r = 0; r < RM; r++) acc[r] = 0.f;
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const float4 a = wa[u];
+#pragma unroll
+            for (int r = 0; r < RM; r++)
+                acc[r] = fmaf(a.x, x[r][u].x, fmaf(a.y, x[r][u].y, fmaf(a.z, x[r][u].z, fmaf(a.w, x[r][u].w, acc[r]))));
+        }
+        return inv * warp_sum_rows<RM>(acc);
+    }
+};
+
+template <int RM>
+__global__ void __launch_bounds__(kScThreads, 1) small_mlp_kernel(const SmallMlp a) {
+    DBT_TL_DECL;
+    extern __shared__ __align__(16) float sm[];
+    __shared__ __align__(8) unsigned long long bar_mem[7];  // four groups of weights, three exchanges
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, R = a.R;
+    constexpr int NW = kScThreads / 32;
+    const uint32_t rank = cluster_rank();
+    const int n_next = a.n_next[0] + a.n_next[1] + a.n_next[2];
+    const SmallClusterLayout l = small_cluster_layout(R, a.d, a.qd, a.F, n_next);
+    auto bar = [&](int i) { return smem_u32(&bar_mem[i]); };
+    if (tid == 0) {
+        for (int i = 0; i < 7; i++) mbar_init(bar(i), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        // what the other 15 CTAs will send in the three exchanges
+        mbar_expect_tx(bar(4), (kScCtas - 1) * R * l.dO * 4);
+        mbar_expect_tx(bar(5), (kScCtas - 1) * R * l.Fs * 4);
+        if (a.g_next) mbar_expect_tx(bar(6), (kScCtas - 1) * R * l.dO * 4);
+        // this CTA's slice of every matrix: whole rows, contiguous in memory
+        auto slice = [&](int off, const float *W, int f0, int nf, int K, int b) {
+            if (nf > 0) bulk_load(smem_u32(sm + off), W + (size_t)f0 * K, (uint32_t)(nf * K * 4), bar(b));
+        };
+        mbar_expect_tx(bar(0), l.dO * a.qd * 4);
+        slice(l.wo, a.wo, rank * l.dO, l.dO, a.qd, 0);
+        mbar_expect_tx(bar(1), 2 * l.Fs * a.d * 4);
+        slice(l.wg, a.wg, rank * l.Fs, l.Fs, a.d, 1);
+        slice(l.wu, a.wu, rank * l.Fs, l.Fs, a.d, 1);
+        mbar_expect_tx(bar(2), l.dO * a.F * 4);
+        slice(l.wd, a.wd, rank * l.dO, l.dO, a.F, 2);
+        if (a.g_next) {
+            mbar_expect_tx(bar(3), l.qs * a.d * 4);
+            int base = 0;
+            for (int s = 0; s < 3; s++) {  // the slice may span two of Q, K, V
+                const int lo = max((int)rank * l.qs, base), hi = min(((int)rank + 1) * l.qs, base + a.n_next[s]);
+                if (hi > lo) slice(l.wn + (lo - (int)rank * l.qs) * a.d, a.w_next[s], lo - base, hi - lo, a.d, 3);
+                base += a.n_next[s];
+            }
+        }
+    }
+    pdl_launch_dependents();
+    const int f_o = rank * l.dO, f_h = rank * l.Fs;
+    for (int i = tid; i < a.d; i += kScThreads) {  // gains and couplings come with the weights, before the wait
+        sm[l.g1 + i] = a.g_mlp[i];
+        if (a.g_next) sm[l.g2 + i] = a.g_next[i];
+    }
+    for (int i = tid; i < l.Fs; i += kScThreads) sm[l.cb + i] = a.coup_b[f_h + i];
+    for (int i = tid; i < l.dO; i += kScThreads) sm[l.cc + i] = a.coup_c[f_o + i];
+    __syncthreads();
+    cluster_sync_all();  // every CTA of the cluster runs: its shared memory may be written
+    pdl_wait();
+    DBT_TL_WAITED;
+    bool ok = true;
+    for (int i = tid; i < R * a.qd / 4; i += kScThreads) *reinterpret_cast<float4 *>(sm + l.x + 4 * i) = ldcg4(a.O + 4 * i);
+    // a lane's row in the sums over a warp, and the lane that writes it
+    const int row = lane / (32 / RM);
+    const bool writes = lane % (32 / RM) == 0 && row < R;
+    const int twin = row >= a.Bc ? row % a.Bc * (32 / RM) : lane;  // lane of a branch row's primary twin
+    // S of this warp's first O-projection feature, requested with the rows
+    float s_in = warp < l.dO && writes ? __ldcg(a.S + (size_t)row * a.d + f_o + warp) : 0.f;
+    __syncthreads();
+    // Sends this CTA's slice [r][f0 .. f0 + n) of the rows at float offset off (row stride K) to all CTAs, warp w to CTA w, in
+    // 16-byte pieces (single words were three times as slow), and waits for the bytes of the other slices: exchange e of three.
+    static_assert(NW == kScCtas, "a warp per CTA");
+    auto share = [&](int off, int K, int f0, int n, int e) {
+        __syncthreads();
+        const int pieces = n / 4;
+        if (warp != (int)rank)
+            for (int i = lane; i < R * pieces; i += 32) {
+                const float *src = sm + off + i / pieces * K + f0 + 4 * (i % pieces);
+                st_async4(mapa_u32(smem_u32(src), warp), *reinterpret_cast<const float4 *>(src), mapa_u32(bar(4 + e), warp));
+            }
+        ok = mbar_wait_cluster(bar(4 + e), 0) && ok;
+    };
+    DBT_TL_MARK(0);
+    // O projection + residual
+    ok = mbar_wait(bar(0), 0) && ok;
+    for (int i = warp; i < l.dO; i += NW) {
+        const float y = sc_dot<RM>(sm + l.wo + i * a.qd, sm + l.x, a.qd, R);
+        if (i != warp) s_in = writes ? __ldcg(a.S + (size_t)row * a.d + f_o + i) : 0.f;
+        if (writes) sm[l.s + row * a.d + f_o + i] = s_in + y;
+    }
+    share(l.s, a.d, f_o, l.dO, 0);
+    DBT_TL_MARK(1);
+    // gate | up, SwiGLU, b coupling
+    ok = mbar_wait(bar(1), 0) && ok;
+    ScRows<RM> xr;
+    xr.load(sm + l.s, sm + l.g1, a.d, R, a.eps);
+    for (int i = warp; i < l.Fs; i += NW) {
+        const float *wg = sm + l.wg + i * a.d, *wu = sm + l.wu + i * a.d;
+        const float gt = xr.dot(wg, a.d), up = xr.dot(wu, a.d);
+        float h = silu(gt) * up;
+        const float h1 = __shfl_sync(0xffffffffu, h, twin);
+        if (row >= a.Bc) h = fmaf(sm[l.cb + i], h1, h);
+        if (writes) sm[l.h + row * a.F + f_h + i] = h;
+    }
+    share(l.h, a.F, f_h, l.Fs, 1);
+    DBT_TL_MARK(2);
+    // down, c coupling, residual
+    ok = mbar_wait(bar(2), 0) && ok;
+    for (int i = warp; i < l.dO; i += NW) {
+        const int f = f_o + i;
+        float mv = sc_dot<RM>(sm + l.wd + i * a.F, sm + l.h, a.F, R);
+        const float m1 = __shfl_sync(0xffffffffu, mv, twin);
+        if (row >= a.Bc) mv = fmaf(sm[l.cc + i], m1, mv);
+        if (writes) {
+            const float y = sm[l.s + row * a.d + f] + mv;
+            sm[l.s + row * a.d + f] = y;
+            if (ok) a.S[(size_t)row * a.d + f] = y;
+        }
+    }
+    if (a.g_next) {
+        share(l.s, a.d, f_o, l.dO, 2);
+        DBT_TL_MARK(3);
+        // the next layer's Q | K | V
+        ok = mbar_wait(bar(3), 0) && ok;
+        xr.load(sm + l.s, sm + l.g2, a.d, R, a.eps);
+        for (int i = warp; i < l.qs; i += NW) {
+            const float y = xr.dot(sm + l.wn + i * a.d, a.d);
+            int f = rank * l.qs + i, s = 0;
+            while (f >= a.n_next[s]) f -= a.n_next[s++];
+            if (ok && writes && row < a.rows_next[s]) a.y_next[s][(size_t)row * a.n_next[s] + f] = y;
+        }
+    }
+    if (!ok && lane == 0) report(a.status, kStatusWaitExpired, 800 + warp);
+    DBT_TL_END("smlp");
+}
+
+// The shared output matrix at up to 8 rows and 256 columns: a warp takes four features, whose weights it requests before the
+// dependency wait, and keeps the rows in registers (a warp per feature, 4096 of them, ran in waves: 17 us by events, now 7.5).
+template <int RM>
+__global__ void __launch_bounds__(256) logits_small_kernel(const SmallLin a) {
+    pdl_launch_dependents();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, K = a.K, R = a.rows[0], V = a.n_out[0];
+    const int f0 = (blockIdx.x * 8 + warp) * 4;
+    const float *W = reinterpret_cast<const float *>(a.W[0]);
+    typedef ScRows<RM, true> Rows;
+    float4 w[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; j++) Rows::weights(W + (size_t)min(f0 + j, V - 1) * K, K, w[j]);
+    pdl_wait();
+    Rows xr;
+    xr.load(a.X, a.g, K, R, a.eps, a.g != nullptr);
+    const int row = lane / (32 / RM), sub = lane % (32 / RM);
+    float y[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) y[j] = xr.dot(w[j]);
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+        if (sub == j % (32 / RM) && row < R && f0 + j < V) a.Y[0][(size_t)row * V + f0 + j] = y[j];
 }
 
 }  // namespace dbt

@@ -1,5 +1,5 @@
-"""GPU: decode steps of fp32 dense models at few rows (the five-kernel chain) against the oracle, around the sizes where
-its kernels change: row groups, weight rows longer than the registered pieces, key splits, passes of 256 keys."""
+"""GPU: decode steps of fp32 dense models at few rows (the five-kernel chain and the cluster kernel) against the oracle, around
+the sizes where its kernels change: row groups, weight rows longer than the registered pieces, key splits, passes of 256 keys."""
 import pytest
 import torch
 
@@ -18,6 +18,9 @@ pytestmark = pytest.mark.gpu
     (dict(n_q_heads=2, n_kv_heads=1, head_dim=128, d_ff=1032), 1, 700, 697),  # several splits, long weight rows
     (dict(n_q_heads=4, n_kv_heads=1, final_norm=0), 2, 40, 36),     # four heads per KV head, no final norm
     (dict(n_paths=4, n_kv_heads=2), 3, 24, 20),                     # three branches
+    (dict(n_paths=3, n_kv_heads=2), 2, 24, 20),                     # six rows of three paths through the cluster kernel
+    (dict(d_ff=1024), 2, 24, 20),                                   # matrices beyond the cluster's shared memory
+    (dict(d_model=128, n_q_heads=6, n_kv_heads=2, d_ff=192), 4, 24, 20),  # a slice over Q and K, eight rows
 ])
 def test_few_row_decode_matches_the_oracle(kw, B, T, npre):
     cfg = tiny_dense_fp32().replace(n_layers=2, vocab=1003, **kw)
