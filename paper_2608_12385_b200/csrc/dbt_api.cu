@@ -136,6 +136,7 @@ struct dbt_model {
     std::vector<GraphEntry> graphs;
     // where a decode step finds sequence b's token: tokens[b * tok_stride + tok_p0] (1, 0 except inside dbt_prefill_boundary)
     int tok_stride = 1, tok_p0 = 0;
+    int clusters_at_once[4] = {74, 33, 22, 15};  // clusters of 2, 4, 6, 8 CTAs of a paired-SM GEMM resident at a time (count_clusters)
     bool cluster16 = false;    // clusters of 16 CTAs can run here (see small_cluster)
     bool att_planned = false;  // inside a decode step whose attention work split has been computed (run_embed_wide)
 };
@@ -281,8 +282,9 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
         w.P_floats = want < cap ? want : cap;
         if (w.P_floats < (size_t)Rd * widest) w.P_floats = (size_t)Rd * widest;
         w.P = k.take<float>(w.P_floats);
-        // shares of sum(S^2): 256 columns each in decode steps, up to eight per 256-feature tile in prompt chunks
-        w.ss = k.take<float>((size_t)((d + 255) / 256 * 8) * Rmax);
+        // shares of sum(S^2): 256 columns each in decode steps, 2 * splits per feature tile in prompt chunks (see plan_gemm_prompt)
+        const int sh256 = (d + 255) / 256 * 8, sh192 = (d + 191) / 192 * 6;
+        w.ss = k.take<float>((size_t)(sh256 > sh192 ? sh256 : sh192) * Rmax);
         if (moe) {
             const size_t Rk = sorted_rows(c);
             w.Xs = k.take<__nv_bfloat16>(2 * Rk * d);
@@ -834,27 +836,31 @@ const CUtensorMap *weight_view(dbt_model *m, const CUtensorMap *W, int box_rows)
 // Tile width and split of one such GEMM, by the time it takes (us, measured on its parts): a k-tile costs the MMAs of N
 // columns (4 N cycles) or what an SM takes in for it (32 KB of rows and 64 N bytes of weights at ~50 bytes per cycle); a
 // tile's first loads and its end 4.5 us, its epilogue up to 4; an exchange 4.4 at N = 256.  Unsplit tiles follow each other
-// on persistent pairs, split ones start anew: 15 clusters of 8 CTAs and about 34 of 4 are resident at a time.
+// on persistent pairs, split ones start anew, as many clusters at a time as the device holds (m->clusters_at_once).
 struct PgPlan {
     int N, splits;
 };
 PgPlan plan_gemm_prompt(const dbt_model *m, PgMode mode, const int (&n_out)[3], int nseg, int K, int R) {
-    const int widths[] = {256, 192, 128};
+    // widths and splits whose slices are whole 32-column chunks of a warp, and which are built for the mode
+    auto built = [&](int N, int S) {
+        if (mode == PG_COMBINE) return N == 256 && S == 1;
+        if (mode == PG_GATEUP) return S == 1 && N >= 192;
+        if (mode == PG_QKV) return N == 256 && S <= 2 && N / S % m->cfg.head_dim == 0;
+        if (mode == PG_RESID) return N == 256 ? S != 3 : N == 192 && S == 3;
+        return N == 256 || N == 128 ? S != 3 : N == 192 ? S == 1 || S == 3 : S == 3;
+    };
     const int total_kt = (K + kTcK - 1) / kTcK, mt = (R + kPgM - 1) / kPgM;
     PgPlan best{256, 1};
     double best_cost = 1e30;
-    for (int N : widths) {
-        if (N == 128 && mode != PG_STORE) continue;
-        if (N == 192 && mode != PG_STORE && mode != PG_GATEUP) continue;
-        for (int S = 1; S <= 4; S *= 2) {
-            if (S > 1 && (mode == PG_GATEUP || mode == PG_COMBINE || N == 192)) continue;  // (slices are multiples of 32 columns)
-            if (mode == PG_QKV && N / S % m->cfg.head_dim) continue;
+    for (int N : {256, 192, 128, 96}) {
+        for (int S = 1; S <= 4; S++) {
+            if (!built(N, S)) continue;
             const int kps = (total_kt + S - 1) / S;
             if ((S - 1) * kps >= total_kt) continue;
             int tiles = 0;
             for (int s = 0; s < nseg; s++) tiles += (n_out[s] + (mode == PG_GATEUP ? N / 2 : N) - 1) / (mode == PG_GATEUP ? N / 2 : N);
             tiles *= mt;
-            const int at_once = S == 1 ? m->num_sms / 2 : S == 2 ? 34 : 15, waves = (tiles + at_once - 1) / at_once;
+            const int at_once = m->clusters_at_once[S - 1], waves = (tiles + at_once - 1) / at_once;
             const double feed = (32768.0 + 64.0 * N) / 50, per_kt = (feed > 4.0 * N ? feed : 4.0 * N) / 1900;
             const double fixed = 4.5 + (S == 1 ? 4.0 : 4.4 + 2.7) * N / 256;
             const double cost = S == 1 ? waves * kps * per_kt + fixed : waves * (kps * per_kt + fixed);
@@ -906,12 +912,13 @@ dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0,
     int widest = 0;
     for (int s = 0; s < nseg; s++) widest = n_out[s] > widest ? n_out[s] : widest;
     PgPlan pl = plan_gemm_prompt(m, MODE, n_out, nseg, K, R);
-    if (shares) *shares = 2 * pl.splits * ((n_out[0] + 255) / 256);
+    if (shares) *shares = 2 * pl.splits * ((n_out[0] + pl.N - 1) / pl.N);
     if constexpr (MODE == PG_STORE) {
         if (widest <= 64) return launch_gemm_prompt<64, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, 1, p);
+        if (pl.N == 96) return launch_gemm_prompt<96, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
         if (pl.N == 128) return launch_gemm_prompt<128, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
     }
-    if constexpr (MODE == PG_STORE || MODE == PG_GATEUP)
+    if constexpr (MODE == PG_STORE || MODE == PG_GATEUP || MODE == PG_RESID)
         if (pl.N == 192) return launch_gemm_prompt<192, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
     return launch_gemm_prompt<256, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
 }
@@ -1820,9 +1827,31 @@ bool allow_smem_pg() {
 bool allow_smem_prompt() {
     return allow_smem_pg<256, PG_QKV>() && allow_smem_pg<256, PG_RESID>() && allow_smem_pg<256, PG_GATEUP>() &&
            allow_smem_pg<192, PG_GATEUP>() && allow_smem_pg<256, PG_COMBINE>() && allow_smem_pg<64, PG_STORE>() &&
-           allow_smem_pg<128, PG_STORE>() && allow_smem_pg<192, PG_STORE>() && allow_smem_pg<256, PG_STORE>() &&
+           allow_smem_pg<96, PG_STORE>() && allow_smem_pg<192, PG_RESID>() && allow_smem_pg<128, PG_STORE>() && allow_smem_pg<192, PG_STORE>() && allow_smem_pg<256, PG_STORE>() &&
            cudaFuncSetAttribute(gemm_group_kernel<GG_GATEUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess &&
            cudaFuncSetAttribute(gemm_group_kernel<GG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess;
+}
+
+// Clusters of 2 S CTAs, one CTA per SM, that this device holds at a time.
+void count_clusters(dbt_model *m) {
+    for (int S = 1; S <= 4; S++) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(2 * S * 74);
+        cfg.blockDim = dim3(kPgThreads);
+        cfg.dynamicSmemBytes = PgCfg<256>::kSmemBytes;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2 * S;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_prompt_kernel<256, PG_STORE>, &cfg) == cudaSuccess && n > 0)
+            m->clusters_at_once[S - 1] = n;
+        else
+            cudaGetLastError();
+    }
+    if (m->clusters_at_once[0] > m->num_sms / 2) m->clusters_at_once[0] = m->num_sms / 2;  // (the persistent grid)
 }
 
 // Build the TMA descriptors of a bf16 model.  Returns false when the path cannot be used.
@@ -1923,6 +1952,7 @@ bool setup_tc(dbt_model *m) {
     m->act_parts = 2;
     const char *pa = getenv("DBT_PROMPT_ATTN");
     const int G = c.n_q_heads / c.n_kv_heads;
+    if (m->att_fast) count_clusters(m);
     m->prompt_attn_tc = m->att_fast && 16 % G == 0 && !(pa && strcmp(pa, "tile") == 0) &&
                         make_prompt_q_map(&m->map_pq, w.Q, m->Rmax, c.n_q_heads, c.head_dim, G) &&
                         make_prompt_kv_map(&m->map_pkv, m->kv_pool, (uint64_t)c.n_layers * 2 * c.num_pages * c.n_kv_heads * c.page_size, c.head_dim);

@@ -16,7 +16,7 @@
 // and append 61 + 25 -> 62, O + residual 41 + 15 -> 39.
 //
 // Few row tiles (decode steps of more than 64 stacked rows, short prompts) leave too few tiles for the chip: the contracted
-// width of a tile is then split over 2 or 4 pairs of one cluster.  Each CTA owns a slice of the tile's columns, the others
+// width of a tile is then split over 2 to 4 pairs of one cluster.  Each CTA owns a slice of the tile's columns, the others
 // write their partial sums of it into its (by then idle) ring through distributed shared memory, and it adds them in split
 // order and runs the epilogue of that slice: no partials in memory, no kernel to sum them.
 //
@@ -55,7 +55,7 @@ struct PgParams {
     // once then share about as many row tiles as weight tiles (9 x 8 of 74), whatever the chunk: with all 32 row tiles of
     // an 8192-row chunk side by side the 8B shape's gate|up re-read its 134 MB of activations from HBM (97 us per row tile).
     int m_group;
-    int splits, kt_per_split;  // pairs per tile (1, 2, 4; a cluster is 2 * splits CTAs); k-tiles of each
+    int splits, kt_per_split;  // pairs per tile (1 to 4; a cluster is 2 * splits CTAs); k-tiles of each
     PgSeg seg[3];
     int nseg;
     int *status;
@@ -98,8 +98,10 @@ struct PgCfg {
     static constexpr int kStageBytes = kPgABytes + kBBytes;
     static constexpr int kStages = N >= 128 ? 4 : 5;
     static constexpr int kStagingBytes = kPgEpiWarps * 4096;
-    static constexpr int kAccStride = N > 128 ? 256 : N;  // TMEM columns between the two accumulators
+    static constexpr int kAccStride = N > 128 ? 256 : N > 64 ? 128 : 64;  // TMEM columns between the two accumulators
     static constexpr int kTmemCols = 2 * kAccStride;
+    static_assert((kTmemCols & (kTmemCols - 1)) == 0 && kTmemCols >= 32 && kTmemCols <= 512, "an allocation of tensor memory");
+    static_assert(N % 32 == 0 && N <= 256, "N of a cta_group::2 MMA with M = 256");
     static constexpr int kSmemBytes = kStages * kStageBytes + kStagingBytes + 1024 + 256;
     static_assert(kSmemBytes <= 227 * 1024, "shared memory of one SM");
 };
