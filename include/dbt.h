@@ -194,7 +194,8 @@ dbt_status dbt_last_expert_union(dbt_model *m, int32_t *count_per_layer_host);
  * shared-memory barrier that a TMA copy or a tensor-core commit completes) ran out after about two
  * seconds: *detail = the wait site (100 + warp: operand ring of the GEMM, 200 + warp: its accumulator,
  * 300..: the decode attention kernel's page ring, 400..: the prompt attention kernel's, 500..: the
- * persistent per-expert GEMM's rings and accumulators), the CTA skipped its stores, released its tensor memory and
+ * persistent per-expert GEMM's rings and accumulators, 600..: the paired-SM GEMMs, 700..: the experts' paired-SM GEMMs,
+ * 800..: the cluster kernel of small fp32 steps), the CTA skipped its stores, released its tensor memory and
  * returned, so the step's results are invalid but the context stays usable: returns DBT_ERR_TIMEOUT.
  * The first code recorded wins until dbt_reset clears the word.  HOST pointers, may be NULL. */
 dbt_status dbt_sync_status(dbt_model *m, int32_t *device_status, int32_t *detail);
