@@ -91,6 +91,7 @@ struct dbt_model {
     bool tc;
     std::vector<LayerMaps> maps;
     CUtensorMap map_lm, map_Xb, map_Ob, map_Hb, map_kv, map_Xs, map_Hs;
+    GgRowMaps rows_Xs, rows_Hs;   // the sorted rows as the experts' GEMMs of a prompt chunk read them
     CUtensorMap map_pq, map_pkv;  // prompt attention: queries, pages
     // prompt chunks take attn_prompt_kernel (bf16 queries, see prompt_q); off for head ratios that do not divide 16 and by
     // DBT_PROMPT_ATTN=tile: the 16-row kernel's packed tiles
@@ -1677,12 +1678,12 @@ dbt_status run_layers_moe_prompt(dbt_model *m, const RowMap &rm) {
         LAUNCH(m, "moe_gather", 0, moe_gather_rows_kernel, R, 256, 0, w.Xb, lo_x, w.ridx, w.epos, km, c.k_primary, d, w.Xs, lo_xs, w.ss, ss_tiles,
                m->Rmax, c.rms_eps, w.rs_sorted);
         GgParams g{};
-        g.E = E; g.cnt = w.ecnt; g.off = w.eoff; g.lo_row0 = Rk; g.status = w.status;
+        g.E = E; g.cnt = w.ecnt; g.off = w.eoff; g.status = w.status;
         g.K = d; g.n_feat = Fe; g.rs = w.rs_sorted; g.H = w.Hs; g.h_lo = lo_hs;
         const int grid = m->num_sms / 2 * 2;
-        LAUNCH(m, "expert_gateup", 0, gemm_group_kernel<GG_GATEUP>, grid, kPgThreads, kGgSmemBytes, mp.eg64, mp.eu64, m->map_Xs, g);
+        LAUNCH(m, "expert_gateup", 0, gemm_group_kernel<GG_GATEUP>, grid, kPgThreads, kGgSmemBytes, mp.eg64, mp.eu64, m->rows_Xs, g);
         g.K = Fe; g.n_feat = d; g.Y = w.Yexp;
-        LAUNCH(m, "expert_down", 0, gemm_group_kernel<GG_DOWN>, grid, kPgThreads, kGgSmemBytes, mp.ed, mp.ed, m->map_Hs, g);
+        LAUNCH(m, "expert_down", 0, gemm_group_kernel<GG_DOWN>, grid, kPgThreads, kGgSmemBytes, mp.ed, mp.ed, m->rows_Hs, g);
         const float *g_next = l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : nullptr;
         if (Fs > 0) {
             PgParams sg{};
@@ -1897,6 +1898,8 @@ bool setup_tc(dbt_model *m) {
         }
         mok = mok && make_bf16_map(&m->map_Xs, w.Xs, 2 * (uint64_t)Rk, d, 16) &&
               make_bf16_map(&m->map_Hs, w.Hs, 2 * (uint64_t)Rk, Fe, 16);
+        for (int j = 0; j < 8; j++)
+            mok = mok && make_act_map(&m->rows_Xs.m[j], w.Xs, Rk, d, 16 * (j + 1)) && make_act_map(&m->rows_Hs.m[j], w.Hs, Rk, Fe, 16 * (j + 1));
         if (mok && Fs > 0) mok = make_bf16_map(&m->map_Hb, w.Hb, 2 * m->Rmax, Fs, 16);
         // (a weight tile that runs past its expert's last row only computes features that the
         // epilogue never stores)

@@ -2,16 +2,20 @@
 //
 // A chunk's rows, sorted by expert, are many short lists (a few dozen to a few hundred rows each), so here the weights
 // take the M side -- a pair's tile is 256 weight rows -- and an expert's rows the N side, whose width follows the list:
-// the list is cut into the fewest tiles of at most 256 rows, equally, rounded up to 32.  Little work is done for
+// the list is cut into the fewest tiles of at most 256 rows, equally, rounded up to 32 (the step of N in an MMA of M = 256).  Little work is done for
 // padding at any list length (with the rows on the M side every list would pay for a multiple of 256), and every
 // expert's matrices are read once per row tile.  Otherwise as gemm_prompt_kernel: each CTA of the pair brings half of
 // the weight tile and half of the rows (both planes), persistent CTAs walk the (expert, feature tile, row tile) units
 // of the experts that have rows, two accumulators overlap one unit's epilogue with the next unit's MMAs.
 //
-// What bounds it: the tensor pipe from about 170 rows per expert on, the expert matrices' HBM stream below.
+// What bounds it: the tensor pipe from about 170 rows per expert on, the expert matrices' HBM stream below.  How many
+// boxes a k-tile is cut into matters as much: with both planes' rows in 2 KB boxes of 16 rows (12 instructions per CTA and
+// k-tile) gate|up of 9472 rows took 508 us with the tensor pipe 49 % busy, and each further box, even a prefetch, cost it
+// about 37 cycles; one box of exactly the tile's rows of both planes (a tensor map per width, GgRowMaps): 384 us, 73 %; down
+// 231 -> 192 us.  The ring holds as many stages as the widest tile allows: 1000 rows 2.19 -> 2.15 ms per 4 layers.
 //
 // Measured on the MoE model (64 experts x 1408, 2 per row), per layer and 2048 rows of a long prompt: gate|up with SwiGLU
-// 269 + 31 -> 107 us (9472-row chunks), down 158 -> 50 us, against 64-row tiles on one SM in 2048-row chunks, which
+// 269 + 31 -> 83 us (9472-row chunks), down 158 -> 41 us, against 64-row tiles on one SM in 2048-row chunks, which
 // streamed every expert's matrices for 64 rows at a time.
 //
 //   GG_GATEUP: a CTA's 128 weight rows are 64 gate rows and the 64 up rows of the same features, so the gate and the up
@@ -26,16 +30,15 @@ namespace dbt {
 
 enum GgMode { GG_GATEUP = 0, GG_DOWN = 1 };
 
-constexpr int kGgStageBytes = 3 * 16384;  // 128 weight rows, 128 rows of each plane, one k-tile
-constexpr int kGgStages = 4;
+constexpr int kGgRingBytes = 4 * 3 * 16384;  // at the widest 4 stages of 128 weight rows and 128 rows of each plane
+constexpr int kGgMaxStages = 8;  // a launch has as many stages, up to this, as its widest row tile leaves room for
 constexpr int kGgMaxExperts = 1024;
 constexpr int kGgScratchBytes = kPgEpiWarps * (2048 + 512);
-constexpr int kGgSmemBytes = kGgStages * kGgStageBytes + kGgScratchBytes + (kGgMaxExperts + 1) * 4 + 1024 + 256;
+constexpr int kGgSmemBytes = kGgRingBytes + kGgScratchBytes + (kGgMaxExperts + 2) * 4 + 1024 + 256;
 static_assert(kGgSmemBytes <= 227 * 1024, "shared memory of one SM");
 
 struct GgParams {
     int K, E, n_feat;           // contracted width; experts; features of one expert (GG_GATEUP: of each matrix)
-    int lo_row0;                // row of the lo plane in the activation map
     const int *cnt, *off;       // rows per expert, first sorted row
     const float *rs;            // GG_GATEUP: 1/rms per sorted row (nullptr: 1)
     __nv_bfloat16 *H;           // GG_GATEUP: [sorted row][n_feat], two planes
@@ -51,6 +54,11 @@ __device__ __forceinline__ void tma2_load_2d(uint32_t dst, const CUtensorMap *ma
         : "memory");
 }
 
+// The sorted rows as [plane][row][K]: map j brings a k-tile of 16 (j + 1) rows of both planes in one box.
+struct GgRowMaps {
+    CUtensorMap m[8];
+};
+
 // A unit of work: rows [row0, row0 + rows) of the sorted list against features f0.. of expert e; n: MMA width.
 struct GgUnit {
     int e, f0, row0, rows, n;
@@ -59,14 +67,14 @@ struct GgUnit {
 template <int MODE>
 __global__ void __launch_bounds__(kPgThreads, 1) __cluster_dims__(2, 1, 1)
 gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
-                  const __grid_constant__ CUtensorMap tmX, const GgParams p) {
-    constexpr int STAGES = kGgStages;
+                  const __grid_constant__ GgRowMaps tmX, const GgParams p) {
+    constexpr int STAGES = kGgMaxStages;
     constexpr int kTileF = MODE == GG_GATEUP ? 128 : 256;  // features of a pair's tile
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t ring = (raw + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (ring - raw);
-    constexpr int kBarOff = STAGES * kGgStageBytes + kGgScratchBytes;
+    constexpr int kBarOff = kGgRingBytes + kGgScratchBytes;
     const uint32_t bars = ring + kBarOff;
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
@@ -74,7 +82,7 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
     auto acc_empty = [&](int a) { return bars + 8u * (2 * STAGES + 2 + a); };
     auto swap_bar = [&](int i) { return bars + 8u * (2 * STAGES + 4 + i); };
     uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(gen + kBarOff + 8 * (2 * STAGES + 8));
-    int *first = reinterpret_cast<int *>(gen + kBarOff + 256);  // first unit of each expert, [E] = all units
+    int *first = reinterpret_cast<int *>(gen + kBarOff + 256);  // first unit of each expert, [E] = all units, [E + 1] = the widest row tile
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
@@ -99,9 +107,10 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
     }
     pdl_wait();  // the row lists
     if (warp == 2) {
-        int base = 0;
+        int base = 0, widest = 32;
         for (int e0 = 0; e0 < p.E; e0 += 32) {
-            const int e = e0 + lane, u = e < p.E ? (ld_mut(p.cnt + e) + 255) / 256 * nft : 0;
+            const int e = e0 + lane, cnt = e < p.E ? ld_mut(p.cnt + e) : 0, rt = (cnt + 255) / 256, u = rt * nft;
+            if (rt) widest = max(widest, ((cnt + rt - 1) / rt + 31) & ~31);
             int incl = u;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -111,7 +120,8 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
             if (e < p.E) first[e] = base + incl - u;
             base += __shfl_sync(0xffffffffu, incl, 31);
         }
-        if (lane == 0) first[p.E] = base;
+        widest = __reduce_max_sync(0xffffffffu, widest);
+        if (lane == 0) first[p.E] = base, first[p.E + 1] = widest;
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -121,6 +131,7 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
     pdl_launch_dependents();
 
     const int units = first[p.E];
+    const int slot = 16384 + first[p.E + 1] * 128, stages = min(STAGES, kGgRingBytes / slot);
     // Units in order of expert, feature tile, row tile: the row tiles that share a weight tile run side by side.
     auto unit_of = [&](int t) {
         int lo = 0, hi = p.E - 1;  // the last expert whose first unit is not past t
@@ -142,40 +153,37 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
 
     bool ok = true;
     if (warp == 0) {
-        // ---- TMA: lanes 16, 17 the weight tile, lanes 0..15 16-row boxes of the two planes
+        // ---- TMA: lane 0 the rows (both planes), lanes 1, 2 the weight tile
         if (lane == 0) {
             tma_prefetch_desc(&tmW0);
-            tma_prefetch_desc(&tmX);
         }
-        int it = 0;
+        int s = 0, ph = 1;
         for (int t = pair; t < units && ok; t += npairs) {
             const GgUnit u = unit_of(t);
-            const int nb = u.n / 32;  // boxes per plane of this CTA
-            const int pl = lane / 8, bx = lane % 8;
-            for (int kt = 0; kt < nkt; kt++, it++) {
-                const int s = it % STAGES;
+            const CUtensorMap *mx = &tmX.m[u.n / 32 - 1];
+            for (int kt = 0; kt < nkt; kt++) {
                 if (lane == 0) {
-                    if (it >= STAGES) ok = mbar_wait_cluster(empty_bar(s), ((it / STAGES) - 1) & 1);
-                    if (ok && rank == 0) mbar_expect_tx(full_bar(s), 2 * (16384 + 2 * nb * 2048));
+                    ok = mbar_wait_cluster(empty_bar(s), ph);  // a fresh barrier's phase before the first is over
+                    if (ok && rank == 0) mbar_expect_tx(full_bar(s), 2 * (16384 + u.n * 128));
                 }
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) break;
-                const uint32_t st = ring + s * kGgStageBytes, bar = mapa_u32(full_bar(s), 0);
-                if (pl < 2 && bx < nb)
-                    tma2_load_2d(st + 16384 * (1 + pl) + bx * 2048, &tmX, bar, kt * kTcK, pl * p.lo_row0 + u.row0 + (int)rank * (u.n / 2) + bx * 16);
+                const uint32_t st = ring + s * slot, bar = mapa_u32(full_bar(s), 0);
+                if (lane == 0) tma2_load_3d(st + 16384, mx, bar, kt * kTcK, u.row0 + (int)rank * (u.n / 2), 0);
                 if (MODE == GG_GATEUP) {
-                    if (lane == 16) tma2_load_2d(st, &tmW0, bar, kt * kTcK, u.e * p.n_feat + u.f0 + (int)rank * 64);
-                    if (lane == 17) tma2_load_2d(st + 8192, &tmW1, bar, kt * kTcK, u.e * p.n_feat + u.f0 + (int)rank * 64);
+                    if (lane == 1) tma2_load_2d(st, &tmW0, bar, kt * kTcK, u.e * p.n_feat + u.f0 + (int)rank * 64);
+                    if (lane == 2) tma2_load_2d(st + 8192, &tmW1, bar, kt * kTcK, u.e * p.n_feat + u.f0 + (int)rank * 64);
                 } else {
-                    if (lane == 16) tma2_load_2d(st, &tmW0, bar, kt * kTcK, u.e * p.n_feat + u.f0 + (int)rank * 128);
+                    if (lane == 1) tma2_load_2d(st, &tmW0, bar, kt * kTcK, u.e * p.n_feat + u.f0 + (int)rank * 128);
                 }
+                if (++s == stages) s = 0, ph ^= 1;
             }
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 700);
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
             // ---- MMA issuer of the pair
-            int it = 0, n_acc = 0;
+            int s = 0, ph = 0, n_acc = 0;
             for (int t = pair; t < units && ok; t += npairs, n_acc++) {
                 const GgUnit u = unit_of(t);
                 const uint32_t idesc = umma2_idesc(u.n);
@@ -184,20 +192,20 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc = tmem_base + a * 256;
-                for (int kt = 0; kt < nkt; kt++, it++) {
-                    const int s = it % STAGES;
-                    ok = mbar_wait_cluster(full_bar(s), (it / STAGES) & 1);
+                for (int kt = 0; kt < nkt; kt++) {
+                    ok = mbar_wait_cluster(full_bar(s), ph);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t st = ring + s * kGgStageBytes;
+                    const uint32_t st = ring + s * slot;
                     const uint64_t adesc = umma_smem_desc(st);
 #pragma unroll
                     for (int part = 0; part < 2; part++) {
-                        const uint64_t bdesc = umma_smem_desc(st + 16384 * (1 + part));
+                        const uint64_t bdesc = umma_smem_desc(st + 16384 + part * u.n * 64);
 #pragma unroll
                         for (int k = 0; k < kTcK / 16; k++) umma2_f16(acc, adesc + 2 * k, bdesc + 2 * k, idesc, (kt | part | k) != 0);
                     }
                     umma2_commit(empty_bar(s));
+                    if (++s == stages) s = 0, ph ^= 1;
                 }
                 if (ok) umma2_commit(acc_full(a));
             }
@@ -206,7 +214,7 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
     } else {
         // ---- epilogue: TMEM lane = weight row, TMEM column = activation row; two warps per lane quadrant share the columns
         const int quad = warp & 3, half = (warp - 2) >> 2;
-        float *xch = reinterpret_cast<float *>(gen + STAGES * kGgStageBytes);          // [warp][2][8][32]
+        float *xch = reinterpret_cast<float *>(gen + kGgRingBytes);          // [warp][2][8][32]
         float *rs_s = xch + kPgEpiWarps * 512 + (warp - 2) * 128;                       // this warp's rows' factors
         const int me = warp - 2, mate = half * 4 + (((quad ^ 2) + 2) & 3);              // the warp 64 lanes away, same columns
         int n_acc = 0, c_run = 0;

@@ -63,6 +63,7 @@ def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
     (dict(n_experts=64, d_expert=136, k_branch=2), 2, 150),                     # short lists, some experts without a row
     (dict(n_experts=8, d_expert=328, n_shared_experts=0, k_branch=8), 1, 513),  # no shared expert: the combine kernel
     (dict(n_experts=8, d_expert=128, n_shared_experts=2, k_primary=3, d_model=328), 1, 300),
+    (dict(n_experts=5, d_expert=264, k_primary=2), 1, 290),                     # row tiles of 96 to 160 rows: a ring of five or six stages
 ])
 def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n):
     from test_gpu_parity import small_moe, test_moe_prompt_chunks_of_more_than_one_row_tile_match_the_oracle as check
