@@ -2,8 +2,8 @@
 // item 1: the primary path alone walks the prompt and writes the cache; sm_100a).
 //
 // A CTA owns two query tiles of 128 rows -- 128 / G consecutive positions x the G heads of a KV head -- and streams the
-// keys they may see in tiles of 128 (eight 16-token pages: a 2 KB TMA box per page, 64-column piece and K|V plane, so
-// that a tile is an ordinary 128-byte-swizzled operand).  Per key tile: S = Q K^T into tensor memory, one thread per
+// keys they may see in tiles of 128 (eight 16-token pages: a TMA box per page and K|V plane, laid out as 128-byte-swizzled
+// groups of eight rows a fixed distance apart).  Per key tile: S = Q K^T into tensor memory, one thread per
 // row takes the softmax of its 128 scores (no shuffle), writes P back over S as bf16, and O += P V takes P from tensor
 // memory.  The two query tiles alternate: while the threads of one work on its scores the tensor cores run the other's
 // products.  O stays in tensor memory; it is rescaled only when a row's maximum has grown by more than 2^8 since the
@@ -11,6 +11,8 @@
 //
 // What bounds it: 4 x 128 x 128 x d_h FLOPs per (query tile, key tile) take 1024 cycles of the tensor pipe at d_h 128,
 // the 16384 exponentials as many cycles of the special-function unit.
+// Copy instructions count too: a page's 16 rows arrive as one 4 KB box at d_h 128 (two 2 KB boxes, one per 64 columns:
+// one 8192-token prompt of the 1B model, 2 layers, 2.96 -> 2.92 ms).
 // Measured per layer and 2048 rows: 1B model at 16 sequences of up to 2048 keys 112 -> 41 us; 8B shape, one sequence at 0..8192
 // keys 644 -> 190 us (720 useful TFLOP/s) against warps of mma.sync m16n8k16 that shared the staged pages.
 //
@@ -72,13 +74,13 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t *r) {
         : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// MN-major, 128B-swizzled operand: 64 elements of the non-contracted dimension per 128-byte row, 8-row groups of the
-// contracted dimension 1024 bytes apart, the next 64 elements lbo bytes further.
-__device__ __forceinline__ uint64_t umma_smem_desc_mn(uint32_t saddr, uint32_t lbo) {
+// 128B-swizzled operand of 8-row groups `group` bytes apart.  K-major (the keys): lbo unused.  MN-major (the values): 64
+// elements of the non-contracted dimension per 128-byte row, the next 64 lbo bytes further, groups along the contraction.
+__device__ __forceinline__ uint64_t umma_smem_desc_groups(uint32_t saddr, uint32_t group, uint32_t lbo) {
     uint64_t d = 0;
     d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
     d |= (uint64_t)(lbo >> 4) << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)(group >> 4) << 32;
     d |= (uint64_t)1 << 46;
     d |= (uint64_t)2 << 61;
     return d;
@@ -100,7 +102,8 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
                                                                     const __grid_constant__ CUtensorMap tmKV, const PromptAttnParams p) {
     using Cfg = PromptAttCfg<DH>;
     constexpr int STAGES = Cfg::kStages, HALVES = Cfg::kHalves, KS = DH / 16;
-    constexpr uint32_t kHalfBytes = 128 * 128;  // 128 rows of one 64-column piece
+    constexpr uint32_t kHalfBytes = 128 * 128;       // queries: 128 rows of one 64-column piece
+    constexpr uint32_t kGroup = HALVES * 1024;       // keys, values: 8 rows, their 64-column pieces one after the other
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t q_s = (raw + 1023u) & ~1023u, k_s = q_s + 2 * Cfg::kTileBytes, v_s = k_s + STAGES * Cfg::kTileBytes;
@@ -163,7 +166,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
 
     bool ok = true;
     if (warp == 8) {
-        // ---- TMA: lane l brings page l / HALVES of the tile, 64-column piece l % HALVES
+        // ---- TMA: lane l brings page l of the tile
         if (lane == 0) {
             tma_prefetch_desc(&tmQ);
             tma_prefetch_desc(&tmKV);
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
                     tma_load_4d(q_s + i * Cfg::kTileBytes + h * kHalfBytes, &tmQ, q_full, 0, g * p.G, b * p.cn + c0 + i * PT, h);
         }
         __syncwarp();
-        const int pages_total = (n_keys + 15) >> 4, my_h = lane % HALVES, my_pg = lane / HALVES;
+        const int pages_total = (n_keys + 15) >> 4, my_pg = lane;
         const bool loads = my_pg < 8;
         int page = loads && my_pg < pages_total ? p.page_table[(size_t)b * p.pt_stride + my_pg] : 0;
         for (int t = 0; t < T && ok; t++) {
@@ -183,7 +186,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
                 page = 0;
             }
             const int row = (int)(((long long)page * p.n_kv + g) * 16);
-            const uint32_t off = s * Cfg::kTileBytes + my_h * kHalfBytes + my_pg * 2048;
+            const uint32_t off = s * Cfg::kTileBytes + my_pg * 2 * kGroup;
             const int nx = (t + 1) * 8 + my_pg;
             const int next_page = loads && nx < pages_total ? p.page_table[(size_t)b * p.pt_stride + nx] : 0;
             if (lane == 0) {
@@ -191,13 +194,13 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
                 if (ok) mbar_expect_tx(k_full(s), (uint32_t)np * HALVES * 2048);
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (ok && loads && my_pg < np) tma_load_3d(k_s + off, &tmKV, k_full(s), 0, (int)(p.k_row0 + row), my_h);
+            if (ok && loads && my_pg < np) tma_load_4d(k_s + off, &tmKV, k_full(s), 0, 0, 0, (int)((p.k_row0 + row) >> 3));
             if (lane == 0 && ok) {
                 if (t >= STAGES) ok = mbar_wait(v_empty(s), ((t / STAGES) - 1) & 1);
                 if (ok) mbar_expect_tx(v_full(s), (uint32_t)np * HALVES * 2048);
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (ok && loads && my_pg < np) tma_load_3d(v_s + off, &tmKV, v_full(s), 0, (int)(p.v_row0 + row), my_h);
+            if (ok && loads && my_pg < np) tma_load_4d(v_s + off, &tmKV, v_full(s), 0, 0, 0, (int)((p.v_row0 + row) >> 3));
             page = next_page;
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 400);
@@ -217,9 +220,9 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
             const int s = t % STAGES;
 #pragma unroll
             for (int k = 0; k < KS; k++) {
-                const uint32_t off = (k >> 2) * kHalfBytes;
-                umma_f16(t_s(i), umma_smem_desc(q_s + i * Cfg::kTileBytes + off) + 2 * (k & 3), umma_smem_desc(k_s + s * Cfg::kTileBytes + off) + 2 * (k & 3),
-                         idesc_qk, k != 0);
+                const int h = k >> 2;
+                umma_f16(t_s(i), umma_smem_desc(q_s + i * Cfg::kTileBytes + h * kHalfBytes) + 2 * (k & 3),
+                         umma_smem_desc_groups(k_s + s * Cfg::kTileBytes + h * 1024, kGroup, 0) + 2 * (k & 3), idesc_qk, k != 0);
             }
             umma_commit(s_full(i));
         };
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
                 const int v0 = n_keys - t * kPaKeys;
                 for (int h = 0; h < HALVES; h++)
                     for (int idx = v0 * 8 + lane; idx < kPaKeys * 8; idx += 32)
-                        asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(v_s + s * Cfg::kTileBytes + h * kHalfBytes + idx * 16), "r"(0u)
+                        asm volatile("st.shared.v4.b32 [%0], {%1,%1,%1,%1};" ::"r"(v_s + s * Cfg::kTileBytes + (idx >> 6) * kGroup + h * 1024 + (idx & 63) * 16), "r"(0u)
                                      : "memory");
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -250,9 +253,9 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
                 ok = wait(p_full(i), t & 1);
                 if (!ok) break;
                 if (lane == 0) {
-                    const uint64_t vd = umma_smem_desc_mn(v_s + s * Cfg::kTileBytes, kHalfBytes);
+                    const uint64_t vd = umma_smem_desc_groups(v_s + s * Cfg::kTileBytes, kGroup, 1024);
 #pragma unroll
-                    for (int k = 0; k < kPaKeys / 16; k++) umma_f16_ts(t_o(i), t_s(i) + 8 * k, vd + 128 * k, idesc_pv, (t | k) != 0);
+                    for (int k = 0; k < kPaKeys / 16; k++) umma_f16_ts(t_o(i), t_s(i) + 8 * k, vd + (2 * kGroup >> 4) * k, idesc_pv, (t | k) != 0);
                     if (t + 1 == Tn[i]) umma_commit(o_full(i));
                 }
                 if (t + 1 < Tn[i]) qk(i, t + 1);
@@ -378,15 +381,16 @@ inline bool make_prompt_q_map(CUtensorMap *map, const void *base, uint64_t rows,
     return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-// The pool as rows of one head: a box is the 16 rows of a page, one 64-column piece.
+// The pool as groups of 8 rows of one head: a box is a page's 16 rows as two groups, in each the 64-column pieces of the
+// eight rows one after the other.
 inline bool make_prompt_kv_map(CUtensorMap *map, const void *base, uint64_t rows, uint64_t dh) {
     EncodeTiledFn fn = encode_tiled_fn();
     if (!fn) return false;
-    cuuint64_t dims[3] = {64, rows, dh / 64};
-    cuuint64_t strides[2] = {dh * 2, 128};
-    cuuint32_t box[3] = {64, 16, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    cuuint64_t dims[4] = {64, 8, dh / 64, rows / 8};
+    cuuint64_t strides[3] = {dh * 2, 128, 8 * dh * 2};
+    cuuint32_t box[4] = {64, 8, (cuuint32_t)(dh / 64), 2};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
