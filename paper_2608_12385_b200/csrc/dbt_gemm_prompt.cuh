@@ -430,8 +430,12 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                 // so that global memory sees 128-byte row pieces: lane l then holds columns 4 (l % 8) .. of row 4 i + l / 8.
                 // What a chunk adds to the accumulator is requested a chunk ahead (the first before the accumulator is
                 // there): the epilogue would otherwise wait for memory once per chunk, longer than the next tile's MMAs take.
+                // PG_COMBINE has three times the rows in flight and takes them half a chunk at a time: with a whole chunk's 96
+                // registers of them some spilled, and a spill waits for its load (9472 rows of the MoE model, K = 1408: 180 us, now
+                // 132; 81 of it are left without the routed rows).  Fetching those rows into L2 a tile ahead made it 151.
                 constexpr bool kResid = MODE != PG_STORE;
                 constexpr int kPre = MODE == PG_COMBINE ? 2 : 0;  // selections whose rows are requested ahead
+                constexpr int kAhead = MODE == PG_COMBINE ? 4 : 8;  // in groups of this many of a lane's eight rows
                 const int c4 = (lane & 7) * 4, rsub = lane >> 3;
                 float sq[8];
 #pragma unroll
@@ -449,13 +453,13 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         wt[j] = sel ? __ldcg(p.sel_wts + o) : 0.f;
                     }
                 }
-                float4 s4[8], y4[kPre > 0 ? kPre : 1][8];
-                auto request = [&](int c) {
+                float4 s4[kAhead], y4[kPre > 0 ? kPre : 1][kAhead];
+                auto request = [&](int c, int i0) {
                     const int col = f0 + cbase + c + c4;
                     const bool con = col < p.seg[sg].n_out;
 #pragma unroll
-                    for (int i = 0; i < 8; i++) {
-                        const int rl = i * 4 + rsub, r = row0 + rl;
+                    for (int i = 0; i < kAhead; i++) {
+                        const int rl = (i0 + i) * 4 + rsub, r = row0 + rl;
                         s4[i] = con && r < p.R ? ldcg4(p.S + (size_t)r * p.d + col) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                         for (int j = 0; j < kPre; j++) {
@@ -464,7 +468,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         }
                     }
                 };
-                if (kResid && cend > 0) request(0);
+                if (kResid && cend > 0) request(0, 0);
                 if (!acc_ready()) break;
 #pragma unroll 1
                 for (int c = 0; c < cend; c += 32) {
@@ -488,49 +492,53 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         *reinterpret_cast<float4 *>(stg + lane * 32 + ((j ^ (lane & 7)) << 2)) = x;
                     }
                     __syncwarp();
-                    float4 add[8];
-                    if (kResid) {
 #pragma unroll
-                        for (int i = 0; i < 8; i++) {
-                            float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int i0 = 0; i0 < 8; i0 += kAhead) {
+                        float4 add[kAhead];
+                        if (kResid) {
 #pragma unroll
-                            for (int j = 0; j < kPre; j++) {
-                                const float g = __shfl_sync(0xffffffffu, wt[j], i * 4 + rsub);
-                                m.x = fmaf(g, y4[j][i].x, m.x), m.y = fmaf(g, y4[j][i].y, m.y);
-                                m.z = fmaf(g, y4[j][i].z, m.z), m.w = fmaf(g, y4[j][i].w, m.w);
+                            for (int i = 0; i < kAhead; i++) {
+                                float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                                for (int j = 0; j < kPre; j++) {
+                                    const float g = __shfl_sync(0xffffffffu, wt[j], (i0 + i) * 4 + rsub);
+                                    m.x = fmaf(g, y4[j][i].x, m.x), m.y = fmaf(g, y4[j][i].y, m.y);
+                                    m.z = fmaf(g, y4[j][i].z, m.z), m.w = fmaf(g, y4[j][i].w, m.w);
+                                }
+                                add[i] = make_float4(s4[i].x + m.x, s4[i].y + m.y, s4[i].z + m.z, s4[i].w + m.w);
                             }
-                            add[i] = make_float4(s4[i].x + m.x, s4[i].y + m.y, s4[i].z + m.z, s4[i].w + m.w);
-                        }
-                        if (MODE == PG_COMBINE && p.k > kPre && con) {  // wider fan-outs: the further selections' rows
+                            if (MODE == PG_COMBINE && p.k > kPre && con) {  // wider fan-outs: the further selections' rows
 #pragma unroll
-                            for (int i = 0; i < 8; i++) {
-                                const int r = row0 + i * 4 + rsub;
-                                if (r >= p.R) continue;
-                                for (int j = kPre; j < p.k; j++) {
-                                    const size_t o = (size_t)r * p.kmax + j;
-                                    if (__ldcg(p.sel_idx + o) < 0) continue;
-                                    const float g = __ldcg(p.sel_wts + o);
-                                    const float4 y = ldcg4(p.Y + (size_t)__ldcg(p.sel_pos + o) * p.d + col);
-                                    add[i].x = fmaf(g, y.x, add[i].x), add[i].y = fmaf(g, y.y, add[i].y);
-                                    add[i].z = fmaf(g, y.z, add[i].z), add[i].w = fmaf(g, y.w, add[i].w);
+                                for (int i = 0; i < kAhead; i++) {
+                                    const int r = row0 + (i0 + i) * 4 + rsub;
+                                    if (r >= p.R) continue;
+                                    for (int j = kPre; j < p.k; j++) {
+                                        const size_t o = (size_t)r * p.kmax + j;
+                                        if (__ldcg(p.sel_idx + o) < 0) continue;
+                                        const float g = __ldcg(p.sel_wts + o);
+                                        const float4 y = ldcg4(p.Y + (size_t)__ldcg(p.sel_pos + o) * p.d + col);
+                                        add[i].x = fmaf(g, y.x, add[i].x), add[i].y = fmaf(g, y.y, add[i].y);
+                                        add[i].z = fmaf(g, y.z, add[i].z), add[i].w = fmaf(g, y.w, add[i].w);
+                                    }
                                 }
                             }
+                            if (i0 + kAhead < 8) request(c, i0 + kAhead);
+                            else if (c + 32 < cend) request(c + 32, 0);
                         }
-                        if (c + 32 < cend) request(c + 32);
-                    }
 #pragma unroll
-                    for (int i = 0; i < 8; i++) {
-                        const int rl = i * 4 + rsub, r = row0 + rl;
-                        float4 x = *reinterpret_cast<const float4 *>(stg + rl * 32 + (((lane & 7) ^ (rl & 7)) << 2));
-                        if (!con || r >= p.R) continue;
-                        if (MODE == PG_STORE) {
-                            *reinterpret_cast<float4 *>(p.P + (size_t)r * p.ldp + p.seg[sg].col0 + col) = x;
-                        } else {
-                            const size_t o = (size_t)r * p.d + col;
-                            x.x += add[i].x, x.y += add[i].y, x.z += add[i].z, x.w += add[i].w;
-                            *reinterpret_cast<float4 *>(p.S + o) = x;
-                            store_split4(p.X, o, p.x_lo, make_float4(gn.x * x.x, gn.y * x.y, gn.z * x.z, gn.w * x.w));
-                            sq[i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+                        for (int i = 0; i < kAhead; i++) {
+                            const int rl = (i0 + i) * 4 + rsub, r = row0 + rl;
+                            float4 x = *reinterpret_cast<const float4 *>(stg + rl * 32 + (((lane & 7) ^ (rl & 7)) << 2));
+                            if (!con || r >= p.R) continue;
+                            if (MODE == PG_STORE) {
+                                *reinterpret_cast<float4 *>(p.P + (size_t)r * p.ldp + p.seg[sg].col0 + col) = x;
+                            } else {
+                                const size_t o = (size_t)r * p.d + col;
+                                x.x += add[i].x, x.y += add[i].y, x.z += add[i].z, x.w += add[i].w;
+                                *reinterpret_cast<float4 *>(p.S + o) = x;
+                                store_split4(p.X, o, p.x_lo, make_float4(gn.x * x.x, gn.y * x.y, gn.z * x.z, gn.w * x.w));
+                                sq[i0 + i] += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+                            }
                         }
                     }
                 }
