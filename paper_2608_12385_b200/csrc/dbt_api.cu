@@ -168,11 +168,12 @@ unsigned branch_blocks(int grouped) { return grouped > 1 ? (unsigned)(grouped - 
 int kmax_of(const dbt_config &c) { return c.k_primary > c.k_branch ? c.k_primary : c.k_branch; }
 // Rows that the decode kernels and the short prompt chunks in their form work on.
 int decode_rows(const dbt_config &c) { return paths_of(c) * c.max_batch > 256 ? paths_of(c) * c.max_batch : 256; }
-// Rows of the activation buffers of bf16 models: a decode step's, or one prompt chunk.  A chunk is at most 37 row tiles
-// of 256: with the 74 pairs of SMs the tiles of a GEMM of any even number of feature tiles are then whole waves (a 1B
-// layer's four GEMMs take 1.22 tile times per row tile; 1.34 at 8 row tiles, 1.31 at 32), an expert's matrices serve
-// four times the rows of a 2048-row chunk, and the buffers stay below a gigabyte at the 1B width.
-constexpr int kPromptRows = 37 * 256;
+// Rows of the activation buffers of bf16 models: a decode step's, or one prompt chunk.  A chunk is at most 74 row tiles
+// of 256: with the 74 pairs of SMs the tiles of any GEMM are then whole waves, and an expert's matrices serve nearly 600
+// rows.  16 prompts of 2048 into the 1B model 88.3 ms in chunks of 37 row tiles, 85.3 of 74, 84.8 of 111; 32 of 1024 into the
+// MoE model 89.4, 81.8, 82.4 (of 18: 106); chunks of equal length changed neither.  The buffers take 1.1 GB at the 1B
+// width, 2.3 GB at the 8B width.
+constexpr int kPromptRows = 74 * 256;
 int prefill_rows(const dbt_config &c) {
     if (c.weight_dtype != DBT_DTYPE_BF16) return decode_rows(c);
     const long long all = ((long long)c.max_batch * c.max_seq + 255) / 256 * 256;
