@@ -29,6 +29,8 @@
 // new K,V row from the Q|K|V GEMM's split-K partials.  All waits are bounded.
 #pragma once
 
+#include <type_traits>
+
 #include "dbt_fused.cuh"
 #include "dbt_gemm_tc.cuh"
 
@@ -1032,43 +1034,47 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         // A thread takes four consecutive outputs of up to two query rows, eight partials of each in flight: up to eight
         // query rows need one round of loads per eight partials.  (Two single outputs per thread took a round per 256
         // outputs: 5 us behind the last segment at 4 query rows, 9 at 8; now about 2.)
-        auto merge = [&](float *pbase, int slot_stride, int n, bool final) {
+        // Four query rows at d_h 128 (or eight at 64) leave one such piece per thread: then sixteen partials of it.  (Eight, and the
+        // second piece's idle arithmetic, made a primary-only step of two sequences of 9139 positions 12 us slower.)
+        auto merge_rows = [&](auto pieces, float *pbase, int slot_stride, int n, bool final) {
+            constexpr int A = decltype(pieces)::value, J = 16 / A;  // pieces of a thread, partials of each in flight
             const size_t sstr = (size_t)slot_stride * 16 * (DH + 2);
             constexpr int VQ = DH / 4;  // 16-byte pieces of a query row
-            for (int idx0 = tid; idx0 < nq_act * VQ; idx0 += 2 * 128) {
-                float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f};
-                float4 X[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-                bool act[2];
-                int ee[2], qq[2];
+            for (int idx0 = tid; idx0 < nq_act * VQ; idx0 += A * 128) {
+                float M[A], L[A];
+                float4 X[A];
+                bool act[A];
+                int ee[A], qq[A];
 #pragma unroll
-                for (int a = 0; a < 2; a++) {
+                for (int a = 0; a < A; a++) {
                     const int idx = idx0 + a * 128;
+                    M[a] = -INFINITY, L[a] = 0.f, X[a] = make_float4(0.f, 0.f, 0.f, 0.f);
                     act[a] = idx < nq_act * VQ;
                     qq[a] = act[a] ? idx / VQ : 0;
                     ee[a] = act[a] ? idx % VQ * 4 : 0;
                 }
-                for (int sb = 0; sb < n; sb += 8) {
-                    float2 ml[2][8];
-                    float4 ov[2][8];
+                for (int sb = 0; sb < n; sb += J) {
+                    float2 ml[A][J];
+                    float4 ov[A][J];
 #pragma unroll
-                    for (int a = 0; a < 2; a++)
+                    for (int a = 0; a < A; a++)
 #pragma unroll
-                        for (int j = 0; j < 8; j++) {
+                        for (int j = 0; j < J; j++) {
                             const bool on = act[a] && sb + j < n;
                             const float *pp = pbase + (size_t)(sb + j) * sstr;
                             ml[a][j] = on ? __ldcg(reinterpret_cast<const float2 *>(pp + 16 * DH) + qq[a]) : make_float2(-INFINITY, 0.f);
                             ov[a][j] = on ? ldcg4(pp + (size_t)qq[a] * DH + ee[a]) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
 #pragma unroll
-                    for (int a = 0; a < 2; a++) {
+                    for (int a = 0; a < A; a++) {
                         float Mn = M[a];
 #pragma unroll
-                        for (int j = 0; j < 8; j++) Mn = fmaxf(Mn, ml[a][j].x);
+                        for (int j = 0; j < J; j++) Mn = fmaxf(Mn, ml[a][j].x);
                         const float sc = M[a] == -INFINITY ? 0.f : exp2f(M[a] - Mn);
                         L[a] *= sc;
                         X[a].x *= sc, X[a].y *= sc, X[a].z *= sc, X[a].w *= sc;
 #pragma unroll
-                        for (int j = 0; j < 8; j++) {
+                        for (int j = 0; j < J; j++) {
                             const float f = ml[a][j].x == -INFINITY ? 0.f : exp2f(ml[a][j].x - Mn);
                             L[a] = fmaf(ml[a][j].y, f, L[a]);
                             X[a].x = fmaf(ov[a][j].x, f, X[a].x), X[a].y = fmaf(ov[a][j].y, f, X[a].y);
@@ -1078,7 +1084,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                     }
                 }
 #pragma unroll
-                for (int a = 0; a < 2; a++) {
+                for (int a = 0; a < A; a++) {
                     if (!act[a]) continue;
                     if (final) {
                         const int row = packed ? item_row0(item) + qq[a] / p.G : (qq[a] / p.G) * Bc + item;
@@ -1103,6 +1109,10 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 }
                 __threadfence();
             }
+        };
+        auto merge = [&](float *pbase, int slot_stride, int n, bool final) {
+            if (nq_act * (DH / 4) <= 128) merge_rows(std::integral_constant<int, 1>{}, pbase, slot_stride, n, final);
+            else merge_rows(std::integral_constant<int, 2>{}, pbase, slot_stride, n, final);
         };
         auto arrive = [&](int *counter, int arrivals) {  // true in the CTA that arrives last
             consumer_sync();

@@ -61,3 +61,11 @@ def test_dealt_pairs_grouped_and_primary_only_write_the_same_cache():
         gm.decode_full(tok, grouped=grouped)
         caches.append(gm.kv_pool.clone())
     assert torch.equal(caches[0], caches[1])
+
+
+@pytest.mark.parametrize("heads,kv_heads,dh,paths", [(2, 2, 64, 2), (8, 2, 64, 2), (4, 2, 128, 2), (4, 2, 128, 3), (8, 2, 128, 2)])
+def test_merge_of_many_segments_at_few_and_more_query_rows(heads, kv_heads, dh, paths):
+    """2 to 8 query rows: one 16-byte piece of the output per thread (sixteen partials at once) up to 4 rows at d_h 128 or 8 at
+    64, two pieces above; 40 segments go through groups, 10 through one merge."""
+    cfg = cfg_of(n_q_heads=heads, n_kv_heads=kv_heads, head_dim=dh, n_paths=paths)
+    test_dealt_pairs_match_the_oracle_on_sampled_sequences(cfg, [2570, 650])
