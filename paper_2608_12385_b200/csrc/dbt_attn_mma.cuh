@@ -1036,6 +1036,8 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         // outputs: 5 us behind the last segment at 4 query rows, 9 at 8; now about 2.)
         // Four query rows at d_h 128 (or eight at 64) leave one such piece per thread: then sixteen partials of it.  (Eight, and the
         // second piece's idle arithmetic, made a primary-only step of two sequences of 9139 positions 12 us slower.)
+        // The number of query rows is the step's, so the choice differs between a grouped and a primary-only step of the same
+        // batch: both forms fold eight partials per common maximum, in the same order, and round alike.
         auto merge_rows = [&](auto pieces, float *pbase, int slot_stride, int n, bool final) {
             constexpr int A = decltype(pieces)::value, J = 16 / A;  // pieces of a thread, partials of each in flight
             const size_t sstr = (size_t)slot_stride * 16 * (DH + 2);
@@ -1066,21 +1068,25 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                             ov[a][j] = on ? ldcg4(pp + (size_t)qq[a] * DH + ee[a]) : make_float4(0.f, 0.f, 0.f, 0.f);
                         }
 #pragma unroll
-                    for (int a = 0; a < A; a++) {
-                        float Mn = M[a];
+                    for (int h = 0; h < J; h += 8) {  // eight at a time, however many are in flight
+                        if (sb + h >= n) break;
 #pragma unroll
-                        for (int j = 0; j < J; j++) Mn = fmaxf(Mn, ml[a][j].x);
-                        const float sc = M[a] == -INFINITY ? 0.f : exp2f(M[a] - Mn);
-                        L[a] *= sc;
-                        X[a].x *= sc, X[a].y *= sc, X[a].z *= sc, X[a].w *= sc;
+                        for (int a = 0; a < A; a++) {
+                            float Mn = M[a];
 #pragma unroll
-                        for (int j = 0; j < J; j++) {
-                            const float f = ml[a][j].x == -INFINITY ? 0.f : exp2f(ml[a][j].x - Mn);
-                            L[a] = fmaf(ml[a][j].y, f, L[a]);
-                            X[a].x = fmaf(ov[a][j].x, f, X[a].x), X[a].y = fmaf(ov[a][j].y, f, X[a].y);
-                            X[a].z = fmaf(ov[a][j].z, f, X[a].z), X[a].w = fmaf(ov[a][j].w, f, X[a].w);
+                            for (int j = h; j < h + 8; j++) Mn = fmaxf(Mn, ml[a][j].x);
+                            const float sc = M[a] == -INFINITY ? 0.f : exp2f(M[a] - Mn);
+                            L[a] *= sc;
+                            X[a].x *= sc, X[a].y *= sc, X[a].z *= sc, X[a].w *= sc;
+#pragma unroll
+                            for (int j = h; j < h + 8; j++) {
+                                const float f = ml[a][j].x == -INFINITY ? 0.f : exp2f(ml[a][j].x - Mn);
+                                L[a] = fmaf(ml[a][j].y, f, L[a]);
+                                X[a].x = fmaf(ov[a][j].x, f, X[a].x), X[a].y = fmaf(ov[a][j].y, f, X[a].y);
+                                X[a].z = fmaf(ov[a][j].z, f, X[a].z), X[a].w = fmaf(ov[a][j].w, f, X[a].w);
+                            }
+                            M[a] = Mn;
                         }
-                        M[a] = Mn;
                     }
                 }
 #pragma unroll

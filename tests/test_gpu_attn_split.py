@@ -69,3 +69,27 @@ def test_merge_of_many_segments_at_few_and_more_query_rows(heads, kv_heads, dh, 
     64, two pieces above; 40 segments go through groups, 10 through one merge."""
     cfg = cfg_of(n_q_heads=heads, n_kv_heads=kv_heads, head_dim=dh, n_paths=paths)
     test_dealt_pairs_match_the_oracle_on_sampled_sequences(cfg, [2570, 650])
+
+
+@pytest.mark.parametrize("kw,lens", [
+    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [640, 777, 1024]),       # 8 query rows against 4: nine to sixteen segments
+    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [4700]),                 # more than eight groups of segments
+    (dict(n_q_heads=4, n_kv_heads=2, head_dim=128, n_paths=3), [900, 650]),  # 6 against 2
+    (dict(n_q_heads=16, n_kv_heads=2, head_dim=64), [5000, 700]),            # 16 against 8 at d_h 64
+])
+def test_merge_of_many_segments_is_the_same_bits_grouped_and_primary_only(kw, lens):
+    """The primary path must not depend on the step's mode.  How many partials a thread keeps in flight does, so the merge's
+    rounding must not follow it: three layers, so that a differing bit of one reaches the cache of the next; several steps."""
+    cfg = cfg_of(n_layers=3, **kw)
+    w = make_weights(cfg, seed=47, matrix_std=0.05)
+    k, v = make_synthetic_kv(cfg, len(lens), max(lens), seed=48)
+    tok = make_tokens(cfg, len(lens), 4, seed=49)
+    kv, z1 = [], []
+    for grouped in (True, False):
+        gm = make_gpu_model(cfg, w, len(lens), max(lens) + 8)
+        gm.write_kv(k, v)
+        gm.set_seq_lens(lens)
+        z1.append([gm.decode_full(tok[:, t].cuda().contiguous(), grouped=grouped)["z1"] for t in range(4)])
+        kv.append(gm.kv_pool.clone())
+    assert torch.equal(kv[0], kv[1])
+    assert all(torch.equal(a, b) for a, b in zip(*z1))
