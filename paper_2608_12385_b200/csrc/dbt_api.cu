@@ -990,6 +990,7 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     // us, Q|K|V 23 -> 21, O 19 -> 19, output matrix 80 -> 56, down 25 -> 29 (its sums then need no second pass); a step is
     // 5 % faster at 132 rows, 20 % at 234.  Up to 128 rows half of M would be idle and the row tile of 128 keeps four stages
     // of both planes as one operand: a step of 128 rows is 13 % faster that way, of 80 rows 17 %.
+    if (e.Z && c.R > 256) return fail(m, DBT_ERR_UNSUPPORTED, "the output-matrix epilogue takes at most 256 rows");
     if (!c.grp_cnt && c.parts == 2 && n_tile >= 256 && many_rows_ok(c)) {
         PgParams q{};
         q.P = e.Z ? e.Z : c.P;
@@ -1042,7 +1043,6 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     // more rows than the widest tile (prompt chunks): several row tiles per weight tile, no split-K
     int row_tiles = 1;
     if (!c.grp_cnt && c.R > 256) {
-        if (e.Z) return fail(m, DBT_ERR_UNSUPPORTED, "the output-matrix epilogue takes at most 256 rows");
         n_tile = 256;
         row_tiles = (c.R + 255) / 256;
         force_split = 1;
@@ -2026,6 +2026,15 @@ dbt_status check_step_args(dbt_model *m, const int32_t *tokens, int B, int n) {
     return DBT_OK;
 }
 
+// Rows that a step of dense bf16 models may stack: the row tiles, the attention plan and the split of the paired-SM GEMMs are
+// chosen from at most 256 rows, and the same for grouped and primary-only steps.  Checked before anything is launched.
+dbt_status check_step_rows(dbt_model *m, int B, int grouped) {
+    if (!m->wide) return DBT_OK;
+    if (B > kAttMaxItems) return fail(m, DBT_ERR_CAPACITY, "attention rows %d exceed %d", B, kAttMaxItems);
+    if (npaths(grouped) * B > 256) return fail(m, DBT_ERR_UNSUPPORTED, "a step takes at most 256 stacked rows (%d)", npaths(grouped) * B);
+    return DBT_OK;
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------------------
@@ -2380,14 +2389,14 @@ static dbt_status step_graphed(dbt_model *m, const int32_t *tokens_dev, int B, i
 dbt_status dbt_decode_step(dbt_model *m, const int32_t *tokens_dev, int32_t B, int32_t *next_tokens_dev,
                            float *logits_primary_dev, float *logits_branch_dev, float *alpha_dev) {
     dbt_status st = check_step_args(m, tokens_dev, B, 1);
-    if (st != DBT_OK) return st;
+    if (st != DBT_OK || (st = check_step_rows(m, B, paths_of(m->cfg))) != DBT_OK) return st;
     return step_graphed(m, tokens_dev, B, paths_of(m->cfg), next_tokens_dev, logits_primary_dev, logits_branch_dev, alpha_dev);
 }
 
 dbt_status dbt_prefill_boundary(dbt_model *m, const int32_t *tokens_dev, int32_t B, int32_t S, int32_t *next_tokens_dev,
                                 float *logits_primary_dev, float *logits_branch_dev, float *alpha_dev) {
     dbt_status st = check_step_args(m, tokens_dev, B, S);
-    if (st != DBT_OK) return st;
+    if (st != DBT_OK || (st = check_step_rows(m, B, paths_of(m->cfg))) != DBT_OK) return st;
     if (S > 1) {
         // positions 1..S-1 of every row of tokens_dev [B][S]: the prompt-wide prefill walks rows of stride S
         m->tok_stride = S;
@@ -2411,7 +2420,7 @@ dbt_status dbt_prefill_boundary(dbt_model *m, const int32_t *tokens_dev, int32_t
 dbt_status dbt_decode_step_primary_only(dbt_model *m, const int32_t *tokens_dev, int32_t B, int32_t *next_tokens_dev,
                                         float *logits_primary_dev) {
     dbt_status st = check_step_args(m, tokens_dev, B, 1);
-    if (st != DBT_OK) return st;
+    if (st != DBT_OK || (st = check_step_rows(m, B, 0)) != DBT_OK) return st;
     return step_graphed(m, tokens_dev, B, 0, next_tokens_dev, logits_primary_dev, nullptr, nullptr);
 }
 

@@ -934,6 +934,25 @@ def test_capacity_and_argument_errors():
         gm.set_page_table(torch.tensor([[0, 0], [1, 2]]))
 
 
+@pytest.mark.parametrize("vocab", [2048, 1000, 2049])
+def test_dense_steps_of_more_than_256_stacked_rows_are_refused_before_anything_is_launched(vocab):
+    """130 sequences x 2 paths: refused whatever the vocabulary (widths that the paired-SM GEMMs take and widths that they do
+    not), with nothing enqueued and no length advanced; the same batch primary-only and 128 sequences grouped still run."""
+    cfg = small_bf16(n_layers=1, vocab=vocab)
+    w = make_weights(cfg, seed=26, matrix_std=0.05)
+    gm = make_gpu_model(cfg, w, 130, 8)
+    tok = make_tokens(cfg, 130, 4, seed=27).cuda()
+    before = gm.launch_count()
+    for call in (lambda: gm.decode_step(tok[:, 0].contiguous()), lambda: gm.prefill_boundary(tok.contiguous())):
+        with pytest.raises(binding.DbtError) as e:
+            call()
+        assert e.value.status == 2
+    assert gm.launch_count() == before and gm.seq_len(0) == 0
+    gm.decode_full(tok[:, 0].contiguous(), grouped=False)
+    gm.decode_full(tok[:128, 1].contiguous())
+    assert gm.seq_len(0) == 2 and gm.sync_status() == (0, 0)
+
+
 def test_out_of_range_token_is_reported_not_faulted():
     cfg = small_bf16(n_layers=1)
     w = make_weights(cfg, seed=25, matrix_std=0.05)
