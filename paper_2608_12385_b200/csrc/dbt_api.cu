@@ -180,6 +180,8 @@ int prefill_rows(const dbt_config &c) {
     const int chunk = all < kPromptRows ? (int)all : kPromptRows;
     return decode_rows(c) > chunk ? decode_rows(c) : chunk;
 }
+// Row pitch of a prompt chunk's router logits: the paired-SM GEMM stores whole 16-byte pieces.
+int router_ld(const dbt_config &c) { return (c.n_experts + 3) / 4 * 4; }
 // Expert-sorted rows of the two-plane buffers: every selection of a decode step's rows, or of a prompt chunk's (the
 // primary path alone, fan-out k_1).
 size_t sorted_rows(const dbt_config &c) {
@@ -260,7 +262,7 @@ size_t carve(const dbt_config &c, char *base, Workspace *ws, int *Rmax_out, int 
     w.att_plan = k.take<int32_t>(kAttPlanInts);
     if (moe) {
         int km = kmax_of(c);
-        w.rlogits = k.take<float>((size_t)Rmax * c.n_experts);
+        w.rlogits = k.take<float>((size_t)Rmax * router_ld(c));
         w.rwts = k.take<float>((size_t)Rmax * km);
         w.ridx = k.take<int32_t>((size_t)Rmax * km);
         w.Hexp = k.take<float>((size_t)Rd * km * c.d_expert);
@@ -507,7 +509,7 @@ dbt_status run_moe(dbt_model *m, int l, const RowMap &rm, int grouped, bool reco
     if (last && !grouped)
         CUDA_TRY(m, cudaMemsetAsync(last + (size_t)c.max_batch * km, 0xff,
                                     sizeof(int32_t) * (paths_of(c) - 1) * c.max_batch * km, m->stream));
-    LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.rlogits, 1, (size_t)0, E, Bc, c.k_primary, c.k_branch, km,
+    LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.rlogits, 1, (size_t)0, E, E, Bc, c.k_primary, c.k_branch, km,
            c.router_mode == DBT_ROUTER_REPLAY, w.ridx, w.rwts, last, c.max_batch * km, (const float *)nullptr, 0, 0, d, c.rms_eps);
     int32_t *ucnt = record_experts ? w.union_cnt + l : nullptr;
     if (ucnt) CUDA_TRY(m, cudaMemsetAsync(ucnt, 0, sizeof(int32_t), m->stream));
@@ -1290,7 +1292,7 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
     if (last && !grouped)
         CUDA_TRY(m, cudaMemsetAsync(last + (size_t)c.max_batch * km, 0xff, sizeof(int32_t) * (paths_of(c) - 1) * c.max_batch * km,
                                     m->stream));
-    LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.P, rnsp, rstride, E, Bc, c.k_primary, c.k_branch, km,
+    LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.P, rnsp, rstride, E, E, Bc, c.k_primary, c.k_branch, km,
            c.router_mode == DBT_ROUTER_REPLAY, w.ridx, w.rwts, last, c.max_batch * km, ssp, ss_tiles, ss_ld, d, c.rms_eps);
     LAUNCH(m, "moe_sort", 0, moe_sort_kernel, 1, R * km > 512 || E > 256 ? 1024 : 256, 0, w.ridx, R, km, E, w.ecnt, w.eoff, w.epos,
            record_experts ? w.union_cnt + l : (int32_t *)nullptr);
@@ -1640,7 +1642,7 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
 // Whether they take the paired-SM chain (otherwise 256-row chunks through the decode step's kernels).
 bool moe_prompt_ok(const dbt_model *m) {
     const dbt_config &c = m->cfg;
-    return c.n_experts > 0 && m->moe_tc && m->moe_wide && m->att_fast && c.d_model <= 8192 && c.n_experts % 4 == 0;
+    return c.n_experts > 0 && m->moe_tc && m->moe_wide && m->att_fast;
 }
 
 // One chunk of a prompt through all layers (Eq. moe_layer, primary path alone: fan-out k_1): Q|K|V, attention, O, router,
@@ -1671,9 +1673,9 @@ dbt_status run_layers_moe_prompt(dbt_model *m, const RowMap &rm) {
             return st;
         PgParams rt{};
         rt.ss_in = w.ss; rt.ss_tiles = ss_tiles; rt.ss_ld = m->Rmax; rt.d_norm = d; rt.eps = c.rms_eps;
-        rt.P = w.rlogits; rt.ldp = E;
+        rt.P = w.rlogits; rt.ldp = router_ld(c);
         if ((st = run_gemm_prompt<PG_STORE>(m, "router", &mp.rt, nullptr, nullptr, {E, 0, 0}, 1, &m->map_Xb, d, R, rt)) != DBT_OK) return st;
-        LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.rlogits, 1, (size_t)0, E, R, c.k_primary, c.k_branch, km, 0, w.ridx,
+        LAUNCH(m, "route", 0, route_kernel, R, 32, 2 * E * sizeof(float), w.rlogits, 1, (size_t)0, rt.ldp, E, R, c.k_primary, c.k_branch, km, 0, w.ridx,
                w.rwts, (int32_t *)nullptr, 0, (const float *)nullptr, 0, 0, d, c.rms_eps);
         LAUNCH(m, "moe_sort", 0, moe_sort_kernel, 1, 1024, 0, w.ridx, R, km, E, w.ecnt, w.eoff, w.epos, (int32_t *)nullptr);
         LAUNCH(m, "moe_gather", 0, moe_gather_rows_kernel, R, 256, 0, w.Xb, lo_x, w.ridx, w.epos, km, c.k_primary, d, w.Xs, lo_xs, w.ss, ss_tiles,

@@ -578,8 +578,8 @@ __global__ void __launch_bounds__(256) moe_gather_kernel(const __nv_bfloat16 *Xb
     DBT_TL_END("moe_gath");
 }
 
-// moe_gather_kernel for a prompt chunk: a block takes a row, requests it before its positions are known, and writes a
-// copy per selection.  d % 8 == 0, d <= 8192.
+// moe_gather_kernel for a prompt chunk: a block takes a row, requests it (8192 columns at a time) before its positions are
+// known, and writes a copy per selection.  d % 8 == 0.
 __global__ void __launch_bounds__(256) moe_gather_rows_kernel(const __nv_bfloat16 *Xb, size_t lo_in, const int32_t *idx, const int32_t *pos,
                                                               int kmax, int k, int d, __nv_bfloat16 *Xs, size_t lo_out, const float *ss,
                                                               int ss_tiles, int ss_ld, float eps, float *rs_sorted) {
@@ -587,33 +587,35 @@ __global__ void __launch_bounds__(256) moe_gather_rows_kernel(const __nv_bfloat1
     const int row = blockIdx.x, nv = d / 8;
     const uint4 *src = reinterpret_cast<const uint4 *>(Xb + (size_t)row * d);
     constexpr int NV = 4;
-    uint4 hi[NV], lo[NV];
-#pragma unroll
-    for (int u = 0; u < NV; u++) {
-        const int i = threadIdx.x + u * 256;
-        if (i < nv) {
-            hi[u] = __ldcg(src + i);
-            lo[u] = __ldcg(src + lo_in / 8 + i);
-        }
-    }
-    float a = 0.f;
-    if (threadIdx.x < 32)
-        for (int t = threadIdx.x; t < ss_tiles; t += 32) a += __ldcg(ss + (size_t)t * ss_ld + row);
-    for (int j = 0; j < k; j++) {
-        if (__ldcg(idx + (size_t)row * kmax + j) < 0) continue;
-        const int ps = __ldcg(pos + (size_t)row * kmax + j);
-        uint4 *dst = reinterpret_cast<uint4 *>(Xs + (size_t)ps * d);
+    for (int v0 = 0; v0 < nv; v0 += NV * 256) {
+        uint4 hi[NV], lo[NV];
 #pragma unroll
         for (int u = 0; u < NV; u++) {
-            const int i = threadIdx.x + u * 256;
+            const int i = v0 + threadIdx.x + u * 256;
             if (i < nv) {
-                dst[i] = hi[u];
-                dst[i + lo_out / 8] = lo[u];
+                hi[u] = __ldcg(src + i);
+                lo[u] = __ldcg(src + lo_in / 8 + i);
             }
         }
-        if (threadIdx.x < 32) {
-            const float q = warp_sum(a);
-            if (threadIdx.x == 0) rs_sorted[ps] = 1.f / sqrtf(q / (float)d + eps);
+        float a = 0.f;
+        if (v0 == 0 && threadIdx.x < 32)
+            for (int t = threadIdx.x; t < ss_tiles; t += 32) a += __ldcg(ss + (size_t)t * ss_ld + row);
+        for (int j = 0; j < k; j++) {
+            if (__ldcg(idx + (size_t)row * kmax + j) < 0) continue;
+            const int ps = __ldcg(pos + (size_t)row * kmax + j);
+            uint4 *dst = reinterpret_cast<uint4 *>(Xs + (size_t)ps * d);
+#pragma unroll
+            for (int u = 0; u < NV; u++) {
+                const int i = v0 + threadIdx.x + u * 256;
+                if (i < nv) {
+                    dst[i] = hi[u];
+                    dst[i + lo_out / 8] = lo[u];
+                }
+            }
+            if (v0 == 0 && threadIdx.x < 32) {
+                const float q = warp_sum(a);
+                if (threadIdx.x == 0) rs_sorted[ps] = 1.f / sqrtf(q / (float)d + eps);
+            }
         }
     }
 }

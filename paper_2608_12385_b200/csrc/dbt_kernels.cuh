@@ -748,7 +748,7 @@ __global__ void advance_len_kernel(int32_t *seq_len, int B, int n) {
 // as split-K partials [nsplit][R][E] (summed in split order).
 // ss != nullptr: the router GEMM ran on g * S (not yet divided by rms(S)); the row's factor comes
 // from its per-tile shares of sum(S^2) and multiplies the logits here (the GEMM is linear).
-__global__ void __launch_bounds__(32) route_kernel(const float *logits, int nsplit, size_t split_stride, int E, int Bc,
+__global__ void __launch_bounds__(32) route_kernel(const float *logits, int nsplit, size_t split_stride, int ld, int E, int Bc,
                                                    int k_p, int k_b, int kmax, int replay, int32_t *idx, float *wts,
                                                    int32_t *last, int last_stride_path, const float *ss, int ss_tiles,
                                                    int ss_ld, int d_norm, float eps) {
@@ -781,8 +781,8 @@ __global__ void __launch_bounds__(32) route_kernel(const float *logits, int nspl
                 for (int j = 0; j < 16; j++) {
                     const int e = e0 + u * 32 + lane;
                     const bool on = e < E && s0 + j < nsplit;
-                    va[u][j] = on ? __ldcg(logits + (size_t)(s0 + j) * split_stride + (size_t)r * E + e) : 0.f;
-                    vb[u][j] = on && twin ? __ldcg(logits + (size_t)(s0 + j) * split_stride + (size_t)sel_row * E + e) : 0.f;
+                    va[u][j] = on ? __ldcg(logits + (size_t)(s0 + j) * split_stride + (size_t)r * ld + e) : 0.f;
+                    vb[u][j] = on && twin ? __ldcg(logits + (size_t)(s0 + j) * split_stride + (size_t)sel_row * ld + e) : 0.f;
                 }
 #pragma unroll
             for (int u = 0; u < 2; u++)

@@ -64,10 +64,26 @@ def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
     (dict(n_experts=8, d_expert=328, n_shared_experts=0, k_branch=8), 1, 513),  # no shared expert: the combine kernel
     (dict(n_experts=8, d_expert=128, n_shared_experts=2, k_primary=3, d_model=328), 1, 300),
     (dict(n_experts=5, d_expert=264, k_primary=2), 1, 290),                     # row tiles of 96 to 160 rows: a ring of five or six stages
+    (dict(n_experts=67, d_expert=64, k_primary=3), 1, 260),                     # a router row of 67 logits
+    (dict(n_experts=6, d_expert=64, d_model=8456, n_layers=1, n_q_heads=2), 1, 257),  # rows of more than 8192 columns
 ])
 def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n):
     from test_gpu_parity import small_moe, test_moe_prompt_chunks_of_more_than_one_row_tile_match_the_oracle as check
     check(small_moe(**kw), B, n, 0.05)
+
+
+def test_moe_prompt_chunks_take_the_same_kernels_at_any_number_of_experts():
+    """A prompt of more than 256 rows goes through the paired-SM chain whether or not the experts come in fours."""
+    from test_gpu_parity import small_moe
+    names = {}
+    for E in (5, 8):
+        cfg = small_moe(n_experts=E)
+        gm = make_gpu_model(cfg, make_weights(cfg, seed=97, matrix_std=0.05), 1, 400)
+        gm.profile_begin()
+        gm.prefill(make_tokens(cfg, 1, 300, seed=98).cuda().contiguous())
+        names[E] = {(e["name"], e["launches"]) for e in gm.profile_end()}
+    assert names[5] == names[8]
+    assert ("expert_gateup", cfg.n_layers) in names[5] and not any(n.startswith("resid") for n, _ in names[5])
 
 
 @pytest.mark.parametrize("n_out,K,R", [(2048, 2048, 70), (2048, 2048, 256), (1028, 520, 129), (4096, 5632, 234), (1024, 64, 200),
