@@ -618,6 +618,7 @@ __global__ void __launch_bounds__(kScThreads, 1) small_mlp_kernel(const SmallMlp
         if (writes) sm[l.h + row * a.F + f_h + i] = h;
     }
     share(l.h, a.F, f_h, l.Fs, 1);
+    if (!a.g_next) cluster_arrive();
     DBT_TL_MARK(2);
     // down, c coupling, residual
     ok = mbar_wait(bar(2), 0) && ok;
@@ -634,6 +635,7 @@ __global__ void __launch_bounds__(kScThreads, 1) small_mlp_kernel(const SmallMlp
     }
     if (a.g_next) {
         share(l.s, a.d, f_o, l.dO, 2);
+        cluster_arrive();
         DBT_TL_MARK(3);
         // the next layer's Q | K | V
         ok = mbar_wait(bar(3), 0) && ok;
@@ -646,6 +648,11 @@ __global__ void __launch_bounds__(kScThreads, 1) small_mlp_kernel(const SmallMlp
         }
     }
     if (!ok && lane == 0) report(a.status, kStatusWaitExpired, 800 + warp);
+    // No CTA leaves before all have sent what they had to send (the arrivals stand behind the last exchange).  Where a wait ran out,
+    // the bytes on their way here are waited for once more, so that none lands in the memory of a CTA that has gone.
+    cluster_wait();
+    if (!ok)
+        for (int e = 0; e < (a.g_next ? 3 : 2); e++) mbar_wait_cluster(bar(4 + e), 0);
     DBT_TL_END("smlp");
 }
 
