@@ -98,6 +98,17 @@ __device__ __forceinline__ void load8(const __nv_bfloat16 *p, float (&v)[8]) {
         v[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
     }
 }
+// Four and eight consecutive elements of a caller's fp32 vector (a gain, a coupling): any alignment, 16-byte loads where
+// the vector has it (a caller may keep them one after the other in one buffer).
+__device__ __forceinline__ float4 load_vec4(const float *p) {
+    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) return *reinterpret_cast<const float4 *>(p);
+    return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ void load_vec8(const float *p, float (&v)[8]) {
+    const float4 a = load_vec4(p), b = load_vec4(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
 __device__ __forceinline__ float load1(const float *p) { return *p; }
 __device__ __forceinline__ float load1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
 __device__ __forceinline__ void store1(float *p, float v) { *p = v; }

@@ -413,8 +413,8 @@ __global__ void __launch_bounds__(256) resid_many_kernel(float *S, const float *
     const bool act = i < d, first = blockIdx.z == 0;
     const int r2 = ((int)blockIdx.z + 1) * Bc + b;
     float4 gn = make_float4(1.f, 1.f, 1.f, 1.f), cc = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (act && g_next) gn = *reinterpret_cast<const float4 *>(g_next + i);
-    if (act && mode >= 2) cc = *reinterpret_cast<const float4 *>(coup_c + i);
+    if (act && g_next) gn = load_vec4(g_next + i);
+    if (act && mode >= 2) cc = load_vec4(coup_c + i);
     pdl_wait();
     float q1 = 0.f, q2 = 0.f;
     if (act) {
@@ -462,7 +462,7 @@ __global__ void __launch_bounds__(256) swiglu_many_kernel(const float *P, int F,
     const bool act = f < F, first = blockIdx.z == 0;
     const int rb = grouped ? ((int)blockIdx.z + 1) * Bc + b : b;
     float4 cb = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (act && grouped && coup_b) cb = *reinterpret_cast<const float4 *>(coup_b + f);
+    if (act && grouped && coup_b) cb = load_vec4(coup_b + f);
     pdl_wait();
     float a = 0.f;  // the norm shares of the block's two rows, a half warp each
     if (ss && threadIdx.x < 32)
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(256) moe_combine_rows_kernel(const float *Ys, 
     const int sub = threadIdx.x >> 6, row = blockIdx.x * 4 + sub, i = blockIdx.y * 256 + (threadIdx.x & 63) * 4;
     const bool act = row < R && i < d;
     float4 gn = make_float4(1.f, 1.f, 1.f, 1.f);
-    if (act && Xn) gn = *reinterpret_cast<const float4 *>(g_next + i);
+    if (act && Xn) gn = load_vec4(g_next + i);
     pdl_wait();
     float q = 0.f;
     if (act) {

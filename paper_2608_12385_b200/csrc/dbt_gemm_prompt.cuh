@@ -488,7 +488,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     tmem_ld16_issue(tacc + cbase + c, v[0]);
                     tmem_ld16_issue(tacc + cbase + c + 16, v[1]);
                     float4 gn = make_float4(1.f, 1.f, 1.f, 1.f);
-                    if (kResid && p.g_next && con) gn = *reinterpret_cast<const float4 *>(p.g_next + col);
+                    if (kResid && p.g_next && con) gn = load_vec4(p.g_next + col);
                     tmem_ld_wait();
                     if (S > 1) {
                         add_peers(v[0], cbase + c);

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32) linear_small_kernel(const Sm
         if (k < K) {
             load8(w0 + k, wa[c]);
             if (SWIGLU) load8(w1 + k, wb[c]);
-            if (a.g) load8(a.g + k, gn[c]);
+            if (a.g) load_vec8(a.g + k, gn[c]);
         }
     }
     const float cp = a.coup ? a.coup[f] : 0.f;
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(kSmallWarps * 32) linear_small_kernel(const Sm
             for (int i = 0; i < 8; i++) gv[i] = 1.f, uv[i] = 0.f;
             load8(w0 + k, wv);
             if (SWIGLU) load8(w1 + k, uv);
-            if (a.g) load8(a.g + k, gv);
+            if (a.g) load_vec8(a.g + k, gv);
             piece(wv, uv, gv, k);
         }
 #pragma unroll
@@ -484,7 +484,7 @@ struct ScRows {
 #pragma unroll
         for (int u = 0; u < 2; u++) {
             const int k = (threadIdx.x & 31) * 4 + u * 128;
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), gv = !norm ? make_float4(1.f, 1.f, 1.f, 1.f) : k < K ? *reinterpret_cast<const float4 *>(g + k) : z;
+            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f), gv = !norm ? make_float4(1.f, 1.f, 1.f, 1.f) : k < K ? load_vec4(g + k) : z;
 #pragma unroll
             for (int r = 0; r < RM; r++) {
                 const float *p = S + (size_t)min(r, R - 1) * K + k;
