@@ -172,13 +172,19 @@ int decode_rows(const dbt_config &c) { return paths_of(c) * c.max_batch > 256 ? 
 // of 256: with the 74 pairs of SMs the tiles of any GEMM are then whole waves, and an expert's matrices serve nearly 600
 // rows.  16 prompts of 2048 into the 1B model 88.3 ms in chunks of 37 row tiles, 85.3 of 74, 84.8 of 111; 32 of 1024 into the
 // MoE model 89.4, 81.8, 82.4 (of 18: 106); chunks of equal length changed neither.  The buffers take 1.1 GB at the 1B
-// width, 2.3 GB at the 8B width.
-constexpr int kPromptRows = 74 * 256;
+// width, 2.3 GB at the 8B width.  Wide fan-outs hold k_1 sorted copies of every row: a chunk has as many rows as fit
+// kPromptBytes (74 row tiles at the widths above), but not fewer than 2048 (at k_1 = 8, d 2048 and experts of 1408: 43 row tiles).
+constexpr int kPromptRows = 74 * 256, kPromptMinRows = 2048;
+constexpr long long kPromptBytes = 2304ll << 20;
 int prefill_rows(const dbt_config &c) {
     if (c.weight_dtype != DBT_DTYPE_BF16) return decode_rows(c);
+    const long long d = c.d_model, qd = (long long)c.n_q_heads * c.head_dim, F = c.n_experts > 0 ? c.n_shared_experts * c.d_expert : c.d_ff;
+    const long long row = 4 * (2 * d + 2 * qd + F) + (c.n_experts > 0 ? c.k_primary * 4ll * (2 * d + c.d_expert) + 4ll * c.n_experts : 0);
+    long long chunk = kPromptBytes / row / 256 * 256;
+    chunk = chunk < kPromptMinRows ? kPromptMinRows : chunk > kPromptRows ? kPromptRows : chunk;
     const long long all = ((long long)c.max_batch * c.max_seq + 255) / 256 * 256;
-    const int chunk = all < kPromptRows ? (int)all : kPromptRows;
-    return decode_rows(c) > chunk ? decode_rows(c) : chunk;
+    if (all < chunk) chunk = all;
+    return decode_rows(c) > chunk ? decode_rows(c) : (int)chunk;
 }
 // Row pitch of a prompt chunk's router logits: the paired-SM GEMM stores whole 16-byte pieces.
 int router_ld(const dbt_config &c) { return (c.n_experts + 3) / 4 * 4; }

@@ -49,6 +49,14 @@ def test_query_sizes_matches_pool_layout(lib):
     assert kv32 == 4 * 2 * 10 * 4 * 16 * 64 * 4
 
 
+@pytest.mark.parametrize("k_primary,limit_gib", [(2, 2), (8, 2.5), (64, 3.5)])
+def test_workspace_of_wide_fan_outs_is_bounded(lib, k_primary, limit_gib):
+    """A prompt chunk keeps k_primary sorted copies of every row; its rows are cut so that the caller is not asked for tens of
+    gigabytes.  The limits: 2.25 GiB of chunk buffers (at least 2048 rows: 1.46 MB each at fan-out 64) beside some 0.3 GiB."""
+    _, ws = binding.query_sizes(moe_1b().replace(k_primary=k_primary), max_batch=8, max_seq=4100, num_pages=8 * 257)
+    assert ws < limit_gib * 2 ** 30
+
+
 @pytest.mark.parametrize("mutate,status", [
     (dict(head_dim=96), 2), (dict(page_size=32), 2), (dict(n_kv_heads=3), 2), (dict(d_model=0), 1),
     (dict(n_q_heads=32, n_kv_heads=2), 2), (dict(weight_dtype="fp32", d_ff=100), 2),
