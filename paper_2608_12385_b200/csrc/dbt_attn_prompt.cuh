@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
         const int pages_total = (n_keys + 15) >> 4, my_pg = lane;
         const bool loads = my_pg < 8;
         int page = loads && my_pg < pages_total ? p.page_table[(size_t)b * p.pt_stride + my_pg] : 0;
+        int nk = 0, nv = 0;  // tiles of keys, of values requested
         for (int t = 0; t < T && ok; t++) {
             const int s = t % STAGES, np = min(8, pages_total - t * 8);
             if (loads && my_pg < np && (page < 0 || page >= p.num_pages)) {
@@ -195,15 +196,23 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (ok && loads && my_pg < np) tma_load_4d(k_s + off, &tmKV, k_full(s), 0, 0, 0, (int)((p.k_row0 + row) >> 3));
+            nk += ok;
             if (lane == 0 && ok) {
                 if (t >= STAGES) ok = mbar_wait(v_empty(s), ((t / STAGES) - 1) & 1);
                 if (ok) mbar_expect_tx(v_full(s), (uint32_t)np * HALVES * 2048);
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (ok && loads && my_pg < np) tma_load_4d(v_s + off, &tmKV, v_full(s), 0, 0, 0, (int)((p.v_row0 + row) >> 3));
+            nv += ok;
             page = next_page;
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 400);
+        // the last loads have landed before the CTA leaves, also where a wait ran out
+        if (lane == 0) {
+            mbar_wait(q_full, 0);
+            for (int j = max(0, nk - STAGES); j < nk; j++) mbar_wait(k_full(j % STAGES), (j / STAGES) & 1, kWaitCycles / STAGES);
+            for (int j = max(0, nv - STAGES); j < nv; j++) mbar_wait(v_full(j % STAGES), (j / STAGES) & 1, kWaitCycles / STAGES);
+        }
     } else if (warp == 9) {
         // ---- MMA issuer (lane 0; the whole warp clears V rows behind the last key)
         constexpr uint32_t idesc_qk = umma_idesc(kPaKeys);

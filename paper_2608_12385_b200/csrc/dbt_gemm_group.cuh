@@ -180,6 +180,14 @@ gemm_group_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
             }
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 700);
+        // The pair's last loads have landed before either CTA leaves, see gemm_prompt_kernel.  (ph: parity of a stage's last fill; of a
+        // stage that had none, that of the phase before a fresh barrier's first.)
+        if (lane == 0 && rank == 0) {
+            for (int j = 0; j < stages; j++) {
+                mbar_wait_cluster(full_bar(s), ph, kWaitCycles / STAGES);
+                if (++s == stages) s = 0, ph ^= 1;
+            }
+        }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
             // ---- MMA issuer of the pair

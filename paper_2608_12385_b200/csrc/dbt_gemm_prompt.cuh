@@ -22,7 +22,8 @@
 //
 // Roles: warp 0 TMA producer, warp 1 MMA issuer (of the pair's first CTA) and TMEM owner, warps 2..9 epilogue (two per
 // TMEM lane quadrant, each taking half of the tile's columns).  Every wait is bounded: on expiry the CTA records
-// kStatusWaitExpired, stops storing, and still reaches the cluster barrier that the pair leaves by.
+// kStatusWaitExpired, stops storing, waits (bounded) for the loads in flight, and still reaches the cluster barrier that the pair
+// leaves by.
 #pragma once
 
 #include "dbt_gemm_tc.cuh"
@@ -133,7 +134,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // mbar_wait with cluster scope: the arrivals come from both CTAs of the pair.
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, uint64_t limit = kWaitCycles) {
     uint32_t done = 0;
     long long t0 = 0;
     while (true) {
@@ -149,7 +150,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
         if (done) return true;
         const long long t = clock64();
         if (t0 == 0) t0 = t;
-        else if ((unsigned long long)(t - t0) > kWaitCycles) return false;
+        else if ((unsigned long long)(t - t0) > limit) return false;
     }
 }
 // Loads of a CTA pair: into this CTA's shared memory, completing on a barrier of either CTA (no multicast).
@@ -328,6 +329,10 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
             }
             DBT_TL_MARK(0);
             if (!ok) report(p.status, kStatusWaitExpired, 600);
+            // The pair's last loads have landed before either CTA leaves, also where a wait ran out (they complete on the first CTA's
+            // barriers; the second leaves by the cluster barrier).
+            if (rank == 0)
+                for (int j = max(0, it - STAGES); j < it; j++) mbar_wait_cluster(full_bar(j % STAGES), (j / STAGES) & 1, kWaitCycles / STAGES);
         }
     } else if (warp == 1) {
         if (lane == 0 && rank == 0) {
