@@ -66,20 +66,21 @@ def test_dealt_pairs_grouped_and_primary_only_write_the_same_cache():
 @pytest.mark.parametrize("heads,kv_heads,dh,paths", [(2, 2, 64, 2), (8, 2, 64, 2), (4, 2, 128, 2), (4, 2, 128, 3), (8, 2, 128, 2)])
 def test_merge_of_many_segments_at_few_and_more_query_rows(heads, kv_heads, dh, paths):
     """2 to 8 query rows: one 16-byte piece of the output per thread (sixteen partials at once) up to 4 rows at d_h 128 or 8 at
-    64, two pieces above; 40 segments go through groups, 10 through one merge."""
+    64, two pieces above; 40 segments (of 256 positions) go through groups, 10 through one merge."""
     cfg = cfg_of(n_q_heads=heads, n_kv_heads=kv_heads, head_dim=dh, n_paths=paths)
-    test_dealt_pairs_match_the_oracle_on_sampled_sequences(cfg, [2570, 650])
+    test_dealt_pairs_match_the_oracle_on_sampled_sequences(cfg, [10250, 2570])
 
 
 @pytest.mark.parametrize("kw,lens", [
-    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [640, 777, 1024]),       # 8 query rows against 4: nine to sixteen segments
-    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [4700]),                 # more than eight groups of segments
-    (dict(n_q_heads=4, n_kv_heads=2, head_dim=128, n_paths=3), [900, 650]),  # 6 against 2
-    (dict(n_q_heads=16, n_kv_heads=2, head_dim=64), [5000, 700]),            # 16 against 8 at d_h 64
+    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [2400, 3000, 4090]),       # 8 query rows against 4: nine to sixteen segments
+    (dict(n_q_heads=8, n_kv_heads=2, head_dim=128), [18500]),                  # 72 segments: more than eight groups
+    (dict(n_q_heads=4, n_kv_heads=2, head_dim=128, n_paths=3), [3600, 2500]),  # 6 against 2
+    (dict(n_q_heads=16, n_kv_heads=2, head_dim=64), [19000, 2700]),            # 16 against 8 at d_h 64
 ])
 def test_merge_of_many_segments_is_the_same_bits_grouped_and_primary_only(kw, lens):
     """The primary path must not depend on the step's mode.  How many partials a thread keeps in flight does, so the merge's
-    rounding must not follow it: three layers, so that a differing bit of one reaches the cache of the next; several steps."""
+    rounding must not follow it.  Segments are of 256 positions here; three layers and four steps, so that a differing bit
+    reaches the cache."""
     cfg = cfg_of(n_layers=3, **kw)
     w = make_weights(cfg, seed=47, matrix_std=0.05)
     k, v = make_synthetic_kv(cfg, len(lens), max(lens), seed=48)

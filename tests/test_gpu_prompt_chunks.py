@@ -58,18 +58,20 @@ def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
     assert torch.equal(a.export_kv(1, 333)[0], b.export_kv(1, 333)[0])
 
 
-@pytest.mark.parametrize("kw,B,n", [
-    (dict(n_experts=4, d_expert=200), 1, 700),                                  # lists of several row tiles of an expert
-    (dict(n_experts=64, d_expert=136, k_branch=2), 2, 150),                     # short lists, some experts without a row
-    (dict(n_experts=8, d_expert=328, n_shared_experts=0, k_branch=8), 1, 513),  # no shared expert: the combine kernel
-    (dict(n_experts=8, d_expert=128, n_shared_experts=2, k_primary=3, d_model=328), 1, 300),
-    (dict(n_experts=5, d_expert=264, k_primary=2), 1, 290),                     # row tiles of 96 to 160 rows: a ring of five or six stages
-    (dict(n_experts=67, d_expert=64, k_primary=3), 1, 260),                     # a router row of 67 logits
-    (dict(n_experts=6, d_expert=64, d_model=8456, n_layers=1, n_q_heads=2), 1, 257),  # rows of more than 8192 columns
+@pytest.mark.parametrize("kw,B,n,std", [
+    (dict(n_experts=4, d_expert=200), 1, 700, 0.05),                                  # lists of several row tiles of an expert
+    (dict(n_experts=64, d_expert=136, k_branch=2), 2, 150, 0.05),                     # short lists, some experts without a row
+    (dict(n_experts=8, d_expert=328, n_shared_experts=0, k_branch=8), 1, 513, 0.05),  # no shared expert: the combine kernel
+    (dict(n_experts=8, d_expert=128, n_shared_experts=2, k_primary=3, d_model=328), 1, 300, 0.05),
+    (dict(n_experts=5, d_expert=264, k_primary=2), 1, 290, 0.05),                     # row tiles of 96 to 160 rows: a ring of five or six stages
+    (dict(n_experts=67, d_expert=64, k_primary=3), 1, 260, 0.05),                     # a router row of 67 logits
+    # rows of more than 8192 columns.  Logits are sums of d products of unit-scale states and weights of deviation std: the stated
+    # tolerance is for std sqrt(d) = 0.05 sqrt(256) = 0.8, which at d = 8456 is std = 0.0087.
+    (dict(n_experts=6, d_expert=64, d_model=8456, n_layers=1, n_q_heads=2), 1, 257, 0.0087),
 ])
-def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n):
+def test_moe_prompt_chunk_edges_match_the_oracle(kw, B, n, std):
     from test_gpu_parity import small_moe, test_moe_prompt_chunks_of_more_than_one_row_tile_match_the_oracle as check
-    check(small_moe(**kw), B, n, 0.05)
+    check(small_moe(**kw), B, n, std)
 
 
 def test_moe_prompt_chunks_take_the_same_kernels_at_any_number_of_experts():
