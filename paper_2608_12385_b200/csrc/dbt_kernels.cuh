@@ -832,7 +832,7 @@ __global__ void __launch_bounds__(32) route_kernel(const float *logits, int nspl
         int bi = 0x7fffffff;
         for (int e = lane; e < E; e += 32) {
             float v = sel[e];
-            if (v > bv || (v == bv && e < bi)) {  // NaN-free: taken entries are -inf
+            if (v > bv || (v == bv && e < bi)) {  // (taken entries are -inf; a NaN is never chosen)
                 bv = v;
                 bi = e;
             }
@@ -846,6 +846,7 @@ __global__ void __launch_bounds__(32) route_kernel(const float *logits, int nspl
                 bi = oi;
             }
         }
+        if (bi >= E) break;  // nothing but NaN is left: the row's further slots stay empty
         if (lane == 0) sel[bi] = -INFINITY;
         __syncwarp();
         tot += own[bi] / sum;
@@ -856,7 +857,7 @@ __global__ void __launch_bounds__(32) route_kernel(const float *logits, int nspl
     for (int j = lane; j < kmax; j += 32) {
         int e = j < k ? (j < 32 ? mine : mine2) : -1;
         idx[(size_t)r * kmax + j] = e;
-        wts[(size_t)r * kmax + j] = j < k ? (own[e] / sum) / tot : 0.f;
+        wts[(size_t)r * kmax + j] = e >= 0 ? (own[e] / sum) / tot : 0.f;
         if (last) last[(size_t)path * last_stride_path + (size_t)(r - path * Bc) * kmax + j] = e;
     }
     DBT_TL_END("route");

@@ -966,6 +966,34 @@ def test_out_of_range_token_is_reported_not_faulted():
     assert gm.sync_status() == (0, 0)
 
 
+@pytest.mark.parametrize("moe,cfg", [("", small_moe()), ("simt", small_moe()), ("", small_moe(weight_dtype="fp32")),
+                                     ("", small_moe(router_mode=1, k_branch=8))])
+def test_a_row_of_nan_router_logits_stays_within_its_row(monkeypatch, moe, cfg):
+    """A token whose embedding is NaN has no top-k: its row selects no expert, and its own outputs are NaN.  The other sequences'
+    outputs are the bits they are without it, in decode steps and in prompt chunks of every form."""
+    if moe:
+        monkeypatch.setenv("DBT_MOE", moe)
+    w = make_weights(cfg, seed=28, matrix_std=0.05)
+    w["embed_primary"][7] = float("nan")
+    w["embed_branch"][7] = float("nan")
+    B, n = 3, 120
+    tok = make_tokens(cfg, B, n + 1, seed=29)
+    tok[tok == 7] = 8
+    out = []
+    for bad in (False, True):
+        t = tok.clone()
+        if bad:
+            t[1, -2:] = 7  # the last position of the prompt, and the step after it
+        gm = make_gpu_model(cfg, w, B, n + 1)
+        z = gm.prefill(t[:, :n].cuda().contiguous(), want_logits=True)
+        g = gm.decode_full(t[:, n].cuda().contiguous())
+        assert gm.sync_status()[0] == 0
+        out.append([z, g["z1"], g["z2"]])
+    for a, b in zip(*out):
+        assert torch.equal(a[[0, 2]], b[[0, 2]]) and torch.isfinite(a).all()
+        assert torch.isnan(b[1]).all()
+
+
 def test_fresh_models_give_bitwise_identical_results():
     """Three handles built one after another run the same prefill and grouped steps: every logit
     is bit-identical (kernels overlap through programmatic dependent launch; a read issued
