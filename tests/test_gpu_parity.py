@@ -67,18 +67,17 @@ def test_prefill_longer_than_one_chunk_and_page_boundaries():
 
 
 @pytest.mark.parametrize("cfg,B,n", [
-    (small_bf16(n_layers=2), 2, 2100),                                    # three chunks of <= 1024 positions, 4 positions per query tile
-    (small_bf16(n_layers=2), 3, 700),                                     # ragged chunks (682 + 18) and tail tiles
-    (small_bf16(n_layers=1, n_q_heads=4, n_kv_heads=4), 1, 2500),         # MHA: 16 positions per tile, 2048 + 452
-    (small_bf16(n_layers=1, n_q_heads=2, n_kv_heads=1, head_dim=128, d_model=128, vocab=777), 5, 1000),  # 8 per tile
-    (small_bf16(n_layers=1, n_q_heads=8, n_kv_heads=1), 2, 333),          # 2 positions per tile
+    (small_bf16(n_layers=2), 2, 2100),                                    # 4 heads per KV head: 32 positions per query tile; 17 row tiles
+    (small_bf16(n_layers=2), 3, 700),                                     # row tiles that span sequences
+    (small_bf16(n_layers=1, n_q_heads=4, n_kv_heads=4), 1, 2500),         # MHA: 128 positions per query tile
+    (small_bf16(n_layers=1, n_q_heads=2, n_kv_heads=1, head_dim=128, d_model=128, vocab=777), 5, 1000),  # 64 per query tile
+    (small_bf16(n_layers=1, n_q_heads=8, n_kv_heads=1), 2, 333),          # 16 per query tile
     (small_bf16(n_layers=1, n_q_heads=3, n_kv_heads=1), 2, 400),          # 3 heads per KV head: 5 positions per tile (the 16-row kernel)
 ])
 def test_long_prompt_prefill_matches_the_oracle(cfg, B, n):
-    """Section 4.4 item 1, prompt-wide prefill: prompts of up to 2500 positions go through in chunks of up to
-    2048 rows (GEMMs over several row tiles per weight tile, vector kernels between them, causal attention
-    with 16 / G consecutive positions per query tile and eight tiles per CTA).  Last-position logits and the
-    whole cache against the oracle's position-by-position primary pass, then two grouped steps on top of the
+    """Section 4.4 item 1, prompt-wide prefill: prompts of up to 2500 positions, each in one chunk (paired-SM GEMMs with
+    their epilogues, causal attention with two 128-row query tiles of 128 / G positions per CTA; chunk borders are
+    crossed in test_gpu_prompt_chunks.py).  Last-position logits and the whole cache against the oracle's position-by-position primary pass, then two grouped steps on top of the
     device's own cache."""
     w = make_weights(cfg, seed=51, matrix_std=0.05)
     tok = make_tokens(cfg, B, n + 2, seed=52)
@@ -130,16 +129,9 @@ def test_prefill_boundary_is_prefill_of_all_but_one_plus_the_grouped_step(cfg):
 
 
 def test_prompt_chunks_through_the_16_row_attention_kernel(monkeypatch):
-    """DBT_PROMPT_ATTN=tile: the earlier form of the prompt attention (one 16-row tile per CTA pass) still
-    serves head ratios that do not divide 16, and computes the same prefill."""
+    """DBT_PROMPT_ATTN=tile: the 16-row decode attention kernel (one tile per CTA pass), which serves head ratios
+    that do not divide 16, computes the same prefill."""
     monkeypatch.setenv("DBT_PROMPT_ATTN", "tile")
-    test_long_prompt_prefill_matches_the_oracle(small_bf16(n_layers=2), 3, 700)
-
-
-def test_prompt_chunks_with_the_swiglu_as_a_kernel_of_its_own(monkeypatch):
-    """DBT_PROMPT_FUSE_SWIGLU=0: the gate|up GEMM of a prompt chunk leaves fp32 partials and the vector SwiGLU
-    kernel follows (the default applies it in the GEMM's epilogue)."""
-    monkeypatch.setenv("DBT_PROMPT_FUSE_SWIGLU", "0")
     test_long_prompt_prefill_matches_the_oracle(small_bf16(n_layers=2), 3, 700)
 
 
@@ -302,7 +294,7 @@ def test_sequences_of_different_lengths_in_one_batch(cfg, lens):
                                    (small_bf16(n_layers=1, n_paths=3), 85)])
 def test_large_batches_up_to_256_stacked_rows(cfg, B):
     """The widest decode tiles: 256 stacked rows (128 sequences x 2 paths), an odd 154, and 255 rows over three
-    paths; prefill of 20 positions (a chunk of more than 2048 rows is cut), three grouped steps."""
+    paths; prefill of 20 positions, three grouped steps."""
     w = make_weights(cfg, seed=43, matrix_std=0.05)
     tok = make_tokens(cfg, B, 23, seed=44)
     teacher_forced_compare(cfg, w, tok, n_prefill=20, grouped=True)
@@ -340,11 +332,11 @@ def test_1b_width_three_paths_at_batch_16_on_sampled_sequences():
     assert gm.sync_status() == (0, 0)
 
 
-def test_8b_width_prompt_pass_with_two_weight_tiles_per_cta():
+def test_8b_width_prompt_pass():
     """The prompt pass at the 8B shape's width (one layer; d 4096, 32 query / 8 KV heads of 128, F 14336): two
-    sequences of 520 positions are one chunk of 1040 rows = five row tiles, where every GEMM of the layer takes
-    two weight tiles per CTA (the Q|K|V launch across its three weight matrices), and the prompt attention
-    kernel runs four heads per KV head.  Last-position logits and the cache against the oracle, then a grouped
+    sequences of 520 positions are one chunk of 1038 rows behind the last position: four whole row tiles of the
+    paired-SM GEMMs and one of 14 rows (the Q|K|V launch across its three weight matrices), and the prompt
+    attention kernel runs four heads per KV head.  Last-position logits and the cache against the oracle, then a grouped
     step on the device's cache."""
     from paper_2608_12385_b200.inputs import dense_8b
     cfg = dense_8b().replace(n_layers=1)
@@ -720,9 +712,8 @@ def test_moe_prefill_matches_the_oracle(cfg):
 @pytest.mark.parametrize("cfg,B,n,std", [(small_moe(), 3, 100, 0.05), (small_moe(), 1, 700, 0.05),
                                          (moe_1b(k_branch=2).replace(n_layers=2), 1, 300, 0.02)])
 def test_moe_prompt_chunks_of_more_than_one_row_tile_match_the_oracle(cfg, B, n, std):
-    """The MoE model's prompt pass in chunks of more than 256 rows (row-tiled GEMMs, the prompt attention kernel,
-    64-row tiles with two weight tiles per CTA in the per-expert GEMMs, the shared-memory-atomic sort, the vector
-    combine) against the oracle's position-by-position primary pass.  With hundreds of prompt rows some router
+    """The MoE model's prompt pass in chunks of more than 256 rows (paired-SM GEMMs with their epilogues, the prompt
+    attention kernel, the experts' paired-SM GEMMs, the combine in the shared down projection's epilogue) against the oracle's position-by-position primary pass.  With hundreds of prompt rows some router
     near-ties are unavoidable, and there the selected set is not unique (Eq. moe_layer fixes it up to rounding):
     a row whose k_1-th and (k_1+1)-th oracle logits are closer than the margin in some layer is left out of the
     cache comparison (its own entries may legitimately differ; its influence on other rows goes through

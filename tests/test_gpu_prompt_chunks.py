@@ -26,9 +26,10 @@ def cfg_of(**kw):
     (cfg_of(n_q_heads=2, n_kv_heads=2), 1, 400, 0),              # one head per KV head: 128 positions per query tile
     (cfg_of(n_q_heads=16, n_kv_heads=2, n_layers=1), 3, 130, 1),  # eight heads per KV head: 16 positions per query tile
     (cfg_of(n_q_heads=4, n_kv_heads=2, head_dim=128, n_layers=1), 1, 650, 0),
+    (cfg_of(n_layers=1), 32, 640, 0),                            # a chunk of 18944 rows and one of 1504
 ])
-def test_prompt_chunk_edges_match_the_oracle(cfg, B, n, past):
-    w = make_weights(cfg, seed=91, matrix_std=0.05)
+def test_prompt_chunk_edges_match_the_oracle(cfg, B, n, past, std=0.05):
+    w = make_weights(cfg, seed=91, matrix_std=std)
     total = past + n
     tok = make_tokens(cfg, B, total, seed=92)
     om = oracle.OracleModel(cfg, w, B, total)
@@ -65,6 +66,7 @@ def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
     (dict(n_experts=8, d_expert=128, n_shared_experts=2, k_primary=3, d_model=328), 1, 300, 0.05),
     (dict(n_experts=5, d_expert=264, k_primary=2), 1, 290, 0.05),                     # row tiles of 96 to 160 rows: a ring of five or six stages
     (dict(n_experts=67, d_expert=64, k_primary=3), 1, 260, 0.05),                     # a router row of 67 logits
+    (dict(n_experts=8, d_expert=128), 32, 640, 0.05),                                 # a chunk of 18944 rows and one of 1536
     # rows of more than 8192 columns.  Logits are sums of d products of unit-scale states and weights of deviation std: the stated
     # tolerance is for std sqrt(d) = 0.05 sqrt(256) = 0.8, which at d = 8456 is std = 0.0087.
     (dict(n_experts=6, d_expert=64, d_model=8456, n_layers=1, n_q_heads=2), 1, 257, 0.0087),
@@ -88,15 +90,51 @@ def test_moe_prompt_chunks_take_the_same_kernels_at_any_number_of_experts():
     assert ("expert_gateup", cfg.n_layers) in names[5] and not any(n.startswith("resid") for n, _ in names[5])
 
 
-@pytest.mark.parametrize("n_out,K,R", [(2048, 2048, 70), (2048, 2048, 256), (1028, 520, 129), (4096, 5632, 234), (1024, 64, 200),
-                                       (11264, 2048, 130)])
+@pytest.mark.parametrize("n_out,K,R", [(2048, 2048, 256), (1028, 520, 129), (4096, 2816, 234), (1024, 64, 200), (11264, 2048, 130)])
 def test_many_row_decode_widths_match_the_oracle(n_out, K, R):
-    """Decode steps of 129 to 256 stacked rows take the paired-SM GEMMs (fewer: row tiles of 128 on one SM): the split over clusters (2 and 4 pairs per tile),
-    ragged last k-tiles and feature tiles.  One layer whose MLP has the given widths, primary rows and branch rows."""
-    cfg = cfg_of(d_model=K if K <= 2048 else 256, d_ff=max(n_out, K) // 2 // 8 * 8, n_layers=1, vocab=1028)
+    """Decode steps of 129 to 256 stacked rows take the paired-SM GEMMs (fewer: row tiles of 128 on one SM): tiles of 96 to 192
+    features, unsplit and over three and four pairs of a cluster, ragged last k-tiles and feature tiles.  One layer whose MLP has
+    the given widths (K = 2816: the down projection's, behind a d of 256), primary rows and branch rows."""
+    cfg = cfg_of(d_model=K if K <= 2048 else 256, d_ff=max(n_out, 2 * K if K > 2048 else K) // 2 // 8 * 8, n_layers=1, vocab=1028)
     B = (R + 1) // 2
     w = make_weights(cfg, seed=95, matrix_std=0.02)
     tok = make_tokens(cfg, B, 3, seed=96)
     from gpu_util import teacher_forced_compare
     # tokens: logits may be off by the stated 2e-2 each, so two probabilities closer than e^(2 x 2e-2) - 1 may swap
     teacher_forced_compare(cfg, w, tok, n_prefill=1, grouped=True, token_margin=4.1e-2)
+
+
+@pytest.mark.parametrize("model,B", [("1b", 66), ("1b", 117), ("8b", 70), ("moe", 75)])
+def test_many_row_decode_at_the_presets_widths_on_sampled_sequences(model, B):
+    """One layer of the presets at 132 to 234 stacked rows: tiles of 128 features over two pairs (1B and MoE Q|K|V, shared gate|up),
+    of 192 over three (8B O and down), of 96 over three, and the unsplit output matrix in tiles of 256."""
+    from paper_2608_12385_b200.inputs import PRESETS, make_synthetic_kv
+    cfg = PRESETS[model]().replace(n_layers=1, **({"vocab": 8192} if model == "8b" else {}))
+    w = make_weights(cfg, seed=0)
+    lens = [3 + (11 * b) % 60 for b in range(B)]
+    k, v = make_synthetic_kv(cfg, B, max(lens), seed=3)
+    tok = make_tokens(cfg, B, 2, seed=2)
+    gm = make_gpu_model(cfg, w, B, max(lens) + 4)
+    gm.write_kv(k, v)
+    gm.set_seq_lens(lens)
+    out = []
+    for t in range(2):
+        out.append(gm.decode_full(tok[:, t].cuda().contiguous()))
+        out[-1]["experts"] = gm.last_experts(B).numpy() if cfg.is_moe else None
+    for b in (0, B // 2, B - 1):
+        om = oracle.OracleModel(cfg, w, 1, max(lens) + 4)
+        om.inject_kv(k[:, b:b + 1, :lens[b]].float().numpy(), v[:, b:b + 1, :lens[b]].float().numpy(), lens[b])
+        for t in range(2):
+            forced = np.ascontiguousarray(out[t]["experts"][:, :, b:b + 1]) if cfg.is_moe else None
+            o = om.decode_step(tok[b:b + 1, t].numpy(), forced_experts=forced)
+            assert_logits_close(out[t]["z1"][b:b + 1], o["z1"], "bf16", f"row {b} step {t} z1")
+            assert_logits_close(out[t]["z2"][b:b + 1], o["z2"], "bf16", f"row {b} step {t} z2")
+    assert gm.sync_status() == (0, 0)
+
+
+@pytest.mark.parametrize("n", [201, 801])
+def test_1b_width_prompts_of_a_few_row_tiles(n):
+    """One layer of the 1B model at 200 and 800 rows: the residual GEMMs over three and four pairs per tile (192 and 256 features)
+    and over two; Q|K|V split and unsplit."""
+    from paper_2608_12385_b200.inputs import PRESETS
+    test_prompt_chunk_edges_match_the_oracle(PRESETS["1b"]().replace(n_layers=1), 1, n, 0, std=0.02)
