@@ -1014,8 +1014,8 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     TcParams p{};
     int tiles = 0, col = 0;
     double bytes = 0;
-    // prompt chunks (more rows than the widest tile): two weight tiles per CTA share every activation box where
-    // that pays -- such a CTA takes ~1.6x as long as a one-tile CTA, so the choice goes by full waves of CTAs
+    // more rows than the widest tile: two weight tiles per CTA share every activation box where that pays -- such a CTA
+    // takes ~1.6x as long as a one-tile CTA, so the choice goes by full waves of CTAs
     int mt = 1;
     if (!c.grp_cnt && c.R > 256) {
         int t1 = 0, t2 = 0;
@@ -1048,7 +1048,8 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     p.status = m->ws.status;
     p.evict_first = m->evict_first ? 1 : 0;
     p.test_skip_load = test_skip_load;
-    // more rows than the widest tile (prompt chunks): several row tiles per weight tile, no split-K
+    // More rows than the widest tile (MoE steps of more than 256 stacked rows, whose router and whose outputs of odd widths do
+    // not take the paired-SM GEMMs): several row tiles per weight tile, no split-K.
     int row_tiles = 1;
     if (!c.grp_cnt && c.R > 256) {
         n_tile = 256;
@@ -1703,9 +1704,8 @@ dbt_status run_layers_moe_prompt(dbt_model *m, const RowMap &rm) {
             sd.Y = w.Yexp; sd.sel_idx = w.ridx; sd.sel_pos = w.epos; sd.sel_wts = w.rwts; sd.kmax = km; sd.k = c.k_primary;
             if ((st = run_gemm_prompt<PG_COMBINE>(m, "shared_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, Fs, R, sd, &ss_tiles)) != DBT_OK) return st;
         } else {
-            LAUNCH(m, "moe_combine", 0, moe_combine_rows_kernel, dim3((R + 3) / 4, (d + 255) / 256), 256, 0, w.Yexp, (const float *)nullptr, 1,
-                   (size_t)0, w.ridx, w.epos, w.rwts, km, R, d, w.S, g_next, g_next ? w.Xb : (__nv_bfloat16 *)nullptr, lo_x,
-                   g_next ? w.ss : (float *)nullptr, m->Rmax);
+            LAUNCH(m, "moe_combine", 0, moe_combine_rows_kernel, dim3((R + 3) / 4, (d + 255) / 256), 256, 0, w.Yexp, w.ridx, w.epos, w.rwts,
+                   km, R, d, w.S, g_next, g_next ? w.Xb : (__nv_bfloat16 *)nullptr, lo_x, g_next ? w.ss : (float *)nullptr, m->Rmax);
             ss_tiles = wide_ss_tiles(m);
         }
     }

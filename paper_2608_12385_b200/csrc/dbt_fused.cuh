@@ -391,19 +391,10 @@ __device__ __forceinline__ void store_split4(__nv_bfloat16 *dst, size_t idx, siz
     }
 }
 
-__device__ __forceinline__ float4 sum_splits4(const float *P, size_t split_stride, int nsplit, size_t off) {
-    float4 m = ldcg4(P + off);
-    for (int s = 1; s < nsplit; s++) {
-        float4 v = ldcg4(P + (size_t)s * split_stride + off);
-        m.x += v.x, m.y += v.y, m.z += v.z, m.w += v.w;
-    }
-    return m;
-}
-
-// resid_wide_kernel and swiglu_couple_kernel for steps of more than 64 stacked rows, whose GEMMs leave one finished sum per
+// resid_wide_kernel and swiglu_couple_kernel for dense steps of 129 to 256 stacked rows, whose GEMMs leave one finished sum per
 // output (no splits): a few MB per launch, so a thread takes four consecutive columns of a row and of its branch twin.
 // At 117 sequences of the 1B model the one-column forms ran in three waves: 6.8 and 11.7 us of the step each.
-// grid (primary rows, ceil(columns / 1024), branches), 256 threads.  Columns % 4 == 0.
+// grid (primary rows, ceil(columns / 1024), branches), 256 threads.  Columns % 4 == 0.  resid_many: modes 1 and 2.
 __global__ void __launch_bounds__(256) resid_many_kernel(float *S, const float *P, int mode, const float *__restrict__ coup_c, int Bc,
                                                          int grouped, const float *__restrict__ g_next, int d, __nv_bfloat16 *Xb,
                                                          size_t lo_off, float *ss_out, int ss_ld) {
@@ -422,7 +413,7 @@ __global__ void __launch_bounds__(256) resid_many_kernel(float *S, const float *
         float4 s1 = ldcg4(S + o1), m1 = ldcg4(P + o1), s2 = s1, m2 = m1;
         if (grouped) {
             s2 = ldcg4(S + o2);
-            if (mode != 3) m2 = ldcg4(P + o2);
+            m2 = ldcg4(P + o2);
         }
         s1.x += m1.x, s1.y += m1.y, s1.z += m1.z, s1.w += m1.w;
         if (first) {
@@ -432,7 +423,6 @@ __global__ void __launch_bounds__(256) resid_many_kernel(float *S, const float *
         q1 = s1.x * s1.x + s1.y * s1.y + s1.z * s1.z + s1.w * s1.w;
         if (grouped) {
             if (mode == 2) m2.x += cc.x * m1.x, m2.y += cc.y * m1.y, m2.z += cc.z * m1.z, m2.w += cc.w * m1.w;
-            if (mode == 3) m2 = make_float4(cc.x * m1.x, cc.y * m1.y, cc.z * m1.z, cc.w * m1.w);  // Eq. matched_attention
             s2.x += m2.x, s2.y += m2.y, s2.z += m2.z, s2.w += m2.w;
             *reinterpret_cast<float4 *>(S + o2) = s2;
             store_split4(Xb, o2, lo_off, make_float4(gn.x * s2.x, gn.y * s2.y, gn.z * s2.z, gn.w * s2.w));
@@ -754,11 +744,11 @@ __global__ void __launch_bounds__(256) moe_combine_sorted_kernel(const float *Ys
     DBT_TL_END("moe_comb");
 }
 
-// moe_combine_sorted_kernel for R primary rows of a prompt chunk (no branch): S += sum_j w_j Expert_j(m) + G(m); the next
-// layer's GEMM input g_next * S as two planes and the shares of sum(S^2).  grid (ceil(R / 4), d / 256), 64 threads
-// per row, four consecutive columns per thread.  d % 4 == 0.
-__global__ void __launch_bounds__(256) moe_combine_rows_kernel(const float *Ys, const float *Psh, int nsplit, size_t split_stride,
-                                                               const int32_t *idx, const int32_t *pos, const float *wts,
+// moe_combine_sorted_kernel for R primary rows of a prompt chunk (no branch) without a shared expert (with one, the combine is in
+// the epilogue of its down projection, PG_COMBINE): S += sum_j w_j Expert_j(m); the next layer's GEMM input g_next * S as two
+// planes and the shares of sum(S^2).  grid (ceil(R / 4), d / 256), 64 threads per row, four consecutive columns per thread.
+// d % 4 == 0.
+__global__ void __launch_bounds__(256) moe_combine_rows_kernel(const float *Ys, const int32_t *idx, const int32_t *pos, const float *wts,
                                                                int kmax, int R, int d, float *S,
                                                                const float *__restrict__ g_next, __nv_bfloat16 *Xn,
                                                                size_t lo_off, float *ss_out, int ss_ld) {
@@ -796,10 +786,6 @@ __global__ void __launch_bounds__(256) moe_combine_rows_kernel(const float *Ys, 
                     m.z = fmaf(w1[j], y[j].z, m.z);
                     m.w = fmaf(w1[j], y[j].w, m.w);
                 }
-        }
-        if (Psh) {
-            float4 sh = sum_splits4(Psh, split_stride, nsplit, o);
-            m.x += sh.x, m.y += sh.y, m.z += sh.z, m.w += sh.w;
         }
         s.x += m.x, s.y += m.y, s.z += m.z, s.w += m.w;
         *reinterpret_cast<float4 *>(S + o) = s;

@@ -1,7 +1,7 @@
 // GEMMs of a prompt chunk on pairs of SMs (tcgen05 cta_group::2), each with the elementwise work that follows it.
 //
-// A prompt chunk (Section 4.4 item 1: the primary path alone walks the prompt) is a dense contraction: up to a few
-// thousand rows against every matrix of the layer.  Its bound is the tensor pipe, at twice the useful FLOPs because the
+// A prompt chunk (Section 4.4 item 1: the primary path alone walks the prompt) is a dense contraction: up to 18944
+// rows against every matrix of the layer.  Its bound is the tensor pipe, at twice the useful FLOPs because the
 // activations are two bf16 planes (x = hi + lo, see dbt_gemm_tc.cuh).  What keeps the pipe busy here:
 //   - a pair of CTAs (a cluster of two on neighbouring SMs) works on one 256-row x N-feature tile: one MMA of M = 256
 //     reads 128 activation rows from each CTA and half of the weight tile from each, so a k-tile of 64 costs an SM
@@ -15,7 +15,7 @@
 // between: gate|up with SwiGLU 204 -> 122 us (1.55 PFLOP/s of tensor work), down + residual 86 + 15 -> 74, Q|K|V + rotation
 // and append 61 + 25 -> 62, O + residual 41 + 15 -> 39.
 //
-// Few row tiles (decode steps of more than 64 stacked rows, short prompts) leave too few tiles for the chip: the contracted
+// Few row tiles (decode steps of 129 to 256 stacked rows, short prompts) leave too few tiles for the chip: the contracted
 // width of a tile is then split over 2 to 4 pairs of one cluster.  Each CTA owns a slice of the tile's columns, the others
 // write their partial sums of it into its (by then idle) ring through distributed shared memory, and it adds them in split
 // order and runs the epilogue of that slice: no partials in memory, no kernel to sum them.

@@ -59,7 +59,7 @@ struct TcParams {
     // launch chain guarantees complete before any CTA of this launch can be resident), so they may be read, and
     // the first ring of weight tiles requested, before the dependency wait
     int grp_prewait;
-    // dense mode with more rows than one tile holds (prompt chunks): blockIdx.x = weight tile * row_tiles + row
+    // dense mode with more rows than one tile holds (MoE steps of more than 256 stacked rows): blockIdx.x = weight tile * row_tiles + row
     // tile, so that the CTAs sharing a weight tile are neighbours in launch order and all but the first find it
     // in L2; 0 or 1: blockIdx.x is the weight tile
     int row_tiles;
@@ -198,7 +198,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 // Activations may arrive as two bf16 terms, x = hi + lo (hi = bf16(x), lo = bf16(x - hi)): the
 // weight tile is then multiplied by both and the two products land in the same fp32
 // accumulator, which restores fp32-level accuracy of the activations at no extra HBM traffic.
-// MT: weight tiles per CTA.  A prompt chunk's GEMM (256-row activation tiles, no split-K) is bound by the
+// MT: weight tiles per CTA.  A GEMM of more than 256 rows (256-row activation tiles, no split-K) is bound by the
 // bytes its CTAs pull from L2 per MMA; with two weight tiles (two accumulators, 2 x 256 TMEM columns) sharing
 // every activation box, a stage carries 96 KB for twice the MMAs of the 80 KB stage of one tile.
 template <int N_TILE, int MT = 1>
@@ -207,9 +207,7 @@ struct TcCfg {
     static constexpr int kStageBytes = MT * kTcABytes + 2 * kBBytes;
     // small row counts: keep one CTA near 100 KB so that a dependent kernel's CTA can become
     // resident beside it; large row counts take the whole SM
-    // (64-row tiles with two weight tiles per CTA -- the per-expert GEMMs of a prompt chunk -- keep two CTAs per SM
-    // with two stages of 48 KB each)
-    static constexpr int kStages = N_TILE <= 16 ? 5 : N_TILE <= 32 ? 4 : N_TILE <= 64 ? (MT == 2 ? 2 : 3) : N_TILE <= 128 ? 4 : 2;
+    static constexpr int kStages = N_TILE <= 16 ? 5 : N_TILE <= 32 ? 4 : N_TILE <= 64 ? 3 : N_TILE <= 128 ? 4 : 2;
     // room for the two planes' accumulators side by side (see `stacked` in the kernel)
     static constexpr int kStackable = N_TILE <= 128;
     static constexpr int kAccCols = kStackable ? 2 * N_TILE : N_TILE;  // accumulator columns of one weight tile

@@ -665,6 +665,13 @@ def test_moe_at_batch_40(monkeypatch, rowtile):
     _moe_compare(small_moe(k_primary=2, k_branch=2), B=40, T=7, npre=5)
 
 
+@pytest.mark.parametrize("vocab", [1000, 32001])
+def test_moe_steps_of_more_than_256_stacked_rows(vocab):
+    """140 sequences, 280 stacked rows: MoE models take them (paired-SM GEMMs where an output is whole 16-byte pieces, several row
+    tiles per weight tile otherwise; two weight tiles per CTA at the odd vocabulary)."""
+    _moe_compare(small_moe(k_primary=2, k_branch=2, vocab=vocab), B=140, T=5, npre=3)
+
+
 def test_moe_1b_shape_two_layers():
     cfg = moe_1b(k_branch=4).replace(n_layers=2)
     _moe_compare(cfg, B=2, T=8, npre=6, matrix_std=0.02)
