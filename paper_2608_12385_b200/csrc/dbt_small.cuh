@@ -36,6 +36,10 @@ struct SmallLin {
     float *S;            // EPI_RESID, EPI_DOWN
 };
 
+// The rows are read through L1, and only those that are there: every warp of the launch reads all of them, and straight from L2
+// (with the last row in place of missing ones) the same few lines were asked for by all SMs at once.  fp32 models of 4 layers, per
+// step at 64 positions: d 2048, 2 rows 1110 -> 482 us, 10 rows 2410 -> 1131 (the generic chain 631 and 1252); d 256, 9 rows
+// 303 -> 191 (283).
 template <typename WT, int RT, bool SWIGLU>
 __global__ void __launch_bounds__(kSmallWarps * 32) linear_small_kernel(const SmallLin a) {
     pdl_launch_dependents();
@@ -79,10 +83,12 @@ __global__ void __launch_bounds__(kSmallWarps * 32) linear_small_kernel(const Sm
             float x[RT][8];
 #pragma unroll
             for (int r = 0; r < RT; r++) {
-                const float *xp = a.X + (size_t)min(r0 + r, rows - 1) * K + k;
-                const float4 x0 = ldcg4(xp), x1 = ldcg4(xp + 4);
-                x[r][0] = x0.x, x[r][1] = x0.y, x[r][2] = x0.z, x[r][3] = x0.w;
-                x[r][4] = x1.x, x[r][5] = x1.y, x[r][6] = x1.z, x[r][7] = x1.w;
+                if (r0 + r < rows) {
+                    load8(a.X + (size_t)(r0 + r) * K + k, x[r]);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; i++) x[r][i] = 0.f;
+                }
             }
 #pragma unroll
             for (int r = 0; r < RT; r++)
