@@ -47,16 +47,65 @@ def test_prompt_chunk_edges_match_the_oracle(cfg, B, n, past, std=0.05):
     assert gm.sync_status() == (0, 0)
 
 
+@pytest.mark.parametrize("cfg,B,n,past", [
+    (cfg_of(), 1, 129, 0),                                        # 128 rows: the most of the short form
+    (cfg_of(), 1, 130, 0),                                        # one row more
+    (cfg_of(), 1, 100, 1),                                        # behind one cached position: the other kernel
+    (cfg_of(), 1, 3, 0),                                          # two positions
+    (cfg_of(), 4, 33, 0),                                         # 4 x 32 rows, whole pages
+    (cfg_of(), 3, 18, 0),
+    (cfg_of(n_q_heads=2, n_kv_heads=2, head_dim=128), 1, 100, 0),  # one head per KV head: 128 positions per block
+    (cfg_of(n_q_heads=8, n_kv_heads=1, head_dim=128), 2, 50, 0),   # eight: 16 positions per block
+    (cfg_of(n_q_heads=16, n_kv_heads=2, n_layers=1), 1, 90, 0),
+])
+def test_short_prompts_match_the_oracle(cfg, B, n, past):
+    """First chunks of at most 128 rows, around the edges of their eight 16-row query tiles and 64-key stages."""
+    test_prompt_chunk_edges_match_the_oracle(cfg, B, n, past)
+
+
+def test_a_captured_short_prompt_replayed_behind_a_longer_cache():
+    """The short form is chosen from the lengths that the host knows when the call is made; a replay of the captured call works on
+    the device's lengths, whatever they are by then."""
+    from paper_2608_12385_b200 import binding
+    from paper_2608_12385_b200.inputs import make_synthetic_kv
+    cfg = cfg_of()
+    w = make_weights(cfg, seed=99, matrix_std=0.05)
+    tok = make_tokens(cfg, 1, 40, seed=100)
+    k, v = make_synthetic_kv(cfg, 1, 300, seed=101)
+    dev = tok.cuda().contiguous()
+    stream = torch.cuda.Stream()
+    gm = binding.Model(cfg, binding.weights_to_device(w), 1, 400, stream=stream)
+    gm.prefill(dev)
+    torch.cuda.synchronize()
+    gm.reset()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        gm.prefill(dev)
+    gm.import_kv(k, v)  # the capture ran nothing: 300 positions, as the replay finds them
+    graph.replay()
+    torch.cuda.synchronize()
+    om = oracle.OracleModel(cfg, w, 1, 400)
+    om.inject_kv(k.float().numpy(), v.float().numpy(), 300)
+    om.prefill(tok.numpy())
+    gm.set_seq_lens([340])
+    k_dev, v_dev = gm.export_kv(1, 340)
+    np.testing.assert_allclose(k_dev.float().numpy(), om.k_cache[:, :1, :340], rtol=2.0 ** -8, atol=5e-3)
+    np.testing.assert_allclose(v_dev.float().numpy(), om.v_cache[:, :1, :340], rtol=2.0 ** -8, atol=5e-3)
+    assert gm.sync_status() == (0, 0)
+
+
 def test_stale_pool_contents_behind_the_prompt_do_not_reach_it():
     """Pages past the last key hold whatever the pool held before; NaN there must change nothing."""
     cfg = cfg_of()
     w = make_weights(cfg, seed=93, matrix_std=0.05)
-    tok = make_tokens(cfg, 1, 333, seed=94).cuda().contiguous()
-    a, b = make_gpu_model(cfg, w, 1, 512), make_gpu_model(cfg, w, 1, 512)
-    b.kv_pool.fill_(float("nan"))
-    za, zb = a.prefill(tok, want_logits=True), b.prefill(tok, want_logits=True)
-    assert torch.equal(za, zb) and torch.isfinite(za).all()
-    assert torch.equal(a.export_kv(1, 333)[0], b.export_kv(1, 333)[0])
+    for n in (333, 71):
+        tok = make_tokens(cfg, 1, n, seed=94).cuda().contiguous()
+        a, b = make_gpu_model(cfg, w, 1, 512), make_gpu_model(cfg, w, 1, 512)
+        b.kv_pool.fill_(float("nan"))
+        za, zb = a.prefill(tok, want_logits=True), b.prefill(tok, want_logits=True)
+        assert torch.equal(za, zb) and torch.isfinite(za).all()
+        assert torch.equal(a.export_kv(1, n)[0], b.export_kv(1, n)[0])
 
 
 @pytest.mark.parametrize("kw,B,n,std", [
