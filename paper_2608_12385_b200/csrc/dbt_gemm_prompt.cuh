@@ -121,10 +121,10 @@ __device__ __forceinline__ uint32_t mapa_u32(uint32_t addr, uint32_t rank) {
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 }
-// The two halves of it: all threads arrive, and wait later.
+// The two halves of it: all threads arrive, and wait later.  The arrival orders no data (relaxed).
 __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();
-    asm volatile("barrier.cluster.arrive.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
     __syncwarp();
