@@ -139,6 +139,7 @@ struct dbt_model {
     int tok_stride = 1, tok_p0 = 0;
     int clusters_at_once[4] = {74, 33, 22, 15};  // clusters of 2, 4, 6, 8 CTAs of a paired-SM GEMM resident at a time (count_clusters)
     bool cluster16 = false;    // clusters of 16 CTAs can run here (see small_cluster)
+    int step_rows = 0;  // inside a decode step of step_tc: the stacked rows of all paths, whatever the mode (see plan_rows)
     bool att_planned = false;  // inside a decode step whose attention work split has been computed (run_embed_wide)
 };
 
@@ -843,6 +844,10 @@ const CUtensorMap *weight_view(dbt_model *m, const CUtensorMap *W, int box_rows)
     return &hit->second;
 }
 
+// The rows that tiles and splits are chosen from.  In decode steps those of all paths, so that a primary-only step adds the same
+// partials in the same order as the grouped step and writes the same K/V bits, also where the two differ in row tiles.
+int plan_rows(const dbt_model *m, int R) { return m->step_rows > R ? m->step_rows : R; }
+
 // Tile width and split of one such GEMM, by the time it takes (us, measured on its parts): a k-tile costs the MMAs of N
 // columns (4 N cycles) or what an SM takes in for it (32 KB of rows and 64 N bytes of weights at ~50 bytes per cycle); a
 // tile's first loads and its end 4.5 us, its epilogue up to 4; an exchange 4.4 at N = 256.  Unsplit tiles follow each other
@@ -921,7 +926,7 @@ dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0,
     p.R = R;
     int widest = 0;
     for (int s = 0; s < nseg; s++) widest = n_out[s] > widest ? n_out[s] : widest;
-    PgPlan pl = plan_gemm_prompt(m, MODE, n_out, nseg, K, R);
+    PgPlan pl = plan_gemm_prompt(m, MODE, n_out, nseg, K, plan_rows(m, R));
     if (shares) *shares = 2 * pl.splits * ((n_out[0] + pl.N - 1) / pl.N);
     if constexpr (MODE == PG_STORE) {
         if (widest <= 64) return launch_gemm_prompt<64, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, 1, p);
@@ -1017,13 +1022,14 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     // more rows than the widest tile: two weight tiles per CTA share every activation box where that pays -- such a CTA
     // takes ~1.6x as long as a one-tile CTA, so the choice goes by full waves of CTAs
     int mt = 1;
-    if (!c.grp_cnt && c.R > 256) {
+    const int plan_R = plan_rows(m, c.R);
+    if (!c.grp_cnt && plan_R > 256) {
         int t1 = 0, t2 = 0;
         for (int s = 0; s < c.nseg; s++) {
             t1 += (c.n_out[s] + kTcM - 1) / kTcM;
             t2 += (c.n_out[s] + 2 * kTcM - 1) / (2 * kTcM);
         }
-        const int rt = (c.R + 255) / 256, sms = m->num_sms;
+        const int rt = (plan_R + 255) / 256, sms = m->num_sms;
         const int w1 = (t1 * rt + sms - 1) / sms, w2 = (t2 * rt + sms - 1) / sms;
         if (16 * w2 < 10 * w1) mt = 2;
     }
@@ -1051,7 +1057,7 @@ dbt_status run_gemm_tc(dbt_model *m, const TcCall &c, int n_tile, int *nsplit_ou
     // More rows than the widest tile (MoE steps of more than 256 stacked rows, whose router and whose outputs of odd widths do
     // not take the paired-SM GEMMs): several row tiles per weight tile, no split-K.
     int row_tiles = 1;
-    if (!c.grp_cnt && c.R > 256) {
+    if (!c.grp_cnt && plan_R > 256) {
         n_tile = 256;
         row_tiles = (c.R + 255) / 256;
         force_split = 1;
@@ -1524,10 +1530,12 @@ dbt_status step_tc(dbt_model *m, const int32_t *tokens_dev, int B, int grouped, 
     }
     int mode, nsp;
     size_t sstride;
+    m->step_rows = paths_of(c) * B;
     st = run_layers_tc(m, rm, grouped, n_tile, true, &mode, &nsp, &sstride);
     m->att_planned = false;
+    if (st == DBT_OK) st = run_head_tc(m, B, grouped, B, 1, 0, n_tile, mode, nsp, sstride);
+    m->step_rows = 0;
     if (st != DBT_OK) return st;
-    if ((st = run_head_tc(m, B, grouped, B, 1, 0, n_tile, mode, nsp, sstride)) != DBT_OK) return st;
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
     if ((st = run_readout(m, B, grouped, next_dev, alpha_dev, z1_dev, z2_dev)) != DBT_OK) return st;
     for (int b = 0; b < B; b++) m->len_host[b] += 1;

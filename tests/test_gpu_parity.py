@@ -467,6 +467,27 @@ def test_moe_kv_cache_bit_identical_at_a_batch_with_row_tiled_expert_gemms():
     assert torch.equal(va.view(torch.int16), vb.view(torch.int16))
 
 
+@pytest.mark.parametrize("kw", [dict(), dict(vocab=32001), dict(d_model=1024, n_q_heads=16, n_kv_heads=4, n_layers=3)])
+def test_moe_kv_cache_bit_identical_beyond_256_stacked_rows(kw):
+    """140 sequences: 280 stacked rows grouped (two row tiles), 140 primary-only (one).  Tiles, weight tiles per CTA and splits come
+    from the batch, so the cache and the primary logits are the same bits."""
+    cfg = small_moe(k_primary=2, k_branch=2, **kw)
+    w = make_weights(cfg, seed=18, matrix_std=0.05)
+    B, T, npre = 140, 7, 4
+    tok = make_tokens(cfg, B, T, seed=19).cuda()
+    wd = binding.weights_to_device(w)
+    a = binding.Model(cfg, wd, B, T)
+    b = binding.Model(cfg, wd, B, T)
+    oa = _run_steps(a, tok, npre, True)
+    ob = _run_steps(b, tok, npre, False)
+    for x, y in zip(oa, ob):
+        assert torch.equal(x["z1"], y["z1"])
+    ka, va = a.export_kv(B, T)
+    kb, vb = b.export_kv(B, T)
+    assert torch.equal(ka.view(torch.int16), kb.view(torch.int16))
+    assert torch.equal(va.view(torch.int16), vb.view(torch.int16))
+
+
 def test_moe_kv_bit_identical_at_full_width_where_the_resident_cta_count_changes_with_the_tile():
     """One layer at the MoE model's width (d 2048, experts of 1408) and 34 sequences: the grouped step's 68
     stacked rows need a row tile of 128 (one GEMM CTA per SM), the 34 primary-only rows alone would fit a tile
