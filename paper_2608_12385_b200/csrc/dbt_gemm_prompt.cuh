@@ -83,7 +83,8 @@ struct PgParams {
     __nv_bfloat16 *H;
     size_t h_lo;
     int F;
-    // PG_QKV (segments 0, 1, 2 = Q, K, V)
+    // PG_QKV: the segments are Q, K, V from number `first` on (1: K and V alone, the last layer of a chunk)
+    int first;
     float *Q;
     __nv_bfloat16 *Qb;  // the prompt attention kernel's queries: bf16, times q_scale (nullptr: Q, fp32)
     float q_scale;
@@ -596,16 +597,16 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                 if (!acc_ready()) break;
                 // PG_QKV: the tile holds N / dh whole heads of one of Q, K, V; the two warps of a lane quadrant take the
                 // first and the second half of every head's rotation pairs (i, i + dh / 2)
-                const int hd = p.dh, hh2 = hd >> 1, span = hd >> 2;
-                const int nh = sg == 0 ? p.n_q : p.n_kv;
+                const int hd = p.dh, hh2 = hd >> 1, span = hd >> 2, mat = sg + p.first;
+                const int nh = mat == 0 ? p.n_q : p.n_kv;
                 const int b = on ? row / p.cn : 0, pos = ld_mut(p.seq_len + b) + (on ? row % p.cn : 0);
                 __nv_bfloat16 *kv = nullptr;
-                if (sg != 0 && on) {
+                if (mat != 0 && on) {
                     const int page = p.page_table[(size_t)b * p.pt_stride + (pos >> 4)];
                     if (page < 0 || page >= p.num_pages) {
                         report(p.status, kStatusBadPage, page);
                     } else {
-                        kv = (sg == 1 ? p.kpool : p.vpool) + ((size_t)page * p.n_kv * 16 + (pos & 15)) * hd;
+                        kv = (mat == 1 ? p.kpool : p.vpool) + ((size_t)page * p.n_kv * 16 + (pos & 15)) * hd;
                     }
                 }
 #pragma unroll 1
@@ -619,7 +620,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         tmem_ld16_issue(tacc + hc * hd + i0, v0);
                         tmem_ld16_issue(tacc + hc * hd + hh2 + i0, v1);
                         float4 cs[8];
-                        if (sg != 2) {
+                        if (mat != 2) {
                             const float4 *tab = reinterpret_cast<const float4 *>(p.rope + (size_t)pos * hh2 + i0);
 #pragma unroll
                             for (int i = 0; i < 8; i++) cs[i] = tab[i];
@@ -633,7 +634,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
 #pragma unroll
                         for (int i = 0; i < 16; i++) {
                             const float u = rs * __uint_as_float(v0[i]), w = rs * __uint_as_float(v1[i]);
-                            if (sg != 2) {
+                            if (mat != 2) {
                                 const float cc = i & 1 ? cs[i >> 1].z : cs[i >> 1].x, sn = i & 1 ? cs[i >> 1].w : cs[i >> 1].y;
                                 x0[i] = u * cc - w * sn;
                                 x1[i] = w * cc + u * sn;
@@ -643,7 +644,7 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                             }
                         }
                         if (head >= nh) continue;
-                        if (sg == 0) {
+                        if (mat == 0) {
                             if (on && p.Qb) {
                                 __nv_bfloat16 *q0 = p.Qb + (size_t)row * p.n_q * hd + (size_t)head * hd + i0;
 #pragma unroll

@@ -187,3 +187,23 @@ def test_1b_width_prompts_of_a_few_row_tiles(n):
     and over two; Q|K|V split and unsplit."""
     from paper_2608_12385_b200.inputs import PRESETS
     test_prompt_chunk_edges_match_the_oracle(PRESETS["1b"]().replace(n_layers=1), 1, n, 0, std=0.02)
+
+
+@pytest.mark.parametrize("kw,n", [
+    (dict(n_q_heads=4, n_kv_heads=1, head_dim=64), 300),    # K and V share one tile of features
+    (dict(n_q_heads=6, n_kv_heads=3, head_dim=64), 258),    # 192 features of each, one row in the second row tile
+    (dict(n_q_heads=6, n_kv_heads=3, head_dim=128), 515),   # a tile and a half of each
+    (dict(n_q_heads=4, n_kv_heads=2, head_dim=128), 90),    # a chunk on the decode step's GEMMs
+])
+def test_prompts_whose_outputs_nobody_reads_fill_the_whole_cache(kw, n):
+    """The last layer of such a prompt forms keys and values alone; a decode step behind it sees them."""
+    cfg = cfg_of(**kw)
+    w = make_weights(cfg, seed=41, matrix_std=0.05)
+    tok = make_tokens(cfg, 2, n + 1, seed=42)
+    om = oracle.OracleModel(cfg, w, 2, n + 1)
+    gm = make_gpu_model(cfg, w, 2, n + 1)
+    om.prefill(tok[:, :n].numpy())
+    gm.prefill(tok[:, :n].cuda().contiguous())
+    want, got = om.decode_step(tok[:, n].numpy()), gm.decode_full(tok[:, n].cuda().contiguous())
+    for name in ("z1", "z2"):
+        assert_logits_close(got[name], want[name], cfg.weight_dtype, name)
