@@ -1390,7 +1390,7 @@ dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0
            (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S,
            m->layers[0].attn_norm_g, w.Xb, m->act_parts == 2 ? (size_t)m->Rmax * c.d_model : (size_t)0, w.ss, m->Rmax,
            (c.d_model + 255) / 256, w.status, w.seq_len, c.n_kv_heads, attn_deep(m, items) ? m->num_sms : 2 * m->num_sms,
-           plan ? w.att_plan : (int32_t *)nullptr);
+           plan ? w.att_plan : (int32_t *)nullptr, 0);
     m->att_planned = plan;  // cleared by the step function when its layers have been enqueued
     return DBT_OK;
 }

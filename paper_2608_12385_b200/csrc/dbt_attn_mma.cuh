@@ -70,6 +70,10 @@ struct AttnParams {
     int pack, cn, nbk;
     const int *plan;   // the step's precomputed work split (embed_fused_kernel), or nullptr
     int plan_prewait;  // the plan may be read before the dependency wait
+    // The producer does not wait for the kernel before (with plan_prewait): the pages it reads were written by earlier steps, which
+    // are complete (the step's embedding kernel lets its dependents in only after its own wait), and the row that this step
+    // adds to them is patched in shared memory.
+    int early;
 };
 
 constexpr int kAttTile = 64;       // tokens per pipeline stage (4 pages)
@@ -151,7 +155,7 @@ __device__ __forceinline__ void consumer_sync() { asm volatile("bar.sync 1, 128;
 // place i, segcum[i] = segments (per KV head) of the rows before place i.
 // The same for every layer of a decode step, so a step computes it once (embed_fused_kernel) and the attention
 // launches copy it; launches without a plan (prompt chunks) compute it themselves.
-__device__ __forceinline__ void att_plan_warp(int lane, int items, int n_kv, int C0_arg, int *cum, const unsigned *nk_s, int *segcum) {
+__device__ __forceinline__ void att_plan_warp(int lane, int items, int n_kv, int C0_arg, int min_units, int *cum, const unsigned *nk_s, int *segcum) {
     int running = 0, longest = 0;
     if (lane == 0) cum[0] = 0;
     for (int base = 0; base < items; base += 32) {
@@ -180,11 +184,11 @@ __device__ __forceinline__ void att_plan_warp(int lane, int items, int n_kv, int
         int n = mode == 0 ? (2 * u + q) / (2 * q) : u / q;
         return min(max(n, 1), min(max(u, 1), kAttMaxSeg));
     };
-    int best_q = max((U0 + C0 - 1) / C0, kAttMinUnits), best_mode = 0;
+    int best_q = max((U0 + C0 - 1) / C0, min_units), best_mode = 0;
     int best_cost = -1, best_sg = 0;
     for (int cand = 0; cand < 6; cand++) {
         const int k = cand / 2 + 1, mode = cand & 1;
-        const int q = max((U0 + k * C0 - 1) / (k * C0), kAttMinUnits);
+        const int q = max((U0 + k * C0 - 1) / (k * C0), min_units);
         int sg = 0, longest_seg = 0;
         for (int base = 0; base < items; base += 32) {
             int i = base + lane;
@@ -225,7 +229,7 @@ __device__ __forceinline__ void att_plan_warp(int lane, int items, int n_kv, int
     if (lane == 0) segcum[0] = 0;
     for (int base = 0; base < items; base += 32) {
         int i = base + lane, n = 0;
-        if (i < items) n = i >= tail0 ? max(1, min(tail_n, (cum[i + 1] - cum[i]) / kAttMinUnits)) : seg_count(cum[i + 1] - cum[i], best_q, best_mode);
+        if (i < items) n = i >= tail0 ? max(1, min(tail_n, (cum[i + 1] - cum[i]) / min_units)) : seg_count(cum[i + 1] - cum[i], best_q, best_mode);
         int incl = n;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -239,10 +243,16 @@ __device__ __forceinline__ void att_plan_warp(int lane, int items, int n_kv, int
 
 constexpr int kAttPlanInts = 3 * kAttMaxItems + 2;  // cum [items + 1] | nk [items] | segcum [items + 1], at fixed offsets
 
+// The shortest segment where the producers fill their rings before the queries exist (see AttnParams::early): what the ring holds,
+// and less where eight segments, one round of the merge's loads, still cover the pair.  1B, one sequence, with 2 / 3 / 4 stages:
+// context 700 592 / 609 / 617 us per step, context 2048 636 / 613 / 625.
+__device__ __forceinline__ int att_min_early(int stages) { return stages <= 2 * kAttGroup ? 2 : 3; }
+
 // A decode step's plan (one position per sequence), by one block of at least 256 threads: rows by falling length.
-__device__ __forceinline__ void att_plan_block(int B, const int32_t *seq_len, int n_kv, int C0, int *plan) {
+__device__ __forceinline__ void att_plan_block(int B, const int32_t *seq_len, int n_kv, int C0, bool early, int *plan) {
     __shared__ int len[kAttMaxItems], cum[kAttMaxItems + 1], segcum[kAttMaxItems + 1];
     __shared__ unsigned nk[kAttMaxItems];
+    __shared__ int min_units;
     const int i = threadIdx.x;
     if (i < B) len[i] = ld_mut(seq_len + i) + 1;
     __syncthreads();
@@ -250,9 +260,10 @@ __device__ __forceinline__ void att_plan_block(int B, const int32_t *seq_len, in
         int rank = 0;
         for (int j = 0; j < B; j++) rank += len[j] > len[i] || (len[j] == len[i] && j < i);
         nk[rank] = (unsigned)len[i] | (unsigned)i << 24;
+        if (rank == 0) min_units = early ? att_min_early((len[i] + kAttTile - 1) / kAttTile) : kAttMinUnits;
     }
     __syncthreads();
-    if (i < 32) att_plan_warp(i, B, n_kv, C0, cum, nk, segcum);
+    if (i < 32) att_plan_warp(i, B, n_kv, C0, min_units, cum, nk, segcum);
     __syncthreads();
     if (i <= B && i <= kAttMaxItems) {
         plan[i] = cum[i];
@@ -275,12 +286,16 @@ __global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens,
                                                           const float *__restrict__ g, float eps, int d, int V,
                                                           float *S, const float *__restrict__ g_next,
                                                           __nv_bfloat16 *Xb, size_t lo_off, float *ss_out, int ss_ld,
-                                                          int ss_tiles, int *status, const int32_t *seq_len, int n_kv, int C0, int *plan) {
-    pdl_enter();
+                                                          int ss_tiles, int *status, const int32_t *seq_len, int n_kv, int C0, int *plan,
+                                                          int barrier) {
+    // barrier: the kernels of this step may rely on all earlier steps being complete, also before their own waits
+    if (!barrier) pdl_launch_dependents();
+    pdl_wait();
+    if (barrier) pdl_launch_dependents();
     __shared__ float scratch[32];
     int r = blockIdx.x;
     if (plan && r == (int)gridDim.x - 1) {
-        att_plan_block(rm.B, seq_len, n_kv, C0, plan);
+        att_plan_block(rm.B, seq_len, n_kv, C0, barrier != 0, plan);
         return;
     }
     int path = r / rm.Bc();  // 0 primary; j >= 1: decode branch j with its own table E2[j-1] (Appendix C.1)
@@ -365,14 +380,11 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         for (int i = lane; i < items; i += 32)
             nk_s[i] = (unsigned)(ld_mut(p.seq_len + p.rm.seq(i)) + p.rm.off(i) + 1) | (unsigned)i << 24;
         __syncwarp();
-        att_plan_warp(lane, items, p.n_kv, (int)gridDim.x, cum, nk_s, segcum);
+        att_plan_warp(lane, items, p.n_kv, (int)gridDim.x, kAttMinUnits, cum, nk_s, segcum);
     }
     __syncthreads();
-    if (use_plan && p.plan_prewait) pdl_wait();
-    DBT_TL_WAITED;
     const int C = gridDim.x, Sg = packed ? items * p.n_kv : segcum[items] * p.n_kv;  // all segments, ordered (row, KV head, segment)
-    DBT_TL_MARK(3);
-    if ((int)blockIdx.x >= Sg) return;
+    if ((int)blockIdx.x >= Sg) return;  // (CTAs with work wait for the kernel before, so this one does not complete before it either way)
     // segment sidx -> its row and the keys it sees, KV head, stage range and the pair's segment count
     auto locate = [&](int sidx, int &item, int &nkeys, int &g, int &seg, int &n, int &ui, int &t0, int &t1) {
         if (packed) {  // one pass per (tile, KV head) over all its keys
@@ -401,6 +413,26 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         t0 = (int)(((long long)seg * ui) / n);
         t1 = (int)(((long long)(seg + 1) * ui) / n);
     };
+    // What the first queries and the new K, V row need besides the partials -- rotation, coupling, the page -- is requested before the
+    // dependency wait: weights, a table and the plan (its positions), none of which this step's kernels write.
+    float2 rope0 = make_float2(1.f, 0.f);
+    float ca00 = 0.f, ca01 = 0.f;
+    int page0 = 0;
+    const bool ahead = use_plan && p.plan_prewait && p.qkv_P != nullptr;
+    if (ahead && warp < kAttWarps) {
+        constexpr int half = DH / 2;
+        int item, nkeys, g, seg, n, ui, t0, t1;
+        locate((int)blockIdx.x, item, nkeys, g, seg, n, ui, t0, t1);
+        const int i = tid % half, o0 = (g * p.G + min(tid, p.G * half - 1) / half) * DH + i;
+        rope0 = p.rope[(size_t)(nkeys - 1) * half + i];
+        if (P > 1) {
+            ca00 = p.coup_a[o0];
+            ca01 = p.coup_a[o0 + half];
+        }
+        if (seg == n - 1 && tid < half) page0 = __ldg(p.page_table + (size_t)p.rm.seq(item) * p.pt_stride + ((nkeys - 1) >> 4));
+    }
+    if (use_plan && p.plan_prewait && !(p.early && warp == kAttWarps)) pdl_wait();
+    DBT_TL_WAITED;
     // this CTA's segment of a round: every second round is dealt backwards
     auto dealt = [&](int round) { return round * C + ((round & 1) ? C - 1 - (int)blockIdx.x : (int)blockIdx.x); };
 
@@ -452,6 +484,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 // at once instead, with the small loads issued first, was measured slower: the queries are ready
                 // 0.8 us sooner but the stream then runs 10 % slower; pausing after one, two, four or six stages
                 // gave 1.0446, 1.0384, 1.0420 and 1.0462 ms per step of the 1B model at batch 16.)
+                if (p.early) continue;  // (the ring was filled before the queries' loads went out)
                 if (it == kAttPauseAt || (it < kAttPauseAt && dealt(round + 1) >= Sg && t == t1 - 1)) asm volatile("bar.sync 2, 160;" ::: "memory");
             }
         }
@@ -516,7 +549,8 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
             const bool do_kv = owns_last && tid < half;
             float *rs_s = reinterpret_cast<float *>(flag + 8);  // [path]
             // the page of this step's position: requested with the first round of loads, used after it
-            const int page_new = do_kv ? __ldg(p.page_table + (size_t)p.rm.seq(item) * p.pt_stride + (pos >> 4)) : 0;
+            const bool pre = ahead && round == 0;
+            const int page_new = pre ? page0 : do_kv ? __ldg(p.page_table + (size_t)p.rm.seq(item) * p.pt_stride + (pos >> 4)) : 0;
             float rs1 = 1.f, rs2 = 1.f, kvs[4] = {0.f, 0.f, 0.f, 0.f};
             float2 t_kv = make_float2(1.f, 0.f);
             for (int it0 = 0; it0 * 128 < nitems; it0++) {
@@ -524,16 +558,29 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 bool act = idx < nitems;
                 int j = act ? idx / half : 0, i = act ? idx % half : tid % half;
                 int o0 = (g * p.G + j) * DH + i, o1 = o0 + half;
-                float2 t = p.rope[(size_t)pos * half + i];
-                float ca0 = grp ? p.coup_a[o0] : 0.f, ca1 = grp ? p.coup_a[o1] : 0.f;
+                const bool here = pre && it0 == 0;
+                float2 t = here ? rope0 : p.rope[(size_t)pos * half + i];
+                float ca0 = here ? ca00 : grp ? p.coup_a[o0] : 0.f, ca1 = here ? ca01 : grp ? p.coup_a[o1] : 0.f;
                 const size_t offs[4] = {p1 + o0, p1 + o1, p2 + o0, p2 + o1};
                 float sm[4] = {0.f, 0.f, 0.f, 0.f};
-                if (act) sum_splits_k<4, 12>(p.qkv_P, p.qkv_stride, p.qkv_nsplit, offs, sm);
+                if (act) {
+                    if (p.qkv_nsplit == 1) {  // (finished sums: the code of the general form alone is a microsecond of instruction misses)
+#pragma unroll
+                        for (int k = 0; k < 4; k++) sm[k] = __ldcg(p.qkv_P + offs[k]);
+                    } else {
+                        sum_splits_k<4, 12>(p.qkv_P, p.qkv_stride, p.qkv_nsplit, offs, sm);
+                    }
+                }
                 if (it0 == 0) {
                     if (do_kv) {  // K_1 and V_1 of this step's token for this KV head (tid = rotation pair)
                         size_t ko = p1 + q_dim + (size_t)g * DH + tid, vo = ko + kv_dim;
                         const size_t koffs[4] = {ko, ko + half, vo, vo + half};
-                        sum_splits_k<4, 12>(p.qkv_P, p.qkv_stride, p.qkv_nsplit, koffs, kvs);
+                        if (p.qkv_nsplit == 1) {
+#pragma unroll
+                            for (int k = 0; k < 4; k++) kvs[k] = __ldcg(p.qkv_P + koffs[k]);
+                        } else {
+                            sum_splits_k<4, 12>(p.qkv_P, p.qkv_stride, p.qkv_nsplit, koffs, kvs);
+                        }
                         t_kv = t;  // idx = tid < half in the first round: the same rotation pair
                     }
                     if (warp == 0) {
@@ -558,6 +605,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                             __syncwarp();
                         }
                     }
+                    DBT_TL_MARK(3);
                     consumer_sync();
                     rs1 = rs_s[0];
                     rs2 = rs_s[1];
@@ -608,7 +656,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         }
         consumer_sync();
         if (round == 0) {
-            asm volatile("bar.arrive 2, 160;" ::: "memory");  // the producer may stream on
+            if (!p.early) asm volatile("bar.arrive 2, 160;" ::: "memory");  // the producer may stream on
             DBT_TL_MARK(0);
         }
         int pair = item * p.n_kv + g;
@@ -868,7 +916,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                     }
                     if (owns_last && t == ui - 1 && ((nkeys - 1) >> 4 & 3) == warp) patch_new_row(kpage, vpage, (nkeys - 1) & 15);
                     // S^T = K Q^T: K rows as the A operand
-                    float sacc[4] = {0.f, 0.f, 0.f, 0.f};
+                    float sacc[4] = {0.f, 0.f, 0.f, 0.f}, sodd[4] = {0.f, 0.f, 0.f, 0.f};  // (two chains of products)
                     {
                         int r = (lane & 7) + (((lane >> 3) & 1) << 3);  // key row this lane addresses
                         int cb = lane >> 4;                              // which 8-dim chunk of the k-step
@@ -879,8 +927,10 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                             uint32_t a = kpage + sg * 128 + (((chunk & 7) ^ (sg & 7)) << 4);
                             uint32_t ka[4];
                             ldsm_x4(a, ka);
-                            mma_bf16(sacc, ka, qb[ks][0], qb[ks][1]);
+                            mma_bf16(ks & 1 ? sodd : sacc, ka, qb[ks][0], qb[ks][1]);
                         }
+#pragma unroll
+                        for (int e = 0; e < 4; e++) sacc[e] += sodd[e];
                     }
                     // sacc: keys g8, g8+8 (rows) x queries 2t, 2t+1 (columns)
                     if (valid < 16) {
@@ -929,7 +979,8 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                     }
                 }
                 __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(s)) : "memory");
+                // (the last stage is the fold's scratch first)
+                if (lane == 0 && t + 1 < t1) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(s)) : "memory");
             }
             if (!ok) {
                 if (lane == 0) report(p.status, kStatusWaitExpired, 310 + warp);
@@ -941,89 +992,66 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 l_run[j] += __shfl_xor_sync(0xffffffffu, l_run[j], 8);
                 l_run[j] += __shfl_xor_sync(0xffffffffu, l_run[j], 16);
             }
-            // ---- fold the four warps' states, (0+2) + (1+3), through the scratch ([8 queries][DH + 4])
+            if (round == 0) DBT_TL_MARK(1);
+            // ---- fold the four warps' states.  Each leaves its own in its page of the last stage, which nobody else touches
+            // ([8 queries][DH + 4], then (m, l) of each), and every thread adds four consecutive outputs of a query over the
+            // four.  (Three rounds through one slot of scratch with six barriers, the outputs written by one warp in 4-byte
+            // pieces, made a step of one sequence 3 % slower.)
             {
                 constexpr int FN = DH + 4;
-                int c = (lane & 3) * 2;
-                auto put = [&]() {
+                static_assert((8 * FN + 16) * 4 <= 2 * Cfg::kPageBytes, "a warp's state fits its page");
+                const int c = (lane & 3) * 2;
+                float *last = reinterpret_cast<float *>(gen + (it - 1) % STAGES * Cfg::kStageBytes);
+                constexpr int WS = 2 * Cfg::kPageBytes / 4;  // floats between two warps' states
+                float *st = last + warp * WS;
+                __syncwarp();
 #pragma unroll
-                    for (int mb = 0; mb < MB; mb++) {
-                        sc_o[(size_t)c * FN + mb * 16 + g8] = o[mb][0];
-                        sc_o[(size_t)(c + 1) * FN + mb * 16 + g8] = o[mb][1];
-                        sc_o[(size_t)c * FN + mb * 16 + g8 + 8] = o[mb][2];
-                        sc_o[(size_t)(c + 1) * FN + mb * 16 + g8 + 8] = o[mb][3];
-                    }
-                    if (g8 == 0) {
-                        sc_m[c] = m_run[0];
-                        sc_m[c + 1] = m_run[1];
-                        sc_l[c] = l_run[0];
-                        sc_l[c + 1] = l_run[1];
-                    }
-                };
-                auto take = [&]() {
-                    float fa[2], fb[2];
-#pragma unroll
-                    for (int j = 0; j < 2; j++) {
-                        float mb2 = sc_m[c + j], lb = sc_l[c + j];
-                        float M = fmaxf(m_run[j], mb2);
-                        fa[j] = m_run[j] == -INFINITY ? 0.f : exp2f(m_run[j] - M);
-                        fb[j] = mb2 == -INFINITY ? 0.f : exp2f(mb2 - M);
-                        l_run[j] = l_run[j] * fa[j] + lb * fb[j];
-                        m_run[j] = M;
-                    }
-#pragma unroll
-                    for (int mb = 0; mb < MB; mb++) {
-                        o[mb][0] = o[mb][0] * fa[0] + sc_o[(size_t)c * FN + mb * 16 + g8] * fb[0];
-                        o[mb][1] = o[mb][1] * fa[1] + sc_o[(size_t)(c + 1) * FN + mb * 16 + g8] * fb[1];
-                        o[mb][2] = o[mb][2] * fa[0] + sc_o[(size_t)c * FN + mb * 16 + g8 + 8] * fb[0];
-                        o[mb][3] = o[mb][3] * fa[1] + sc_o[(size_t)(c + 1) * FN + mb * 16 + g8 + 8] * fb[1];
-                    }
-                };
-                for (int step = 0; step < 3; step++) {  // 2 -> 0, 3 -> 1, 1 -> 0
-                    int src = step == 0 ? 2 : step == 1 ? 3 : 1, dst = step == 1 ? 1 : 0;
-                    if (warp == src) put();
-                    consumer_sync();
-                    if (warp == dst) take();
-                    consumer_sync();
+                for (int mb = 0; mb < MB; mb++) {
+                    st[(size_t)c * FN + mb * 16 + g8] = o[mb][0];
+                    st[(size_t)(c + 1) * FN + mb * 16 + g8] = o[mb][1];
+                    st[(size_t)c * FN + mb * 16 + g8 + 8] = o[mb][2];
+                    st[(size_t)(c + 1) * FN + mb * 16 + g8 + 8] = o[mb][3];
                 }
-                if (warp == 0) {
+                if (g8 == 0) {
+                    *reinterpret_cast<float2 *>(st + 8 * FN + 2 * c) = make_float2(m_run[0], l_run[0]);
+                    *reinterpret_cast<float2 *>(st + 8 * FN + 2 * c + 2) = make_float2(m_run[1], l_run[1]);
+                }
+                consumer_sync();
+                constexpr int VQ = DH / 4;
+                for (int idx = tid; idx < nq_act * VQ; idx += 128) {
+                    const int q = idx / VQ, e = idx % VQ * 4;
+                    float2 ml[kAttWarps];
+                    float M = -INFINITY, L = 0.f;
+                    float4 X = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                    for (int j = 0; j < 2; j++) {
-                        int q = c + j;
-                        if (q < nq_act) {
-                            if (nseg == 1) {
-                                int row = packed ? item_row0(item) + q / p.G : (q / p.G) * Bc + item;
-                                int hq = g * p.G + q % p.G;
-                                size_t ob = (size_t)row * q_dim + (size_t)hq * DH;
-                                float inv = 1.f / l_run[j];
-#pragma unroll
-                                for (int mb = 0; mb < MB; mb++)
-#pragma unroll
-                                    for (int e = 0; e < 2; e++) {
-                                        float x = o[mb][2 * e + j] * inv;
-                                        size_t oi = ob + mb * 16 + g8 + 8 * e;
-                                        __nv_bfloat16 hi = __float2bfloat16_rn(x);
-                                        p.Ob[oi] = hi;
-                                        if (p.lo_off) p.Ob[oi + p.lo_off] = __float2bfloat16_rn(x - __bfloat162float(hi));
-                                    }
-                            } else {
-#pragma unroll
-                                for (int mb = 0; mb < MB; mb++) {
-                                    out[(size_t)q * DH + mb * 16 + g8] = o[mb][j];
-                                    out[(size_t)q * DH + mb * 16 + g8 + 8] = o[mb][2 + j];
-                                }
-                                if (g8 == 0) {
-                                    out[16 * DH + 2 * q] = m_run[j];  // base-2 units
-                                    out[16 * DH + 2 * q + 1] = l_run[j];
-                                }
-                            }
-                        }
+                    for (int w = 0; w < kAttWarps; w++) {
+                        ml[w] = *reinterpret_cast<const float2 *>(last + w * WS + 8 * FN + 2 * q);
+                        M = fmaxf(M, ml[w].x);
                     }
-                    if (nseg > 1) __threadfence();
+#pragma unroll
+                    for (int w = 0; w < kAttWarps; w++) {
+                        const float f = ml[w].x == -INFINITY ? 0.f : exp2f(ml[w].x - M);
+                        const float4 y = *reinterpret_cast<const float4 *>(last + w * WS + q * FN + e);
+                        L = fmaf(ml[w].y, f, L);
+                        X.x = fmaf(y.x, f, X.x), X.y = fmaf(y.y, f, X.y), X.z = fmaf(y.z, f, X.z), X.w = fmaf(y.w, f, X.w);
+                    }
+                    if (nseg == 1) {
+                        // the pair's only segment: normalise and write the head's output
+                        const int row = (q / p.G) * Bc + item, hq = g * p.G + q % p.G;
+                        const float inv = 1.f / L;
+                        store_split4(p.Ob, (size_t)row * q_dim + (size_t)hq * DH + e, p.lo_off, make_float4(X.x * inv, X.y * inv, X.z * inv, X.w * inv));
+                    } else {
+                        *reinterpret_cast<float4 *>(out + (size_t)q * DH + e) = X;
+                        if (e == 0) *reinterpret_cast<float2 *>(out + 16 * DH + 2 * q) = make_float2(M, L);  // base-2 units
+                    }
+                }
+                if (nseg > 1) __threadfence();
+                if (dealt(round + 1) < Sg) {  // the stage goes back to the producer
+                    consumer_sync();
+                    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar((it - 1) % STAGES)) : "memory");
                 }
             }
         }
-        if (round == 0) DBT_TL_MARK(1);
         // ---- merging a pair's segments.  Up to kAttSingle segments: the last one to arrive merges them
         // all, in segment order, and writes the output.  More: the segments form groups of kAttGroup;
         // the last arrival of a group merges it in place into the group's first slot, and the last
