@@ -17,6 +17,7 @@
 
 #include "dbt_attn_mma.cuh"
 #include "dbt_attn_prompt.cuh"
+#include "dbt_few.cuh"
 #include "dbt_fused.cuh"
 #include "dbt_gemm_tc.cuh"
 #include "dbt_gemm_persist.cuh"
@@ -64,6 +65,7 @@ struct LayerMaps {
     CUtensorMap eg, eu, ed;                  // all routed experts as [E*Fe, d], [E*Fe, d], [E*d, Fe]
     CUtensorMap rt;                          // router [E, d]
     CUtensorMap eg64, eu64;                  // the experts' in boxes of 64 rows (prompt chunks)
+    CUtensorMap fq, fk, fv, fo, fg, fu, fd;  // decode steps at few rows (dbt_few.cuh)
 };
 
 }  // namespace
@@ -91,6 +93,8 @@ struct dbt_model {
     bool tc;
     std::vector<LayerMaps> maps;
     CUtensorMap map_lm, map_Xb, map_Ob, map_Hb, map_kv, map_Xs, map_Hs;
+    CUtensorMap few_lm, few_X[3], few_O[3], few_H[3];  // the same of the output matrix and of the rows (boxes of 2, 4, 8)
+    bool few_ok;                  // every contracted width comes in whole 64-element columns
     GgRowMaps rows_Xs, rows_Hs;   // the sorted rows as the experts' GEMMs of a prompt chunk read them
     CUtensorMap map_pq, map_pkv;  // prompt attention: queries, pages
     // prompt chunks take attn_prompt_kernel (bf16 queries, see prompt_q); off for head ratios that do not divide 16 and by
@@ -1098,6 +1102,7 @@ struct QkvFuse {
     const float *ss;
     int ss_tiles, ss_ld;
     const float *coup_a;
+    bool early = false;  // the pages may be requested before the Q|K|V kernel is done (see AttnParams)
 };
 
 // One deep-ring CTA per SM instead of two CTAs per SM: when the (sequence, KV head) pairs fill one wave of SMs,
@@ -1200,6 +1205,7 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
     if (planned && !packed) {  // from the second layer on the plan may be read before the dependency wait
         p.plan = m->ws.att_plan;
         p.plan_prewait = layer > 0 ? 1 : 0;
+        p.early = qf && qf->early && layer > 0 ? 1 : 0;
     }
     if (!packed && items > kAttMaxItems) return fail(m, DBT_ERR_CAPACITY, "attention rows %d exceed %d", items, kAttMaxItems);
     dim3 grid(2 * m->num_sms);  // two resident CTAs per SM; each takes an equal share of all K/V tiles
@@ -1381,16 +1387,16 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
 
 // Embeddings and the first layer's GEMM input; plan: also the attention work split of a decode step, once for all its layers.
 template <typename WT>
-dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0, const RowMap &rm, int R, bool plan) {
+dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0, const RowMap &rm, int R, bool plan, bool few = false) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
     const int items = rm.B * rm.cn;
     plan = plan && items <= kAttMaxItems;  // (the attention launch reports the capacity error)
     LAUNCH(m, "embed", 0, embed_fused_kernel<WT>, R + (plan ? 1 : 0), 256, 0, tokens_dev, n, p0, rm, (const WT *)m->w.embed_primary,
            (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S,
-           m->layers[0].attn_norm_g, w.Xb, m->act_parts == 2 ? (size_t)m->Rmax * c.d_model : (size_t)0, w.ss, m->Rmax,
-           (c.d_model + 255) / 256, w.status, w.seq_len, c.n_kv_heads, attn_deep(m, items) ? m->num_sms : 2 * m->num_sms,
-           plan ? w.att_plan : (int32_t *)nullptr, 0);
+           m->layers[0].attn_norm_g, w.Xb, m->act_parts == 2 ? (size_t)m->Rmax * c.d_model : (size_t)0, w.ss,
+           few ? kFewRows : m->Rmax, few ? (c.d_model + 15) / 16 : (c.d_model + 255) / 256, w.status, w.seq_len, c.n_kv_heads, attn_deep(m, items) ? m->num_sms : 2 * m->num_sms,
+           plan ? w.att_plan : (int32_t *)nullptr, few ? 1 : 0);
     m->att_planned = plan;  // cleared by the step function when its layers have been enqueued
     return DBT_OK;
 }
@@ -1640,6 +1646,82 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
     return DBT_OK;
 }
 
+// ---- decode steps of dense bf16 models at few stacked rows (dbt_few.cuh) -----------------------------
+// Decided from the batch and the model, never from the mode, so that grouped and primary-only steps do the same arithmetic per row.
+bool few_step(const dbt_model *m, int B) { return m->few_ok && paths_of(m->cfg) * B <= kFewRows; }
+int few_box(int rows) { return rows <= 2 ? 0 : rows <= 4 ? 1 : 2; }
+
+template <int MODE>
+dbt_status run_few(dbt_model *m, const char *tag, int B, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
+                   const CUtensorMap (&X)[3], FewParams p) {
+    double bytes = 0;
+    p.tiles = 0;
+    for (int s = 0; s < p.nseg; s++) {
+        p.tile0[s] = p.tiles;
+        p.tiles += (p.n_out[s] + (MODE == FEW_GATEUP ? 7 : 15)) / (MODE == FEW_GATEUP ? 8 : 16);
+        bytes += (double)p.n_out[s] * p.K * 2 * (MODE == FEW_GATEUP ? 2 : 1);
+    }
+    p.evict_first = m->evict_first ? 1 : 0;
+    p.status = m->ws.status;
+    const int slots = kFewCtas * m->num_sms, grid = p.tiles < slots ? p.tiles : slots, x = few_box(paths_of(m->cfg) * B);
+    const FewLayout lay = few_layout(2 << x, p.K, p.tiles <= grid, p.tiles <= m->num_sms ? kFewSmemOne : kFewSmem);
+    p.ring = lay.ring;
+    p.x_resident = lay.resident;
+    if (x == 0) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 2>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[0], p);
+    else if (x == 1) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 4>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[1], p);
+    else LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 8>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[2], p);
+    return DBT_OK;
+}
+
+// The layer stack and the shared output matrix: five kernels per layer.
+dbt_status run_layers_few(dbt_model *m, const RowMap &rm, int grouped) {
+    typedef __nv_bfloat16 WT;
+    const dbt_config &c = m->cfg;
+    const Workspace &w = m->ws;
+    const int B = rm.B, R = npaths(grouped) * B, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ff;
+    const int ss_tiles = (d + 15) / 16;
+    double kv_bytes = 0;
+    for (int b = 0; b < B; b++) kv_bytes += (double)(m->len_host[b] + 1) * 2 * kvd * sizeof(WT);
+    dbt_status st;
+    auto lin = [&](int n_out, int K) {
+        FewParams p{};
+        p.n_out[0] = n_out; p.rows[0] = R; p.nseg = 1; p.K = K; p.R = R; p.Bc = B; p.d = d; p.F = F;
+        return p;
+    };
+    auto normed = [&](FewParams &p) { p.ss_in = w.ss; p.ss_tiles = ss_tiles; p.d_norm = d; p.eps = c.rms_eps; };
+    auto resid = [&](FewParams &p, const float *g_next, const float *coup) {
+        p.S = w.S; p.g_next = g_next; p.coup = coup; p.Xn = w.Xb; p.xn_lo = (size_t)m->Rmax * d; p.ss_out = w.ss;
+    };
+    for (int l = 0; l < c.n_layers; l++) {
+        const dbt_layer_weights &lw = m->layers[l];
+        const LayerMaps &mp = m->maps[l];
+        FewParams q = lin(qd, d);
+        q.n_out[1] = kvd; q.rows[1] = B; q.col0[1] = qd;
+        q.n_out[2] = kvd; q.rows[2] = B; q.col0[2] = qd + kvd;
+        q.nseg = 3; q.Y = w.P; q.ldy = qd + 2 * kvd;
+        normed(q);
+        if ((st = run_few<FEW_STORE>(m, "gemm_qkv", B, &mp.fq, &mp.fk, &mp.fv, m->few_X, q)) != DBT_OK) return st;
+        const QkvFuse qf{w.P, 1, 0, nullptr, 0, 0, lw.coup_a, true};  // (1/rms is in the rows already)
+        st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, grouped, l, kv_bytes, &qf, false, m->att_planned)
+                               : run_attention_mma<64>(m, rm, grouped, l, kv_bytes, &qf, false, m->att_planned);
+        if (st != DBT_OK) return st;
+        FewParams o = lin(d, qd);
+        resid(o, lw.mlp_norm_g, nullptr);
+        if ((st = run_few<FEW_RESID>(m, "gemm_o", B, &mp.fo, &mp.fo, &mp.fo, m->few_O, o)) != DBT_OK) return st;
+        FewParams gu = lin(F, d);
+        gu.coup = lw.coup_b; gu.H = w.Hb; gu.h_lo = (size_t)m->Rmax * F;
+        normed(gu);
+        if ((st = run_few<FEW_GATEUP>(m, "gemm_gateup", B, &mp.fg, &mp.fu, &mp.fu, m->few_X, gu)) != DBT_OK) return st;
+        FewParams dn = lin(d, F);
+        resid(dn, l + 1 < c.n_layers ? m->layers[l + 1].attn_norm_g : (c.final_norm ? m->w.final_norm_g : (const float *)nullptr), lw.coup_c);
+        if ((st = run_few<FEW_RESID>(m, "gemm_down", B, &mp.fd, &mp.fd, &mp.fd, m->few_H, dn)) != DBT_OK) return st;
+    }
+    FewParams lm = lin(c.vocab, d);
+    lm.Y = w.Z; lm.ldy = c.vocab;
+    if (c.final_norm) normed(lm);
+    return run_few<FEW_STORE>(m, "gemm_lm_head", B, &m->few_lm, &m->few_lm, &m->few_lm, m->few_X, lm);
+}
+
 // ---- prompt chunks of dense bf16 models -------------------------------------------------------------
 
 // One chunk of a prompt through all layers: five kernels per layer, one in the last: nobody reads the chunk's outputs, so that layer
@@ -1779,11 +1861,12 @@ dbt_status step_wide(dbt_model *m, const int32_t *tokens_dev, int B, int grouped
     RowMap rm{B, 1};
     int R = npaths(grouped) * B, n_tile = pad_rows(paths_of(c) * B);
     dbt_status st;
-    if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, true)) != DBT_OK) return st;
-    st = run_layers_wide(m, rm, grouped, n_tile);
+    const bool few = few_step(m, B);
+    if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, true, few)) != DBT_OK) return st;
+    st = few ? run_layers_few(m, rm, grouped) : run_layers_wide(m, rm, grouped, n_tile);
     m->att_planned = false;
     if (st != DBT_OK) return st;
-    if ((st = run_head_wide(m, rm, grouped, n_tile)) != DBT_OK) return st;
+    if (!few && (st = run_head_wide(m, rm, grouped, n_tile)) != DBT_OK) return st;
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
     if ((st = run_readout(m, B, grouped, next_dev, alpha_dev, z1_dev, z2_dev)) != DBT_OK) return st;
     for (int b = 0; b < B; b++) m->len_host[b] += 1;
@@ -1886,6 +1969,13 @@ bool allow_smem_prompt() {
            cudaFuncSetAttribute(gemm_group_kernel<GG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess;
 }
 
+template <int MODE>
+bool allow_smem_few() {
+    return cudaFuncSetAttribute(few_linear_kernel<MODE, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) == cudaSuccess &&
+           cudaFuncSetAttribute(few_linear_kernel<MODE, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) == cudaSuccess &&
+           cudaFuncSetAttribute(few_linear_kernel<MODE, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) == cudaSuccess;
+}
+
 // Clusters of 2 S CTAs, one CTA per SM, that this device holds at a time.
 void count_clusters(dbt_model *m) {
     for (int S = 1; S <= 4; S++) {
@@ -1983,7 +2073,7 @@ bool setup_tc(dbt_model *m) {
         m->act_base[&m->map_Hs] = {w.Hs};
     }
     const char *fa = getenv("DBT_ATTN");
-    m->att_fast = ok && allow_smem_prompt() && c.max_seq < (1 << 24) && !(fa && strcmp(fa, "simt") == 0) &&
+    m->att_fast = ok && allow_smem_prompt() && allow_smem_few<FEW_STORE>() && allow_smem_few<FEW_RESID>() && allow_smem_few<FEW_GATEUP>() && c.max_seq < (1 << 24) && !(fa && strcmp(fa, "simt") == 0) &&
                   make_kv_page_map(&m->map_kv, m->kv_pool, (uint64_t)c.n_layers * 2 * c.num_pages * c.n_kv_heads * c.page_size,
                                    (uint64_t)c.num_pages * c.n_kv_heads * c.page_size, c.head_dim) &&
                   cudaFuncSetAttribute(attn_prompt_short_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2009,6 +2099,18 @@ bool setup_tc(dbt_model *m) {
     // Default chain of a dense bf16 model: the RMSNorm factor is applied after the GEMM, so no kernel
     // reduces over a whole row.
     m->wide = ok && m->att_fast && !moe;
+    m->few_ok = m->wide && make_few_weight_map(&m->few_lm, m->w.lm_head, c.vocab, d, 16);
+    for (int l = 0; l < c.n_layers && m->few_ok; l++) {
+        const dbt_layer_weights &lw = m->layers[l];
+        LayerMaps &mp = m->maps[l];
+        m->few_ok = make_few_weight_map(&mp.fq, lw.wq, qd, d, 16) && make_few_weight_map(&mp.fk, lw.wk, kvd, d, 16) &&
+                    make_few_weight_map(&mp.fv, lw.wv, kvd, d, 16) && make_few_weight_map(&mp.fo, lw.wo, d, qd, 16) &&
+                    make_few_weight_map(&mp.fg, lw.w_gate, F, d, 8) && make_few_weight_map(&mp.fu, lw.w_up, F, d, 8) &&
+                    make_few_weight_map(&mp.fd, lw.w_down, d, F, 16);
+    }
+    for (int i = 0; i < 3 && m->few_ok; i++)
+        m->few_ok = make_few_row_map(&m->few_X[i], w.Xb, m->Rmax, d, 2 << i) && make_few_row_map(&m->few_O[i], w.Ob, m->Rmax, qd, 2 << i) &&
+                    make_few_row_map(&m->few_H[i], w.Hb, m->Rmax, F, 2 << i);
     m->act_parts = 2;
     const char *pa = getenv("DBT_PROMPT_ATTN");
     const int G = c.n_q_heads / c.n_kv_heads;
