@@ -1654,22 +1654,33 @@ int few_box(int rows) { return rows <= 2 ? 0 : rows <= 4 ? 1 : 2; }
 template <int MODE>
 dbt_status run_few(dbt_model *m, const char *tag, int B, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
                    const CUtensorMap (&X)[3], FewParams p) {
+    const int x = few_box(paths_of(m->cfg) * B);
     double bytes = 0;
-    p.tiles = 0;
-    for (int s = 0; s < p.nseg; s++) {
-        p.tile0[s] = p.tiles;
-        p.tiles += (p.n_out[s] + (MODE == FEW_GATEUP ? 7 : 15)) / (MODE == FEW_GATEUP ? 8 : 16);
-        bytes += (double)p.n_out[s] * p.K * 2 * (MODE == FEW_GATEUP ? 2 : 1);
+    int tm = 1;
+    auto cut = [&] {
+        const int per = tm * (MODE == FEW_GATEUP ? 8 : 16);
+        p.tiles = 0;
+        for (int s = 0; s < p.nseg; s++) {
+            p.tile0[s] = p.tiles;
+            p.tiles += (p.n_out[s] + per - 1) / per;
+        }
+    };
+    cut();
+    if (x == 2 && p.K >= 4096 && p.tiles / 2 >= m->num_sms * 3 / 4) {
+        tm = 2;
+        cut();
     }
+    for (int s = 0; s < p.nseg; s++) bytes += (double)p.n_out[s] * p.K * 2 * (MODE == FEW_GATEUP ? 2 : 1);
     p.evict_first = m->evict_first ? 1 : 0;
     p.status = m->ws.status;
-    const int slots = kFewCtas * m->num_sms, grid = p.tiles < slots ? p.tiles : slots, x = few_box(paths_of(m->cfg) * B);
-    const FewLayout lay = few_layout(2 << x, p.K, p.tiles <= grid, p.tiles <= m->num_sms ? kFewSmemOne : kFewSmem);
+    const int slots = kFewCtas * m->num_sms, grid = p.tiles < slots ? p.tiles : slots;
+    const FewLayout lay = few_layout(2 << x, tm, p.K, p.tiles <= grid, p.tiles <= m->num_sms ? kFewSmemOne : kFewSmem);
     p.ring = lay.ring;
     p.x_resident = lay.resident;
-    if (x == 0) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 2>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[0], p);
-    else if (x == 1) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 4>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[1], p);
-    else LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 8>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[2], p);
+    if (x == 0) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 2, 1>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[0], p);
+    else if (x == 1) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 4, 1>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[1], p);
+    else if (tm == 1) LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 8, 1>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[2], p);
+    else LAUNCH(m, tag, bytes, (few_linear_kernel<MODE, 8, 2>), grid, kFewThreads, lay.bytes, *W0, *W1, *W2, X[2], p);
     return DBT_OK;
 }
 
@@ -1971,9 +1982,10 @@ bool allow_smem_prompt() {
 
 template <int MODE>
 bool allow_smem_few() {
-    return cudaFuncSetAttribute(few_linear_kernel<MODE, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) == cudaSuccess &&
-           cudaFuncSetAttribute(few_linear_kernel<MODE, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) == cudaSuccess &&
-           cudaFuncSetAttribute(few_linear_kernel<MODE, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) == cudaSuccess;
+    for (const void *f : {(const void *)few_linear_kernel<MODE, 2, 1>, (const void *)few_linear_kernel<MODE, 4, 1>, (const void *)few_linear_kernel<MODE, 8, 1>,
+                          (const void *)few_linear_kernel<MODE, 8, 2>})
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kFewSmemOne) != cudaSuccess) return false;
+    return true;
 }
 
 // Clusters of 2 S CTAs, one CTA per SM, that this device holds at a time.

@@ -83,7 +83,7 @@ __device__ __forceinline__ void tma_load_w(uint32_t dst, const CUtensorMap *map,
 // NR: room for 2, 4 or 8 rows over all paths.
 template <int NR>
 struct FewCfg {
-    static constexpr int kWBytes = 16 * kFewStage * 2;      // a stage of weights
+    static constexpr int kWBytes = 16 * kFewStage * 2;      // a stage of sixteen weight rows
     static constexpr int kXBytes = 2 * NR * kFewStage * 2;  // and of the rows
 };
 // Shared memory of a CTA: the rows as a whole where they take at most kFewRowBytes (each CTA then reads them once, however many tiles it
@@ -91,8 +91,8 @@ struct FewCfg {
 struct FewLayout {
     int resident, ring, bytes;
 };
-inline FewLayout few_layout(int NR, int K, bool single, int smem) {
-    const int stages = (K + kFewStage - 1) / kFewStage, w = 16 * kFewStage * 2, x = 2 * NR * kFewStage * 2;
+inline FewLayout few_layout(int NR, int TM, int K, bool single, int smem) {
+    const int stages = (K + kFewStage - 1) / kFewStage, w = TM * 16 * kFewStage * 2, x = 2 * NR * kFewStage * 2;
     FewLayout l;
     l.resident = !single && stages * x <= kFewRowBytes;
     const int fixed = l.resident ? stages * x : 0, per = l.resident ? w : w + x;
@@ -102,16 +102,20 @@ inline FewLayout few_layout(int NR, int K, bool single, int smem) {
     return l;
 }
 
-template <int MODE, int NR>
+// TM: sixteens of weight rows per tile.  At eight rows a stage of them is as large as a stage of sixteen weight rows; two sixteens
+// share it where the contracted width is long and that leaves enough tiles for the SMs: 8B, four sequences of 32768 / 500 positions
+// 5704 / 3183 -> 5568 / 3100 us per step (at a width of 2048, four stages, it is slower: 1B 699 -> 710).
+template <int MODE, int NR, int TM>
 __global__ void __launch_bounds__(kFewThreads, 2)
 few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
                   const __grid_constant__ CUtensorMap tmX, const FewParams p) {
     using Cfg = FewCfg<NR>;
     constexpr bool FOUR = NR <= 4;
-    constexpr int PL = FOUR ? 1 : 2;
+    constexpr int PL = FOUR ? 1 : 2, QS = TM == 1 ? 2 : 1;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ float sums[2][kFewWarps][kFewRows * kFewColStride];
-    __shared__ float fin[2][kFewRows][16];
+    constexpr int NB = TM == 1 ? 2 : 1;  // buffers of the warps' sums (two sixteens: two CTAs would not fit an SM with two)
+    __shared__ float sums[NB][kFewWarps][TM][kFewRows * kFewColStride];
+    __shared__ float fin[2][TM][kFewRows][16];
     __shared__ float rs_s[kFewRows];
     __shared__ int bad_s;  // a wait ran out: nothing is stored from here on
     __shared__ __align__(8) uint64_t bar_s[2 * kFewMaxRing + 1];
@@ -122,7 +126,7 @@ few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
     const int stages = (p.K + kFewStage - 1) / kFewStage;  // of a tile
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u, bars = smem_u32(bar_s);
     const uint32_t ring = base + (xres ? stages * Cfg::kXBytes : 0);
-    const int stage_bytes = Cfg::kWBytes + (xres ? 0 : Cfg::kXBytes);
+    const int stage_bytes = TM * Cfg::kWBytes + (xres ? 0 : Cfg::kXBytes);
     auto full_bar = [&](int s) { return bars + 8u * s; };
     auto empty_bar = [&](int s) { return bars + 8u * (kFewMaxRing + s); };
     const uint32_t x_bar = bars + 8u * (2 * kFewMaxRing);
@@ -151,15 +155,19 @@ few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
             auto load_w = [&](int s, int tile, int st) {
                 const uint32_t dst = ring + s * stage_bytes;
                 mbar_expect_tx(full_bar(s), stage_bytes);
-                if (MODE == FEW_GATEUP) {
-                    tma_load_w(dst, &tmW0, full_bar(s), tile * 8, st * 8, pol, p.evict_first);
-                    tma_load_w(dst + Cfg::kWBytes / 2, &tmW1, full_bar(s), tile * 8, st * 8, pol, p.evict_first);
-                } else {
-                    const int sg = seg_of(tile);
-                    tma_load_w(dst, sg == 0 ? &tmW0 : sg == 1 ? &tmW1 : &tmW2, full_bar(s), (tile - p.tile0[sg]) * 16, st * 8, pol, p.evict_first);
+                const int sg = seg_of(tile), row = (tile - p.tile0[sg]) * TM;
+#pragma unroll
+                for (int m = 0; m < TM; m++) {  // (rows past the matrix's last arrive as zeros)
+                    if (MODE == FEW_GATEUP) {
+                        tma_load_w(dst + m * Cfg::kWBytes, &tmW0, full_bar(s), (row + m) * 8, st * 8, pol, p.evict_first);
+                        tma_load_w(dst + m * Cfg::kWBytes + Cfg::kWBytes / 2, &tmW1, full_bar(s), (row + m) * 8, st * 8, pol, p.evict_first);
+                    } else {
+                        tma_load_w(dst + m * Cfg::kWBytes, sg == 0 ? &tmW0 : sg == 1 ? &tmW1 : &tmW2, full_bar(s), (row + m) * 16, st * 8, pol,
+                                   p.evict_first);
+                    }
                 }
             };
-            auto load_x = [&](int s, int st) { tma_load_4d(ring + s * stage_bytes + Cfg::kWBytes, &tmX, full_bar(s), 0, 0, st * 8, 0); };
+            auto load_x = [&](int s, int st) { tma_load_4d(ring + s * stage_bytes + TM * Cfg::kWBytes, &tmX, full_bar(s), 0, 0, st * 8, 0); };
             const int mine = (p.tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x, total = mine * stages, npre = min(RING, total);
             int tile = blockIdx.x, st = 0, i = 0;
             for (; i < npre; i++) {
@@ -202,28 +210,31 @@ few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
         q += __shfl_xor_sync(0xffffffffu, q, 16);
         if (lane < kFewRows) rs_s[lane] = p.ss_in ? 1.f / sqrtf(q / (float)p.d_norm + p.eps) : 1.f;
         __syncwarp();
-        asm volatile("bar.arrive 3, 160;" ::: "memory");
+        asm volatile("bar.arrive 3, %0;" ::"n"(32 + 128 * TM) : "memory");
         return;
     }
 
-    // the epilogue's thread: feature ef, row er of a tile
-    const int ef = MODE == FEW_GATEUP ? tid & 7 : tid & 15, er = MODE == FEW_GATEUP ? tid >> 3 : tid >> 4;
+    // the epilogue's thread: feature ef, row er of sixteen `sub` of a tile
+    const int sub = warp >> 2, etid = tid & 127;  // (four warps per sixteen)
+    const int ef = MODE == FEW_GATEUP ? etid & 7 : etid & 15, er = MODE == FEW_GATEUP ? etid >> 3 : etid >> 4;
     float cp = 0.f, gn = 1.f, s_old = 0.f;
     auto load_vecs = [&](int tile) {
         if (MODE == FEW_RESID && er < kFewRows) {
-            const int f = tile * 16 + ef;
+            const int f = (tile * TM + sub) * 16 + ef;
             if (f < p.d) {
                 gn = p.g_next ? p.g_next[f] : 1.f;
                 cp = p.coup ? p.coup[f] : 0.f;
             }
         }
-        if (MODE == FEW_GATEUP && er < kFewRows && tile * 8 + ef < p.F) cp = p.coup ? p.coup[tile * 8 + ef] : 0.f;
+        const int h = (tile * TM + sub) * 8 + ef;
+        if (MODE == FEW_GATEUP && er < kFewRows && h < p.F) cp = p.coup ? p.coup[h] : 0.f;
     };
     load_vecs(blockIdx.x);
     pdl_wait();
     DBT_TL_WAITED;
     auto load_s = [&](int tile) {
-        if (MODE == FEW_RESID && er < p.R && tile * 16 + ef < p.d) s_old = __ldcg(p.S + (size_t)er * p.d + tile * 16 + ef);
+        const int f = (tile * TM + sub) * 16 + ef;
+        if (MODE == FEW_RESID && er < p.R && f < p.d) s_old = __ldcg(p.S + (size_t)er * p.d + f);
     };
     load_s(blockIdx.x);
     int buf = 0, slot = 0, par = 0;
@@ -234,26 +245,32 @@ few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
     auto piece = [&](uint32_t at, uint32_t o, int c) { return lds128(at + ((o + c * 16) ^ ((o >> 3) & 0x70))); };
     bool ok = !xres || mbar_wait(x_bar, 0);
     for (int tile = blockIdx.x; tile < p.tiles; tile += gridDim.x, buf ^= 1) {
-        float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        float acc[TM][2][4];
+#pragma unroll
+        for (int m = 0; m < TM; m++)
+#pragma unroll
+            for (int i = 0; i < 8; i++) acc[m][i >> 2][i & 3] = 0.f;
         const int next = tile + (int)gridDim.x;
 #pragma unroll 1
-        for (int st = 0; st < stages; st += 2) {
-            // two stages at a time: their fragments are read together, their products follow
-            uint4 a[2][2][2], x[2][2][PL];
-            const int nst = min(2, stages - st);
+        for (int st = 0; st < stages; st += QS) {
+            // two stages at a time (two sixteens: one): their fragments are read together, their products follow
+            uint4 a[QS][TM][2][2], x[QS][2][PL];
+            const int nst = min(QS, stages - st);
 #pragma unroll
-            for (int q = 0; q < 2; q++) {
+            for (int q = 0; q < QS; q++) {
                 if (q >= nst) break;
                 ok = ok && mbar_wait(full_bar(slot), par);
                 if (tile == (int)blockIdx.x && st == 0 && q == 0) DBT_TL_MARK(0);
                 // Lane t takes the row's sixteen elements 16 t .. 16 t + 15 of this warp's 64 as two 16-byte pieces: with the swizzle
                 // no two lanes of a quarter warp meet in a bank.
-                const uint32_t at = ring + slot * stage_bytes, xat = xres ? base + (st + q) * Cfg::kXBytes : at + Cfg::kWBytes;
+                const uint32_t at = ring + slot * stage_bytes, xat = xres ? base + (st + q) * Cfg::kXBytes : at + TM * Cfg::kWBytes;
 #pragma unroll
                 for (int blk = 0; blk < 2; blk++) {
 #pragma unroll
-                    for (int h = 0; h < 2; h++)  // (gate|up: the gate rows' columns, then the up rows')
-                        a[q][blk][h] = piece(at, MODE == FEW_GATEUP ? h * (Cfg::kWBytes / 2) + warp * 1024 + g * 128 : warp * 2048 + (g + 8 * h) * 128, 2 * t + blk);
+                    for (int mh = 0; mh < 2 * TM; mh++) {  // (gate|up: the gate rows' columns, then the up rows')
+                        const int m = mh >> 1, h = mh & 1;
+                        a[q][m][blk][h] = piece(at + m * Cfg::kWBytes, MODE == FEW_GATEUP ? h * (Cfg::kWBytes / 2) + warp * 1024 + g * 128 : warp * 2048 + (g + 8 * h) * 128, 2 * t + blk);
+                    }
 #pragma unroll
                     for (int pl = 0; pl < PL; pl++)
                         x[q][blk][pl] = xslot ? piece(xat, (((FOUR ? g >> 2 : pl) * 8 + warp) * NR + xr) * 128, 2 * t + blk) : make_uint4(0, 0, 0, 0);
@@ -263,16 +280,17 @@ few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
                 if (++slot == RING) slot = 0, par ^= 1;
             }
 #pragma unroll
-            for (int q = 0; q < 2; q++) {
+            for (int q = 0; q < QS; q++) {
                 if (q >= nst) break;
 #pragma unroll
-                for (int blk = 0; blk < 2; blk++) {
-                    const uint4 v = a[q][blk][0], w = a[q][blk][1];
+                for (int mb = 0; mb < 2 * TM; mb++) {
+                    const int m = mb >> 1, blk = mb & 1;
+                    const uint4 v = a[q][m][blk][0], w = a[q][m][blk][1];
                     const uint32_t fa[4] = {v.x, w.x, v.y, w.y}, fb[4] = {v.z, w.z, v.w, w.w};
 #pragma unroll
                     for (int pl = 0; pl < PL; pl++) {
-                        mma_bf16(acc[blk], fa, x[q][blk][pl].x, x[q][blk][pl].y);
-                        mma_bf16(acc[blk], fb, x[q][blk][pl].z, x[q][blk][pl].w);
+                        mma_bf16(acc[m][blk], fa, x[q][blk][pl].x, x[q][blk][pl].y);
+                        mma_bf16(acc[m][blk], fb, x[q][blk][pl].z, x[q][blk][pl].w);
                     }
                 }
             }
@@ -282,58 +300,61 @@ few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constan
             bad_s = 1;
         }
         if (tile == (int)blockIdx.x) DBT_TL_MARK(1);
-        float *mine = sums[buf][warp];  // [column][feature]
 #pragma unroll
-        for (int i = 0; i < 4; i++) mine[(2 * t + (i & 1)) * kFewColStride + g + (i >> 1) * 8] = acc[0][i] + acc[1][i];
+        for (int m = 0; m < TM; m++)  // [column][feature]
+#pragma unroll
+            for (int i = 0; i < 4; i++) sums[buf % NB][warp][m][(2 * t + (i & 1)) * kFewColStride + g + (i >> 1) * 8] = acc[m][0][i] + acc[m][1][i];
         asm volatile("bar.sync 2, 256;" ::: "memory");
-        if (warp >= 4) continue;
-        if (MODE != FEW_RESID && tile == (int)blockIdx.x) asm volatile("bar.sync 3, 160;" ::: "memory");  // 1/rms is there
+        if (warp >= 4 * TM) continue;
+        if (MODE != FEW_RESID && tile == (int)blockIdx.x) asm volatile("bar.sync 3, %0;" ::"n"(32 + 128 * TM) : "memory");  // 1/rms is there
         if (bad_s) continue;
         {
-            const int f = tid & 15, r = tid >> 4;
+            const int f = etid & 15, r = etid >> 4;
             float v = 0.f;
 #pragma unroll
             for (int w = 0; w < kFewWarps; w++) {
                 if (FOUR) {
-                    if (r < 4) v += sums[buf][w][r * kFewColStride + f] + sums[buf][w][(r + 4) * kFewColStride + f];
+                    if (r < 4) v += sums[buf % NB][w][sub][r * kFewColStride + f] + sums[buf % NB][w][sub][(r + 4) * kFewColStride + f];
                 } else {
-                    v += sums[buf][w][r * kFewColStride + f];
+                    v += sums[buf % NB][w][sub][r * kFewColStride + f];
                 }
             }
+            if (NB == 1) asm volatile("bar.sync 2, 256;" ::: "memory");  // all have read: the next tile's sums may be written
             if (MODE == FEW_STORE) {
-                const int sg = seg_of(tile), o = (tile - p.tile0[sg]) * 16 + f;
+                const int sg = seg_of(tile), o = ((tile - p.tile0[sg]) * TM + sub) * 16 + f;
                 if (r < min(p.rows[sg], p.R) && o < p.n_out[sg]) p.Y[(size_t)r * p.ldy + p.col0[sg] + o] = rs_s[r] * v;
                 continue;
             }
-            fin[buf][r][f] = v;
+            fin[buf][sub][r][f] = v;
         }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (TM == 1 || sub == 0) asm volatile("bar.sync 1, 128;" ::: "memory");
+        else asm volatile("bar.sync 4, 128;" ::: "memory");
         if (MODE == FEW_RESID) {
-            const int o = tile * 16 + ef;
+            const int o = (tile * TM + sub) * 16 + ef;
             const bool on = er < p.R && o < p.d;
             float s = 0.f;
             if (on) {
-                s = s_old + fin[buf][er][ef];
-                if (er >= p.Bc && p.coup) s += cp * fin[buf][er % p.Bc][ef];
+                s = s_old + fin[buf][sub][er][ef];
+                if (er >= p.Bc && p.coup) s += cp * fin[buf][sub][er % p.Bc][ef];
                 p.S[(size_t)er * p.d + o] = s;
                 store_split(p.Xn, (size_t)er * p.d + o, p.xn_lo, gn * s);
             }
             float q = s * s;
 #pragma unroll
             for (int i = 8; i > 0; i >>= 1) q += __shfl_xor_sync(0xffffffffu, q, i);
-            if (ef == 0) p.ss_out[(size_t)tile * kFewRows + er] = q;
+            if (ef == 0) p.ss_out[(size_t)(tile * TM + sub) * kFewRows + er] = q;
             if (next < p.tiles) {
                 load_vecs(next);
                 load_s(next);
             }
         } else {
-            const int o = tile * 8 + ef;
+            const int o = (tile * TM + sub) * 8 + ef;
             if (er < p.R && o < p.F) {
                 const float rs = rs_s[er];
-                float h = silu(rs * fin[buf][er][ef]) * (rs * fin[buf][er][8 + ef]);
+                float h = silu(rs * fin[buf][sub][er][ef]) * (rs * fin[buf][sub][er][8 + ef]);
                 if (er >= p.Bc && p.coup) {
                     const int b = er % p.Bc;
-                    h += cp * (silu(rs_s[b] * fin[buf][b][ef]) * (rs_s[b] * fin[buf][b][8 + ef]));
+                    h += cp * (silu(rs_s[b] * fin[buf][sub][b][ef]) * (rs_s[b] * fin[buf][sub][b][8 + ef]));
                 }
                 store_split(p.H, (size_t)er * p.F + o, p.h_lo, h);
             }
