@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
     float ca00 = 0.f, ca01 = 0.f;
     int page0 = 0;
     // (Not in the deep form: there it gained 0.5 % at 16 sequences of 2048 and lost 1 % at 8000.)
-    const bool ahead = !DEEP && use_plan && p.plan_prewait && p.qkv_P != nullptr;
+    const bool ahead = NARROW && !DEEP && use_plan && p.plan_prewait && p.qkv_P != nullptr;
     if (ahead && warp < kAttWarps) {
         constexpr int half = DH / 2;
         int item, nkeys, g, seg, n, ui, t0, t1;
@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 const size_t offs[4] = {p1 + o0, p1 + o1, p2 + o0, p2 + o1};
                 float sm[4] = {0.f, 0.f, 0.f, 0.f};
                 if (act) {
-                    if (p.qkv_nsplit == 1) {  // (finished sums: the code of the general form alone is a microsecond of instruction misses)
+                    if (NARROW && p.qkv_nsplit == 1) {  // (finished sums: the code of the general form alone is a microsecond of instruction misses)
 #pragma unroll
                         for (int k = 0; k < 4; k++) sm[k] = __ldcg(p.qkv_P + offs[k]);
                     } else {
@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                     if (do_kv) {  // K_1 and V_1 of this step's token for this KV head (tid = rotation pair)
                         size_t ko = p1 + q_dim + (size_t)g * DH + tid, vo = ko + kv_dim;
                         const size_t koffs[4] = {ko, ko + half, vo, vo + half};
-                        if (p.qkv_nsplit == 1) {
+                        if (NARROW && p.qkv_nsplit == 1) {
 #pragma unroll
                             for (int k = 0; k < 4; k++) kvs[k] = __ldcg(p.qkv_P + koffs[k]);
                         } else {
