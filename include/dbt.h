@@ -146,7 +146,8 @@ dbt_status dbt_prefill(dbt_model *m, const int32_t *tokens_dev, int32_t B, int32
  * (tokens_dev DEVICE int32 [B][S], sequences 0..B-1 from their current lengths), and the continuation boundary
  * -- one branch evaluation at the final prompt token, coupled to the primary's Q_1, H_1, M_1 of that position
  * and read against the completed cache -- predicts x_{S+1} from the mixture.  Outputs as dbt_decode_step.
- * How it runs: positions 1..S-1 as the prompt-wide prefill, position S as one grouped step.  The boundary
+ * How it runs: positions 1..S-1 as the prompt-wide prefill, position S as one grouped step, whose rows go
+ * through the GEMMs of the last prompt chunk where they fit its row tiles (dense bf16 models).  The boundary
  * evaluation has to stream every shared matrix once for the branch row anyway; letting the primary row of
  * position S ride in that same pass produces the "retained intermediates" where they are consumed, costs no
  * extra memory traffic and needs no per-layer retention buffers.  The values are those of the paper's form

@@ -143,6 +143,8 @@ struct dbt_model {
     int tok_stride = 1, tok_p0 = 0;
     int clusters_at_once[4] = {74, 33, 22, 15};  // clusters of 2, 4, 6, 8 CTAs of a paired-SM GEMM resident at a time (count_clusters)
     bool cluster16 = false;    // clusters of 16 CTAs can run here (see small_cluster)
+    RideRows ride{};    // inside dbt_prefill_boundary: the boundary step's rows that rode in the last chunk (see ride_rows)
+    int step_l0 = 0;    // inside a decode step: its first layer (the others' work is done where its rows rode in a prompt chunk)
     int step_rows = 0;  // inside a decode step of step_tc: the stacked rows of all paths, whatever the mode (see plan_rows)
     bool att_planned = false;  // inside a decode step whose attention work split has been computed (run_embed_wide)
 };
@@ -895,7 +897,7 @@ PgPlan plan_gemm_prompt(const dbt_model *m, PgMode mode, const int (&n_out)[3], 
     return best;
 }
 
-template <int N, int MODE>
+template <int N, int MODE, bool RIDE = false>
 dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0, const CUtensorMap *W1, const CUtensorMap *W2,
                               const int (&n_out)[3], int nseg, const CUtensorMap *X, int S, PgParams p) {
     constexpr int kTileF = MODE == PG_GATEUP ? N / 2 : N;
@@ -919,7 +921,7 @@ dbt_status launch_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *
     p.m_group = (p.m_tiles + groups - 1) / groups;
     p.status = m->ws.status;
     const int grid = S > 1 ? 2 * S * p.tiles : 2 * (p.tiles < pairs ? p.tiles : pairs);
-    LAUNCH_CLUSTER(m, tag, bytes, 2 * S, (gemm_prompt_kernel<N, MODE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *w[0], *w[1], *w[2], *x, p);
+    LAUNCH_CLUSTER(m, tag, bytes, 2 * S, (gemm_prompt_kernel<N, MODE, RIDE>), grid, kPgThreads, (PgCfg<N>::kSmemBytes), *w[0], *w[1], *w[2], *x, p);
     return DBT_OK;
 }
 
@@ -935,6 +937,13 @@ dbt_status run_gemm_prompt(dbt_model *m, const char *tag, const CUtensorMap *W0,
     for (int s = 0; s < nseg; s++) widest = n_out[s] > widest ? n_out[s] : widest;
     PgPlan pl = plan_gemm_prompt(m, MODE, n_out, nseg, K, plan_rows(m, R));
     if (shares) *shares = 2 * pl.splits * ((n_out[0] + pl.N - 1) / pl.N);
+    if constexpr (MODE == PG_QKV || MODE == PG_RESID || MODE == PG_GATEUP) {
+        if (p.ride.K > 0) {
+            if constexpr (MODE != PG_QKV)
+                if (pl.N == 192) return launch_gemm_prompt<192, MODE, true>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
+            return launch_gemm_prompt<256, MODE, true>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
+        }
+    }
     if constexpr (MODE == PG_STORE) {
         if (widest <= 64) return launch_gemm_prompt<64, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, 1, p);
         if (pl.N == 96) return launch_gemm_prompt<96, MODE>(m, tag, W0, W1, W2, n_out, nseg, X, pl.splits, p);
@@ -1131,7 +1140,8 @@ bool short_prompt(const dbt_model *m, const RowMap &rm) {
 
 template <int DH>
 dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int layer, double kv_bytes,
-                             const QkvFuse *qf = nullptr, bool pack_prompt = false, bool planned = false) {
+                             const QkvFuse *qf = nullptr, bool pack_prompt = false, bool planned = false, const RideRows *ride = nullptr,
+                             int ahead = 0) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
     int items = rm.B * rm.cn, G = c.n_q_heads / c.n_kv_heads;
@@ -1154,6 +1164,11 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
     p.lo_off = m->act_parts == 2 ? (size_t)m->Rmax * c.n_q_heads * c.head_dim : (size_t)0;
     p.status = w.status;
     p.evict_first = m->evict_first ? 1 : 0;
+    if (ride) {
+        p.Q = w.O;
+        p.ride = *ride;
+        p.ahead = ahead;
+    }
     if (qf) {
         p.qkv_P = qf->P;
         p.qkv_nsplit = qf->nsplit;
@@ -1186,6 +1201,7 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
         q.lo_off = p.lo_off;
         q.status = w.status;
         q.Q = prompt_q(m);
+        q.let_in_late = m->ride.K > 0;
         if (short_prompt(m, rm)) {
             q.nqb = (rm.cn + 128 / G - 1) / (128 / G);
             LAUNCH(m, "attention", kv_bytes, attn_prompt_short_kernel<DH>, dim3(rm.B * c.n_kv_heads * q.nqb), (kPsWarps + 1) * 32,
@@ -1204,8 +1220,8 @@ dbt_status run_attention_mma(dbt_model *m, const RowMap &rm, int grouped, int la
     }
     if (planned && !packed) {  // from the second layer on the plan may be read before the dependency wait
         p.plan = m->ws.att_plan;
-        p.plan_prewait = layer > 0 ? 1 : 0;
-        p.early = qf && qf->early && layer > 0 ? 1 : 0;
+        p.plan_prewait = layer > m->step_l0 ? 1 : 0;
+        p.early = qf && qf->early && layer > m->step_l0 ? 1 : 0;
     }
     if (!packed && items > kAttMaxItems) return fail(m, DBT_ERR_CAPACITY, "attention rows %d exceed %d", items, kAttMaxItems);
     dim3 grid(2 * m->num_sms);  // two resident CTAs per SM; each takes an equal share of all K/V tiles
@@ -1387,7 +1403,7 @@ dbt_status run_moe_tc(dbt_model *m, int l, const RowMap &rm, int grouped, bool r
 
 // Embeddings and the first layer's GEMM input; plan: also the attention work split of a decode step, once for all its layers.
 template <typename WT>
-dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0, const RowMap &rm, int R, bool plan, bool few = false) {
+dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0, const RowMap &rm, int R, bool plan, bool few = false, RideRows ride = RideRows{}) {
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
     const int items = rm.B * rm.cn;
@@ -1396,7 +1412,7 @@ dbt_status run_embed_wide(dbt_model *m, const int32_t *tokens_dev, int n, int p0
            (const WT *)m->w.embed_branch, m->w.embed_norm_g, c.rms_eps, c.d_model, c.vocab, w.S,
            m->layers[0].attn_norm_g, w.Xb, m->act_parts == 2 ? (size_t)m->Rmax * c.d_model : (size_t)0, w.ss,
            few ? kFewRows : m->Rmax, few ? (c.d_model + 15) / 16 : (c.d_model + 255) / 256, w.status, w.seq_len, c.n_kv_heads, attn_deep(m, items) ? m->num_sms : 2 * m->num_sms,
-           plan ? w.att_plan : (int32_t *)nullptr, few ? 1 : 0);
+           plan ? w.att_plan : (int32_t *)nullptr, few ? 1 : 0, ride);
     m->att_planned = plan;  // cleared by the step function when its layers have been enqueued
     return DBT_OK;
 }
@@ -1582,7 +1598,7 @@ dbt_status run_layers_wide(dbt_model *m, const RowMap &rm, int grouped, int n_ti
         t.parts = m->act_parts; t.lo_row0 = m->Rmax;
         return t;
     };
-    for (int l = 0; l < c.n_layers; l++) {
+    for (int l = m->step_l0; l < c.n_layers; l++) {
         const dbt_layer_weights &lw = m->layers[l];
         const LayerMaps &mp = m->maps[l];
         WT *kpool = reinterpret_cast<WT *>(m->kv_pool) + (size_t)l * pool_layer_elems;
@@ -1685,7 +1701,7 @@ dbt_status run_few(dbt_model *m, const char *tag, int B, const CUtensorMap *W0, 
 }
 
 // The layer stack and the shared output matrix: five kernels per layer.
-dbt_status run_layers_few(dbt_model *m, const RowMap &rm, int grouped) {
+dbt_status run_layers_few(dbt_model *m, const RowMap &rm, int grouped) {  // (from layer m->step_l0 on)
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
@@ -1703,7 +1719,7 @@ dbt_status run_layers_few(dbt_model *m, const RowMap &rm, int grouped) {
     auto resid = [&](FewParams &p, const float *g_next, const float *coup) {
         p.S = w.S; p.g_next = g_next; p.coup = coup; p.Xn = w.Xb; p.xn_lo = (size_t)m->Rmax * d; p.ss_out = w.ss;
     };
-    for (int l = 0; l < c.n_layers; l++) {
+    for (int l = m->step_l0; l < c.n_layers; l++) {
         const dbt_layer_weights &lw = m->layers[l];
         const LayerMaps &mp = m->maps[l];
         FewParams q = lin(qd, d);
@@ -1735,6 +1751,24 @@ dbt_status run_layers_few(dbt_model *m, const RowMap &rm, int grouped) {
 
 // ---- prompt chunks of dense bf16 models -------------------------------------------------------------
 
+// The boundary step's K*B rows behind the `own` rows of the last prompt chunk, where they ride in its GEMMs: they stand in groups of
+// 32 and must not open another row tile of 256 (which costs a large chunk more than the step it saves).  All that is left of the
+// boundary step is then an attention launch per layer beside the chunk's own, the last layer and the readout.
+// prefill_boundary, the step by itself / riding, us: 1B, one prompt of 150 / 333 / 700 / 2000 tokens 2285 / 1790, 2521 / 2106, 3292 / 2824,
+// 6120 / 5450; four of 100 2481 / 2034; 200 behind 500 2448 / 1985; 8B, 333 / 3000 15050 / 12650, 70800 / 68000.
+RideRows ride_rows(const dbt_model *m, int B, int own) {
+    RideRows r{};
+    const int K = paths_of(m->cfg), spg = 32 / K, row0 = (own + 31) / 32 * 32, end = row0 + (B + spg - 1) / spg * 32;
+    if (!m->prompt_attn_tc || m->cfg.n_layers < 2 || end > m->Rmax || (end + kPgM - 1) / kPgM != (own + kPgM - 1) / kPgM) return r;
+    r.row0 = row0;
+    r.spg = spg;
+    r.K = K;
+    r.B = B;
+    return r;
+}
+// Rows of a chunk's GEMMs: its own, and the groups that ride behind them.
+int ride_end(const dbt_model *m, int own) { return m->ride.K > 0 ? m->ride.row0 + (m->ride.B + m->ride.spg - 1) / m->ride.spg * 32 : own; }
+
 // One chunk of a prompt through all layers: five kernels per layer, one in the last: nobody reads the chunk's outputs, so that layer
 // is done when its keys and values are in the cache (16 prompts of 2048 into the 1B model 86.1 -> 81.5 ms, 32 of 1024 into the MoE
 // model 83.1 -> 78.2, one of 8192 into the 8B shape 191.0 -> 186.2).
@@ -1742,7 +1776,16 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
-    const int R = rm.B * rm.cn, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ff;
+    const int own = rm.B * rm.cn, d = c.d_model, qd = c.n_q_heads * c.head_dim, kvd = c.n_kv_heads * c.head_dim, F = c.d_ff;
+    const RideRows ride = m->ride;  // (the rows that go through all but the last layer with the chunk)
+    const int R = ride_end(m, own);
+    auto riding = [&](PgParams p, const float *coup) {
+        p.ride = ride;
+        p.own = own;
+        p.ride_coup = coup;
+        p.ride_q = w.O;
+        return p;
+    };
     const size_t lo_h = (size_t)m->Rmax * F;
     double kv_bytes = 0;
     for (int b = 0; b < rm.B; b++)
@@ -1755,21 +1798,28 @@ dbt_status run_layers_prompt(dbt_model *m, const RowMap &rm) {
         PgParams q = prompt_qkv_params(m, rm, l, ss_tiles);
         if (l + 1 == c.n_layers) {
             q.first = 1;
-            return run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wk, &mp.wv, nullptr, {kvd, kvd, 0}, 2, &m->map_Xb, d, R, q);
+            return run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wk, &mp.wv, nullptr, {kvd, kvd, 0}, 2, &m->map_Xb, d, own, q);
         }
-        if ((st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, R, q)) != DBT_OK) return st;
+        if ((st = run_gemm_prompt<PG_QKV>(m, "gemm_qkv", &mp.wq, &mp.wk, &mp.wv, {qd, kvd, kvd}, 3, &m->map_Xb, d, R, riding(q, lw.coup_a))) != DBT_OK) return st;
         st = c.head_dim == 128 ? run_attention_mma<128>(m, rm, 0, l, kv_bytes, nullptr, true, false)
                                : run_attention_mma<64>(m, rm, 0, l, kv_bytes, nullptr, true, false);
         if (st != DBT_OK) return st;
-        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R, prompt_resid_params(m, lw.mlp_norm_g), &ss_tiles)) != DBT_OK)
+        if (ride.K > 0) {
+            const RowMap step{rm.B, 1};
+            st = c.head_dim == 128 ? run_attention_mma<128>(m, step, ride.K, l, kv_bytes, nullptr, false, false, &ride, rm.cn)
+                                   : run_attention_mma<64>(m, step, ride.K, l, kv_bytes, nullptr, false, false, &ride, rm.cn);
+            if (st != DBT_OK) return st;
+        }
+        if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_o", &mp.wo, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Ob, qd, R,
+                                            riding(prompt_resid_params(m, lw.mlp_norm_g), nullptr), &ss_tiles)) != DBT_OK)
             return st;
         PgParams g{};
         g.ss_in = w.ss; g.ss_tiles = ss_tiles; g.ss_ld = m->Rmax; g.d_norm = d; g.eps = c.rms_eps;
         g.H = w.Hb; g.h_lo = lo_h; g.F = F;
-        st = run_gemm_prompt<PG_GATEUP>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, 0, 0}, 1, &m->map_Xb, d, R, g);
+        st = run_gemm_prompt<PG_GATEUP>(m, "gemm_gateup", &mp.wg, &mp.wu, nullptr, {F, 0, 0}, 1, &m->map_Xb, d, R, riding(g, lw.coup_b));
         if (st != DBT_OK) return st;
         if ((st = run_gemm_prompt<PG_RESID>(m, "gemm_down", &mp.wd, nullptr, nullptr, {d, 0, 0}, 1, &m->map_Hb, F, R,
-                                            prompt_resid_params(m, m->layers[l + 1].attn_norm_g), &ss_tiles)) != DBT_OK)
+                                            riding(prompt_resid_params(m, m->layers[l + 1].attn_norm_g), lw.coup_c), &ss_tiles)) != DBT_OK)
             return st;
     }
     return DBT_OK;
@@ -1873,9 +1923,22 @@ dbt_status step_wide(dbt_model *m, const int32_t *tokens_dev, int B, int grouped
     int R = npaths(grouped) * B, n_tile = pad_rows(paths_of(c) * B);
     dbt_status st;
     const bool few = few_step(m, B);
-    if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, true, few)) != DBT_OK) return st;
+    if (m->ride.K > 0) {  // its rows went through all layers but the last with the prompt's last chunk
+        const Workspace &w = m->ws;
+        const RideRows ride = m->ride;
+        m->ride = RideRows{};
+        const int d = c.d_model;
+        m->step_l0 = c.n_layers - 1;
+        LAUNCH(m, "embed", 0, ride_take_kernel, R + 1, 256, 0, ride, w.S, m->layers[m->step_l0].attn_norm_g, d, w.Xb, (size_t)m->Rmax * d, w.ss,
+               few ? kFewRows : m->Rmax, few ? (d + 15) / 16 : wide_ss_tiles(m), w.seq_len, c.n_kv_heads,
+               attn_deep(m, B) ? m->num_sms : 2 * m->num_sms, w.att_plan, few ? 1 : 0);
+        m->att_planned = true;
+    } else if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride, m->tok_p0, rm, R, true, few)) != DBT_OK) {
+        return st;
+    }
     st = few ? run_layers_few(m, rm, grouped) : run_layers_wide(m, rm, grouped, n_tile);
     m->att_planned = false;
+    m->step_l0 = 0;
     if (st != DBT_OK) return st;
     if (!few && (st = run_head_wide(m, rm, grouped, n_tile)) != DBT_OK) return st;
     // the readout also bumps the sequence lengths: nothing after it in the step reads them
@@ -1924,7 +1987,8 @@ dbt_status prefill_tc(dbt_model *m, const int32_t *tokens_dev, int B, int n, flo
     return DBT_OK;
 }
 
-dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, float *last_logits) {
+// boundary: a boundary step on the position behind the prompt follows (dbt_prefill_boundary); m->ride says whether its rows rode along.
+dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, float *last_logits, bool boundary) {
     typedef __nv_bfloat16 WT;
     const dbt_config &c = m->cfg;
     const Workspace &w = m->ws;
@@ -1938,9 +2002,10 @@ dbt_status prefill_wide(dbt_model *m, const int32_t *tokens_dev, int B, int n, f
         int cn = p0 < n_bulk ? (n_bulk - p0 < cn_max ? n_bulk - p0 : cn_max) : 1;
         RowMap rm{B, cn};
         int R = B * cn, n_tile = pad_rows(R < 256 ? R : 256);
-        if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, R, false)) != DBT_OK) return st;
         // (measured on the 1B model: 128 rows 7 % slower than the decode step's kernels, 199 rows 23 % faster)
         const bool pairs = cn > 1 && R > 128;
+        if (boundary && pairs && p0 + cn >= n) m->ride = ride_rows(m, B, R);
+        if ((st = run_embed_wide<WT>(m, tokens_dev, m->tok_stride > 1 ? m->tok_stride : n, p0, rm, ride_end(m, R), false, false, m->ride)) != DBT_OK) return st;
         const bool head = last_logits && p0 + cn >= n;
         if ((st = pairs ? run_layers_prompt(m, rm) : run_layers_wide(m, rm, 0, n_tile, !head)) != DBT_OK) return st;
         if (head) {
@@ -1968,13 +2033,14 @@ bool allow_smem_all() {
                cudaSuccess;
 }
 
-template <int N, int MODE>
+template <int N, int MODE, bool RIDE = false>
 bool allow_smem_pg() {
-    return cudaFuncSetAttribute(gemm_prompt_kernel<N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PgCfg<N>::kSmemBytes) == cudaSuccess;
+    return cudaFuncSetAttribute(gemm_prompt_kernel<N, MODE, RIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, PgCfg<N>::kSmemBytes) == cudaSuccess;
 }
 bool allow_smem_prompt() {
     return allow_smem_pg<256, PG_QKV>() && allow_smem_pg<256, PG_RESID>() && allow_smem_pg<256, PG_GATEUP>() &&
-           allow_smem_pg<192, PG_GATEUP>() && allow_smem_pg<256, PG_COMBINE>() && allow_smem_pg<64, PG_STORE>() &&
+           allow_smem_pg<256, PG_QKV, true>() && allow_smem_pg<256, PG_RESID, true>() && allow_smem_pg<192, PG_RESID, true>() &&
+           allow_smem_pg<256, PG_GATEUP, true>() && allow_smem_pg<192, PG_GATEUP, true>() && allow_smem_pg<192, PG_GATEUP>() && allow_smem_pg<256, PG_COMBINE>() && allow_smem_pg<64, PG_STORE>() &&
            allow_smem_pg<96, PG_STORE>() && allow_smem_pg<192, PG_RESID>() && allow_smem_pg<128, PG_STORE>() && allow_smem_pg<192, PG_STORE>() && allow_smem_pg<256, PG_STORE>() &&
            cudaFuncSetAttribute(gemm_group_kernel<GG_GATEUP>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess &&
            cudaFuncSetAttribute(gemm_group_kernel<GG_DOWN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGgSmemBytes) == cudaSuccess;
@@ -2490,7 +2556,7 @@ dbt_status dbt_prefill(dbt_model *m, const int32_t *tokens_dev, int32_t B, int32
     dbt_status st = check_step_args(m, tokens_dev, B, n);
     if (st != DBT_OK) return st;
     if (m->cfg.weight_dtype == DBT_DTYPE_F32) return prefill_impl<float>(m, tokens_dev, B, n, last_primary_logits_dev);
-    if (m->wide) return prefill_wide(m, tokens_dev, B, n, last_primary_logits_dev);
+    if (m->wide) return prefill_wide(m, tokens_dev, B, n, last_primary_logits_dev, false);
     if (m->tc) return prefill_tc(m, tokens_dev, B, n, last_primary_logits_dev, false);
     return prefill_impl<__nv_bfloat16>(m, tokens_dev, B, n, last_primary_logits_dev);
 }
@@ -2571,11 +2637,14 @@ dbt_status dbt_prefill_boundary(dbt_model *m, const int32_t *tokens_dev, int32_t
         // positions 1..S-1 of every row of tokens_dev [B][S]: the prompt-wide prefill walks rows of stride S
         m->tok_stride = S;
         st = m->cfg.weight_dtype == DBT_DTYPE_F32 ? prefill_impl<float>(m, tokens_dev, B, S - 1, nullptr)
-             : m->wide                             ? prefill_wide(m, tokens_dev, B, S - 1, nullptr)
+             : m->wide                             ? prefill_wide(m, tokens_dev, B, S - 1, nullptr, true)
              : m->tc                               ? prefill_tc(m, tokens_dev, B, S - 1, nullptr, true)
                                                    : prefill_impl<__nv_bfloat16>(m, tokens_dev, B, S - 1, nullptr);
         m->tok_stride = 1;
-        if (st != DBT_OK) return st;
+        if (st != DBT_OK) {
+            m->ride = RideRows{};
+            return st;
+        }
     }
     // position S: the primary's step and the branch's boundary evaluation in one grouped pass (launched
     // directly: the token addressing differs from a decode step's, so the captured graphs do not apply)
@@ -2584,6 +2653,8 @@ dbt_status dbt_prefill_boundary(dbt_model *m, const int32_t *tokens_dev, int32_t
     st = step_direct(m, tokens_dev, B, paths_of(m->cfg), next_tokens_dev, logits_primary_dev, logits_branch_dev, alpha_dev);
     m->tok_stride = 1;
     m->tok_p0 = 0;
+    m->step_l0 = 0;
+    m->ride = RideRows{};
     return st;
 }
 

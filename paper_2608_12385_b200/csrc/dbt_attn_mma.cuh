@@ -33,6 +33,7 @@
 
 #include "dbt_fused.cuh"
 #include "dbt_gemm_tc.cuh"
+#include "dbt_gemm_prompt.cuh"
 
 namespace dbt {
 
@@ -68,6 +69,11 @@ struct AttnParams {
     // limit; a chunk holds cn positions per sequence, nbk = ceil(cn / pack) tiles per sequence, one CTA pass per
     // (tile, KV head) over all its keys, no split.  Q rows and output rows are seq * cn + position.
     int pack, cn, nbk;
+    // Rows of a boundary step that ride behind a prompt chunk (ride.K > 0; K rows per sequence, path-major queries in Q): they see
+    // `ahead` positions more than seq_len says, the chunk's, and their outputs go to their places in the chunk.  The launch
+    // starts beside the chunk's own attention (whose CTAs let it in behind their wait) and waits for that one at its end.
+    RideRows ride;
+    int ahead;
     const int *plan;   // the step's precomputed work split (embed_fused_kernel), or nullptr
     int plan_prewait;  // the plan may be read before the dependency wait
     // The producer does not wait for the kernel before (with plan_prewait): the pages it reads were written by earlier steps, which
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens,
                                                           float *S, const float *__restrict__ g_next,
                                                           __nv_bfloat16 *Xb, size_t lo_off, float *ss_out, int ss_ld,
                                                           int ss_tiles, int *status, const int32_t *seq_len, int n_kv, int C0, int *plan,
-                                                          int barrier) {
+                                                          int barrier, RideRows ride) {
     // barrier: the kernels of this step may rely on all earlier steps being complete, also before their own waits
     if (!barrier) pdl_launch_dependents();
     pdl_wait();
@@ -299,7 +305,12 @@ __global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens,
         return;
     }
     int path = r / rm.Bc();  // 0 primary; j >= 1: decode branch j with its own table E2[j-1] (Appendix C.1)
-    int tok = ld_mut(tokens + (size_t)rm.seq(r) * n + p0 + rm.off(r));
+    int seq = rm.seq(r), off = rm.off(r);
+    if (ride.K > 0 && r >= rm.Bc()) {  // behind a prompt chunk: the boundary step's rows, and rows of no sequence between
+        if (r < ride.row0 || !ride.locate(r, path, seq)) return;
+        off = rm.cn;
+    }
+    int tok = ld_mut(tokens + (size_t)seq * n + p0 + off);
     if (tok < 0 || tok >= V) {
         if (threadIdx.x == 0) report(status, kStatusBadToken, tok);
         tok = min(max(tok, 0), V - 1);
@@ -317,6 +328,31 @@ __global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens,
         S[(size_t)r * d + i] = s0;
         store_split(Xb, (size_t)r * d + i, lo_off, g_next[i] * s0);
         sq += s0 * s0;
+    }
+    sq = block_sum(sq, scratch);
+    for (int t = threadIdx.x; t < ss_tiles; t += blockDim.x) ss_out[(size_t)t * ss_ld + r] = t == 0 ? sq : 0.f;
+}
+
+// Boundary step behind a chunk that its rows rode in: they leave for the decode kernels' places (path-major), with the last layer's
+// input g * S and sum(S^2) as embed_fused_kernel leaves them; one more block computes the step's attention work split.
+__global__ void __launch_bounds__(256) ride_take_kernel(RideRows ride, float *S, const float *__restrict__ g, int d, __nv_bfloat16 *Xb, size_t lo_off,
+                                                        float *ss_out, int ss_ld, int ss_tiles, const int32_t *seq_len, int n_kv, int C0,
+                                                        int *plan, int early) {
+    pdl_wait();
+    pdl_launch_dependents();  // (behind the wait: see AttnParams::early)
+    __shared__ float scratch[32];
+    const int r = blockIdx.x;
+    if (r == (int)gridDim.x - 1) {
+        att_plan_block(ride.B, seq_len, n_kv, C0, early != 0, plan);
+        return;
+    }
+    const float *src = S + (size_t)ride.row(r / ride.B, r % ride.B) * d;
+    float sq = 0.f;
+    for (int i = threadIdx.x; i < d; i += blockDim.x) {
+        const float x = __ldcg(src + i);
+        S[(size_t)r * d + i] = x;
+        store_split(Xb, (size_t)r * d + i, lo_off, g[i] * x);
+        sq += x * x;
     }
     sq = block_sum(sq, scratch);
     for (int t = threadIdx.x; t < ss_tiles; t += blockDim.x) ss_out[(size_t)t * ss_ld + r] = t == 0 ? sq : 0.f;
@@ -367,8 +403,10 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
     // A decode step's work split comes precomputed (the same for all its layers).  From the second layer on
     // it is read before the dependency wait: the kernel that wrote it finished long before any kernel that
     // could still be running now; in the first layer that kernel may still be running, so the wait comes first.
-    const bool use_plan = p.plan != nullptr && !packed;
-    if (!(use_plan && p.plan_prewait)) pdl_wait();  // sequence lengths, Q and the freshly appended K/V come from earlier kernels of the step
+    const bool use_plan = p.plan != nullptr && !packed, riding = p.ride.K > 0;
+    // output row of a path of an item
+    auto out_row = [&](int path, int item) { return riding ? p.ride.row(path, item) : path * Bc + item; };
+    if (!riding && !(use_plan && p.plan_prewait)) pdl_wait();  // sequence lengths, Q and the freshly appended K/V come from earlier kernels of the step
     if (use_plan) {
         if (!p.plan_prewait) pdl_wait();
         for (int i = tid; i <= items; i += blockDim.x) {
@@ -378,7 +416,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         }
     } else if (warp == 0 && !packed) {
         for (int i = lane; i < items; i += 32)
-            nk_s[i] = (unsigned)(ld_mut(p.seq_len + p.rm.seq(i)) + p.rm.off(i) + 1) | (unsigned)i << 24;
+            nk_s[i] = (unsigned)(ld_mut(p.seq_len + p.rm.seq(i)) + p.rm.off(i) + 1 + p.ahead) | (unsigned)i << 24;
         __syncwarp();
         att_plan_warp(lane, items, p.n_kv, (int)gridDim.x, kAttMinUnits, cum, nk_s, segcum);
     }
@@ -845,7 +883,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                         if (q < nq_act) {
                             if (nseg == 1) {
                                 // the pair's only segment: normalise and write the head's output
-                                int row = packed ? item_row0(item) + q / p.G : (q / p.G) * Bc + item;
+                                int row = packed ? item_row0(item) + q / p.G : out_row(q / p.G, item);
                                 int hq = g * p.G + q % p.G;
                                 size_t ob = (size_t)row * q_dim + (size_t)hq * DH;
                                 float inv = 1.f / l_run[h];
@@ -1038,7 +1076,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                     }
                     if (nseg == 1) {
                         // the pair's only segment: normalise and write the head's output
-                        const int row = (q / p.G) * Bc + item, hq = g * p.G + q % p.G;
+                        const int row = out_row(q / p.G, item), hq = g * p.G + q % p.G;
                         const float inv = 1.f / L;
                         store_split4(p.Ob, (size_t)row * q_dim + (size_t)hq * DH + e, p.lo_off, make_float4(X.x * inv, X.y * inv, X.z * inv, X.w * inv));
                     } else {
@@ -1122,7 +1160,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 for (int a = 0; a < A; a++) {
                     if (!act[a]) continue;
                     if (final) {
-                        const int row = packed ? item_row0(item) + qq[a] / p.G : (qq[a] / p.G) * Bc + item;
+                        const int row = packed ? item_row0(item) + qq[a] / p.G : out_row(qq[a] / p.G, item);
                         const int h = g * p.G + qq[a] % p.G;
                         store_split4(p.Ob, (size_t)row * q_dim + (size_t)h * DH + ee[a], p.lo_off,
                                      make_float4(X[a].x / L[a], X[a].y / L[a], X[a].z / L[a], X[a].w / L[a]));
@@ -1178,6 +1216,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         }
         if (round == 0) DBT_TL_MARK(2);
     }
+    if (riding) pdl_wait();
 #ifdef DBT_TL_ATT_ALL
     {  // every CTA leaves a record: mark 3 carries (SM id << 16 | block index)
         unsigned smid;

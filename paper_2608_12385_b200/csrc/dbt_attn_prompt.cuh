@@ -32,6 +32,7 @@ struct PromptAttnParams {
     __nv_bfloat16 *Ob;  // [B * cn][q_dim] attention output, hi plane (+ lo plane at lo_off)
     size_t lo_off;
     int *status;
+    int let_in_late;  // the next launch starts behind this one's wait: it reads what the kernel before wrote without a wait of its own
     int nqb;  // query blocks per sequence: ceil(cn / (256 / G)); attn_prompt_short_kernel: ceil(cn / (128 / G))
 };
 
@@ -154,8 +155,9 @@ __global__ void __launch_bounds__(kPaThreads, 1) attn_prompt_kernel(const __grid
     const uint32_t tmem = *tmem_holder;
     auto t_s = [&](int i) { return tmem + 128u * i; };
     auto t_o = [&](int i) { return tmem + 256u + (uint32_t)DH * i; };
-    pdl_launch_dependents();
+    if (!p.let_in_late) pdl_launch_dependents();
     pdl_wait();  // the chunk's Q rows and its K, V rows in the cache come from the kernel before
+    if (p.let_in_late) pdl_launch_dependents();
 
     const int len0 = ld_mut(p.seq_len + b);
     const int c0 = jb * PB;

@@ -50,6 +50,21 @@ struct PgSeg {
     int col0;   // PG_STORE: its first column of P
 };
 
+// Rows of the boundary step that ride behind a chunk's own rows (RIDE): sequence b's K rows -- the primary's and its branches' at the
+// position behind the chunk -- stand in one group of 32, row row0 + b / spg * 32 + path * spg + b % spg, so that one warp of an
+// epilogue holds them and a branch reaches its primary row by a shuffle.
+struct RideRows {
+    int row0, spg, K, B;  // (K == 0: none)
+    __host__ __device__ int row(int path, int b) const { return row0 + b / spg * 32 + path * spg + b % spg; }
+    // the path and the sequence of a row; false: a row of no sequence
+    __device__ bool locate(int r, int &path, int &b) const {
+        const int q = r - row0, l = q & 31;
+        path = l / spg;
+        b = (q >> 5) * spg + l % spg;
+        return path < K && b < B;
+    }
+};
+
 struct PgParams {
     int K, R, m_tiles, tiles;  // tiles: m_tiles x feature tiles
     // Order of the tiles: groups of m_group row tiles, in a group feature tile by feature tile.  The pairs that run at
@@ -92,6 +107,11 @@ struct PgParams {
     const float2 *rope;
     const int32_t *seq_len, *page_table;
     __nv_bfloat16 *kpool, *vpool;
+    // RIDE: R counts the riding rows, `own` the chunk's
+    RideRows ride;
+    int own;
+    const float *ride_coup;  // a, b or c (nullptr: no coupling)
+    float *ride_q;           // PG_QKV: their queries, fp32, [path * B + sequence][q_dim]
 };
 
 template <int N>
@@ -217,7 +237,7 @@ __device__ __forceinline__ void store16(__nv_bfloat16 *dst, const float *x) {
                                                              pack2(x[8 * i + 4], x[8 * i + 5]), pack2(x[8 * i + 6], x[8 * i + 7]));
 }
 
-template <int N, int MODE>
+template <int N, int MODE, bool RIDE = false>
 __global__ void __launch_bounds__(kPgThreads, 1)
 gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1,
                    const __grid_constant__ CUtensorMap tmW2, const __grid_constant__ CUtensorMap tmX, const PgParams p) {
@@ -385,7 +405,19 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
             tile_of(t, mt, nt);
             const int sg = seg_of(nt), f0 = (nt - p.seg[sg].tile0) * kTileF;
             const int row0 = mt * kPgM + (int)rank * 128 + quad * 32, row = row0 + lane;
-            const bool on = row < p.R;
+            // riding rows: this warp's 32 rows are a group of them; the lane's path and sequence, the lane of its primary row
+            const bool rides = RIDE && p.ride.K > 0 && row0 >= p.ride.row0;
+            int path = 0, rb = 0;
+            const bool on = !RIDE ? row < p.R : rides ? p.ride.locate(row, path, rb) : row < p.own;
+            const int twin = rides ? lane % p.ride.spg : lane;
+            // adds coup[f + i] times the primary row's value to a branch row's, of sixteen features
+            auto couple = [&](float *x, int f, int n_feat) {
+#pragma unroll
+                for (int i = 0; i < 16; i++) {
+                    const float y = __shfl_sync(0xffffffffu, x[i], twin), a = f + i < n_feat ? p.ride_coup[f + i] : 0.f;
+                    if (path > 0) x[i] = fmaf(a, y, x[i]);
+                }
+            };
             float rs = 1.f;
             if (MODE == PG_QKV || MODE == PG_GATEUP || MODE == PG_STORE)
                 rs = row_scale(p.ss_in, p.ss_tiles, p.ss_ld, on ? row : 0, p.d_norm, p.eps);
@@ -500,6 +532,12 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         add_peers(v[0], cbase + c);
                         add_peers(v[1], cbase + c + 16);
                     }
+                    if constexpr (RIDE && MODE == PG_RESID) {
+                        if (rides && p.ride_coup) {
+#pragma unroll
+                            for (int h = 0; h < 2; h++) couple(reinterpret_cast<float *>(v[h]), f0 + cbase + c + 16 * h, p.seg[sg].n_out);
+                        }
+                    }
 #pragma unroll
                     for (int j = 0; j < 8; j++) {
                         float4 x = make_float4(rs * __uint_as_float(v[j >> 2][(j & 3) * 4]), rs * __uint_as_float(v[j >> 2][(j & 3) * 4 + 1]),
@@ -581,6 +619,8 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                     float h[16];
 #pragma unroll
                     for (int i = 0; i < 16; i++) h[i] = silu(rs * __uint_as_float(vg[i])) * (rs * __uint_as_float(vu[i]));
+                    if constexpr (RIDE)
+                        if (rides) couple(h, f0 + fbase + c, p.F);
 #pragma unroll
                     for (int q = 0; q < 2; q++) {  // F % 8 == 0: pieces of eight features are whole
                         const int f = f0 + fbase + c + q * 8;
@@ -599,9 +639,9 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                 // first and the second half of every head's rotation pairs (i, i + dh / 2)
                 const int hd = p.dh, hh2 = hd >> 1, span = hd >> 2, mat = sg + p.first;
                 const int nh = mat == 0 ? p.n_q : p.n_kv;
-                const int b = on ? row / p.cn : 0, pos = ld_mut(p.seq_len + b) + (on ? row % p.cn : 0);
+                const int b = !on ? 0 : rides ? rb : row / p.cn, pos = ld_mut(p.seq_len + b) + (!on ? 0 : rides ? p.cn : row % p.cn);
                 __nv_bfloat16 *kv = nullptr;
-                if (mat != 0 && on) {
+                if (mat != 0 && on && path == 0) {
                     const int page = p.page_table[(size_t)b * p.pt_stride + (pos >> 4)];
                     if (page < 0 || page >= p.num_pages) {
                         report(p.status, kStatusBadPage, page);
@@ -645,6 +685,20 @@ gemm_prompt_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_consta
                         }
                         if (head >= nh) continue;
                         if (mat == 0) {
+                            if constexpr (RIDE)
+                                if (rides) {  // Q~_j = Q_j + a * Q_1
+                                    couple(x0, head * hd + i0, p.n_q * hd);
+                                    couple(x1, head * hd + hh2 + i0, p.n_q * hd);
+                                    if (on) {
+                                        float *q0 = p.ride_q + ((size_t)path * p.ride.B + rb) * p.n_q * hd + (size_t)head * hd + i0;
+#pragma unroll
+                                        for (int i = 0; i < 4; i++) {
+                                            *reinterpret_cast<float4 *>(q0 + 4 * i) = make_float4(x0[4 * i], x0[4 * i + 1], x0[4 * i + 2], x0[4 * i + 3]);
+                                            *reinterpret_cast<float4 *>(q0 + hh2 + 4 * i) = make_float4(x1[4 * i], x1[4 * i + 1], x1[4 * i + 2], x1[4 * i + 3]);
+                                        }
+                                    }
+                                    continue;
+                                }
                             if (on && p.Qb) {
                                 __nv_bfloat16 *q0 = p.Qb + (size_t)row * p.n_q * hd + (size_t)head * hd + i0;
 #pragma unroll

@@ -207,3 +207,42 @@ def test_prompts_whose_outputs_nobody_reads_fill_the_whole_cache(kw, n):
     want, got = om.decode_step(tok[:, n].numpy()), gm.decode_full(tok[:, n].cuda().contiguous())
     for name in ("z1", "z2"):
         assert_logits_close(got[name], want[name], cfg.weight_dtype, name)
+
+
+@pytest.mark.parametrize("kw,B,S,past", [
+    (dict(), 1, 160, 0),                                        # one sequence's rows behind 159
+    (dict(), 1, 225, 0),                                        # the last group of the row tile (224 + 32 rows)
+    (dict(), 1, 226, 0),                                        # no room in the row tile: the step runs by itself
+    (dict(n_paths=3), 12, 30, 0),                               # 360 - 12 rows, two groups of ten sequences' three paths
+    (dict(n_paths=4, n_q_heads=4, n_kv_heads=2), 9, 40, 0),     # eight sequences to a group
+    (dict(n_layers=3), 20, 41, 0),                              # two paths of twenty sequences: the last layer on the wider chain
+    (dict(n_layers=3), 2, 400, 133),                            # behind a cached prefix
+    (dict(n_q_heads=4, n_kv_heads=2, head_dim=128, d_ff=704), 3, 300, 0),
+    (dict(n_q_heads=16, n_kv_heads=2), 1, 333, 0),              # sixteen query rows per KV head
+    (dict(d_model=328, d_ff=1032), 2, 150, 0),                  # ragged feature tiles
+    (dict(n_q_heads=2, n_kv_heads=2, d_ff=2048, n_layers=2), 1, 650, 0),
+])
+def test_boundary_step_whose_rows_ride_in_the_prompts_last_chunk(kw, B, S, past):
+    """The boundary evaluation, the cache it leaves and a step behind it against the oracle."""
+    cfg = cfg_of(**kw)
+    w = make_weights(cfg, seed=51, matrix_std=0.05)
+    tok = make_tokens(cfg, B, past + S + 1, seed=52)
+    om = oracle.OracleModel(cfg, w, B, past + S + 1)
+    gm = make_gpu_model(cfg, w, B, past + S + 1)
+    if past:
+        gm.prefill(tok[:, :past].cuda().contiguous())
+    om.prefill(tok[:, :past + S - 1].numpy(), want_logits=False)
+    want = om.decode_step(tok[:, past + S - 1].numpy())
+    got = gm.prefill_boundary(tok[:, past:past + S].cuda().contiguous())
+    for name in ("z1", "z2"):
+        assert_logits_close(got[name], want[name], cfg.weight_dtype, name)
+    k_dev, v_dev = gm.export_kv(B, past + S)
+    # two layers: one attention, whose queries and weights are bf16, lies before the deepest keys and values, up to 5e-3 as in the
+    # tests above; every further layer adds another one's
+    atol = 5e-3 * (cfg.n_layers - 1)
+    np.testing.assert_allclose(k_dev.float().numpy(), om.k_cache[:, :B, :past + S], rtol=2.0 ** -8, atol=atol)
+    np.testing.assert_allclose(v_dev.float().numpy(), om.v_cache[:, :B, :past + S], rtol=2.0 ** -8, atol=atol)
+    want, got = om.decode_step(tok[:, past + S].numpy()), gm.decode_full(tok[:, past + S].cuda().contiguous())
+    for name in ("z1", "z2"):
+        assert_logits_close(got[name], want[name], cfg.weight_dtype, name)
+    assert gm.sync_status() == (0, 0)
