@@ -56,8 +56,9 @@ def prefill_flops(cfg, B: int, n: int) -> float:
         per_layer += 3 * cfg.d_expert * cfg.d_model * (cfg.k_primary + cfg.n_shared_experts) + cfg.n_experts * cfg.d_model
     else:
         per_layer += 3 * cfg.d_ff * cfg.d_model
-    gemm = 2.0 * per_layer * cfg.n_layers * B * n
-    attn = 4.0 * cfg.q_dim * cfg.n_layers * B * (n * (n + 1) / 2.0)
+    layers = cfg.n_layers if cfg.is_moe else cfg.n_layers - 1  # dense models' last layer forms keys and values alone
+    gemm = 2.0 * (per_layer * layers + (0 if cfg.is_moe else 2 * cfg.kv_dim * cfg.d_model)) * B * n
+    attn = 4.0 * cfg.q_dim * layers * B * (n * (n + 1) / 2.0)
     return gemm + attn
 
 
