@@ -548,6 +548,13 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         }
         __syncwarp();
     };
+    // A segment's last stage is written by ordinary stores too -- zeros behind the last key, the new row, in the narrow form the
+    // warps' states -- and the next segment's pages then arrive in it by TMA, through the async proxy: every thread that wrote (each
+    // comes here) orders its accesses before those ahead of the barrier arrival that gives the stage back.  Without a next
+    // segment nothing arrives there any more.
+    auto hand_over = [&](int round) {
+        if (dealt(round + 1) < Sg) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    };
     for (int round = 0, sidx; (sidx = dealt(round)) < Sg; round++) {
         int item, nkeys, g, seg, nseg, ui, t0, t1;
         locate(sidx, item, nkeys, g, seg, nseg, ui, t0, t1);
@@ -825,6 +832,8 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                         }
                     }
                 }
+                // (the row's last stage may hold zeros and the new row: see hand_over)
+                if (t + 1 == t1) hand_over(round);
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar(s)) : "memory");
             }
@@ -1086,6 +1095,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 }
                 if (nseg > 1) __threadfence();
                 if (dealt(round + 1) < Sg) {  // the stage goes back to the producer
+                    hand_over(round);
                     consumer_sync();
                     if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(empty_bar((it - 1) % STAGES)) : "memory");
                 }

@@ -94,3 +94,24 @@ def test_merge_of_many_segments_is_the_same_bits_grouped_and_primary_only(kw, le
         kv.append(gm.kv_pool.clone())
     assert torch.equal(kv[0], kv[1])
     assert all(torch.equal(a, b) for a, b in zip(*z1))
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(head_dim=128, n_q_heads=16), dict(n_q_heads=32, n_kv_heads=4)])  # (the last: 16 query rows)
+def test_stages_that_segments_wrote_take_the_next_segments_pages(kw):
+    """Several segments per CTA, whose last stages hold zeros, the new row and (up to eight query rows) the warps' states when the
+    next segment's pages arrive in them: what the first sequences give is right, and twenty runs leave the same bits."""
+    cfg = cfg_of(**kw)
+    lens = [17 + (53 * i) % 650 for i in range(117)]
+    test_dealt_pairs_match_the_oracle_on_sampled_sequences(cfg, lens)
+    w = make_weights(cfg, seed=41, matrix_std=0.05)
+    k, v = make_synthetic_kv(cfg, len(lens), max(lens), seed=42)
+    tok = make_tokens(cfg, len(lens), 1, seed=43)[:, 0].cuda().contiguous()
+    gm = make_gpu_model(cfg, w, len(lens), max(lens) + 4)
+    gm.write_kv(k, v)
+    first = None
+    for _ in range(20):
+        gm.set_seq_lens(lens)
+        out = gm.decode_full(tok)
+        got = [out["z1"].clone(), out["z2"].clone(), gm.kv_pool.clone()]
+        first = first or got
+        assert all(torch.equal(a, b) for a, b in zip(first, got))
