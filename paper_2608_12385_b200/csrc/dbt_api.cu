@@ -1760,6 +1760,8 @@ RideRows ride_rows(const dbt_model *m, int B, int own) {
     RideRows r{};
     const int K = paths_of(m->cfg), spg = 32 / K, row0 = (own + 31) / 32 * 32, end = row0 + (B + spg - 1) / spg * 32;
     if (!m->prompt_attn_tc || m->cfg.n_layers < 2 || end > m->Rmax || (end + kPgM - 1) / kPgM != (own + kPgM - 1) / kPgM) return r;
+    if (K * B > row0) return r;  // ride_take_kernel moves them to rows 0 .. K*B - 1.  (Chunks of more than 128 rows never come here: up
+                                 // to 256 rows of their own leave room for 96 in the tile, and a step has at most 256)
     r.row0 = row0;
     r.spg = spg;
     r.K = K;

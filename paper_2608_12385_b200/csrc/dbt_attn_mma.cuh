@@ -71,7 +71,8 @@ struct AttnParams {
     int pack, cn, nbk;
     // Rows of a boundary step that ride behind a prompt chunk (ride.K > 0; K rows per sequence, path-major queries in Q): they see
     // `ahead` positions more than seq_len says, the chunk's, and their outputs go to their places in the chunk.  The launch
-    // starts beside the chunk's own attention (whose CTAs let it in behind their wait) and waits for that one at its end.
+    // starts beside the chunk's own attention and waits for that one at its end: it reads the Q|K|V kernel's queries, keys and
+    // values without a wait of its own, so both prompt attention kernels let it in behind theirs (PromptAttnParams::let_in_late).
     RideRows ride;
     int ahead;
     const int *plan;   // the step's precomputed work split (embed_fused_kernel), or nullptr
@@ -335,6 +336,7 @@ __global__ void __launch_bounds__(256) embed_fused_kernel(const int32_t *tokens,
 
 // Boundary step behind a chunk that its rows rode in: they leave for the decode kernels' places (path-major), with the last layer's
 // input g * S and sum(S^2) as embed_fused_kernel leaves them; one more block computes the step's attention work split.
+// (In place: the destinations, rows 0 .. K*B - 1, end before the first source, see ride_rows.)
 __global__ void __launch_bounds__(256) ride_take_kernel(RideRows ride, float *S, const float *__restrict__ g, int d, __nv_bfloat16 *Xb, size_t lo_off,
                                                         float *ss_out, int ss_ld, int ss_tiles, const int32_t *seq_len, int n_kv, int C0,
                                                         int *plan, int early) {

@@ -427,8 +427,9 @@ __global__ void __launch_bounds__((kPsWarps + 1) * 32, 1) attn_prompt_short_kern
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    pdl_launch_dependents();
+    if (!p.let_in_late) pdl_launch_dependents();
     pdl_wait();  // the chunk's Q rows and its K, V rows in the cache come from the kernel before
+    if (p.let_in_late) pdl_launch_dependents();
     const int len0 = ld_mut(p.seq_len + b);
     const int c0 = jb * PB, c_last = min(c0 + PB, p.cn) - 1;  // chunk positions of this block
     const int nkeys_max = len0 + c_last + 1;                  // keys visible to the block's last position
