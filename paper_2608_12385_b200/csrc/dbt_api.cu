@@ -1689,7 +1689,13 @@ dbt_status run_few(dbt_model *m, const char *tag, int B, const CUtensorMap *W0, 
     for (int s = 0; s < p.nseg; s++) bytes += (double)p.n_out[s] * p.K * 2 * (MODE == FEW_GATEUP ? 2 : 1);
     p.evict_first = m->evict_first ? 1 : 0;
     p.status = m->ws.status;
-    const int slots = kFewCtas * m->num_sms, grid = p.tiles < slots ? p.tiles : slots;
+    // Long tiles (128 KB of weights and more) are dealt so that all CTAs walk about equally many: in a last round of a few CTAs each
+    // streams at its own pace, a fraction of HBM's.  320 tiles of 885 KB (d 5120, F 27648) on 296 CTAs left 24 of them a second
+    // tile: 1230 us per step, 1164 on the split-K chain, 1140 on 160 CTAs; d 5120, F 17408 872 / 829 / 815; d 6144, F 16384
+    // 1003 / 993 / 961; 8B, four sequences of 2048 3208 / 3425 / 3136.  A shorter tile's successor is in the ring by then, and
+    // fewer CTAs have less in flight (d 2560: 448 us, dealt equally 457; d 3072 498 / 504; 1B, four sequences 700 / 705).
+    const int slots = kFewCtas * m->num_sms, rounds = tm * p.K >= 4096 ? (p.tiles + slots - 1) / slots : 1;
+    const int share = (p.tiles + rounds - 1) / rounds, grid = share < slots ? share : slots;
     const FewLayout lay = few_layout(2 << x, tm, p.K, p.tiles <= grid, p.tiles <= m->num_sms ? kFewSmemOne : kFewSmem);
     p.ring = lay.ring;
     p.x_resident = lay.resident;
