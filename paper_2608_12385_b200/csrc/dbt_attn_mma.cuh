@@ -485,6 +485,9 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
         const uint64_t pol = l2_evict_first_policy();
         bool ok = true;
         int it = 0;
+        // early: the ring is filled before the queries' loads go out.  (Asked of p.early at every stage instead, the deep form at d_h 64
+        // streamed 7 % slower: 16 sequences of 6000 722 us per step, 707 now.)
+        const int pause_at = p.early ? -1 : kAttPauseAt;
         for (int round = 0, sidx; ok && (sidx = dealt(round)) < Sg; round++) {
             int item, nkeys, g, seg, n, ui, t0, t1;
             locate(sidx, item, nkeys, g, seg, n, ui, t0, t1);
@@ -525,8 +528,7 @@ __global__ void __launch_bounds__(160, DEEP ? 1 : 2) attn_mma_kernel(const __gri
                 // at once instead, with the small loads issued first, was measured slower: the queries are ready
                 // 0.8 us sooner but the stream then runs 10 % slower; pausing after one, two, four or six stages
                 // gave 1.0446, 1.0384, 1.0420 and 1.0462 ms per step of the 1B model at batch 16.)
-                if (p.early) continue;  // (the ring was filled before the queries' loads went out)
-                if (it == kAttPauseAt || (it < kAttPauseAt && dealt(round + 1) >= Sg && t == t1 - 1)) asm volatile("bar.sync 2, 160;" ::: "memory");
+                if (it == pause_at || (it < pause_at && dealt(round + 1) >= Sg && t == t1 - 1)) asm volatile("bar.sync 2, 160;" ::: "memory");
             }
         }
         if (!ok && lane == 0) report(p.status, kStatusWaitExpired, 300);
