@@ -254,8 +254,8 @@ constexpr int kAttPlanInts = 3 * kAttMaxItems + 2;  // cum [items + 1] | nk [ite
 // where eight segments, one round of the merge's loads, still cover the pair.  One sequence of the 1B model (d_h 128, a ring of three)
 // with 2 / 3 / 4 stages: context 700 592 / 609 / 617 us per step, context 2048 636 / 613 / 625.  Rings of six stages (d_h 64)
 // want no longer ones: 2 and 3 / 4 and 6 stages, d 2048 at 700 positions 315 / 323 us and at 2048 323 / 328, d 512 with four
-// sequences of 700 225 / 238; nor does d 3072 at d_h 128, 476 / 493.  In the 16-row form, whose fold takes longer, both ways: 64 heads of
-// 64 764 / 777 (700 positions), 48 of 128 971 / 983 (700), 1002 / 997 (2048), two sequences 996 / 986.
+// sequences of 700 225 / 238; nor does d 3072 at d_h 128, 476 / 493.  In the 16-row form the same: 64 heads of 64 748 / 760 (700
+// positions), 763 / 764 (2048), 48 of 128 939 / 949 and 966 / 965.
 __device__ __forceinline__ int att_min_early(int stages) { return stages <= 2 * kAttGroup ? 2 : 3; }
 
 // A decode step's plan (one position per sequence), by one block of at least 256 threads: rows by falling length.

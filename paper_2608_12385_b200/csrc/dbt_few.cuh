@@ -103,8 +103,10 @@ inline FewLayout few_layout(int NR, int TM, int K, bool single, int smem) {
 }
 
 // TM: sixteens of weight rows per tile.  At eight rows a stage of them is as large as a stage of sixteen weight rows; two sixteens
-// share it where the contracted width is long and that leaves enough tiles for the SMs: 8B, four sequences of 32768 / 500 positions
-// 5704 / 3183 -> 5568 / 3100 us per step (at a width of 2048, four stages, it is slower: 1B 699 -> 710).
+// share it where the contracted width is long and that leaves enough tiles for the SMs.  One / two sixteens from 4096 elements on,
+// us per step of four sequences: 8B at 2048 positions 3330 / 3146, at 32768 5695 / 5525, d 4096 F 11008 881 / 863, d 5120 F 27648
+// 1305 / 1168, d 6144 F 16384 1060 / 983, d 8192 F 28672 1408 / 1309.  From 1024 elements on they would give 1 to 4 % more (1B 704 / 699,
+// d 3072 556 / 532, d 3584 700 / 675); before long tiles were dealt equally they cost 1.5 % there, and the line has not moved.
 template <int MODE, int NR, int TM>
 __global__ void __launch_bounds__(kFewThreads, 2)
 few_linear_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant__ CUtensorMap tmW1, const __grid_constant__ CUtensorMap tmW2,
